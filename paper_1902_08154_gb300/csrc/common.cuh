@@ -73,12 +73,38 @@ struct CtxView {
 int ctx_view(const struct ::qp_pt2_ctx* x, CtxView* v);
 int report(int code, const char* msg);
 
-// Bucket entries per coarse-filter record: a record with holes Q of I
-// (d = |Q|) is listed once in the shared bucket (d <= 2), once per hole
-// (d = 3) or once per pair of holes (d = 4).
+// Bucket entries per coarse-filter record with holes Q of I (d = |Q|), at
+// most: d = 1 the shared list and its hole's, d = 2 the shared list, two
+// holes' and the pair's, d = 3 three holes' and three pairs', d = 4 six pairs'.
 __host__ __device__ inline long long bucket_entries_per_record(int nel) {
-  return nel >= 4 ? 6 : (nel == 3 ? 3 : 1);
+  return nel >= 3 ? 6 : (nel == 2 ? 4 : 2);
 }
+
+// Bit masks of the cells that J ranked before I ban, per generator slot (see
+// prep_slot).  Words of one set: a bit per cell of a spin-up pair batch (ca),
+// a spin-down pair batch (cb) and an opposite-spin batch (cm).  A slot holds
+// the base set [ca | cb | cm], then per hole of I [same spin | opposite spin]
+// with stride hs.
+struct MaskDims {
+  int ca, cb, cm, hs;
+};
+__host__ __device__ inline MaskDims mask_dims(int norb, int na, int nb) {
+  const int va = norb - na, vb = norb - nb;
+  MaskDims m;
+  m.ca = (va * (va - 1) / 2 + 31) / 32;
+  m.cb = (vb * (vb - 1) / 2 + 31) / 32;
+  m.cm = (va * vb + 31) / 32;
+  m.hs = (m.ca > m.cb ? m.ca : m.cb) + m.cm;
+  return m;
+}
+__host__ __device__ inline int mask_words(int norb, int na, int nb) {  // even: 64-bit masks follow
+  const MaskDims m = mask_dims(norb, na, nb);
+  return (m.ca + m.cb + m.cm + (na + nb) * m.hs + 1) & ~1;
+}
+// 64-bit orbital masks per slot: rows banned in every pair batch [2][nint],
+// cells banned in every one-hole batch [2][nint], and per hole its rows
+// [2][nint] and one-hole cells [nint].
+__host__ __device__ inline int orb_mask_words(int nint, int nel) { return (4 + 3 * nel) * nint; }
 
 // Dynamic shared memory of the one-state batch kernel for mc cells: A_alpha
 // as a 96-bit integer per cell (a 64-bit low word and a 32-bit high word; the
@@ -90,12 +116,14 @@ __host__ __device__ inline size_t sweep_smem(int mc) {
 
 struct GenMeta;
 // Device bytes per generator slot of a wave: metadata, nd coarse-filter
-// records (words, nst coefficients, hole mask, particles, flag), bucket
-// offsets, ent_cap self-contained entries (20 bytes), the dead-batch bits and
-// the nper items' FP64 sums (2 per state).
-inline size_t wave_slot_bytes(size_t meta_bytes, int nel, int nbat, int nw, size_t nd, int nst, int nper) {
+// records (words, nst coefficients, hole mask, particles), bucket offsets,
+// ent_cap self-contained entries (20 bytes), the ban masks, the dead-batch
+// bits and the nper items' FP64 sums (2 per state).
+inline size_t wave_slot_bytes(size_t meta_bytes, int norb, int na, int nb, int nbat, size_t nd, int nst, int nper) {
+  const int nint = (norb - 1) / 64 + 1, nw = 2 * nint, nel = na + nb;
   const size_t ent_cap = nd * (size_t)bucket_entries_per_record(nel);
-  return meta_bytes + nd * (8 * (size_t)nw + 8 * (size_t)nst + 8 + 8 + 4) + 4 * (size_t)(nbat + 2) + 20 * ent_cap +
+  return meta_bytes + nd * (8 * (size_t)nw + 8 * (size_t)nst + 8 + 8) + 4 * (size_t)(nbat + 2) + 20 * ent_cap +
+         4 * (size_t)mask_words(norb, na, nb) + 8 * (size_t)orb_mask_words(nint, nel) +
          4 * (size_t)((nbat + 31) / 32) + 16 * (size_t)nper * (size_t)nst;
 }
 
@@ -166,8 +194,10 @@ struct SweepParams {
   double* r_coef;                 // [slots][ndet]
   uint64_t* r_hmask;              // [slots][ndet]  holes of I missing from J (occupied index bits)
   uint64_t* r_part;               // [slots][ndet]  up to 4 particle codes of J outside I, 16 bits each
-  uint32_t* r_flag;               // [slots][ndet]  bit 0: rank(J) < rank(I)
-  int* b_ofs;                     // [slots][nbat + 2]  bucket offsets (bucket nbat: J within degree 2)
+  int* b_ofs;                     // [slots][nbat + 2]  bucket offsets (bucket nbat: the shared list)
+  uint32_t* b_mask;               // [slots][mask_w]  cells banned by J ranked before I (MaskDims)
+  uint64_t* o_mask;               // [slots][orb_w]   rows and one-hole cells banned (orb_mask_words)
+  int mask_w, orb_w;
   // bucket entries, self-contained so that the batch kernel classifies a
   // bucket by streaming it: the record's hole mask and particle codes, and
   // its index with the rank flag (rank(J) < rank(I)) in bit 31

@@ -192,77 +192,107 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   if (batch_blocks_per_sm_packed(nint, smem) < 1) return nfail(QP_ENOTSUP, "batch accumulator exceeds shared memory");
   int nsm = 0;
   NTRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const int grid = nsm;  // one CTA per SM keeps the selection buffers small
   const size_t nd = (size_t)ndet;
-  const int64_t cap = k > 0 ? k + max_cells : 1;
-  const size_t maxc = (size_t)grid * (size_t)(k > 0 ? k : 1);
-  size_t tmp1 = 0, tmp2 = 0;
-  cub::DeviceRadixSort::SortPairs(nullptr, tmp1, (unsigned long long*)nullptr, (unsigned long long*)nullptr,
-                                  (int32_t*)nullptr, (int32_t*)nullptr, (int)ndet, 0, 64, st);
-  cub::DeviceRadixSort::SortPairs(nullptr, tmp2, (unsigned long long*)nullptr, (unsigned long long*)nullptr,
-                                  (int32_t*)nullptr, (int32_t*)nullptr, (int)maxc, 0, 64, st);
-  Carve cv{base};
-  double* d_J = cv.take<double>((size_t)norb * norb);
-  double* d_K = cv.take<double>((size_t)norb * norb);
-  unsigned long long* hkey = cv.take<unsigned long long>(nd);
-  unsigned long long* hkey2 = cv.take<unsigned long long>(nd);
-  unsigned long long* rkey = cv.take<unsigned long long>(nd);
-  unsigned long long* rkey2 = cv.take<unsigned long long>(nd);
-  int32_t* hidx = cv.take<int32_t>(nd);
-  int32_t* hidx2 = cv.take<int32_t>(nd);
-  int32_t* order = cv.take<int32_t>(nd);
-  int32_t* rank_of = cv.take<int32_t>(nd);
-  unsigned char* cub_tmp = cv.take<unsigned char>(tmp1 > tmp2 ? tmp1 : tmp2);
-  double* eps = cv.take<double>(nd);
-  double* s2 = cv.take<double>(nd);
-  unsigned long long* na = cv.take<unsigned long long>(nd);
-  unsigned long long* ncon = cv.take<unsigned long long>(nd);
-  unsigned long long* acc = cv.take<unsigned long long>(9);
-  DevResult* dres = cv.take<DevResult>(1);
-  int* queues = cv.take<int>(nd + 1);
-  double* tk_e = cv.take<double>((size_t)cap * grid);
-  double* tk_a = cv.take<double>((size_t)cap * grid);
-  uint64_t* tk_key = cv.take<uint64_t>((size_t)cap * grid * nw);
-  int* tk_cnt = cv.take<int>(grid);
-  unsigned long long* tk_tau = cv.take<unsigned long long>(grid);
-  unsigned long long* d_hmax = cv.take<unsigned long long>(2);
-  unsigned int* sel_hist = cv.take<unsigned int>(kSelBins);
-  double* cand_e = cv.take<double>(maxc);
-  double* cand_a = cv.take<double>(maxc);
-  uint64_t* cand_key = cv.take<uint64_t>(maxc * nw);
-  unsigned long long* skey = cv.take<unsigned long long>(maxc);
-  unsigned long long* skey2 = cv.take<unsigned long long>(maxc);
-  int32_t* perm = cv.take<int32_t>(maxc);
-  int32_t* perm2 = cv.take<int32_t>(maxc);
-  if (!cv.ok)
-    return nfail(QP_EINVAL, "ndet or k too large for the 64 MiB static scratch of qp_pt2_eval_noalloc");
-  const int64_t ent_per = bucket_entries_per_record(nel);
-  const int64_t ent_cap = (int64_t)nd * ent_per;
+  const int64_t cap = k > 0 ? k + max_cells : 1, ngen = ndet;
+  const int64_t ent_cap = (int64_t)nd * bucket_entries_per_record(nel);
   const size_t dwords = (size_t)(nbat + 31) / 32;
   const int nper = nbat;
-  const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), nel, nbat, nw, nd, 1, nper);
-  // each of the 12 per-slot arrays carved below may start with up to 255
-  // bytes of alignment padding: keep 12 x 256 bytes aside for them
-  const size_t left = kScratchBytes > cv.off + 12 * 256 ? kScratchBytes - cv.off - 12 * 256 : 0;
-  int64_t W = (int64_t)(left / per_slot);
-  if (W < 1)
-    return nfail(QP_EINVAL, "ndet too large for the 64 MiB static scratch of qp_pt2_eval_noalloc");
-  const int64_t ngen = ndet;
-  if (W > ngen) W = ngen;
-  const int64_t nwaves = (ngen + W - 1) / W;
-  const size_t wsl = (size_t)W;
-  GenMeta* meta = cv.take<GenMeta>(wsl);
-  uint64_t* r_words = cv.take<uint64_t>(nd * nw * wsl);
-  double* r_coef = cv.take<double>(nd * wsl);
-  uint64_t* r_hmask = cv.take<uint64_t>(nd * wsl);
-  uint64_t* r_part = cv.take<uint64_t>(nd * wsl);
-  uint32_t* r_flag = cv.take<uint32_t>(nd * wsl);
-  int* b_ofs = cv.take<int>((size_t)(nbat + 2) * wsl);
-  ulonglong2* e_hp = cv.take<ulonglong2>((size_t)ent_cap * wsl);
-  uint32_t* e_rec = cv.take<uint32_t>((size_t)ent_cap * wsl);
-  double* it_sum = cv.take<double>((size_t)2 * nper * wsl);
-  uint32_t* b_dead = cv.take<uint32_t>(dwords * wsl);
-  if (!cv.ok) return nfail(QP_EINVAL, "ndet too large for the 64 MiB static scratch of qp_pt2_eval_noalloc");
+  size_t maxc = 0, tmp1 = 0, tmp2 = 0;
+  int64_t W = 0, nwaves = 0;
+  double *d_J = nullptr, *d_K = nullptr, *eps = nullptr, *s2 = nullptr, *tk_e = nullptr;
+  double *tk_a = nullptr, *cand_e = nullptr, *cand_a = nullptr, *r_coef = nullptr;
+  double *it_sum = nullptr;
+  unsigned long long *hkey = nullptr, *hkey2 = nullptr, *rkey = nullptr, *rkey2 = nullptr, *na = nullptr;
+  unsigned long long *ncon = nullptr, *acc = nullptr, *tk_tau = nullptr, *d_hmax = nullptr, *skey = nullptr;
+  unsigned long long *skey2 = nullptr;
+  int32_t *hidx = nullptr, *hidx2 = nullptr, *order = nullptr, *rank_of = nullptr, *perm = nullptr, *perm2 = nullptr;
+  unsigned char *cub_tmp = nullptr, *cub_tmp2 = nullptr;
+  DevResult *dres = nullptr;
+  int *queues = nullptr, *tk_cnt = nullptr, *b_ofs = nullptr;
+  uint64_t *tk_key = nullptr, *cand_key = nullptr, *r_words = nullptr, *r_hmask = nullptr;
+  uint64_t *r_part = nullptr, *o_mask = nullptr;
+  unsigned int *sel_hist = nullptr;
+  GenMeta *meta = nullptr;
+  uint32_t *b_mask = nullptr, *e_rec = nullptr, *b_dead = nullptr;
+  ulonglong2 *e_hp = nullptr;
+  // Lays the arrays out for `grid` sweep CTAs; 0, or which size does not fit.
+  auto layout = [&](int grid) -> int {
+    maxc = (size_t)grid * (size_t)(k > 0 ? k : 1);
+    tmp1 = tmp2 = 0;
+    cub::DeviceRadixSort::SortPairs(nullptr, tmp1, (unsigned long long*)nullptr, (unsigned long long*)nullptr,
+                                    (int32_t*)nullptr, (int32_t*)nullptr, (int)ndet, 0, 64, st);
+    cub::DeviceRadixSort::SortPairs(nullptr, tmp2, (unsigned long long*)nullptr, (unsigned long long*)nullptr,
+                                    (int32_t*)nullptr, (int32_t*)nullptr, (int)maxc, 0, 64, st);
+    // kept for the whole call
+    Carve cv{base};
+    d_J = cv.take<double>((size_t)norb * norb);
+    d_K = cv.take<double>((size_t)norb * norb);
+    order = cv.take<int32_t>(nd);
+    rank_of = cv.take<int32_t>(nd);
+    eps = cv.take<double>(nd);
+    s2 = cv.take<double>(nd);
+    na = cv.take<unsigned long long>(nd);
+    ncon = cv.take<unsigned long long>(nd);
+    acc = cv.take<unsigned long long>(9);
+    dres = cv.take<DevResult>(1);
+    queues = cv.take<int>(nd + 1);
+    tk_e = cv.take<double>((size_t)cap * grid);
+    tk_a = cv.take<double>((size_t)cap * grid);
+    tk_key = cv.take<uint64_t>((size_t)cap * grid * nw);
+    tk_cnt = cv.take<int>(grid);
+    tk_tau = cv.take<unsigned long long>(grid);
+    d_hmax = cv.take<unsigned long long>(2);
+    sel_hist = cv.take<unsigned int>(kSelBins);
+    // the validation's arrays, the waves' and the selection's share the rest,
+    // one phase after another on the stream
+    Carve c1 = cv, c3 = cv;
+    hkey = c1.take<unsigned long long>(nd);
+    hkey2 = c1.take<unsigned long long>(nd);
+    rkey = c1.take<unsigned long long>(nd);
+    rkey2 = c1.take<unsigned long long>(nd);
+    hidx = c1.take<int32_t>(nd);
+    hidx2 = c1.take<int32_t>(nd);
+    cub_tmp = c1.take<unsigned char>(tmp1);
+    cand_e = c3.take<double>(maxc);
+    cand_a = c3.take<double>(maxc);
+    cand_key = c3.take<uint64_t>(maxc * nw);
+    skey = c3.take<unsigned long long>(maxc);
+    skey2 = c3.take<unsigned long long>(maxc);
+    perm = c3.take<int32_t>(maxc);
+    perm2 = c3.take<int32_t>(maxc);
+    cub_tmp2 = c3.take<unsigned char>(tmp2);
+    if (!cv.ok || !c1.ok || !c3.ok) return 1;
+    const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), norb, n_alpha, n_beta, nbat, nd, 1, nper);
+    // each of the 13 per-slot arrays carved below may start with up to 255
+    // bytes of alignment padding: keep 13 x 256 bytes aside for them
+    const size_t left = kScratchBytes > cv.off + 13 * 256 ? kScratchBytes - cv.off - 13 * 256 : 0;
+    W = (int64_t)(left / per_slot);
+    if (W < 1) return 2;
+    if (W > ngen) W = ngen;
+    nwaves = (ngen + W - 1) / W;
+    const size_t wsl = (size_t)W;
+    meta = cv.take<GenMeta>(wsl);
+    r_words = cv.take<uint64_t>(nd * nw * wsl);
+    r_coef = cv.take<double>(nd * wsl);
+    r_hmask = cv.take<uint64_t>(nd * wsl);
+    r_part = cv.take<uint64_t>(nd * wsl);
+    b_mask = cv.take<uint32_t>((size_t)mask_words(norb, n_alpha, n_beta) * wsl);
+    o_mask = cv.take<uint64_t>((size_t)orb_mask_words(nint, nel) * wsl);
+    b_ofs = cv.take<int>((size_t)(nbat + 2) * wsl);
+    e_hp = cv.take<ulonglong2>((size_t)ent_cap * wsl);
+    e_rec = cv.take<uint32_t>((size_t)ent_cap * wsl);
+    it_sum = cv.take<double>((size_t)2 * nper * wsl);
+    b_dead = cv.take<uint32_t>(dwords * wsl);
+    return cv.ok ? 0 : 2;
+  };
+  // one CTA per SM keeps the selection buffers small; one CTA less where a
+  // generator slot would not fit otherwise (with k > 0 its buffer is larger
+  // than the slot's ban masks)
+  int grid = nsm, lay = layout(grid);
+  if (lay && grid > 1) lay = layout(--grid);
+  if (lay == 1)
+    return nfail(QP_EINVAL, "ndet or k too large for the 64 MiB static scratch of qp_pt2_eval_noalloc");
+  if (lay) return nfail(QP_EINVAL, "ndet too large for the 64 MiB static scratch of qp_pt2_eval_noalloc");
 
   // ---- clear what must start at zero; integral tables; validation ----
   // accumulator words: 0, 1 digest, 2 min |D|, 3 tiny, 4 threshold, 6 error
@@ -336,7 +366,10 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   p.r_coef = r_coef;
   p.r_hmask = r_hmask;
   p.r_part = r_part;
-  p.r_flag = r_flag;
+  p.b_mask = b_mask;
+  p.o_mask = o_mask;
+  p.mask_w = mask_words(norb, n_alpha, n_beta);
+  p.orb_w = orb_mask_words(nint, nel);
   p.b_ofs = b_ofs;
   p.b_dead = b_dead;
   p.ent_cap = ent_cap;
@@ -387,7 +420,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
       for (int pass = 0; pass <= nw; pass++) {
         const int word = (pass < nw) ? (nw - 1 - pass) : nw;
         sortkey_kernel<<<sb, 256, 0, st>>>(ncand, nint, word, cand_e, cand_key, pa, skey);
-        NTRY_Q(cub::DeviceRadixSort::SortPairs(cub_tmp, tmp2, skey, skey2, pa, pb, ncand, 0, 64, st));
+        NTRY_Q(cub::DeviceRadixSort::SortPairs(cub_tmp2, tmp2, skey, skey2, pa, pb, ncand, 0, 64, st));
         int32_t* t = pa;
         pa = pb;
         pb = t;

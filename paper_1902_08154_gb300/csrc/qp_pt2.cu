@@ -327,7 +327,7 @@ struct qp_pt2_ctx {
   // workspace
   Buf in_dets, in_coefs, hkey, hkey2, hidx, hidx2, rkey, rkey2, order, rank_of, cub_tmp;
   Buf eps, s2, na, ncon, acc, res;
-  Buf meta, r_words, r_coef, r_hmask, r_part, r_flag, b_ofs, e_hp, e_rec, b_dead, queues, it_sum;
+  Buf meta, r_words, r_coef, r_hmask, r_part, b_mask, o_mask, b_ofs, e_hp, e_rec, b_dead, queues, it_sum;
   Buf tk_e, tk_a, tk_key, tk_cnt, tk_tau, sel_hist, gen_list, gen_out, st_cmax;
   Buf cand_e, cand_a, cand_key, skey, skey2, perm, perm2, cub_tmp2;
   Buf out_sel, out_e, out_num, out_eps, out_na, out_ncon, out_rank;
@@ -531,7 +531,7 @@ extern "C" void qp_pt2_destroy(qp_pt2_ctx* x) {
   cudaFree(x->d_hmax);
   Buf* all[] = {&x->in_dets, &x->in_coefs, &x->hkey, &x->hkey2, &x->hidx, &x->hidx2, &x->rkey, &x->rkey2,
                 &x->order, &x->rank_of, &x->cub_tmp, &x->eps, &x->s2, &x->na, &x->ncon, &x->acc,
-                &x->res, &x->meta, &x->r_words, &x->r_coef, &x->r_hmask, &x->r_part, &x->r_flag,
+                &x->res, &x->meta, &x->r_words, &x->r_coef, &x->r_hmask, &x->r_part, &x->b_mask, &x->o_mask,
                 &x->b_ofs, &x->e_hp, &x->e_rec, &x->it_sum, &x->b_dead, &x->queues, &x->tk_e, &x->tk_a, &x->tk_key, &x->tk_cnt, &x->tk_tau, &x->sel_hist, &x->gen_list, &x->gen_out, &x->cand_e, &x->cand_a, &x->cand_key, &x->skey,
                 &x->skey2, &x->perm, &x->perm2, &x->cub_tmp2, &x->out_sel, &x->out_e, &x->out_num,
                 &x->out_eps, &x->out_na, &x->out_ncon, &x->out_rank, &x->g_dh, &x->g_deri, &x->g_wF, &x->g_wH};
@@ -781,7 +781,7 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   const int64_t ent_cap = (int64_t)nd * ent_per;
   const size_t dwords = (size_t)(x->nbat + 31) / 32;
   const int nper = x->nbat + (x->ntile - 1) * x->nalpha * x->nbeta;
-  const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), x->nel, x->nbat, nw, nd, nsts, nper);
+  const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), x->norb, x->nalpha, x->nbeta, x->nbat, nd, nsts, nper);
   int64_t W = (int64_t)(kWaveBudget / per_slot);
   if (W < 1) W = 1;
   if (W > ngen) W = ngen > 0 ? ngen : 1;
@@ -791,7 +791,8 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
       (rc = x->ncon.grow(8 * nd)) || (rc = x->meta.grow(sizeof(GenMeta) * ws)) ||
       (rc = x->r_words.grow(8 * nd * nw * ws)) || (rc = x->r_coef.grow(8 * nd * ws * nsts)) ||
       (rc = x->r_hmask.grow(8 * nd * ws)) || (rc = x->r_part.grow(8 * nd * ws)) ||
-      (rc = x->r_flag.grow(4 * nd * ws)) || (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * ws)) ||
+      (rc = x->b_mask.grow(4 * (size_t)mask_words(x->norb, x->nalpha, x->nbeta) * ws)) ||
+      (rc = x->o_mask.grow(8 * (size_t)orb_mask_words(nint, x->nel) * ws)) || (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * ws)) ||
       (rc = x->e_hp.grow(16 * (size_t)ent_cap * ws)) ||
       (rc = x->e_rec.grow(4 * (size_t)ent_cap * ws)) || (rc = x->it_sum.grow(16 * (size_t)nper * nsts * ws)) ||
       (rc = x->b_dead.grow(4 * dwords * ws)) || (rc = x->queues.grow(4 * (size_t)(nwaves + 1))) ||
@@ -855,7 +856,10 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   p.r_coef = x->r_coef.as<double>();
   p.r_hmask = x->r_hmask.as<uint64_t>();
   p.r_part = x->r_part.as<uint64_t>();
-  p.r_flag = x->r_flag.as<uint32_t>();
+  p.b_mask = x->b_mask.as<uint32_t>();
+  p.o_mask = x->o_mask.as<uint64_t>();
+  p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);
+  p.orb_w = orb_mask_words(x->nint, x->nel);
   p.b_ofs = x->b_ofs.as<int>();
   p.b_dead = x->b_dead.as<uint32_t>();
   p.ent_cap = ent_cap;
@@ -1183,7 +1187,7 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   const int64_t ent_cap = (int64_t)nd * ent_per;
   const size_t dwords = (size_t)(x->nbat + 31) / 32;
   const int nper = x->nbat + (x->ntile - 1) * x->nalpha * x->nbeta;
-  const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), x->nel, x->nbat, nw, nd, 1, nper);
+  const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), x->norb, x->nalpha, x->nbeta, x->nbat, nd, 1, nper);
   int64_t W = (int64_t)(kWaveBudget / per_slot);
   if (W < 1) W = 1;
   if (W > ngen) W = ngen > 0 ? ngen : 1;
@@ -1193,7 +1197,8 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
       (rc = x->ncon.grow(8 * nd)) || (rc = x->meta.grow(sizeof(GenMeta) * wsl)) ||
       (rc = x->r_words.grow(8 * nd * nw * wsl)) || (rc = x->r_coef.grow(8 * nd * wsl)) ||
       (rc = x->r_hmask.grow(8 * nd * wsl)) || (rc = x->r_part.grow(8 * nd * wsl)) ||
-      (rc = x->r_flag.grow(4 * nd * wsl)) || (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * wsl)) ||
+      (rc = x->b_mask.grow(4 * (size_t)mask_words(x->norb, x->nalpha, x->nbeta) * wsl)) ||
+      (rc = x->o_mask.grow(8 * (size_t)orb_mask_words(nint, x->nel) * wsl)) || (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * wsl)) ||
       (rc = x->e_hp.grow(16 * (size_t)ent_cap * wsl)) ||
       (rc = x->e_rec.grow(4 * (size_t)ent_cap * wsl)) || (rc = x->it_sum.grow(16 * (size_t)nper * wsl)) ||
       (rc = x->b_dead.grow(4 * dwords * wsl)) ||
@@ -1252,7 +1257,10 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   p.r_coef = x->r_coef.as<double>();
   p.r_hmask = x->r_hmask.as<uint64_t>();
   p.r_part = x->r_part.as<uint64_t>();
-  p.r_flag = x->r_flag.as<uint32_t>();
+  p.b_mask = x->b_mask.as<uint32_t>();
+  p.o_mask = x->o_mask.as<uint64_t>();
+  p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);
+  p.orb_w = orb_mask_words(x->nint, x->nel);
   p.b_ofs = x->b_ofs.as<int>();
   p.b_dead = x->b_dead.as<uint32_t>();
   p.ent_cap = ent_cap;
@@ -1418,7 +1426,7 @@ struct qp_pt2_batch {
 // Device bytes of one generator slot of instance b's waves.
 static size_t inst_slot_bytes(const BatchInst& b) {
   const qp_pt2_ctx* x = b.x;
-  return wave_slot_bytes(sizeof(GenMeta), x->nel, x->nbat, 2 * x->nint, (size_t)b.ndet, 1, b.nper);
+  return wave_slot_bytes(sizeof(GenMeta), x->norb, x->nalpha, x->nbeta, x->nbat, (size_t)b.ndet, 1, b.nper);
 }
 
 // Workspaces of instance b: W slots per wave (W_fixed > 0) or as many as
@@ -1461,7 +1469,8 @@ static int plan_instance(BatchInst& b, size_t wave_budget, int64_t W_fixed, bool
   if (!pooled &&
       ((rc = x->meta.grow(sizeof(GenMeta) * ws)) || (rc = x->r_words.grow(8 * nd * nw * ws)) ||
       (rc = x->r_coef.grow(8 * nd * ws)) || (rc = x->r_hmask.grow(8 * nd * ws)) ||
-      (rc = x->r_part.grow(8 * nd * ws)) || (rc = x->r_flag.grow(4 * nd * ws)) ||
+      (rc = x->r_part.grow(8 * nd * ws)) || (rc = x->b_mask.grow(4 * (size_t)mask_words(x->norb, x->nalpha, x->nbeta) * ws)) ||
+      (rc = x->o_mask.grow(8 * (size_t)orb_mask_words(nint, x->nel) * ws)) ||
       (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * ws)) || (rc = x->e_hp.grow(16 * (size_t)b.ent_cap * ws)) ||
       (rc = x->e_rec.grow(4 * (size_t)b.ent_cap * ws)) ||
       (rc = x->it_sum.grow(16 * (size_t)nper * ws)) || (rc = x->b_dead.grow(4 * dwords * ws))))
@@ -1528,7 +1537,10 @@ static void make_params(BatchInst& b) {
   p.r_coef = x->r_coef.as<double>();
   p.r_hmask = x->r_hmask.as<uint64_t>();
   p.r_part = x->r_part.as<uint64_t>();
-  p.r_flag = x->r_flag.as<uint32_t>();
+  p.b_mask = x->b_mask.as<uint32_t>();
+  p.o_mask = x->o_mask.as<uint64_t>();
+  p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);
+  p.orb_w = orb_mask_words(x->nint, x->nel);
   p.b_ofs = x->b_ofs.as<int>();
   p.b_dead = x->b_dead.as<uint32_t>();
   p.ent_cap = b.ent_cap;
@@ -1700,7 +1712,7 @@ static int plan_fused(qp_pt2_batch* B, const qp_pt2_batch_options& o, size_t wav
     for (int i : G.members) {
       BatchInst& b = B->inst[i];
       b.grid = G.grid;
-      const size_t per = inst_slot_bytes(b) + 12 * 256;  // a slot and the alignment of its arrays
+      const size_t per = inst_slot_bytes(b) + 13 * 256;  // a slot and the alignment of its arrays
       int64_t start = 0;
       while (start < b.ngen) {
         int64_t fit = (int64_t)((budget > used ? budget - used : 0) / per);
@@ -1760,7 +1772,8 @@ static int plan_fused(qp_pt2_batch* B, const qp_pt2_batch_options& o, size_t wav
       p.r_coef = reinterpret_cast<double*>(take(8 * nd * ws));
       p.r_hmask = reinterpret_cast<uint64_t*>(take(8 * nd * ws));
       p.r_part = reinterpret_cast<uint64_t*>(take(8 * nd * ws));
-      p.r_flag = reinterpret_cast<uint32_t*>(take(4 * nd * ws));
+      p.b_mask = reinterpret_cast<uint32_t*>(take(4 * (size_t)p.mask_w * ws));
+      p.o_mask = reinterpret_cast<uint64_t*>(take(8 * (size_t)p.orb_w * ws));
       p.b_ofs = reinterpret_cast<int*>(take(4 * (size_t)(x->nbat + 2) * ws));
       p.e_hp = reinterpret_cast<ulonglong2*>(take(16 * (size_t)b.ent_cap * ws));
       p.e_rec = reinterpret_cast<uint32_t*>(take(4 * (size_t)b.ent_cap * ws));

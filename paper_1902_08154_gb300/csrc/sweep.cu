@@ -62,8 +62,18 @@ int batch_multi_blocks_per_sm_mixed(int nint, size_t smem);
 cudaError_t launch_wave_multi(int nint, int mixed, const MultiWave& m, const MultiWaveInline& mi, int total_slots,
                               int grid, size_t smem, cudaStream_t st) {
   if (total_slots <= 0) return cudaSuccess;
-  if (nint == 1) prep_multi_kernel<1><<<total_slots, kThreads, 0, st>>>(m);
-  else prep_multi_kernel<2><<<total_slots, kThreads, 0, st>>>(m);
+  size_t ps = 0;
+  for (int i = 0; i < mi.n; i++) {
+    const size_t b = 4 * (size_t)mi.ps[i].mask_w + 8 * (size_t)mi.ps[i].orb_w;
+    ps = b > ps ? b : ps;
+  }
+  if (nint == 1) {
+    cudaFuncSetAttribute(prep_multi_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps);
+    prep_multi_kernel<1><<<total_slots, kThreads, ps, st>>>(m);
+  } else {
+    cudaFuncSetAttribute(prep_multi_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps);
+    prep_multi_kernel<2><<<total_slots, kThreads, ps, st>>>(m);
+  }
   if (mixed) return launch_wave_multi_mixed(nint, mi, total_slots, grid, smem, st);
   return multi_wave_launch<double>(nint, mi, total_slots, grid, smem, st);
 }
@@ -96,9 +106,18 @@ cudaError_t launch_grad_gen(int nint, const SweepParams& p, int ngen, cudaStream
 cudaError_t launch_batch_mixed(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st);
 int batch_blocks_per_sm_mixed(int nint, size_t smem);
 
+// Dynamic shared memory of the prep kernel: a slot's ban masks.
+static size_t prep_smem(const SweepParams& p) { return 4 * (size_t)p.mask_w + 8 * (size_t)p.orb_w; }
+
 cudaError_t launch_prep(int nint, const SweepParams& p, int slots, cudaStream_t st) {
-  if (nint == 1) prep_kernel<1><<<slots, kThreads, 0, st>>>(p);
-  else prep_kernel<2><<<slots, kThreads, 0, st>>>(p);
+  const size_t smem = prep_smem(p);
+  if (nint == 1) {
+    cudaFuncSetAttribute(prep_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    prep_kernel<1><<<slots, kThreads, smem, st>>>(p);
+  } else {
+    cudaFuncSetAttribute(prep_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    prep_kernel<2><<<slots, kThreads, smem, st>>>(p);
+  }
   return cudaGetLastError();
 }
 
