@@ -132,10 +132,10 @@ struct GenMeta {
   uint64_t I[4];            // generator determinant (2*NINT words used)
   int g;                    // rank of the generator (-1: empty slot)
   int nrec;                 // coarse-filter records
-  double hii;               // <I|H|I>
+  long long hii;            // <I|H|I>, fixed point (den_scale in sweep_impl.cuh)
   double cI;                // c_I
   int occ[kMaxElec];        // spin-orbital codes s*norb+q of I, ordered
-  double F[2][kMaxOrb];     // Fock diagonal of I
+  long long F[2][kMaxOrb];  // Fock diagonal of I, fixed point
 };
 
 struct SweepParams {
@@ -166,6 +166,7 @@ struct SweepParams {
   int mixed;              // 1: numerator gathers and products in FP32
   const double* Jm;       // [norb*norb] (pp|qq)
   const double* Km;       // [norb*norb] (pq|qp)
+  long long *Ji, *Wi;     // [norb*norb] Jm and Jm - Km in fixed point (written by the prep kernel)
   double e0;
   int shard_index, shard_count;   // generators of rank shard_index + t*shard_count
   const int32_t* gen_list;        // if set: the generator of slot t has rank gen_list[t]

@@ -207,6 +207,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   unsigned long long *skey2 = nullptr;
   int32_t *hidx = nullptr, *hidx2 = nullptr, *order = nullptr, *rank_of = nullptr, *perm = nullptr, *perm2 = nullptr;
   unsigned char *cub_tmp = nullptr, *cub_tmp2 = nullptr;
+  long long *den_tab = nullptr;
   DevResult *dres = nullptr;
   int *queues = nullptr, *tk_cnt = nullptr, *b_ofs = nullptr;
   uint64_t *tk_key = nullptr, *cand_key = nullptr, *r_words = nullptr, *r_hmask = nullptr;
@@ -227,6 +228,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     Carve cv{base};
     d_J = cv.take<double>((size_t)norb * norb);
     d_K = cv.take<double>((size_t)norb * norb);
+    den_tab = cv.take<long long>(2 * (size_t)norb * norb);
     order = cv.take<int32_t>(nd);
     rank_of = cv.take<int32_t>(nd);
     eps = cv.take<double>(nd);
@@ -285,11 +287,11 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     b_dead = cv.take<uint32_t>(dwords * wsl);
     return cv.ok ? 0 : 2;
   };
-  // one CTA per SM keeps the selection buffers small; one CTA less where a
-  // generator slot would not fit otherwise (with k > 0 its buffer is larger
-  // than the slot's ban masks)
+  // one CTA per SM keeps the selection buffers small; a few CTAs less where a
+  // generator slot would not fit otherwise (with k > 0 the buffer of one or
+  // two CTAs is larger than the ban masks and denominator tables)
   int grid = nsm, lay = layout(grid);
-  if (lay && grid > 1) lay = layout(--grid);
+  for (int i = 0; i < 3 && lay && grid > 1; i++) lay = layout(--grid);
   if (lay == 1)
     return nfail(QP_EINVAL, "ndet or k too large for the 64 MiB static scratch of qp_pt2_eval_noalloc");
   if (lay) return nfail(QP_EINVAL, "ndet too large for the 64 MiB static scratch of qp_pt2_eval_noalloc");
@@ -358,6 +360,8 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   p.eri = eri;
   p.Jm = d_J;
   p.Km = d_K;
+  p.Ji = den_tab;
+  p.Wi = den_tab + (size_t)norb * norb;
   p.e0 = e0;
   p.shard_index = 0;
   p.shard_count = 1;

@@ -327,7 +327,7 @@ struct qp_pt2_ctx {
   // workspace
   Buf in_dets, in_coefs, hkey, hkey2, hidx, hidx2, rkey, rkey2, order, rank_of, cub_tmp;
   Buf eps, s2, na, ncon, acc, res;
-  Buf meta, r_words, r_coef, r_hmask, r_part, b_mask, o_mask, b_ofs, e_hp, e_rec, b_dead, queues, it_sum;
+  Buf den_tab, meta, r_words, r_coef, r_hmask, r_part, b_mask, o_mask, b_ofs, e_hp, e_rec, b_dead, queues, it_sum;
   Buf tk_e, tk_a, tk_key, tk_cnt, tk_tau, sel_hist, gen_list, gen_out, st_cmax;
   Buf cand_e, cand_a, cand_key, skey, skey2, perm, perm2, cub_tmp2;
   Buf out_sel, out_e, out_num, out_eps, out_na, out_ncon, out_rank;
@@ -531,7 +531,7 @@ extern "C" void qp_pt2_destroy(qp_pt2_ctx* x) {
   cudaFree(x->d_hmax);
   Buf* all[] = {&x->in_dets, &x->in_coefs, &x->hkey, &x->hkey2, &x->hidx, &x->hidx2, &x->rkey, &x->rkey2,
                 &x->order, &x->rank_of, &x->cub_tmp, &x->eps, &x->s2, &x->na, &x->ncon, &x->acc,
-                &x->res, &x->meta, &x->r_words, &x->r_coef, &x->r_hmask, &x->r_part, &x->b_mask, &x->o_mask,
+                &x->res, &x->meta, &x->r_words, &x->r_coef, &x->r_hmask, &x->den_tab, &x->r_part, &x->b_mask, &x->o_mask,
                 &x->b_ofs, &x->e_hp, &x->e_rec, &x->it_sum, &x->b_dead, &x->queues, &x->tk_e, &x->tk_a, &x->tk_key, &x->tk_cnt, &x->tk_tau, &x->sel_hist, &x->gen_list, &x->gen_out, &x->cand_e, &x->cand_a, &x->cand_key, &x->skey,
                 &x->skey2, &x->perm, &x->perm2, &x->cub_tmp2, &x->out_sel, &x->out_e, &x->out_num,
                 &x->out_eps, &x->out_na, &x->out_ncon, &x->out_rank, &x->g_dh, &x->g_deri, &x->g_wF, &x->g_wH};
@@ -798,7 +798,8 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
       (rc = x->b_dead.grow(4 * dwords * ws)) || (rc = x->queues.grow(4 * (size_t)(nwaves + 1))) ||
       (rc = x->tk_e.grow(8 * (size_t)cap * grid)) || (rc = x->tk_a.grow(8 * (size_t)cap * grid)) ||
       (rc = x->tk_key.grow(8 * (size_t)cap * grid * nw)) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
-      (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->res.grow(sizeof(DevResult) * nsts)) ||
+      (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
+      (rc = x->res.grow(sizeof(DevResult) * nsts)) ||
       (rc = x->sel_hist.grow(4 * (size_t)kSelBins)))
     return rc;
   CUDA_TRY(cudaMemsetAsync(x->sel_hist.p, 0, 4 * (size_t)kSelBins, st));
@@ -856,6 +857,8 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   p.r_coef = x->r_coef.as<double>();
   p.r_hmask = x->r_hmask.as<uint64_t>();
   p.r_part = x->r_part.as<uint64_t>();
+  p.Ji = x->den_tab.as<long long>();
+  p.Wi = p.Ji + (size_t)x->norb * x->norb;
   p.b_mask = x->b_mask.as<uint32_t>();
   p.o_mask = x->o_mask.as<uint64_t>();
   p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);
@@ -1203,7 +1206,8 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
       (rc = x->e_rec.grow(4 * (size_t)ent_cap * wsl)) || (rc = x->it_sum.grow(16 * (size_t)nper * wsl)) ||
       (rc = x->b_dead.grow(4 * dwords * wsl)) ||
       (rc = x->queues.grow(4 * (size_t)(nwaves + 1))) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
-      (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->res.grow(sizeof(DevResult))) ||
+      (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
+      (rc = x->res.grow(sizeof(DevResult))) ||
       (rc = x->g_wF.grow(8 * nd * 2 * norb)) || (rc = x->g_wH.grow(8 * nd)))
     return rc;
   CUDA_TRY(cudaMemsetAsync(x->eps.p, 0, 8 * nd, st));
@@ -1257,6 +1261,8 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   p.r_coef = x->r_coef.as<double>();
   p.r_hmask = x->r_hmask.as<uint64_t>();
   p.r_part = x->r_part.as<uint64_t>();
+  p.Ji = x->den_tab.as<long long>();
+  p.Wi = p.Ji + (size_t)x->norb * x->norb;
   p.b_mask = x->b_mask.as<uint32_t>();
   p.o_mask = x->o_mask.as<uint64_t>();
   p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);
@@ -1478,7 +1484,8 @@ static int plan_instance(BatchInst& b, size_t wave_budget, int64_t W_fixed, bool
   if ((rc = x->queues.grow(4 * (size_t)(b.nwaves + 1))) ||
       (rc = x->tk_e.grow(8 * (size_t)b.cap * grid)) || (rc = x->tk_a.grow(8 * (size_t)b.cap * grid)) ||
       (rc = x->tk_key.grow(8 * (size_t)b.cap * grid * nw)) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
-      (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->res.grow(sizeof(DevResult))) ||
+      (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
+      (rc = x->res.grow(sizeof(DevResult))) ||
       (rc = x->sel_hist.grow(4 * (size_t)kSelBins)) || (rc = x->cand_e.grow(8 * b.maxc)) || (rc = x->cand_a.grow(8 * b.maxc)) ||
       (rc = x->cand_key.grow(8 * b.maxc * nw)) || (rc = x->skey.grow(8 * b.maxc)) ||
       (rc = x->skey2.grow(8 * b.maxc)) || (rc = x->perm.grow(4 * b.maxc)) || (rc = x->perm2.grow(4 * b.maxc)))
@@ -1537,6 +1544,8 @@ static void make_params(BatchInst& b) {
   p.r_coef = x->r_coef.as<double>();
   p.r_hmask = x->r_hmask.as<uint64_t>();
   p.r_part = x->r_part.as<uint64_t>();
+  p.Ji = x->den_tab.as<long long>();
+  p.Wi = p.Ji + (size_t)x->norb * x->norb;
   p.b_mask = x->b_mask.as<uint32_t>();
   p.o_mask = x->o_mask.as<uint64_t>();
   p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);

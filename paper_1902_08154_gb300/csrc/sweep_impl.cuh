@@ -126,24 +126,77 @@ __device__ __forceinline__ const double* numer_h<double>(const SweepParams& p) {
 template <>
 __device__ __forceinline__ const float* numer_h<float>(const SweepParams& p) { return p.h32; }
 
-// 1/d by Newton-Raphson iteration for the reciprocal, r <- r + r (1 - d r),
-// from the hardware's approximate FP64 reciprocal (PTX rcp.approx.ftz.f64,
-// relative error below 2^-22).  Each step squares the relative error: two
-// steps reach the rounding level of FP64 (a few ulp) with four FMAs on the
-// FP64 pipe instead of a correctly rounded division; one step leaves a
-// relative error near 2^-44, used by the mixed-precision sweep, whose
-// budget is 1e-6 Eh.  |d| must be a normal number (the sweep's denominators
-// are bounded away from 0 and infinity; others take the plain division).
-template <int STEPS>
-__device__ __forceinline__ double recip_nr(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-#pragma unroll
-  for (int i = 0; i < STEPS; i++) {
-    const double e = fma(-d, r, 1.0);
-    r = fma(r, e, r);
+// ---------------------------------------------------------------------------
+// Denominators D = E0 - H_aa as 64-bit integers in units of 2^-S, and A/D by
+// integer arithmetic.  An FP64 warp instruction takes 19 cycles of an SM here
+// (a 64-bit integer add 1, a high 64-bit product 5.5), so the two FP64
+// additions of D and the five operations of its reciprocal were most of the
+// cells pass.  S is the same for a whole sweep:
+// |D| <= |E0| + n_el max|h| + n_el (n_el - 1) max|(pq|rs)| < 2^(62 - S), and
+// sums of table entries on the way may wrap.  The units are finer than the
+// rounding of the same sums in FP64 (2^-51 Eh against 2^-45 on 64 orbitals).
+// Two states at once, 2,000 determinants, 64 orbitals: 43 to 33.8 ms (two
+// quotients per cell); one state, 10^4 determinants 113.3 to 111.8 ms; 10^3
+// determinants, 128 orbitals 87.1 to 84.1 ms.
+// ---------------------------------------------------------------------------
+constexpr int kBadScale = 1 << 20;  // integrals not finite: every quotient is NaN
+__device__ __forceinline__ int den_scale(const SweepParams& p) {
+  const double hmx = __longlong_as_double((long long)p.hmax_bits[0]);
+  const double emx = __longlong_as_double((long long)p.hmax_bits[1]);
+  double e0 = fabs(p.e0);
+  for (int s = 0; s < p.nst; s++) e0 = fmax(e0, fabs(p.st_e0[s]));
+  const double n = (double)(p.nel + 2), bound = e0 + n * hmx + n * (n - 1.0) * emx;
+  if (!(bound < 1e300)) return kBadScale;
+  const int e = (int)((((unsigned long long)__double_as_longlong(bound)) >> 52) & 0x7FF) - 1023;
+  return 62 - e < 900 ? 62 - e : 900;
+}
+// 2^e, e within the normal exponents.
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+// x in units of 2^-S.
+__device__ __forceinline__ long long den_fix(double x, int S) {
+  return S == kBadScale ? 0ll : __double2ll_rn(x * pow2(S));
+}
+__device__ __forceinline__ double den_double(unsigned long long um, int S) {
+  return S == kBadScale ? __longlong_as_double(0x7FF8000000000000ll) : (double)um * pow2(-S);
+}
+
+// a / (d 2^-S) for a quotient outside the normal range, a zero denominator
+// or operands that are not finite.
+static __device__ __noinline__ double div_slow(double a, long long d, int S) {
+  if (S == kBadScale) return __longlong_as_double(0x7FF8000000000000ll);
+  return a / ((double)d * pow2(-S));
+}
+
+// a / (d 2^-S): the reciprocal of the normalised 64-bit magnitude m of d from
+// the FP32 approximation of its top 24 bits (relative error e below 2^-21) by
+// two Newton steps in integers (e^2 and the 32 bits of m left out of the
+// first step, then 2^-60), the product with a's mantissa, one rounding to
+// FP64 (half away from zero).
+__device__ __forceinline__ double div_fix(double a, long long d, int S) {
+  const unsigned long long ab = (unsigned long long)__double_as_longlong(a);
+  const int ea = (int)((ab >> 52) & 0x7FF);
+  unsigned long long m = d < 0 ? 0ull - (unsigned long long)d : (unsigned long long)d;
+  const int n = __clzll((long long)m);
+  m <<= n & 63;
+  const unsigned int mh = (unsigned int)(m >> 32);
+  float rf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(__uint2float_rn(mh)));
+  const unsigned int r0 = __float2uint_rz(rf * 9.223372036854775808e18f);  // 2^63 / mh, at most 2^32 - 1
+  const long long e1 = (long long)(0x8000000000000000ull - (unsigned long long)mh * r0);
+  unsigned long long r = ((unsigned long long)r0 << 32) + (unsigned long long)(((long long)(int)(e1 >> 20) * (long long)r0) >> 11);
+  const long long e2 = (long long)(0x7FFFFFFFFFFFFFFFull - __umul64hi(m, r));
+  r += (unsigned long long)(((long long)(r >> 34) * e2) >> 29);  // 2^127 / m
+  unsigned long long q = __umul64hi(((ab & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 11, r);
+  const int up = (int)(q >> 63);
+  q <<= 1 - up;
+  const int ex = ea + S + n - 64 + up;
+  if (m == 0ull || ex < 1 || ex > 2045 || ea == 0x7FF) {
+    if (ea == 0 && m != 0ull && S != kBadScale) return 0.0;
+    return div_slow(a, d, S);
   }
-  return r;
+  if (ea == 0) return 0.0;
+  const unsigned long long v = ((unsigned long long)(unsigned int)(ex - 1) << 52) + (q >> 11) + ((q >> 10) & 1ull);
+  return __longlong_as_double((long long)(v | ((ab ^ (unsigned long long)d) & 0x8000000000000000ull)));
 }
 
 // Nanoseconds of the device's global timer.
@@ -355,6 +408,7 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   __shared__ uint64_t sI[NW];
   __shared__ int s_occ[kMaxElec];
   __shared__ unsigned char s_vidx[2][kMaxOrb];
+  __shared__ double s_F[2 * kMaxOrb];
   extern __shared__ __align__(16) unsigned char dyn[];
   uint32_t* sm = reinterpret_cast<uint32_t*>(dyn);               // cell masks (MaskDims)
   uint64_t* so = reinterpret_cast<uint64_t*>(sm + p.mask_w);     // orbital masks (orb_mask_words)
@@ -387,6 +441,13 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   }
   __syncthreads();
   if (tid < nel) M->occ[tid] = s_occ[tid];
+  const int S = den_scale(p);
+  if (slot == 0)  // the denominators' tables, once per wave
+    for (int x = tid; x < norb * norb; x += kThreads) {
+      const long long j = den_fix(p.Jm[x], S);
+      p.Ji[x] = j;
+      p.Wi[x] = j - den_fix(p.Km[x], S);
+    }
   // Fock diagonal F_s(q) = h_qq + sum_{j in I} [(qq|jj) - delta_s (qj|jq)]
   for (int x = tid; x < 2 * norb; x += kThreads) {
     const int s = x / norb, q = x - s * norb;
@@ -396,16 +457,17 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
       f += p.Jm[q * norb + j];
       if (sj == s) f -= p.Km[q * norb + j];
     }
-    M->F[s][q] = f;
+    M->F[s][q] = den_fix(f, S);
+    s_F[x] = f;
   }
   __syncthreads();
   if (tid == 0) {  // H_II = 1/2 sum_i (h_ii + F(i))
     double e = 0.0;
     for (int i = 0; i < nel; i++) {
       const int c = s_occ[i], s = c >= norb, q = c - s * norb;
-      e += p.h[q * norb + q] + M->F[s][q];
+      e += p.h[q * norb + q] + s_F[c];
     }
-    M->hii = 0.5 * e;
+    M->hii = den_fix(0.5 * e, S);
   }
 
   // ---- coarse filter: J within degree 4 of I (I itself included) ----
@@ -727,14 +789,15 @@ struct BatchShared {
   int vir[2][kMaxOrb];
   int vidx[2][kMaxOrb];
   int nv[2];
-  double F[2][kMaxOrb];
-  double u0[kMaxOrb], u1[kMaxOrb];  // per-batch row sums for H_aa
-  double dx[kMaxOrb];               // E0 - base - u0[x]
+  // fixed point (den_scale): the Fock diagonal, per-batch row sums for H_aa
+  long long F[2][kMaxOrb];
+  long long u0[kMaxOrb], u1[kMaxOrb];
+  long long dx[kMaxOrb];            // E0 - base - u0[x]
   // two-hole batches: <I|H|I - H + R> by the pair tables of the all-cell
   // fast path, built for J = I (its X is the hole pair H itself)
   int iRow[kMaxOrb], iCol[kMaxOrb];
   NT cI;
-  double hii, base;
+  long long hii, base;
   float inv_nv1;
   uint64_t kbase[2 * NINT];  // I with the batch's holes removed
   int g, slot;
@@ -1344,7 +1407,10 @@ struct ItemEnv {
   int* Ahi;
   uint32_t* ban;
   double *ms_gc, *ms_cI, *ms_w;
+  long long* ms_de;  // E0_s - E0_0, fixed point
   int mc, nst, norb, nel, nbat, nper;
+  int dscale;    // den_scale
+  long long e0;  // E0 (state 0's) in those units
 };
 
 template <bool MS>
@@ -1359,11 +1425,14 @@ __device__ __forceinline__ ItemEnv item_env(const SweepParams& p) {
   E.ms_gc = reinterpret_cast<double*>(E.ban + (((E.mc + 31) / 32 + 1) & ~1));
   E.ms_cI = E.ms_gc + kGroup * kMaxStates;
   E.ms_w = E.ms_cI + kMaxStates;
+  E.ms_de = reinterpret_cast<long long*>(E.ms_w + kMaxStates);
   E.nst = MS ? p.nst : 1;
   E.norb = p.norb;
   E.nel = p.nel;
   E.nbat = p.nbat;
   E.nper = p.nper;
+  E.dscale = den_scale(p);
+  E.e0 = den_fix(MS ? p.st_e0[0] : p.e0, E.dscale);
   return E;
 }
 
@@ -1383,6 +1452,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   double* ms_gc = E.ms_gc;
   double* ms_cI = E.ms_cI;
   double* ms_w = E.ms_w;
+  long long* ms_de = E.ms_de;
   const int mc = E.mc, nst = E.nst;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int norb = E.norb, nel = E.nel, nbat = E.nbat;
@@ -1441,6 +1511,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         ms_cI[tid] = p.coefs[(size_t)tid * p.ndet + p.order[M->g]];
         const double m = __longlong_as_double((long long)p.st_cmax[tid]);
         ms_w[tid] = 1.0 / (m * m);
+        ms_de[tid] = den_fix(p.st_e0[tid], E.dscale) - E.e0;
       }
     }
     __syncthreads();
@@ -1572,11 +1643,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     }
   }
   {
-    auto W = [&](int x, int sx, int y, int sy) {
-      double v = p.Jm[x * norb + y];
-      if (sx == sy) v -= p.Km[x * norb + y];
-      return v;
-    };
+    auto W = [&](int x, int sx, int y, int sy) { return (sx == sy ? p.Wi : p.Ji)[x * norb + y]; };
     if (B.kind == 0) {
       const int s = B.sa;
       for (int x = tid; x < S.nv[s]; x += kThreads) {
@@ -1621,7 +1688,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     }
   }
   __syncthreads();
-  for (int x = tid; x < S.nv[B.sa]; x += kThreads) S.dx[x] = (p.e0 - S.base) - S.u0[x];
+  for (int x = tid; x < S.nv[B.sa]; x += kThreads) S.dx[x] = (E.e0 - S.base) - S.u0[x];
   if (p.tgt_on) {  // cells outside the target space contribute nothing: ban them
     for (int cc = tid; cc < B.nct; cc += kThreads) {
       int ro, so, x, y;
@@ -2169,7 +2236,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   }
   const unsigned long long tau = S.tau;
   double acc_e = 0.0, acc_s2 = 0.0;
-  unsigned long long acc_na = 0, acc_d0 = 0, acc_d1 = 0, acc_min = 0x7FF0000000000000ull, acc_tiny = 0;
+  unsigned long long acc_na = 0, acc_d0 = 0, acc_d1 = 0, acc_min = ~0ull, acc_tiny = 0;  // acc_min: units of 2^-S
   double acc_es[kMaxStates], acc_s2s[kMaxStates];  // multi-state form: sums per state
 #pragma unroll
   for (int st = 0; st < kMaxStates; st++) acc_es[st] = acc_s2s[st] = 0.0;
@@ -2196,25 +2263,21 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         }
         con++;
       }
-      // E0_s - H_aa = ((E0_s - base) - u0[x]) - rest, as the one-state form
-      double rest = 0.0;
-      if (B.kind == 2) rest = S.u1[y] + p.Jm[ro * norb + so];
-      else if (B.kind == 1) rest = S.u0[y] + (p.Jm[ro * norb + so] - p.Km[ro * norb + so]);
+      long long D0 = S.dx[x];  // E0_0 - H_aa
+      if (B.kind == 2) D0 -= S.u1[y] + p.Ji[ro * norb + so];
+      else if (B.kind == 1) D0 -= S.u0[y] + p.Wi[ro * norb + so];
       double crit = 0.0, a0 = 0.0;
 #pragma unroll
       for (int st = 0; st < kMaxStates; st++) {
         if (st >= nst) break;
         const double a = A[st * mc + cc] + ms_cI[st] * vI;
-        double D = (p.st_e0[st] - S.base) - S.u0[x];
-        if (B.kind != 0) D -= rest;
-        const unsigned long long dex = ((unsigned long long)__double_as_longlong(D) >> 52) & 0x7FFull;
-        const double inv = (dex > 523ull && dex < 1523ull) ? recip_nr<2>(D) : 1.0 / D;
-        const double q = a * inv;
+        const long long D = D0 + ms_de[st];
+        const double q = div_fix(a, D, E.dscale);
         const double e = a * q;
         acc_es[st] += e;
         acc_s2s[st] += q * q;
         crit += ms_w[st] * e;  // c_alpha,s A_s / max_I c_Is^2
-        const unsigned long long db = abs_bits(D);
+        const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
         acc_min = db < acc_min ? db : acc_min;
         if (st == 0) a0 = a;
       }
@@ -2268,13 +2331,10 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         con++;
       }
       // D = E0 - H_aa from the per-batch row sums
-      double D = S.dx[x];
-      if (B.kind == 2) D -= S.u1[y] + p.Jm[ro * norb + so];
-      else if (B.kind == 1) D -= S.u0[y] + (p.Jm[ro * norb + so] - p.Km[ro * norb + so]);
-      // |D| in [2^-500, 2^500]: Newton reciprocal; otherwise the division
-      const unsigned long long dex = ((unsigned long long)__double_as_longlong(D) >> 52) & 0x7FFull;
-      const double inv = (dex > 523ull && dex < 1523ull) ? recip_nr<sizeof(NT) == 8 ? 2 : 1>(D) : 1.0 / D;
-      const double q = a * inv;
+      long long D = S.dx[x];
+      if (B.kind == 2) D -= S.u1[y] + p.Ji[ro * norb + so];
+      else if (B.kind == 1) D -= S.u0[y] + p.Wi[ro * norb + so];
+      const double q = div_fix(a, D, E.dscale);
       acc_e = fma(a, q, acc_e);  // e = A q
       acc_s2 += q * q;
       acc_na++;
@@ -2289,8 +2349,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       }
       // |a| < 1e-14, compared on the bit pattern (no FP64 compare)
       if (abs_bits(a) < 0x3D06849B86A12B9Bull) acc_tiny++;
-      // |D| and |e| as bit patterns, off the FP64 pipe
-      const unsigned long long db = abs_bits(D);
+      const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
       acc_min = db < acc_min ? db : acc_min;
       uint64_t key[NW];  // alpha's words; selects keep them in registers
       const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
@@ -2348,7 +2407,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     }
     if (tid == 0) {
       const double te_ = se, ts = ss;
-      unsigned long long tn = 0, tc = 0, x0 = 0, x1 = 0, m = 0x7FF0000000000000ull, tt = 0;
+      unsigned long long tn = 0, tc = 0, x0 = 0, x1 = 0, m = ~0ull, tt = 0;
       for (int w = 0; w < kWarps; w++) {
         tn += S.red_u[w][0];
         tc += S.red_u[w][1];
@@ -2370,7 +2429,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         atomicAdd(&p.ncon[g], tc);
         atomicAdd(&p.digest[0], x0);
         atomicXor(&p.digest[1], x1);
-        atomicMin(p.min_den_bits, m);
+        atomicMin(p.min_den_bits, (unsigned long long)__double_as_longlong(den_double(m, E.dscale)));
         if (tt) atomicAdd(p.n_tiny, tt);
       }
     }

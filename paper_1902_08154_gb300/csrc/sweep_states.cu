@@ -10,11 +10,12 @@ template __global__ void batch_kernel<2, double, false, true>(const __grid_const
 
 // Dynamic shared memory of the multi-state form: nst accumulators of
 // max_cells doubles, the ban bitmap (rounded to 8 bytes), the group's
-// per-state coefficients, c_I per state and the weights.
+// per-state coefficients, c_I per state, the weights and
+// the states' E0 differences.
 size_t states_smem(int max_cells, int nst) {
   const size_t ban_words = (size_t)(((max_cells + 31) / 32 + 1) & ~1);
   return sizeof(double) * (size_t)max_cells * (size_t)nst + sizeof(uint32_t) * ban_words +
-         sizeof(double) * (size_t)(kGroup * kMaxStates + 2 * kMaxStates);
+         sizeof(double) * (size_t)(kGroup * kMaxStates + 3 * kMaxStates);
 }
 
 int batch_blocks_per_sm_states(int nint, size_t smem) {
