@@ -117,14 +117,14 @@ __host__ __device__ inline size_t sweep_smem(int mc) {
 struct GenMeta;
 // Device bytes per generator slot of a wave: metadata, nd coarse-filter
 // records (words, nst coefficients, hole mask, particles), bucket offsets,
-// ent_cap self-contained entries (20 bytes), the ban masks, the dead-batch
-// bits and the nper items' FP64 sums (2 per state).
+// ent_cap self-contained entries (20 bytes), the ban masks, the live-item
+// list and the nper items' FP64 sums (2 per state).
 inline size_t wave_slot_bytes(size_t meta_bytes, int norb, int na, int nb, int nbat, size_t nd, int nst, int nper) {
   const int nint = (norb - 1) / 64 + 1, nw = 2 * nint, nel = na + nb;
   const size_t ent_cap = nd * (size_t)bucket_entries_per_record(nel);
   return meta_bytes + nd * (8 * (size_t)nw + 8 * (size_t)nst + 8 + 8) + 4 * (size_t)(nbat + 2) + 20 * ent_cap +
          4 * (size_t)mask_words(norb, na, nb) + 8 * (size_t)orb_mask_words(nint, nel) +
-         4 * (size_t)((nbat + 31) / 32) + 16 * (size_t)nper * (size_t)nst;
+         4 * (size_t)nper + 16 * (size_t)nper * (size_t)nst;
 }
 
 // Per-generator data built by the prep kernel and read by the batch kernel.
@@ -204,7 +204,10 @@ struct SweepParams {
   // its index with the rank flag (rank(J) < rank(I)) in bit 31
   ulonglong2* e_hp;               // [slots][ent_cap]: hole mask, particles (one 16-byte load)
   uint32_t* e_rec;                // [slots][ent_cap]
-  uint32_t* b_dead;               // [slots][(nbat + 31) / 32]  batches banned as a whole
+  // the wave's work items (slot * nper + item), without those of batches
+  // banned as a whole, in the order the prep kernel finished the slots
+  uint32_t* live;                 // [slots * nper]
+  int* live_cnt;                  // per wave, zero before the prep kernel
   int64_t ent_cap;
 
   // exact accumulation of A_alpha: bits of max_I |c_I| (written by the
@@ -264,6 +267,9 @@ struct MultiWaveInline {
   unsigned long long* t_start;
   int* err;                    // flag 128: the watchdog stopped the launch
 };
+
+// Slots a wave may hold for its work items to be numbered in 31 bits.
+inline long long max_wave_slots(int nper) { return ((1ll << 31) - 1) / (nper > 0 ? nper : 1); }
 
 // One wave of several instances' sweeps in one launch: ps[i] holds instance
 // i's parameters for the wave; slot_ofs / item_ofs number the instances'

@@ -195,7 +195,6 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   const size_t nd = (size_t)ndet;
   const int64_t cap = k > 0 ? k + max_cells : 1, ngen = ndet;
   const int64_t ent_cap = (int64_t)nd * bucket_entries_per_record(nel);
-  const size_t dwords = (size_t)(nbat + 31) / 32;
   const int nper = nbat;
   size_t maxc = 0, tmp1 = 0, tmp2 = 0;
   int64_t W = 0, nwaves = 0;
@@ -214,7 +213,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   uint64_t *r_part = nullptr, *o_mask = nullptr;
   unsigned int *sel_hist = nullptr;
   GenMeta *meta = nullptr;
-  uint32_t *b_mask = nullptr, *e_rec = nullptr, *b_dead = nullptr;
+  uint32_t *b_mask = nullptr, *e_rec = nullptr, *live = nullptr;
   ulonglong2 *e_hp = nullptr;
   // Lays the arrays out for `grid` sweep CTAs; 0, or which size does not fit.
   auto layout = [&](int grid) -> int {
@@ -237,7 +236,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     ncon = cv.take<unsigned long long>(nd);
     acc = cv.take<unsigned long long>(9);
     dres = cv.take<DevResult>(1);
-    queues = cv.take<int>(nd + 1);
+    queues = cv.take<int>(2);  // the wave's item counter and live count
     tk_e = cv.take<double>((size_t)cap * grid);
     tk_a = cv.take<double>((size_t)cap * grid);
     tk_key = cv.take<uint64_t>((size_t)cap * grid * nw);
@@ -271,6 +270,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     W = (int64_t)(left / per_slot);
     if (W < 1) return 2;
     if (W > ngen) W = ngen;
+    if (W > max_wave_slots(nper)) W = max_wave_slots(nper);
     nwaves = (ngen + W - 1) / W;
     const size_t wsl = (size_t)W;
     meta = cv.take<GenMeta>(wsl);
@@ -284,7 +284,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     e_hp = cv.take<ulonglong2>((size_t)ent_cap * wsl);
     e_rec = cv.take<uint32_t>((size_t)ent_cap * wsl);
     it_sum = cv.take<double>((size_t)2 * nper * wsl);
-    b_dead = cv.take<uint32_t>(dwords * wsl);
+    live = cv.take<uint32_t>((size_t)nper * wsl);
     return cv.ok ? 0 : 2;
   };
   // one CTA per SM keeps the selection buffers small; a few CTAs less where a
@@ -330,7 +330,6 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   NTRY(cudaMemsetAsync(s2, 0, 8 * nd, st));
   NTRY(cudaMemsetAsync(na, 0, 8 * nd, st));
   NTRY(cudaMemsetAsync(ncon, 0, 8 * nd, st));
-  NTRY(cudaMemsetAsync(queues, 0, 4 * (nd + 1), st));
   NTRY(cudaMemsetAsync(tk_cnt, 0, 4 * (size_t)grid, st));
   NTRY(cudaMemsetAsync(tk_tau, 0, 8 * (size_t)grid, st));
   NTRY(cudaMemsetAsync(sel_hist, 0, 4 * (size_t)kSelBins, st));
@@ -375,7 +374,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   p.mask_w = mask_words(norb, n_alpha, n_beta);
   p.orb_w = orb_mask_words(nint, nel);
   p.b_ofs = b_ofs;
-  p.b_dead = b_dead;
+  p.live = live;
   p.ent_cap = ent_cap;
   p.eps = eps;
   p.s2 = s2;
@@ -399,8 +398,9 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     p.wave_start = (int)(w * W);
     p.wave_slots = (int)((ngen - w * W) < W ? (ngen - w * W) : W);
     p.last_wave = (w == nwaves - 1);
-    p.queue = queues + w;
-    NTRY_Q(cudaMemsetAsync(it_sum, 0, sizeof(double) * 2 * (size_t)nper * p.wave_slots, st));
+    p.queue = queues;
+    p.live_cnt = queues + 1;
+    NTRY_Q(cudaMemsetAsync(queues, 0, 2 * sizeof(int), st));
     NTRY_Q(launch_prep(nint, p, p.wave_slots, st));
     NTRY_Q(launch_batch_packed(nint, p, grid, smem, st));
     NTRY_Q(launch_reduce_items(p, st));

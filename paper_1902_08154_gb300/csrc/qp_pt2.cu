@@ -327,7 +327,7 @@ struct qp_pt2_ctx {
   // workspace
   Buf in_dets, in_coefs, hkey, hkey2, hidx, hidx2, rkey, rkey2, order, rank_of, cub_tmp;
   Buf eps, s2, na, ncon, acc, res;
-  Buf den_tab, meta, r_words, r_coef, r_hmask, r_part, b_mask, o_mask, b_ofs, e_hp, e_rec, b_dead, queues, it_sum;
+  Buf den_tab, meta, r_words, r_coef, r_hmask, r_part, b_mask, o_mask, b_ofs, e_hp, e_rec, live, queues, it_sum;
   Buf tk_e, tk_a, tk_key, tk_cnt, tk_tau, sel_hist, gen_list, gen_out, st_cmax;
   Buf cand_e, cand_a, cand_key, skey, skey2, perm, perm2, cub_tmp2;
   Buf out_sel, out_e, out_num, out_eps, out_na, out_ncon, out_rank;
@@ -532,7 +532,7 @@ extern "C" void qp_pt2_destroy(qp_pt2_ctx* x) {
   Buf* all[] = {&x->in_dets, &x->in_coefs, &x->hkey, &x->hkey2, &x->hidx, &x->hidx2, &x->rkey, &x->rkey2,
                 &x->order, &x->rank_of, &x->cub_tmp, &x->eps, &x->s2, &x->na, &x->ncon, &x->acc,
                 &x->res, &x->meta, &x->r_words, &x->r_coef, &x->r_hmask, &x->den_tab, &x->r_part, &x->b_mask, &x->o_mask,
-                &x->b_ofs, &x->e_hp, &x->e_rec, &x->it_sum, &x->b_dead, &x->queues, &x->tk_e, &x->tk_a, &x->tk_key, &x->tk_cnt, &x->tk_tau, &x->sel_hist, &x->gen_list, &x->gen_out, &x->cand_e, &x->cand_a, &x->cand_key, &x->skey,
+                &x->b_ofs, &x->e_hp, &x->e_rec, &x->it_sum, &x->live, &x->queues, &x->tk_e, &x->tk_a, &x->tk_key, &x->tk_cnt, &x->tk_tau, &x->sel_hist, &x->gen_list, &x->gen_out, &x->cand_e, &x->cand_a, &x->cand_key, &x->skey,
                 &x->skey2, &x->perm, &x->perm2, &x->cub_tmp2, &x->out_sel, &x->out_e, &x->out_num,
                 &x->out_eps, &x->out_na, &x->out_ncon, &x->out_rank, &x->g_dh, &x->g_deri, &x->g_wF, &x->g_wH};
   for (Buf* b : all) b->release();
@@ -779,10 +779,10 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   }
   const int64_t ent_per = bucket_entries_per_record(x->nel);
   const int64_t ent_cap = (int64_t)nd * ent_per;
-  const size_t dwords = (size_t)(x->nbat + 31) / 32;
   const int nper = x->nbat + (x->ntile - 1) * x->nalpha * x->nbeta;
   const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), x->norb, x->nalpha, x->nbeta, x->nbat, nd, nsts, nper);
   int64_t W = (int64_t)(kWaveBudget / per_slot);
+  W = std::min<int64_t>(W, max_wave_slots(nper));
   if (W < 1) W = 1;
   if (W > ngen) W = ngen > 0 ? ngen : 1;
   const int64_t nwaves = ngen > 0 ? (ngen + W - 1) / W : 0;
@@ -795,7 +795,7 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
       (rc = x->o_mask.grow(8 * (size_t)orb_mask_words(nint, x->nel) * ws)) || (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * ws)) ||
       (rc = x->e_hp.grow(16 * (size_t)ent_cap * ws)) ||
       (rc = x->e_rec.grow(4 * (size_t)ent_cap * ws)) || (rc = x->it_sum.grow(16 * (size_t)nper * nsts * ws)) ||
-      (rc = x->b_dead.grow(4 * dwords * ws)) || (rc = x->queues.grow(4 * (size_t)(nwaves + 1))) ||
+      (rc = x->live.grow(4 * (size_t)nper * ws)) || (rc = x->queues.grow(8 * (size_t)(nwaves + 1))) ||
       (rc = x->tk_e.grow(8 * (size_t)cap * grid)) || (rc = x->tk_a.grow(8 * (size_t)cap * grid)) ||
       (rc = x->tk_key.grow(8 * (size_t)cap * grid * nw)) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
       (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
@@ -807,7 +807,7 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   CUDA_TRY(cudaMemsetAsync(x->s2.p, 0, 8 * nd * nsts, st));
   CUDA_TRY(cudaMemsetAsync(x->na.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->ncon.p, 0, 8 * nd, st));
-  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 4 * (size_t)(nwaves + 1), st));
+  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 8 * (size_t)(nwaves + 1), st));
   CUDA_TRY(cudaMemsetAsync(x->tk_cnt.p, 0, 4 * (size_t)grid, st));
   CUDA_TRY(cudaMemsetAsync(x->tk_tau.p, 0, 8 * (size_t)grid, st));
   SweepParams p{};
@@ -864,7 +864,7 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);
   p.orb_w = orb_mask_words(x->nint, x->nel);
   p.b_ofs = x->b_ofs.as<int>();
-  p.b_dead = x->b_dead.as<uint32_t>();
+  p.live = x->live.as<uint32_t>();
   p.ent_cap = ent_cap;
   p.eps = x->eps.as<double>();
   p.s2 = x->s2.as<double>();
@@ -897,7 +897,7 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
     p.wave_slots = (int)((ngen - w * W) < W ? (ngen - w * W) : W);
     p.last_wave = (w == nwaves - 1);
     p.queue = x->queues.as<int>() + w;
-    CUDA_TRY(cudaMemsetAsync(p.it_sum, 0, sizeof(double) * (size_t)p.wave_slots * p.nper * p.it_stride, st));
+    p.live_cnt = x->queues.as<int>() + (nwaves + 1) + w;
     CUDA_TRY(launch_prep(nint, p, p.wave_slots, st));
     if (ms) CUDA_TRY(launch_batch_states(nint, p, grid, smem, st));
     else CUDA_TRY(launch_batch(nint, p, grid, smem, st));
@@ -1188,10 +1188,10 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   const int64_t ngen = (ndet > shard_index) ? (ndet - shard_index + shard_count - 1) / shard_count : 0;
   const int64_t ent_per = bucket_entries_per_record(x->nel);
   const int64_t ent_cap = (int64_t)nd * ent_per;
-  const size_t dwords = (size_t)(x->nbat + 31) / 32;
   const int nper = x->nbat + (x->ntile - 1) * x->nalpha * x->nbeta;
   const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), x->norb, x->nalpha, x->nbeta, x->nbat, nd, 1, nper);
   int64_t W = (int64_t)(kWaveBudget / per_slot);
+  W = std::min<int64_t>(W, max_wave_slots(nper));
   if (W < 1) W = 1;
   if (W > ngen) W = ngen > 0 ? ngen : 1;
   const int64_t nwaves = ngen > 0 ? (ngen + W - 1) / W : 0;
@@ -1204,8 +1204,8 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
       (rc = x->o_mask.grow(8 * (size_t)orb_mask_words(nint, x->nel) * wsl)) || (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * wsl)) ||
       (rc = x->e_hp.grow(16 * (size_t)ent_cap * wsl)) ||
       (rc = x->e_rec.grow(4 * (size_t)ent_cap * wsl)) || (rc = x->it_sum.grow(16 * (size_t)nper * wsl)) ||
-      (rc = x->b_dead.grow(4 * dwords * wsl)) ||
-      (rc = x->queues.grow(4 * (size_t)(nwaves + 1))) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
+      (rc = x->live.grow(4 * (size_t)nper * wsl)) ||
+      (rc = x->queues.grow(8 * (size_t)(nwaves + 1))) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
       (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
       (rc = x->res.grow(sizeof(DevResult))) ||
       (rc = x->g_wF.grow(8 * nd * 2 * norb)) || (rc = x->g_wH.grow(8 * nd)))
@@ -1214,7 +1214,7 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   CUDA_TRY(cudaMemsetAsync(x->s2.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->na.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->ncon.p, 0, 8 * nd, st));
-  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 4 * (size_t)(nwaves + 1), st));
+  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 8 * (size_t)(nwaves + 1), st));
   CUDA_TRY(cudaMemsetAsync(x->tk_cnt.p, 0, 4 * (size_t)grid, st));
   CUDA_TRY(cudaMemsetAsync(x->tk_tau.p, 0, 8 * (size_t)grid, st));
   CUDA_TRY(cudaMemsetAsync(x->g_wF.p, 0, 8 * nd * 2 * norb, st));
@@ -1268,7 +1268,7 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);
   p.orb_w = orb_mask_words(x->nint, x->nel);
   p.b_ofs = x->b_ofs.as<int>();
-  p.b_dead = x->b_dead.as<uint32_t>();
+  p.live = x->live.as<uint32_t>();
   p.ent_cap = ent_cap;
   p.eps = x->eps.as<double>();
   p.s2 = x->s2.as<double>();
@@ -1295,7 +1295,7 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
     p.wave_slots = (int)((ngen - w * W) < W ? (ngen - w * W) : W);
     p.last_wave = (w == nwaves - 1);
     p.queue = x->queues.as<int>() + w;
-    CUDA_TRY(cudaMemsetAsync(p.it_sum, 0, sizeof(double) * (size_t)p.wave_slots * p.nper * p.it_stride, st));
+    p.live_cnt = x->queues.as<int>() + (nwaves + 1) + w;
     CUDA_TRY(launch_prep(nint, p, p.wave_slots, st));
     CUDA_TRY(launch_batch_grad(nint, p, grid, x->smem, st));
     CUDA_TRY(launch_reduce_items(p, st));
@@ -1410,7 +1410,7 @@ struct FusedGroup {
   SweepParams* d_ps = nullptr;    // [nwaves + 1][nm]: the wave's pieces; row nwaves: all members
   int* d_slot_ofs = nullptr;      // [nwaves][nm + 1]
   long long* d_item_ofs = nullptr;  // [nwaves][nm + 1]
-  unsigned long long* d_words = nullptr;  // [nwaves][npw] pieces' item counters, then the watchdog's start time
+  unsigned long long* d_words = nullptr;  // [nwaves][npw] pieces' item counters, the watchdog's start time, their live counts
   int* d_err = nullptr;
   cudaStream_t st = nullptr;
   cudaEvent_t done = nullptr;
@@ -1450,9 +1450,9 @@ static int plan_instance(BatchInst& b, size_t wave_budget, int64_t W_fixed, bool
   b.ngen = b.ndet;
   const int64_t ent_per = bucket_entries_per_record(x->nel);
   b.ent_cap = (int64_t)nd * ent_per;
-  const size_t dwords = (size_t)(x->nbat + 31) / 32;
   const int nper = b.nper;
   b.W = W_fixed > 0 ? W_fixed : (int64_t)(wave_budget / inst_slot_bytes(b));
+  b.W = std::min<int64_t>(b.W, max_wave_slots(nper));
   if (b.W < 1) b.W = 1;
   if (b.W > b.ngen) b.W = b.ngen;
   b.nwaves = (b.ngen + b.W - 1) / b.W;
@@ -1479,9 +1479,9 @@ static int plan_instance(BatchInst& b, size_t wave_budget, int64_t W_fixed, bool
       (rc = x->o_mask.grow(8 * (size_t)orb_mask_words(nint, x->nel) * ws)) ||
       (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * ws)) || (rc = x->e_hp.grow(16 * (size_t)b.ent_cap * ws)) ||
       (rc = x->e_rec.grow(4 * (size_t)b.ent_cap * ws)) ||
-      (rc = x->it_sum.grow(16 * (size_t)nper * ws)) || (rc = x->b_dead.grow(4 * dwords * ws))))
+      (rc = x->it_sum.grow(16 * (size_t)nper * ws)) || (rc = x->live.grow(4 * (size_t)nper * ws))))
     return rc;
-  if ((rc = x->queues.grow(4 * (size_t)(b.nwaves + 1))) ||
+  if ((rc = x->queues.grow(8 * (size_t)(b.nwaves + 1))) ||
       (rc = x->tk_e.grow(8 * (size_t)b.cap * grid)) || (rc = x->tk_a.grow(8 * (size_t)b.cap * grid)) ||
       (rc = x->tk_key.grow(8 * (size_t)b.cap * grid * nw)) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
       (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
@@ -1551,7 +1551,7 @@ static void make_params(BatchInst& b) {
   p.mask_w = mask_words(x->norb, x->nalpha, x->nbeta);
   p.orb_w = orb_mask_words(x->nint, x->nel);
   p.b_ofs = x->b_ofs.as<int>();
-  p.b_dead = x->b_dead.as<uint32_t>();
+  p.live = x->live.as<uint32_t>();
   p.ent_cap = b.ent_cap;
   p.eps = x->eps.as<double>();
   p.s2 = x->s2.as<double>();
@@ -1601,7 +1601,7 @@ static int enqueue_pre(BatchInst& b, cudaStream_t st) {
   CUDA_TRY(cudaMemsetAsync(x->s2.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->na.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->ncon.p, 0, 8 * nd, st));
-  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 4 * (size_t)(b.nwaves + 1), st));
+  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 8 * (size_t)(b.nwaves + 1), st));
   CUDA_TRY(cudaMemsetAsync(x->tk_cnt.p, 0, 4 * (size_t)b.grid, st));
   CUDA_TRY(cudaMemsetAsync(x->tk_tau.p, 0, 8 * (size_t)b.grid, st));
   return QP_OK;
@@ -1616,6 +1616,7 @@ static int enqueue_waves(BatchInst& b, cudaStream_t st) {
     p.wave_slots = (int)((b.ngen - w * b.W) < b.W ? (b.ngen - w * b.W) : b.W);
     p.last_wave = (w == b.nwaves - 1);
     p.queue = x->queues.as<int>() + w;
+    p.live_cnt = x->queues.as<int>() + (b.nwaves + 1) + w;
     CUDA_TRY(launch_prep(x->nint, p, p.wave_slots, st));  // it zeroes the wave's per-item sums
     CUDA_TRY(launch_batch(x->nint, p, b.grid, b.smem, st));
     CUDA_TRY(launch_reduce_items(p, st));
@@ -1731,6 +1732,7 @@ static int plan_fused(qp_pt2_batch* B, const qp_pt2_batch_options& o, size_t wav
           inwave = 0;
           continue;
         }
+        fit = std::min<int64_t>(fit, max_wave_slots(b.nper));
         if (fit < 1) fit = 1;
         const int64_t take = std::min(fit, b.ngen - start);
         pieces.push_back({wave, i, start, take, used});
@@ -1758,6 +1760,8 @@ static int plan_fused(qp_pt2_batch* B, const qp_pt2_batch_options& o, size_t wav
       for (const Piece& q : pieces) maxp = std::max(maxp, ++cnt[q.wave]);
     }
     G.npw = maxp;
+    if (cudaMalloc(&G.d_words, sizeof(unsigned long long) * (2 * (size_t)G.nwaves * maxp + 1)) != cudaSuccess)
+      return fail(QP_ENOMEM, "device allocation of the batch tables failed");
     std::vector<SweepParams> hp((size_t)G.nwaves * maxp + nm);
     std::vector<int> hs((size_t)G.nwaves * (maxp + 1), 0);
     std::vector<long long> hi((size_t)G.nwaves * (maxp + 1), 0);
@@ -1786,13 +1790,14 @@ static int plan_fused(qp_pt2_batch* B, const qp_pt2_batch_options& o, size_t wav
       p.b_ofs = reinterpret_cast<int*>(take(4 * (size_t)(x->nbat + 2) * ws));
       p.e_hp = reinterpret_cast<ulonglong2*>(take(16 * (size_t)b.ent_cap * ws));
       p.e_rec = reinterpret_cast<uint32_t*>(take(4 * (size_t)b.ent_cap * ws));
-      p.b_dead = reinterpret_cast<uint32_t*>(take(4 * (size_t)((x->nbat + 31) / 32) * ws));
+      p.live = reinterpret_cast<uint32_t*>(take(4 * (size_t)b.nper * ws));
       p.it_sum = reinterpret_cast<double*>(take(16 * (size_t)b.nper * ws));
       p.wave_start = (int)q.start;
       p.wave_slots = (int)q.slots;
       p.last_wave = 0;  // compact_multi_kernel keeps the k best after the last wave
       p.queue = nullptr;
       const int r = q.wave, a = G.nact[r]++;
+      p.live_cnt = reinterpret_cast<int*>(G.d_words + (size_t)G.nwaves * maxp + 1 + (size_t)r * maxp + a);
       hp[(size_t)r * maxp + a] = p;
       int* so = hs.data() + (size_t)r * (maxp + 1);
       long long* io = hi.data() + (size_t)r * (maxp + 1);
@@ -1807,7 +1812,6 @@ static int plan_fused(qp_pt2_batch* B, const qp_pt2_batch_options& o, size_t wav
     if (cudaMalloc(&G.d_ps, sizeof(SweepParams) * hp.size()) != cudaSuccess ||
         cudaMalloc(&G.d_slot_ofs, sizeof(int) * hs.size()) != cudaSuccess ||
         cudaMalloc(&G.d_item_ofs, sizeof(long long) * hi.size()) != cudaSuccess ||
-        cudaMalloc(&G.d_words, sizeof(unsigned long long) * ((size_t)G.nwaves * maxp + 1)) != cudaSuccess ||
         cudaMalloc(&G.d_err, sizeof(int)) != cudaSuccess)
       return fail(QP_ENOMEM, "device allocation of the batch tables failed");
     if (cudaMemcpy(G.d_ps, hp.data(), sizeof(SweepParams) * hp.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
@@ -1827,7 +1831,7 @@ static int plan_fused(qp_pt2_batch* B, const qp_pt2_batch_options& o, size_t wav
 // of the candidate buffers.
 static int enqueue_group(FusedGroup& G) {
   const int nm = (int)G.members.size(), np = G.npw;
-  CUDA_TRY(cudaMemsetAsync(G.d_words, 0, sizeof(unsigned long long) * ((size_t)G.nwaves * np + 1), G.st));
+  CUDA_TRY(cudaMemsetAsync(G.d_words, 0, sizeof(unsigned long long) * (2 * (size_t)G.nwaves * np + 1), G.st));
   CUDA_TRY(cudaMemsetAsync(G.d_err, 0, sizeof(int), G.st));
   for (int r = 0; r < G.nwaves; r++) {
     MultiWave m{};

@@ -53,7 +53,7 @@ namespace qp {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kChunk = 1536;  // bucket entries classified per round
+constexpr int kChunk = 512;  // bucket entries classified per round
 constexpr int kGroup = 8;     // J reaching every cell, handled together
 constexpr unsigned kFull = 0xffffffffu;
 // Bit of a bucket entry's particle word that flags a J ranked before I (see
@@ -310,14 +310,19 @@ __device__ __forceinline__ void fix_add(unsigned long long& lo, int& hi, unsigne
   hi += h2 + (lo < l2 ? 1 : 0);
 }
 
-// Adds (l, h) into the shared-memory accumulator of cell cc: the low words
-// add modulo 2^64 and each carry out of them is added to the high word, so
-// the total is exact whatever the order of the atomics.
-__device__ __forceinline__ void fix_atomic_add(unsigned long long* Alo, int* Ahi, int cc, unsigned long long l,
+// Adds (l, h) into the shared-memory accumulator of a cell, kept as three
+// 32-bit words in arrays of their own (a 64-bit shared-memory add is a
+// compare-and-swap loop: 116 cycles against 44 for a 32-bit one): each carry
+// out of a word is added to the next, so the total is exact whatever the
+// order of the atomics.
+__device__ __forceinline__ void fix_atomic_add(uint32_t* A0, uint32_t* A1, uint32_t* A2, int cc, unsigned long long l,
                                                int h) {
-  const unsigned long long old = atomicAdd(&Alo[cc], l);
-  const int dh = h + ((old + l < old) ? 1 : 0);
-  if (dh) atomicAdd(&Ahi[cc], dh);
+  const uint32_t l0 = (uint32_t)l, l1 = (uint32_t)(l >> 32);
+  const uint32_t o0 = atomicAdd(&A0[cc], l0);
+  const uint32_t c0 = o0 + l0 < o0 ? 1u : 0u, t1 = l1 + c0;
+  const uint32_t o1 = atomicAdd(&A1[cc], t1);
+  const uint32_t dh = (uint32_t)h + (t1 < c0 ? 1u : 0u) + (o1 + t1 < o1 ? 1u : 0u);
+  if (dh) atomicAdd(&A2[cc], dh);
 }
 
 // (lo, hi) * 2^-F rounded to FP64 (nearest, ties away from zero): the top
@@ -394,6 +399,70 @@ __device__ __forceinline__ void for_buckets(uint64_t hm, uint64_t pt, int nel, i
       const int b = pair_batch(nel, Q[i], Q[j]);
       if (!((dead[b >> 5] >> (b & 31)) & 1u)) fn(b);
     }
+}
+
+struct Batch {
+  int h;            // number of holes (1, 2)
+  int kind;         // 0 single, 1 same-spin double, 2 opposite-spin double
+  int ia, ib;       // occupied indices of the holes in I
+  int ca, cb;       // their spin-orbital codes
+  int sa, sb;       // their spins
+  int qa, qb;       // their orbitals
+  uint64_t hm;      // hole mask over I's occupied list
+  int ncell;
+  int clo, nct;     // this work item's cells: [clo, clo + nct) (a tile of the batch)
+};
+
+
+// Batch and tile of work item j of a generator: j < nbat is batch j (the first
+// row tile of a split batch), j >= nbat row tile 1 + (j - nbat) / (n_alpha
+// n_beta) of opposite-spin batch (j - nbat) % (n_alpha n_beta).
+__device__ __forceinline__ int item_batch(const SweepParams& p, int j, int* tile) {
+  *tile = 0;
+  if (j < p.nbat) return j;
+  const int na = p.nalpha, nab = p.nalpha * p.nbeta, k = (j - p.nbat) % nab;
+  *tile = 1 + (j - p.nbat) / nab;
+  const int ia = k % na, ib = na + k / na;
+  return p.nel + ib * (ib - 1) / 2 + ia;
+}
+
+// The holes, kind and cells of batch b, tile `tile` (the orbitals of the
+// holes are filled in from the generator's occupied list).  The occupied list
+// is ordered spin-up first, so the indices give the spins.
+__device__ __forceinline__ void batch_geometry(const SweepParams& p, int b, int tile, Batch& B) {
+  const int nv0 = p.norb - p.nalpha, nv1 = p.norb - p.nbeta;
+  if (b < p.nel) {
+    B.h = 1;
+    B.ia = b;
+    B.ib = -1;
+    B.sa = b >= p.nalpha;
+    B.sb = -1;
+    B.kind = 0;
+    B.hm = 1ull << b;
+    B.ncell = B.sa ? nv1 : nv0;
+  } else {
+    const int t = b - p.nel;
+    int y = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)t)) * 0.5f);
+    while (y * (y - 1) / 2 > t) y--;
+    while ((y + 1) * y / 2 <= t) y++;
+    B.h = 2;
+    B.ib = y;
+    B.ia = t - y * (y - 1) / 2;
+    B.sa = B.ia >= p.nalpha;
+    B.sb = B.ib >= p.nalpha;
+    B.kind = B.sa == B.sb ? 1 : 2;
+    B.hm = (1ull << B.ia) | (1ull << B.ib);
+    const int nv = B.sa ? nv1 : nv0;
+    B.ncell = B.kind == 1 ? nv * (nv - 1) / 2 : nv0 * nv1;
+  }
+  B.clo = 0;
+  B.nct = B.ncell;
+  if (p.ntile > 1 && B.kind == 2) {  // rows [tile h, min((tile + 1) h, nv0))
+    const int h = (nv0 + p.ntile - 1) / p.ntile;
+    const int r0 = tile * h, r1 = min(r0 + h, nv0);
+    B.clo = r0 * nv1;
+    B.nct = (r1 - r0) * nv1;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -638,6 +707,23 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
     }
   }
   __syncthreads();
+  // the slot's work items, without those of batches banned as a whole
+  for (int j0 = 0; j0 < p.nper; j0 += kThreads) {
+    const int j = j0 + tid;
+    bool live = false;
+    if (j < p.nper) {
+      int tile;
+      const int b = item_batch(p, j, &tile);
+      Batch B;
+      batch_geometry(p, b, tile, B);
+      live = B.nct > 0 && !((s_dead[b >> 5] >> (b & 31)) & 1u);
+    }
+    const unsigned lb = __ballot_sync(kFull, live);
+    int at = 0;
+    if ((tid & 31) == 0 && lb) at = atomicAdd(p.live_cnt, __popc(lb));
+    at = __shfl_sync(kFull, at, 0);
+    if (live) p.live[at + __popc(lb & ((1u << (tid & 31)) - 1))] = (uint32_t)(slot * p.nper + j);
+  }
   bool one_alive = false;
   for (int i = 0; i < nel; i++) one_alive |= !((s_dead[i >> 5] >> (i & 31)) & 1u);
 
@@ -714,8 +800,6 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   for (int x = tid; x < p.mask_w; x += kThreads) gm[x] = sm[x];
   uint64_t* go = p.o_mask + (size_t)slot * p.orb_w;
   for (int x = tid; x < p.orb_w; x += kThreads) go[x] = so[x];
-  uint32_t* dead = p.b_dead + (size_t)slot * dw;
-  for (int w = tid; w < dw; w += kThreads) dead[w] = s_dead[w];
   __syncthreads();
   ulonglong2* e_hp = p.e_hp + (size_t)slot * (size_t)p.ent_cap;
   uint32_t* e_rec = p.e_rec + (size_t)slot * (size_t)p.ent_cap;
@@ -784,26 +868,34 @@ __global__ void __launch_bounds__(kThreads) prep_multi_kernel(const __grid_const
 // ---------------------------------------------------------------------------
 template <int NINT, typename NT>
 struct BatchShared {
-  uint64_t I[2 * NINT];
   int occ[kMaxElec];
-  int vir[2][kMaxOrb];
-  int vidx[2][kMaxOrb];
-  int nv[2];
-  // fixed point (den_scale): the Fock diagonal, per-batch row sums for H_aa
-  long long F[2][kMaxOrb];
-  long long u0[kMaxOrb], u1[kMaxOrb];
-  long long dx[kMaxOrb];            // E0 - base - u0[x]
-  // two-hole batches: <I|H|I - H + R> by the pair tables of the all-cell
-  // fast path, built for J = I (its X is the hole pair H itself)
+  // virtual orbitals of I by index and their indices by orbital (255: occupied)
+  unsigned char vir[2][kMaxOrb], vidx[2][kMaxOrb];
+  int nv[2];  // the sweep's virtual orbitals per spin
+  float inv_nv1;
+  // fixed point (den_scale): per-batch row sums for H_aa, E0 - base - u0[x]
+  long long u0[kMaxOrb], u1[kMaxOrb], dx[kMaxOrb];
+  // two-hole batches: <I|H|I - H + R> by pair tables like those of the J
+  // reaching every cell (its particles are the hole pair H itself)
   int iRow[kMaxOrb], iCol[kMaxOrb];
   NT cI;
-  long long hii, base;
-  float inv_nv1;
   uint64_t kbase[2 * NINT];  // I with the batch's holes removed
-  int g, slot;
-  long long item, inext, iend;
-  // storage of one phase of a work item at a time: the J lists of loops 2
-  // and 3, the selection histogram, the per-thread sums of the reduction
+  // rows (and columns) of cells banned as a whole by J ranked before I, bits
+  // by orbital
+  uint64_t rowban[2 * NINT];
+  // the item's records and bucket entries (kept here, not in registers, over
+  // the phases that do not touch them): words, coefficients, hole masks and
+  // particle words; entries; the lists' offsets and first positions
+  const uint64_t *rw, *rhm, *rpt;
+  const double* rc;
+  const ulonglong2* ehp;
+  const uint32_t* erec;
+  int seg_o[4], seg_s[4];
+  Batch bt;  // the item's batch, read again by each phase
+  int item[2];        // this work item and the next (-1: none)
+  int inext, iend, nlive;  // positions left of the last draw; live items of the wave
+  // storage of one phase of a work item at a time: the J lists, the
+  // selection histogram, the per-thread sums of the reduction
   union {
     struct {
       // records of the J reaching every cell; of the J reaching rows (from
@@ -814,14 +906,13 @@ struct BatchShared {
     double red_t[2][kThreads];  // per-thread e and (A/D)^2 sums of the item
   } u;
   int n0, n1, n2;
-  int cnext;  // next row-reaching J (then subset block) to draw
-  // a group of J reaching every cell, processed by the whole CTA
-  uint64_t gJw[kGroup][2 * NINT];
+  int cnext;  // next unit of the row pass to draw
+  // a group of J reaching every cell, J = K + {x1, x2}: per particle orbital
+  // of each slot the offset of its integrals, with the phase parity in bit 31
+  // and, for the particles of J, bit 30 (the gradient's per-orbital weights
+  // use the same storage in the cells pass and after loop 3)
   NT gcj[kGroup];
-  // two-hole batches: J = K + {x1, x2}; per particle orbital of each slot the
-  // pair index tri(x, r) with the phase parity in bit 31
-  // (loop 2); the gradient's per-orbital weights use the same storage in
-  // the cells pass and after loop 3
+  int gx2[kGroup], gB[kGroup];
   union {
     struct {
       int gRow[kGroup][kMaxOrb], gCol[kGroup][kMaxOrb];
@@ -830,13 +921,6 @@ struct BatchShared {
       double rowW2[kMaxOrb], colW2[kMaxOrb];  // sums of (A/D)^2 over the cells of each particle orbital
     } w;
   } v;
-  int gx1[kGroup], gx2[kGroup], gsr[kGroup], gsc[kGroup];
-  // four-index layout: the slab of each J's pair (x1, x2) and of the batch's
-  // holes; the pair tables then hold orbitals, not pair indices
-  int gB[kGroup], ibase;
-  // two-hole batches: bit x of frow (fcol) set when row
-  // (column) x of cells is banned as a whole by a J ranked before I
-  uint32_t frow[kMaxOrb / 32], fcol[kMaxOrb / 32];
   int wsum[kWarps];
   // selection
   int tkcnt;
@@ -844,21 +928,13 @@ struct BatchShared {
   uint64_t pw[1 + 2 * NINT];
   uint64_t thr[1 + 2 * NINT];
   int need, group, found_w, found_sh;
-  // reductions
-  unsigned long long red_u[kWarps][6];
+  // reductions: warps that finished the item, their counts
+  int arrive;
+  unsigned long long red_na[kWarps], red_con[kWarps];
   double sw2;
-};
-
-struct Batch {
-  int h;            // number of holes (1, 2)
-  int kind;         // 0 single, 1 same-spin double, 2 opposite-spin double
-  int ia, ib;       // occupied indices of the holes in I
-  int ca, cb;       // their spin-orbital codes
-  int sa, sb;       // their spins
-  int qa, qb;       // their orbitals
-  uint64_t hm;      // hole mask over I's occupied list
-  int ncell;
-  int clo, nct;     // this work item's cells: [clo, clo + nct) (a tile of the batch)
+  // totals of this thread over the sweep: digest sum and xor, min |D|, |A| < 1e-14
+  unsigned long long td0[kThreads], td1[kThreads], tmin[kThreads];
+  uint32_t ttiny[kThreads];
 };
 
 template <int NINT, typename NT>
@@ -945,22 +1021,33 @@ __device__ __forceinline__ void for_subset_cells(const Batch& B, const BatchShar
   }
 }
 
+// True when the row (column) of cells holding orbital q of spin s is banned
+// as a whole (two-hole batches).
+template <int NINT, typename NT>
+__device__ __forceinline__ bool row_banned(const BatchShared<NINT, NT>& S, int s, int q) {
+  return (S.rowban[s * NINT + (q >> 6)] >> (q & 63)) & 1ull;
+}
+
 // True when some cell inside the particles of J lies in this item's tile and
 // is not banned: a J with t = 2 that reaches no such cell adds nothing and is
-// dropped at classification (most of them: their one cell is usually banned
-// by an earlier generator, or its spins do not match the batch's).
+// dropped at classification.  Rows banned as a whole are tested by their
+// flags (their cells may not be in the ban bits yet).
 template <int NINT, typename NT>
 __device__ __forceinline__ bool subset_live(const Batch& B, const BatchShared<NINT, NT>& S, int norb,
                                             uint64_t part, const uint32_t* ban) {
   bool live = false;
+  if (B.h == 2)
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const int c = part_code(part, i), s = c >= norb;
+      if (c != kNoPart && row_banned<NINT, NT>(S, s, c - s * norb)) part |= 0x7FFFull << (16 * i);
+    }
   for_subset_cells<NINT, NT>(B, S, norb, part, [&](int c) {
     const int cc = c - B.clo;
     live |= (unsigned)cc < (unsigned)B.nct && !((ban[cc >> 5] >> (cc & 31)) & 1u);
   });
   return live;
 }
-
-__device__ __forceinline__ bool flagged(const uint32_t* f, int x) { return (f[x >> 5] >> (x & 31)) & 1u; }
 
 // True when some row or column of cells that a J with t = 1 reaches (the
 // rows of its particles) is not banned as a whole.  Rows flagged in loop 1
@@ -975,8 +1062,7 @@ __device__ __forceinline__ bool row_live(const Batch& B, const BatchShared<NINT,
     const int c = part_code(part, i);
     if (c == kNoPart) continue;
     const int s = c >= norb, q = c - s * norb;
-    if (B.kind == 2) live |= !flagged(s ? S.fcol : S.frow, S.vidx[s][q]);
-    else if (s == B.sa) live |= !flagged(S.frow, S.vidx[s][q]);
+    if (B.kind == 2 || s == B.sa) live |= !row_banned<NINT, NT>(S, s, q);
   }
   return live;
 }
@@ -995,7 +1081,7 @@ __device__ __forceinline__ void for_row_cells(const Batch& B, const BatchShared<
     const int nv = S.nv[B.sa];
     for (int i = 0; i < np; i++) {
       const int x = S.vidx[B.sa][pk(P, i)];
-      if (flagged(S.frow, x)) continue;
+      if (row_banned<NINT, NT>(S, B.sa, pk(P, i))) continue;
       for (int y = lane; y < nv; y += 32) {
         if (y == x) continue;
         bool dup = false;  // pair {P[j], P[i]}, j < i, was visited from P[j]
@@ -1010,12 +1096,12 @@ __device__ __forceinline__ void for_row_cells(const Batch& B, const BatchShared<
     const int nv0 = S.nv[0], nv1 = S.nv[1];
     for (int i = 0; i < na; i++) {
       const int x = S.vidx[0][pk(Pa, i)];
-      if (flagged(S.frow, x)) continue;
+      if (row_banned<NINT, NT>(S, 0, pk(Pa, i))) continue;
       for (int y = lane; y < nv1; y += 32) fn(x * nv1 + y, pk(Pa, i), norb + S.vir[1][y]);
     }
     for (int j = 0; j < nb; j++) {
       const int y = S.vidx[1][pk(Pb, j)];
-      if (flagged(S.fcol, y)) continue;
+      if (row_banned<NINT, NT>(S, 1, pk(Pb, j))) continue;
       for (int x = lane; x < nv0; x += 32) {
         bool dup = false;  // rows of Pa were visited above
         for (int i = 0; i < na; i++) dup |= (S.vidx[0][pk(Pa, i)] == x);
@@ -1051,66 +1137,29 @@ __device__ __forceinline__ void excitation_sets(const Batch& B, const BatchShare
   *nt = b;
 }
 
-// <J|H|alpha> with alpha = K + R, K = I - H.
-// holes(J -> alpha) = X - R, particles = T + (R - X).
-// Kept out of line: one copy serves every caller, which keeps the batch
-// kernel's code small enough for the instruction cache.
-// Jw points to the record's words in global or shared memory; the sets are
-// packed codes; nothing is passed through local memory.
+// <J|H|alpha> for the double substitution u0 u1 -> q0 q1 of J (spin-orbital
+// codes, u0 < u1 occupied, q0 < q1 empty).
 template <int NINT, typename NT, bool E4>
-__device__ __noinline__ NT element(const NT* eri, const NT* hh, int norb, const uint64_t* Jw, uint32_t X, int nx,
-                                   uint32_t T, int nt, int r, int s) {
-  int ho[2], pa[2], nh = 0, npp = 0;
-  bool r_in = false, s_in = false;
-  for (int i = 0; i < nx; i++) {
-    const int x = pk(X, i);
-    r_in |= (x == r);
-    s_in |= (x == s);
-    if (x != r && x != s && nh < 2) ho[nh++] = x;
-  }
-  for (int i = 0; i < nt && npp < 2; i++) pa[npp++] = pk(T, i);
-  if (!r_in && npp < 2) pa[npp++] = r;
-  if (s >= 0 && !s_in && npp < 2) pa[npp++] = s;
-  if (nh == 0 || nh != npp) return NT(0);  // not reached: such cells are banned
-  if (nh == 1) {
-    const int sp = ho[0] >= norb, a = ho[0] - sp * norb, b = pa[0] - sp * norb;
-    const uint64_t* sw = Jw + sp * NINT;
-    const int lo = a < b ? a : b, hi = a < b ? b : a;
-    const bool neg = count_between<NINT>(sw, lo, hi) & 1;
-    NT v = hh[a * norb + b];
+__device__ __forceinline__ NT double_element(const NT* eri, int norb, const uint64_t* Jw, int u0, int u1, int q0,
+                                             int q1) {
+  const int s1 = u0 >= norb, s2 = u1 >= norb;
+  const int h1 = u0 - s1 * norb, p1 = q0 - s1 * norb;
+  const int h2 = u1 - s2 * norb, p2 = q1 - s2 * norb;
+  uint64_t w1[NINT], w2[NINT];
 #pragma unroll
-    for (int t = 0; t < 2; t++) {
-#pragma unroll
-      for (int w = 0; w < NINT; w++) {
-        uint64_t bits = Jw[t * NINT + w];
-        while (bits) {
-          const int q = 64 * w + __ffsll((long long)bits) - 1;
-          bits &= bits - 1;
-          v += eri[gidx<E4>(a, b, q, q, norb)];
-          if (t == sp) v -= eri[gidx<E4>(a, q, q, b, norb)];
-        }
-      }
+  for (int w = 0; w < NINT; w++) {
+    w1[w] = s1 ? Jw[NINT + w] : Jw[w];
+    w2[w] = s2 ? Jw[NINT + w] : Jw[w];
+    if (s1 == s2) {  // the second substitution counts on the result of the first
+      if ((h1 >> 6) == w) w2[w] &= ~(1ull << (h1 & 63));
+      if ((p1 >> 6) == w) w2[w] |= 1ull << (p1 & 63);
     }
-    return flip_sign(v, neg);
   }
-  // double: order holes and particles by spin-orbital code, pair 1-1, 2-2
-  if (ho[0] > ho[1]) { const int t = ho[0]; ho[0] = ho[1]; ho[1] = t; }
-  if (pa[0] > pa[1]) { const int t = pa[0]; pa[0] = pa[1]; pa[1] = t; }
-  const int s1 = ho[0] >= norb, s2 = ho[1] >= norb;
-  const int h1 = ho[0] - s1 * norb, p1 = pa[0] - s1 * norb;
-  const int h2 = ho[1] - s2 * norb, p2 = pa[1] - s2 * norb;
-  uint64_t w1[NINT];
-#pragma unroll
-  for (int w = 0; w < NINT; w++) w1[w] = Jw[s1 * NINT + w];
-  const int n1 = count_between<NINT>(w1, h1 < p1 ? h1 : p1, h1 < p1 ? p1 : h1);
-  // apply h1 -> p1, then count for h2 -> p2 on the result
-  w1[h1 >> 6] &= ~(1ull << (h1 & 63));
-  w1[p1 >> 6] |= (1ull << (p1 & 63));
-  const int n2 = (s2 == s1) ? count_between<NINT>(w1, h2 < p2 ? h2 : p2, h2 < p2 ? p2 : h2)
-                            : count_between<NINT>(Jw + s2 * NINT, h2 < p2 ? h2 : p2, h2 < p2 ? p2 : h2);
+  const int n = count_between<NINT>(w1, h1 < p1 ? h1 : p1, h1 < p1 ? p1 : h1) +
+                count_between<NINT>(w2, h2 < p2 ? h2 : p2, h2 < p2 ? p2 : h2);
   NT v = eri[gidx<E4>(h1, p1, h2, p2, norb)];
   if (s1 == s2) v -= eri[gidx<E4>(h1, p2, h2, p1, norb)];
-  return flip_sign(v, (n1 + n2) & 1);
+  return flip_sign(v, n & 1);
 }
 
 // Phases of the substitutions u -> z of a string w (NINT words, u occupied)
@@ -1400,11 +1449,10 @@ __device__ __noinline__ void compact_selection(const SweepParams& p, BatchShared
 // and kept across work items.  Multi-state form: one FP64 accumulator per
 // state (stride mc), then the ban bits, the CTA group's coefficients per
 // state, c_I per state and the weights w_s; one-state form: the exact 96-bit
-// accumulators (low words, then high words), then the ban bits.
+// accumulators (their low, middle and high words), then the ban bits.
 struct ItemEnv {
   double* A;
-  unsigned long long* Alo;
-  int* Ahi;
+  uint32_t *A0, *A1, *A2;
   uint32_t* ban;
   double *ms_gc, *ms_cI, *ms_w;
   long long* ms_de;  // E0_s - E0_0, fixed point
@@ -1419,9 +1467,10 @@ __device__ __forceinline__ ItemEnv item_env(const SweepParams& p) {
   ItemEnv E;
   E.mc = p.max_cells;
   E.A = reinterpret_cast<double*>(dyn);
-  E.Alo = reinterpret_cast<unsigned long long*>(dyn);
-  E.Ahi = reinterpret_cast<int*>(E.Alo + E.mc);
-  E.ban = MS ? reinterpret_cast<uint32_t*>(E.A + p.nst * E.mc) : reinterpret_cast<uint32_t*>(E.Ahi + ((E.mc + 1) & ~1));
+  E.A0 = reinterpret_cast<uint32_t*>(dyn);
+  E.A1 = E.A0 + E.mc;
+  E.A2 = E.A1 + E.mc;
+  E.ban = MS ? reinterpret_cast<uint32_t*>(E.A + p.nst * E.mc) : E.A2 + ((E.mc + 1) & ~1);
   E.ms_gc = reinterpret_cast<double*>(E.ban + (((E.mc + 31) / 32 + 1) & ~1));
   E.ms_cI = E.ms_gc + kGroup * kMaxStates;
   E.ms_w = E.ms_cI + kMaxStates;
@@ -1440,14 +1489,31 @@ __device__ __forceinline__ ItemEnv item_env(const SweepParams& p) {
 // row tile of one): bans, the accumulation of A_alpha, the cells pass and the
 // item's sums.  Used by the kernel of one sweep and by the kernel whose queue
 // spans the waves of several instances.
+//
+// What bounds an item is latency, not a pipe (issue slots half used, FP64
+// 23%): 256 threads share about 2,000 cells, and every phase that few of them
+// work in, every dependent global load and every barrier shows.  So the
+// set-up reads the generator straight from global memory in two dependent
+// steps, the first round of bucket entries is in registers before the bans
+// are, tables of the J reaching every cell are units of the row pass, their
+// terms are formed in the cells pass, and the item's sums are finished by the
+// last warp to arrive while the others begin the next item: five barriers
+// where there were fifteen.
+// This CTA's candidate buffers of the selection.
+__device__ __forceinline__ double* buf_e(const SweepParams& p) { return p.tk_e + (size_t)blockIdx.x * (size_t)p.cap; }
+__device__ __forceinline__ double* buf_a(const SweepParams& p) { return p.tk_a + (size_t)blockIdx.x * (size_t)p.cap; }
+template <int NINT>
+__device__ __forceinline__ uint64_t* buf_key(const SweepParams& p) {
+  return p.tk_key + (size_t)blockIdx.x * (size_t)p.cap * (2 * NINT);
+}
+
 template <int NINT, typename NT, bool GRAD, bool MS, bool E4>
 __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NINT, NT>& S, const long long item,
-                                           const int F, double* te, double* ta, uint64_t* tk, const ItemEnv& E,
+                                           const int F, const ItemEnv& E,
                                            const NT* eri_n, const NT* h_n) {
   constexpr int NW = 2 * NINT;
-  double* A = E.A;
-  unsigned long long* Alo = E.Alo;
-  int* Ahi = E.Ahi;
+  double* A = E.A;  // multi-state form
+  uint32_t *A0 = E.A0, *A1 = E.A1, *A2 = E.A2;
   uint32_t* ban = E.ban;
   double* ms_gc = E.ms_gc;
   double* ms_cI = E.ms_cI;
@@ -1458,237 +1524,158 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   const int norb = E.norb, nel = E.nel, nbat = E.nbat;
   const int nper = E.nper;
 
-  const int slot = (int)(item / nper), j = (int)(item - (long long)slot * nper);
-  // item j < nbat: batch j (the first row tile of a split batch); j >= nbat:
-  // row tile 1 + (j - nbat) / (n_alpha n_beta) of opposite-spin batch
-  // (j - nbat) % (n_alpha n_beta)
-  int b = j, tile = 0;
-  if (j >= nbat) {
-    const int na = p.nalpha, nab = p.nalpha * p.nbeta;
-    const int k = (j - nbat) % nab;
-    tile = 1 + (j - nbat) / nab;
-    const int ia = k % na, ib = na + k / na;
-    b = nel + ib * (ib - 1) / 2 + ia;
-  }
-  const GenMeta* M = p.meta + slot;
-  if (M->g < 0) return;
-  if ((p.b_dead[(size_t)slot * ((nbat + 31) / 32) + (b >> 5)] >> (b & 31)) & 1u) return;
-  if (slot != S.slot) {  // load the generator
-    __syncthreads();
-    if (tid < NW) S.I[tid] = M->I[tid];
-    if (tid < nel) S.occ[tid] = M->occ[tid];
-    for (int x = tid; x < 2 * norb; x += kThreads) S.F[x / norb][x % norb] = M->F[x / norb][x % norb];
-    __syncthreads();
-    for (int x = tid; x < 2 * norb; x += kThreads) {
-      const int s = x / norb, q = x - s * norb;
-      const uint64_t* sw = S.I + s * NINT;
-      const bool occ = (sw[q >> 6] >> (q & 63)) & 1ull;
-      int below = 0;  // occupied orbitals of spin s below q
-#pragma unroll
-      for (int w = 0; w < NINT; w++) {
-        const int lim = q - 64 * w;
-        if (lim >= 64) below += __popcll(sw[w]);
-        else if (lim > 0) below += __popcll(sw[w] & ((1ull << lim) - 1));
-      }
-      const int v = q - below;
-      S.vidx[s][q] = occ ? -1 : v;
-      if (!occ) S.vir[s][v] = q;
-    }
-    if (tid < 2) {
-      int n = 0;
-#pragma unroll
-      for (int w = 0; w < NINT; w++) n += __popcll(S.I[tid * NINT + w]);
-      S.nv[tid] = norb - n;
-    }
-    if (tid == 0) {
-      S.hii = M->hii;
-      S.cI = (NT)M->cI;
-      S.g = M->g;
-      S.slot = slot;
-    }
-    if constexpr (MS) {
-      if (tid < nst) {
-        ms_cI[tid] = p.coefs[(size_t)tid * p.ndet + p.order[M->g]];
-        const double m = __longlong_as_double((long long)p.st_cmax[tid]);
-        ms_w[tid] = 1.0 / (m * m);
-        ms_de[tid] = den_fix(p.st_e0[tid], E.dscale) - E.e0;
-      }
-    }
-    __syncthreads();
-  }
-  const int g = S.g;
-
-  // ---- batch geometry ----
+  const int slot = (int)(item / nper), jitem = (int)(item - (long long)slot * nper);
+  int tile;
+  const int b = item_batch(p, jitem, &tile);
   Batch B;
-  if (b < nel) {
-    B.h = 1;
-    B.ia = b;
-    B.ib = -1;
-  } else {
-    const int t = b - nel;
-    int y = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)t)) * 0.5f);
-    while (y * (y - 1) / 2 > t) y--;
-    while ((y + 1) * y / 2 <= t) y++;
-    B.h = 2;
-    B.ib = y;
-    B.ia = t - y * (y - 1) / 2;
-  }
-  B.ca = S.occ[B.ia];
-  B.sa = B.ca >= norb;
-  B.qa = B.ca - B.sa * norb;
-  B.hm = 1ull << B.ia;
-  if (B.h == 2) {
-    B.cb = S.occ[B.ib];
-    B.sb = B.cb >= norb;
-    B.qb = B.cb - B.sb * norb;
-    B.hm |= 1ull << B.ib;
-    B.kind = (B.sa == B.sb) ? 1 : 2;
-    const int nv = S.nv[B.sa];
-    B.ncell = (B.kind == 1) ? nv * (nv - 1) / 2 : S.nv[0] * S.nv[1];
-  } else {
-    B.cb = -1;
-    B.sb = -1;
-    B.qb = -1;
-    B.kind = 0;
-    B.ncell = S.nv[B.sa];
-  }
-  B.clo = 0;
-  B.nct = B.ncell;
-  if (p.ntile > 1 && B.kind == 2) {  // rows [tile h, min((tile + 1) h, nv0))
-    const int h = (S.nv[0] + p.ntile - 1) / p.ntile;
-    const int r0 = tile * h, r1 = min(r0 + h, S.nv[0]);
-    B.clo = r0 * S.nv[1];
-    B.nct = (r1 - r0) * S.nv[1];
-  }
-  if (B.nct <= 0) return;
+  batch_geometry(p, b, tile, B);
+  const GenMeta* M = p.meta + slot;
 
+  // ---- set-up ----
   // bucket lists (prep_slot): this batch's bucket (a one-hole batch's is its
   // hole's list), for a two-hole batch the lists of its two holes (a record
   // holding both is in the batch's bucket), then the shared list (a record
   // with a hole of the batch is in that hole's list)
   const int* ofs = p.b_ofs + (size_t)slot * (nbat + 2);
-  const int ob = ofs[b], nb_ = ofs[b + 1] - ob, oa = ofs[nbat], na_ = ofs[nbat + 1] - oa;
-  const int o1 = (B.h == 2) ? ofs[B.ia] : 0, n1_ = (B.h == 2) ? ofs[B.ia + 1] - o1 : 0;
-  const int o2 = (B.h == 2) ? ofs[B.ib] : 0, n2_ = (B.h == 2) ? ofs[B.ib + 1] - o2 : 0;
-  const int s1 = nb_, s2 = s1 + n1_, s3 = s2 + n2_;
-  const int total = s3 + na_;
-  const size_t rb = (size_t)slot * (size_t)p.ndet;
-  const uint64_t* rw = p.r_words + rb * NW;
-  const double* rc = p.r_coef + rb;
-  const uint64_t* rhm = p.r_hmask + rb;  // hole mask and particle word of each record
-  const uint64_t* rpt = p.r_part + rb;
   const size_t eb = (size_t)slot * (size_t)p.ent_cap;
-  const ulonglong2* ehp = p.e_hp + eb;
-  const uint32_t* erec = p.e_rec + eb;
+  ulonglong2 en0 = make_ulonglong2(0ull, 0ull);  // this thread's entry of the first round
+  uint32_t rec0 = 0;
+  {
+    const int ob = ofs[b], nb_ = ofs[b + 1] - ob, oa = ofs[nbat], na_ = ofs[nbat + 1] - oa;
+    const int o1 = (B.h == 2) ? ofs[B.ia] : 0, n1_ = (B.h == 2) ? ofs[B.ia + 1] - o1 : 0;
+    const int o2 = (B.h == 2) ? ofs[B.ib] : 0, n2_ = (B.h == 2) ? ofs[B.ib + 1] - o2 : 0;
+    const int s1 = nb_, s2 = s1 + n1_, s3 = s2 + n2_, s4 = s3 + na_;
+    if (tid < s4) {
+      const int o = tid < s1 ? ob + tid : (tid < s2 ? o1 + tid - s1 : (tid < s3 ? o2 + tid - s2 : oa + tid - s3));
+      en0 = p.e_hp[eb + o];
+      rec0 = p.e_rec[eb + o];
+    }
+    if (tid == 0) {
+      S.seg_o[0] = ob;
+      S.seg_o[1] = o1 - s1;
+      S.seg_o[2] = o2 - s2;
+      S.seg_o[3] = oa - s3;
+      S.seg_s[0] = s1;
+      S.seg_s[1] = s2;
+      S.seg_s[2] = s3;
+      S.seg_s[3] = s4;
+      const size_t rb = (size_t)slot * (size_t)p.ndet;
+      S.rw = p.r_words + rb * NW;
+      S.rc = p.r_coef + rb;
+      S.rhm = p.r_hmask + rb;
+      S.rpt = p.r_part + rb;
+      S.ehp = p.e_hp + eb;
+      S.erec = p.e_rec + eb;
+    }
+  }
+  unsigned long long gtau = 0;
+  if (p.k > 0 && tid == 0) gtau = *((volatile unsigned long long*)p.tau_bits);
   // position of the i-th entry of this batch in the slot's entry arrays
   auto entry = [&](int i) {
-    return i < s1 ? ob + i : (i < s2 ? o1 + i - s1 : (i < s3 ? o2 + i - s2 : oa + i - s3));
+    return i + S.seg_o[i < S.seg_s[0] ? 0 : i < S.seg_s[1] ? 1 : i < S.seg_s[2] ? 2 : 3];
   };
   auto dup = [&](int i, uint64_t hm) {
-    return i >= s1 && (i < s3 ? (hm & B.hm) == B.hm : (hm & B.hm) != 0ull);
+    return i >= S.seg_s[0] && (i < S.seg_s[2] ? (hm & B.hm) == B.hm : (hm & B.hm) != 0ull);
   };
-
-  if (tid == 0) {
-    S.inv_nv1 = S.nv[1] > 0 ? 1.0f / (float)S.nv[1] : 0.0f;
+  B.ca = M->occ[B.ia];
+  B.qa = B.ca - B.sa * norb;
+  B.cb = B.h == 2 ? M->occ[B.ib] : -1;
+  B.qb = B.h == 2 ? B.cb - B.sb * norb : -1;
+  const int ibase = B.h == 2 ? (B.qa * norb + B.qb) * norb * norb : 0;
+  for (int x = tid; x < 2 * norb; x += kThreads) {  // a thread per orbital and spin
+    const int s = x >= norb, q = x - s * norb;
+    uint64_t sw[NINT];
+    int below = 0;  // occupied orbitals of spin s below q
 #pragma unroll
-    for (int w = 0; w < NW; w++) S.kbase[w] = S.I[w];
+    for (int w = 0; w < NINT; w++) {
+      sw[w] = M->I[s * NINT + w];
+      const int lim = q - 64 * w;
+      if (lim >= 64) below += __popcll(sw[w]);
+      else if (lim > 0) below += __popcll(sw[w] & ((1ull << lim) - 1));
+    }
+    if (mask_bit<NINT>(sw, q)) {
+      S.vidx[s][q] = 255;
+      continue;
+    }
+    const int v = q - below;
+    S.vidx[s][q] = (unsigned char)v;
+    S.vir[s][v] = (unsigned char)q;
+    auto W = [&](int y, int sy) { return (s == sy ? p.Wi : p.Ji)[q * norb + y]; };
+    const bool isrow = s == B.sa, iscol = B.h == 2 && s == B.sb;
+    if (isrow || iscol) {
+      long long u = M->F[s][q] - W(B.qa, B.sa);
+      if (B.h == 2) u -= W(B.qb, B.sb);
+      if (isrow) {  // E0 - base - u0, base = H_II - F(a) [- F(b) + W(a, b)]
+        long long base = M->hii - M->F[B.sa][B.qa];
+        if (B.h == 2) base += (B.kind == 1 ? p.Wi : p.Ji)[B.qa * norb + B.qb] - M->F[B.sb][B.qb];
+        S.u0[v] = u;
+        S.dx[v] = (E.e0 - base) - u;
+      }
+      if (iscol) S.u1[v] = u;
+      if (B.h == 2) {  // pair tables of J = I: its particles x1, x2 are the holes a, b
+        if (isrow) {
+          const int par = count_between<NINT>(sw, q < B.qa ? q : B.qa, q < B.qa ? B.qa : q) & 1;
+          S.iRow[v] = (E4 ? ibase + q * norb : tri(B.qa, q)) | (par << 31);
+        }
+        if (iscol) {
+          const int lo = q < B.qb ? q : B.qb, hi = q < B.qb ? B.qb : q;
+          int par = count_between<NINT>(sw, lo, hi) & 1;
+          if (B.kind == 1) par ^= (B.qa > lo && B.qa < hi) ? 1 : 0;
+          S.iCol[v] = (E4 ? q : tri(B.qb, q)) | (par << 31);
+        }
+      }
+    }
+  }
+  if (tid < nel) S.occ[tid] = M->occ[tid];
+  if (lane == 0) S.red_con[warp] = 0ull;
+  if (tid == 0) {
+    S.bt = B;
+    S.cI = (NT)M->cI;
+    S.n0 = S.n1 = S.n2 = S.cnext = 0;
+#pragma unroll
+    for (int w = 0; w < NW; w++) S.kbase[w] = M->I[w];
     S.kbase[B.sa * NINT + (B.qa >> 6)] &= ~(1ull << (B.qa & 63));
     if (B.h == 2) S.kbase[B.sb * NINT + (B.qb >> 6)] &= ~(1ull << (B.qb & 63));
   }
-  // zero the accumulator, the bans; row sums for H_aa
   if constexpr (MS) {
+    if (tid < nst) {
+      ms_cI[tid] = p.coefs[(size_t)tid * p.ndet + p.order[M->g]];
+      const double m = __longlong_as_double((long long)p.st_cmax[tid]);
+      ms_w[tid] = 1.0 / (m * m);
+      ms_de[tid] = den_fix(p.st_e0[tid], E.dscale) - E.e0;
+    }
     for (int st = 0; st < nst; st++)
       for (int c = tid; c < B.nct; c += kThreads) A[st * mc + c] = 0.0;
   } else {
-    for (int c = tid; c < B.nct; c += kThreads) {
-      Alo[c] = 0ull;
-      Ahi[c] = 0;
-    }
+    for (int c = tid; c < B.nct; c += kThreads) A0[c] = A1[c] = A2[c] = 0u;
   }
   // bans by J ranked before I: the masks of the slot and the batch's holes
-  {
+  const uint64_t* om = p.o_mask + (size_t)slot * p.orb_w;
+  if (B.h == 2) {
     const MaskDims md = mask_dims(norb, p.nalpha, p.nbeta);
-    const uint64_t* om = p.o_mask + (size_t)slot * p.orb_w;
-    if (B.kind == 0) {
-      const uint64_t *b1 = om + (2 + B.sa) * NINT, *h1 = om + (6 + 3 * B.ia) * NINT;
-      for (int c0 = 0; c0 < B.nct; c0 += kThreads) {
-        const int c = c0 + tid, r = c < B.nct ? S.vir[B.sa][c] : 0;
-        const unsigned f = __ballot_sync(kFull, c < B.nct && (((b1[r >> 6] | h1[r >> 6]) >> (r & 63)) & 1ull));
-        if (lane == 0 && c < B.nct) ban[c >> 5] = f;
-      }
-    } else {
-      const uint32_t* gm = p.b_mask + (size_t)slot * p.mask_w;
-      const int mbase = md.ca + md.cb + md.cm, mix = md.ca > md.cb ? md.ca : md.cb;
-      const uint32_t* m0 = gm + (B.kind == 2 ? md.ca + md.cb : B.sa ? md.ca : 0);
-      const uint32_t* m1 = gm + mbase + B.ia * md.hs + (B.kind == 2 ? mix : 0);
-      const uint32_t* m2 = gm + mbase + B.ib * md.hs + (B.kind == 2 ? mix : 0);
-      const int nw32 = (B.ncell + 31) / 32;
-      auto word = [&](int w) { return w < nw32 ? m0[w] | m1[w] | m2[w] : 0u; };
-      for (int w = tid; w < (B.nct + 31) / 32; w += kThreads) {
-        const int at = (B.clo >> 5) + w;
-        ban[w] = __funnelshift_r(word(at), (B.clo & 31) ? word(at + 1) : 0u, B.clo & 31);
-      }
-      // rows (and columns) banned as a whole, as bits of virtual indices
-      static_assert(kWarps >= 2 * (kMaxOrb / 32), "one warp per mask word");
-      if (warp < 2 * (kMaxOrb / 32)) {
-        const int s = B.kind == 2 ? warp / (kMaxOrb / 32) : B.sa, w = warp % (kMaxOrb / 32), x = 32 * w + lane;
-        bool f = false;
-        if (x < S.nv[s]) {
-          const int r = S.vir[s][x], o = s * NINT + (r >> 6);
-          f = ((om[o] | om[(4 + 3 * B.ia) * NINT + o] | om[(4 + 3 * B.ib) * NINT + o]) >> (r & 63)) & 1ull;
-        }
-        const unsigned fb = __ballot_sync(kFull, f);
-        if (lane == 0) (warp < kMaxOrb / 32 ? S.frow : S.fcol)[w] = fb;
-      }
+    const uint32_t* gm = p.b_mask + (size_t)slot * p.mask_w;
+    const int mbase = md.ca + md.cb + md.cm, mix = md.ca > md.cb ? md.ca : md.cb;
+    const uint32_t* m0 = gm + (B.kind == 2 ? md.ca + md.cb : B.sa ? md.ca : 0);
+    const uint32_t* m1 = gm + mbase + B.ia * md.hs + (B.kind == 2 ? mix : 0);
+    const uint32_t* m2 = gm + mbase + B.ib * md.hs + (B.kind == 2 ? mix : 0);
+    const int nw32 = (B.ncell + 31) / 32;
+    auto word = [&](int w) { return w < nw32 ? m0[w] | m1[w] | m2[w] : 0u; };
+    for (int w = tid; w < (B.nct + 31) / 32; w += kThreads) {
+      const int at = (B.clo >> 5) + w;
+      ban[w] = __funnelshift_r(word(at), (B.clo & 31) ? word(at + 1) : 0u, B.clo & 31);
     }
-  }
-  {
-    auto W = [&](int x, int sx, int y, int sy) { return (sx == sy ? p.Wi : p.Ji)[x * norb + y]; };
-    if (B.kind == 0) {
-      const int s = B.sa;
-      for (int x = tid; x < S.nv[s]; x += kThreads) {
-        const int r = S.vir[s][x];
-        S.u0[x] = S.F[s][r] - W(r, s, B.qa, s);
-      }
-      if (tid == 0) S.base = S.hii - S.F[s][B.qa];
-    } else {
-      const int s1 = B.sa, s2 = B.sb;
-      for (int x = tid; x < S.nv[s1]; x += kThreads) {
-        const int r = S.vir[s1][x];
-        S.u0[x] = S.F[s1][r] - W(r, s1, B.qa, s1) - W(r, s1, B.qb, s2);
-      }
-      if (B.kind == 2)
-        for (int y = tid; y < S.nv[s2]; y += kThreads) {
-          const int s = S.vir[s2][y];
-          S.u1[y] = S.F[s2][s] - W(s, s2, B.qa, s1) - W(s, s2, B.qb, s2);
-        }
-      if (tid == 0) {
-        S.base = S.hii - S.F[s1][B.qa] - S.F[s2][B.qb] + W(B.qa, s1, B.qb, s2);
-        S.ibase = (B.qa * norb + B.qb) * norb * norb;
-      }
-      // pair tables of J = I: rows tri(qa, r) and columns tri(qb, s) with
-      // the phases of qa -> r and qb -> s on I's strings
-      const int sl2 = (B.kind == 2) ? 1 : s1;
-      const int nva = S.nv[s1];
-      for (int v = tid; v < nva + S.nv[sl2]; v += kThreads) {
-        if (v < nva) {
-          const int r = S.vir[s1][v];
-          const int par = count_between<NINT>(S.I + s1 * NINT, r < B.qa ? r : B.qa, r < B.qa ? B.qa : r) & 1;
-          S.iRow[v] = (E4 ? r : tri(B.qa, r)) | (par << 31);
-        } else {
-          const int sv = S.vir[sl2][v - nva];
-          int par = count_between<NINT>(S.I + sl2 * NINT, sv < B.qb ? sv : B.qb, sv < B.qb ? B.qb : sv) & 1;
-          if (B.kind == 1) {
-            const int lo = sv < B.qb ? sv : B.qb, hi = sv < B.qb ? B.qb : sv;
-            par ^= (B.qa > lo && B.qa < hi) ? 1 : 0;
-          }
-          S.iCol[v - nva] = (E4 ? sv : tri(B.qb, sv)) | (par << 31);
-        }
-      }
-    }
+    if (tid < NW) S.rowban[tid] = om[tid] | om[(4 + 3 * B.ia) * NINT + tid] | om[(4 + 3 * B.ib) * NINT + tid];
   }
   __syncthreads();
-  for (int x = tid; x < S.nv[B.sa]; x += kThreads) S.dx[x] = (E.e0 - S.base) - S.u0[x];
+  if (B.h == 1) {
+    const uint64_t *b1 = om + (2 + B.sa) * NINT, *h1 = om + (6 + 3 * B.ia) * NINT;
+    for (int c0 = 0; c0 < B.nct; c0 += kThreads) {
+      const int c = c0 + tid, r = c < B.nct ? S.vir[B.sa][c] : 0;
+      const unsigned f = __ballot_sync(kFull, c < B.nct && (((b1[r >> 6] | h1[r >> 6]) >> (r & 63)) & 1ull));
+      if (lane == 0 && c < B.nct) ban[c >> 5] = f;
+    }
+    __syncthreads();
+  }
   if (p.tgt_on) {  // cells outside the target space contribute nothing: ban them
     for (int cc = tid; cc < B.nct; cc += kThreads) {
       int ro, so, x, y;
@@ -1707,80 +1694,115 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       if (!ok) atomicOr(&ban[cc >> 5], 1u << (cc & 31));
     }
   }
-
   // ---- loop 1: bans by the entries of the batch's own bucket.  J ranked
   // before I: rows (t = 1) and cells (t = 2); a later J equal to a cell's
   // alpha bans that cell ----
-  for (int i = tid; i < nb_; i += kThreads) {
-    const ulonglong2 en = ehp[ob + i];
+  for (int i = tid; i < S.seg_s[0]; i += kThreads) {
+    const ulonglong2 en = i < kThreads ? en0 : S.ehp[S.seg_o[0] + i];
     const uint64_t hm = en.x, part = en.y;
-    if (part & kBeforeBit) {
-      if (__popcll(hm) == 3) {
-        int na_, nb2;
-        const uint32_t Pa = particles_of_spin(part, norb, B.kind == 2 ? 0 : B.sa, &na_);
-        for (int q = 0; q < na_; q++) {
-          const int x = S.vidx[B.kind == 2 ? 0 : B.sa][pk(Pa, q)];
-          atomicOr(&S.frow[x >> 5], 1u << (x & 31));
-        }
-        if (B.kind == 2) {
-          const uint32_t Pb = particles_of_spin(part, norb, 1, &nb2);
-          for (int q = 0; q < nb2; q++) {
-            const int x = S.vidx[1][pk(Pb, q)];
-            atomicOr(&S.fcol[x >> 5], 1u << (x & 31));
-          }
-        }
-      } else {
-        for_subset_cells<NINT, NT>(B, S, norb, part, [&](int c) { ban_cell(ban, B, c); });
+    if ((part & kBeforeBit) && __popcll(hm) == 3) {
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        const int c = part_code(part, k), s = c >= norb, q = c - s * norb;
+        if (B.kind == 2 || s == B.sa)
+          atomicOr(reinterpret_cast<unsigned long long*>(&S.rowban[s * NINT + (q >> 6)]), 1ull << (q & 63));
       }
-    } else if (hm == B.hm) {
+    } else if ((part & kBeforeBit) || hm == B.hm) {
       for_subset_cells<NINT, NT>(B, S, norb, part, [&](int c) { ban_cell(ban, B, c); });
     }
   }
+  if (gtau > S.tau) S.tau = gtau;  // thread 0
+  const int tkcnt = S.tkcnt;       // unchanged until the last pass over the cells
   __syncthreads();
   if (B.h == 2) {  // flagged rows and columns as cell bans: a row per thread, 32 cells at a time
-    const int y1 = B.kind == 2 ? S.nv[1] : 0;
-    const int x0 = B.kind == 2 ? B.clo / (y1 > 0 ? y1 : 1) : 0;
-    const int x1 = B.kind == 2 ? x0 + B.nct / (y1 > 0 ? y1 : 1) : S.nv[B.sa];
-    const int nch = kMaxOrb / 32;
-    for (int i = tid; i < (x1 - x0) * nch; i += kThreads) {
-      const int x = x0 + i / nch, y = 32 * (i % nch);
-      const int len = B.kind == 2 ? y1 : x;  // same spin: the cells (y, x), y < x
-      if (y >= len) continue;
-      uint32_t pat = flagged(S.frow, x) ? ~0u : (B.kind == 2 ? S.fcol : S.frow)[y >> 5];
-      if (len - y < 32) pat &= (1u << (len - y)) - 1u;
-      if (!pat) continue;
-      const int pos = (B.kind == 2 ? (x - x0) * y1 : x * (x - 1) / 2) + y;
-      atomicOr(&ban[pos >> 5], pat << (pos & 31));
-      if ((pos & 31) && (pat >> (32 - (pos & 31)))) atomicOr(&ban[(pos >> 5) + 1], pat >> (32 - (pos & 31)));
+    const int scol = B.kind == 2 ? 1 : B.sa, srow = B.kind == 2 ? 0 : B.sa, nvc = S.nv[scol];
+    const int x0 = B.kind == 2 ? B.clo / nvc : 0, x1 = B.kind == 2 ? x0 + B.nct / nvc : nvc;
+    for (int y = 0; y < nvc; y += 32) {
+      const unsigned fw =
+          __ballot_sync(kFull, y + lane < nvc && row_banned<NINT, NT>(S, scol, S.vir[scol][(y + lane) & (kMaxOrb - 1)]));
+      for (int x = x0 + tid; x < x1; x += kThreads) {
+        const int len = B.kind == 2 ? nvc : x;  // same spin: the cells (y, x), y < x
+        if (y >= len) continue;
+        uint32_t pat = row_banned<NINT, NT>(S, srow, S.vir[srow][x]) ? ~0u : fw;
+        if (len - y < 32) pat &= (1u << (len - y)) - 1u;
+        if (!pat) continue;
+        const int pos = (B.kind == 2 ? (x - x0) * nvc : x * (x - 1) / 2) + y;
+        atomicOr(&ban[pos >> 5], pat << (pos & 31));
+        if ((pos & 31) && (pat >> (32 - (pos & 31)))) atomicOr(&ban[(pos >> 5) + 1], pat >> (32 - (pos & 31)));
+      }
+      __syncwarp();
     }
-    __syncthreads();
   }
+
+  // Pair table of a J reaching every cell (a two-hole batch; a warp).
+  // J = K + {x1, x2}, x1 < x2; for a cell R disjoint from {x1, x2} the element
+  // is the double substitution x1 x2 -> R, whose integrals and phase split
+  // into a row and a column part.  The cells holding a particle of J (bit 30)
+  // are single substitutions and go with the rows.
+  auto build_table = [&](int j, int r) {
+    uint32_t xs, ts;
+    int nxs, nts;
+    excitation_sets<NINT, NT>(B, S, S.rpt[r], S.rhm[r], &xs, &nxs, &ts, &nts);
+    const int a = pk(xs, 0), bb = pk(xs, 1);
+    const int sr = B.sa, sc = B.kind == 2 ? 1 : B.sa;
+    const int x1 = (a < bb ? a : bb) - sr * norb, x2 = (a < bb ? bb : a) - sc * norb;
+    const int gB = (x1 * norb + x2) * norb * norb;
+    if (lane == 0) {
+      S.gcj[j] = (NT)S.rc[r];
+      S.gx2[j] = x2;
+      S.gB[j] = gB;
+      if constexpr (MS)
+        for (int st = 0; st < nst; st++) ms_gc[j * kMaxStates + st] = S.rc[st * p.rc_stride + r];
+    }
+    uint64_t w1[NINT], w2[NINT], M1[NINT], M2[NINT];
+#pragma unroll
+    for (int w = 0; w < NINT; w++) {
+      w1[w] = S.rw[(size_t)r * NW + sr * NINT + w];
+      w2[w] = S.rw[(size_t)r * NW + sc * NINT + w];
+      if (B.kind == 1 && (x1 >> 6) == w) w2[w] &= ~(1ull << (x1 & 63));
+    }
+    phase_mask<NINT>(w1, x1, 0, M1);
+    phase_mask<NINT>(w2, x2, 0, M2);
+    for (int v = lane; v < S.nv[sr]; v += 32) {
+      const int q = S.vir[sr][v];
+      const int ex = q == x1 || (B.kind == 1 && q == x2) ? 1 << 30 : 0;
+      S.v.g.gRow[j][v] = (E4 ? gB + q * norb : tri(x1, q)) | ex | ((int)mask_bit<NINT>(M1, q) << 31);
+    }
+    for (int v = lane; v < S.nv[sc]; v += 32) {
+      const int q = S.vir[sc][v];
+      const int ex = q == x2 || (B.kind == 1 && q == x1) ? 1 << 30 : 0;
+      S.v.g.gCol[j][v] = (E4 ? q : tri(x2, q)) | ex | ((int)mask_bit<NINT>(M2, q) << 31);
+    }
+  };
+
+  // the gradient's weight 2 A/D of a cell (in place of its accumulator)
+  auto a2d = [&](int cc) {
+    return __longlong_as_double((long long)(A0[cc] | ((unsigned long long)A1[cc] << 32)));
+  };
+  (void)a2d;
 
   // ---- loop 2: A(R) += c_J <J|H|I - H + R> over J ranked at or after I.
   // In the one-state form every term goes into the exact accumulator, so
   // the order in which J are listed and cells are reached does not matter ----
-  unsigned long long con = 0;
-  for (int c0 = 0; c0 < total; c0 += kChunk) {
-    if (tid == 0) {
-      S.n0 = 0;
-      S.n1 = 0;
-      S.n2 = 0;
-      S.cnext = 0;
-    }
-    __syncthreads();
-    const int c1 = min(c0 + kChunk, total);
-    ulonglong2 enx = (c0 + tid < c1) ? ehp[entry(c0 + tid)] : make_ulonglong2(0ull, 0ull);
+  unsigned int con = 0;  // of a round (at most 512 entries); summed per warp after each
+  auto add_con = [&]() {
+    const unsigned int wcon = __reduce_add_sync(kFull, con);
+    if (lane == 0) S.red_con[warp] += wcon;
+    con = 0;
+  };
+  for (int c0 = 0;; c0 += kChunk) {
+    const int total = S.seg_s[3], c1 = min(c0 + kChunk, total);
+    const bool last_round = c0 + kChunk >= total;
     for (int i = c0 + tid; i < c1; i += kThreads) {
-      const ulonglong2 en = enx;
       const int o = entry(i);
-      if (i + kThreads < c1) enx = ehp[entry(i + kThreads)];
+      const ulonglong2 en = i < kThreads ? en0 : S.ehp[o];
       const uint64_t hmr = en.x, part = en.y;
       if (part & kBeforeBit) continue;
       if (dup(i, hmr)) continue;
       if (B.h == 2 && hmr == 0ull) continue;  // J = I: added in the cells pass
       const int t = __popcll(hmr & ~B.hm);
       if (t > 2) continue;
-      const int rec = (int)(erec[o] & 0x7FFFFFFFu);
+      const int rec = (int)((i < kThreads ? rec0 : S.erec[o]) & 0x7FFFFFFFu);
       if (t == 0) S.u.l.L0[atomicAdd(&S.n0, 1)] = rec;
       else if (t == 1) {
         if (B.h == 1 || row_live<NINT, NT>(B, S, norb, part)) S.u.l.L12[atomicAdd(&S.n1, 1)] = rec;
@@ -1788,121 +1810,8 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       else if (subset_live<NINT, NT>(B, S, norb, part, ban)) S.u.l.L12[kChunk - 1 - atomicAdd(&S.n2, 1)] = rec;
     }
     __syncthreads();
-    // J reaching every cell: the whole CTA, kGroup of them per pass.
-    // In a two-hole batch such a J is K + {x1, x2}; for a cell R disjoint
-    // from {x1, x2} the element is a double substitution x1 x2 -> R whose
-    // pair indices and phase split into a row part and a column part,
-    // precomputed once per J; the cells meeting the particles of J are single
-    // substitutions of J and go to the row pass.
     const int n0 = S.n0;
-    for (int g0 = 0; g0 < (B.h == 2 ? n0 : 0); g0 += kGroup) {
-      const int m = min(kGroup, n0 - g0);
-      if (tid < m) {
-        const int r = S.u.l.L0[g0 + tid];
-#pragma unroll
-        for (int w = 0; w < NW; w++) S.gJw[tid][w] = rw[(size_t)r * NW + w];
-        S.gcj[tid] = (NT)rc[r];
-        if constexpr (MS)
-          for (int st = 0; st < nst; st++) ms_gc[tid * kMaxStates + st] = rc[st * p.rc_stride + r];
-        uint32_t xs, ts;
-        int nxs, nts;
-        const ulonglong2 en = make_ulonglong2(rhm[r], rpt[r]);
-        excitation_sets<NINT, NT>(B, S, en.y, en.x, &xs, &nxs, &ts, &nts);
-        const int a = pk(xs, 0), bb = pk(xs, 1);
-        const int x1 = a < bb ? a : bb, x2 = a < bb ? bb : a;
-        S.gx1[tid] = x1;
-        S.gx2[tid] = x2;
-        const int s1 = x1 >= norb, s2 = x2 >= norb;
-        S.gsr[tid] = S.vidx[s1][x1 - s1 * norb];
-        S.gsc[tid] = S.vidx[s2][x2 - s2 * norb];
-        S.gB[tid] = ((x1 - s1 * norb) * norb + (x2 - s2 * norb)) * norb * norb;
-      }
-      __syncthreads();
-      const int sl1 = B.sa, sl2 = (B.kind == 2) ? 1 : B.sa;
-      const int nva = S.nv[sl1], nvb = S.nv[sl2];
-      {
-        const int per = nva + nvb;
-        for (int idx = tid; idx < m * per; idx += kThreads) {
-          const int j = idx / per;
-          const int v = idx - j * per;
-          const uint64_t* Jw = S.gJw[j];
-          const int x1 = S.gx1[j] - sl1 * norb, x2 = S.gx2[j] - sl2 * norb;
-          if (v < nva) {
-            const int r = S.vir[sl1][v];
-            int par = 0;
-            if (r != x1) par = count_between<NINT>(Jw + sl1 * NINT, r < x1 ? r : x1, r < x1 ? x1 : r) & 1;
-            S.v.g.gRow[j][v] = (E4 ? r : tri(x1, r)) | (par << 31);
-          } else {
-            const int sv = S.vir[sl2][v - nva];
-            int par = 0;
-            if (sv != x2) par = count_between<NINT>(Jw + sl2 * NINT, sv < x2 ? sv : x2, sv < x2 ? x2 : sv) & 1;
-            if (B.kind == 1) {
-              const int lo = sv < x2 ? sv : x2, hi = sv < x2 ? x2 : sv;
-              par ^= (x1 > lo && x1 < hi) ? 1 : 0;
-            }
-            S.v.g.gCol[j][v - nva] = (E4 ? sv : tri(x2, sv)) | (par << 31);
-          }
-        }
-        __syncthreads();
-      }
-      for (int cc = tid; cc < B.nct; cc += kThreads) {
-        if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
-        int ro, so, x, y;
-        cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
-        unsigned long long acc_lo = 0ull;  // exact sum of this group's products
-        int acc_hi = 0;
-        double accs[kMaxStates];  // multi-state form: one sum per state
-#pragma unroll
-        for (int st = 0; st < kMaxStates; st++) accs[st] = 0.0;
-        for (int j = 0; j < m; j++) {
-          // a cell touching the particles of J is a single substitution of J
-          // (or J itself, banned): it goes with the rows below
-          NT v;
-          const int sr = S.gsr[j], sc = S.gsc[j];
-          if (B.kind == 2) {
-            if (x == sr || y == sc) continue;
-            const int rt = S.v.g.gRow[j][x], ct = S.v.g.gCol[j][y];
-            v = flip_sign(eri_n[E4 ? S.gB[j] + (rt & 0x7fffffff) * norb + (ct & 0x7fffffff) : tri(rt & 0x7fffffff, ct & 0x7fffffff)],
-                          (rt ^ ct) < 0);
-          } else {
-            if (x == sr || x == sc || y == sr || y == sc) continue;
-            const int a1 = S.v.g.gRow[j][x], b2 = S.v.g.gCol[j][y];
-            const int a2 = S.v.g.gRow[j][y], b1 = S.v.g.gCol[j][x];
-            if constexpr (E4)
-              v = eri_n[S.gB[j] + (a1 & 0x7fffffff) * norb + (b2 & 0x7fffffff)] - eri_n[S.gB[j] + (b2 & 0x7fffffff) * norb + (a1 & 0x7fffffff)];
-            else
-              v = eri_n[tri(a1 & 0x7fffffff, b2 & 0x7fffffff)] - eri_n[tri(a2 & 0x7fffffff, b1 & 0x7fffffff)];
-            const int x2 = S.gx2[j] - B.sa * norb;
-            const int lo = so < x2 ? so : x2, hi = so < x2 ? x2 : so;
-            const int par = ((a1 ^ b2) < 0 ? 1 : 0) ^ ((ro > lo && ro < hi) ? 1 : 0);
-            v = flip_sign(v, par);
-          }
-          con++;
-          if constexpr (MS) {
-#pragma unroll
-            for (int st = 0; st < kMaxStates; st++)
-              if (st < nst) accs[st] = fma(ms_gc[j * kMaxStates + st], (double)v, accs[st]);
-          } else {
-            unsigned long long l;
-            int hh;
-            fix_of(S.gcj[j] * v, F, l, hh);
-            fix_add(acc_lo, acc_hi, l, hh);
-          }
-        }
-        if constexpr (MS) {
-#pragma unroll
-          for (int st = 0; st < kMaxStates; st++)
-            if (st < nst) A[st * mc + cc] += accs[st];
-        } else {
-          unsigned long long lo = Alo[cc];
-          int hi = Ahi[cc];
-          fix_add(lo, hi, acc_lo, acc_hi);
-          Alo[cc] = lo;
-          Ahi[cc] = hi;
-        }
-      }
-      __syncthreads();
-    }
+    B = S.bt;
     // The rest of the J, drawn by the warps as they free up: the rows of J
     // reaching every cell (a two-hole batch: the cells touching their
     // particles; a one-hole batch: all cells), J reaching rows, and J reaching
@@ -1922,8 +1831,9 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     // of 30 dependent loads wherever a row met a single substitution.)
     {
       const int nrow = S.n1, n2 = S.n2;
+      const int ntab = B.h == 2 ? (n0 < kGroup ? n0 : kGroup) : 0;
       const int nvm = S.nv[0] > S.nv[1] ? S.nv[0] : S.nv[1], nch = (nvm + 31) / 32;
-      const int nall = n0 * B.h * nch;  // (J, particle slot, 32 cells)
+      const int nall = ntab + n0 * B.h * nch;  // pair tables, then (J, particle slot, 32 cells)
       int per = (nrow + kWarps - 1) / kWarps;
       per = per > 8 ? 8 : per;
       const int ndraw = nall + (per ? (nrow + per - 1) / per : 0);
@@ -1932,12 +1842,12 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         if constexpr (MS) {
 #pragma unroll
           for (int st = 0; st < kMaxStates; st++)
-            if (st < nst) atomicAdd(&A[st * mc + cc], rc[st * p.rc_stride + rj] * (double)v);
+            if (st < nst) atomicAdd(&A[st * mc + cc], S.rc[st * p.rc_stride + rj] * (double)v);
         } else {
           unsigned long long l;
           int hh;
           fix_of(cjj * v, F, l, hh);
-          fix_atomic_add(Alo, Ahi, cc, l, hh);
+          fix_atomic_add(A0, A1, A2, cc, l, hh);
         }
         con++;
       };
@@ -1946,10 +1856,12 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         int jd = 0;
         if (lane == 0) jd = atomicAdd(&S.cnext, 1);
         jd = __shfl_sync(kFull, jd, 0);
-        if (jd < nall) {
-          const int j = jd / (B.h * nch), rem = jd - j * (B.h * nch), ip = rem / nch, y = (rem - ip * nch) * 32 + lane;
+        if (jd < ntab) {
+          build_table(jd, S.u.l.L0[jd]);
+        } else if (jd < nall) {
+          const int ju = jd - ntab, j = ju / (B.h * nch), rem = ju - j * (B.h * nch), ip = rem / nch, y = (rem - ip * nch) * 32 + lane;
           const int r = S.u.l.L0[j];
-          const uint64_t hm = rhm[r], part = rpt[r];
+          const uint64_t hm = S.rhm[r], part = S.rpt[r];
           uint32_t X, T;
           int nx, nt;
           excitation_sets<NINT, NT>(B, S, part, hm, &X, &nx, &T, &nt);
@@ -1960,11 +1872,11 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           const int s = code >= norb, x = code >= 0 ? S.vidx[s][code - s * norb] : 0;
           if (B.kind == 1 && s != B.sa) continue;
           const int sz = B.kind == 2 ? 1 - s : B.sa;
-          if (B.h == 2 && flagged((B.kind == 2 && s) ? S.fcol : S.frow, x)) continue;
+          if (B.h == 2 && row_banned<NINT, NT>(S, s, code - s * norb)) continue;
           const int x0 = pk(X, 0), uz = (x0 == code ? pk(X, 1) : x0) - sz * norb;
           uint64_t wz[NINT], M[NINT];
 #pragma unroll
-          for (int w = 0; w < NINT; w++) wz[w] = rw[(size_t)r * NW + sz * NINT + w];
+          for (int w = 0; w < NINT; w++) wz[w] = S.rw[(size_t)r * NW + sz * NINT + w];
           phase_mask<NINT>(wz, uz, 0, M);
           if (y >= S.nv[sz]) continue;
           const int z = S.vir[sz][y];
@@ -1976,7 +1888,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           // it), four at a time so that their loads overlap
 #pragma unroll
           for (int w = 0; w < NW; w++) {
-            uint64_t bits = rw[(size_t)r * NW + w];
+            uint64_t bits = S.rw[(size_t)r * NW + w];
             const bool sp = w / NINT == sz;
             while (bits) {
               int o[4];
@@ -1997,7 +1909,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
               }
             }
           }
-          add(cc, flip_sign(v, mask_bit<NINT>(M, z)), r, (NT)rc[r]);
+          add(cc, flip_sign(v, mask_bit<NINT>(M, z)), r, (NT)S.rc[r]);
         } else if (jd < ndraw) {
           const int jl = (jd - nall) * per + (lane >> 2), ip = lane & 3;
           const bool have = (lane >> 2) < per && jl < nrow;
@@ -2019,23 +1931,23 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           for (int w = 0; w < NINT; w++) M[w] = EX[w] = 0;
           if (have) {
             r = S.u.l.L12[jl];
-            part = rpt[r];
-            hm = rhm[r];
-            cj = (NT)rc[r];
+            part = S.rpt[r];
+            hm = S.rhm[r];
+            cj = (NT)S.rc[r];
             uint32_t X, T;
             int nx, nt;
             excitation_sets<NINT, NT>(B, S, part, hm, &X, &nx, &T, &nt);
             const int q = pk(T, 0), sq = q >= norb ? 1 : 0, qo = q - sq * norb;
             uint64_t Jw[NW];
 #pragma unroll
-            for (int w = 0; w < NW; w++) Jw[w] = rw[(size_t)r * NW + w];
+            for (int w = 0; w < NW; w++) Jw[w] = S.rw[(size_t)r * NW + w];
             // the row's particle (a one-hole batch has one row per J and no
             // fixed particle)
             const int code = B.h == 2 ? part_code(part, ip) : (ip == 0 ? -1 : kNoPart);
             if (code != kNoPart) {
               const int s = code >= norb, x = code >= 0 ? S.vidx[s][code - s * norb] : 0;
               const int sz = B.kind == 2 ? 1 - s : B.sa;
-              act = B.h == 1 || ((B.kind == 2 || s == B.sa) && !flagged((B.kind == 2 && s) ? S.fcol : S.frow, x));
+              act = B.h == 1 || ((B.kind == 2 || s == B.sa) && !row_banned<NINT, NT>(S, s, code - s * norb));
               geo = x | (s << 8);
               int u0 = -1, u1 = -1;  // X without the row's particle
 #pragma unroll
@@ -2116,20 +2028,39 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             const int nz = S.nv[sz], nv1 = S.nv[1];
             // the integrals at b1 + z and (same spin) b2 + z
             const int b1 = ((uo * norb + uz) * norb + q) * norb, b2 = ((uz * norb + uo) * norb + q) * norb;
-#pragma unroll 2
-            for (int y = lane; y < nz; y += 32) {
-              const int z = S.vir[sz][y];
-              const int cc = (B.kind == 0 ? y : B.kind == 1 ? pair_cell(x, y) : (s ? y * nv1 + x : x * nv1 + y)) - B.clo;
-              if (mask_bit<NINT>(Er, z) || !live(cc)) continue;
-              NT v;
-              if constexpr (E4) {
-                v = eri_n[b1 + z];
-                if (same) v -= eri_n[b2 + z];
-              } else {
-                v = eri_n[eri_index(uo, q, uz, z)];
-                if (same) v -= eri_n[eri_index(uz, q, uo, z)];
+            // two rounds of 32 cells at a time, their loads in flight together
+            for (int y0 = lane; y0 < nz; y0 += 64) {
+              int cc[2], zz[2];
+              NT v[2], w2[2];
+#pragma unroll
+              for (int i = 0; i < 2; i++) {
+                const int y = y0 + 32 * i;
+                cc[i] = -1;
+                v[i] = w2[i] = NT(0);
+                zz[i] = 0;
+                if (y < nz) {
+                  const int z = S.vir[sz][y];
+                  const int c = (B.kind == 0 ? y : B.kind == 1 ? pair_cell(x, y) : (s ? y * nv1 + x : x * nv1 + y)) - B.clo;
+                  zz[i] = z;
+                  if (!mask_bit<NINT>(Er, z) && live(c)) {
+                    cc[i] = c;
+                    if constexpr (E4) {
+                      v[i] = eri_n[b1 + z];
+                      if (same) w2[i] = eri_n[b2 + z];
+                    } else {
+                      v[i] = eri_n[eri_index(uo, q, uz, z)];
+                      if (same) w2[i] = eri_n[eri_index(uz, q, uo, z)];
+                    }
+                  }
+                }
               }
-              add(cc, flip_sign(v, mask_bit<NINT>(Mr, z)), rj, cjr);
+#pragma unroll
+              for (int i = 0; i < 2; i++)
+                if (cc[i] >= 0) {
+                  NT t = v[i];
+                  if (same) t -= w2[i];
+                  add(cc[i], flip_sign(t, mask_bit<NINT>(Mr, zz[i])), rj, cjr);
+                }
             }
           }
           for (unsigned m = __ballot_sync(kFull, sact); m; m &= m - 1) {
@@ -2157,7 +2088,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
               for (int w = 0; w < 2 * NW; w++) {
                 const int o = 32 * (w % (2 * NINT)) + lane;
                 const bool sp = w / (2 * NINT) == sq;
-                uint32_t bits = (uint32_t)(rw[(size_t)rj * NW + w / 2] >> (32 * (w & 1)));
+                uint32_t bits = (uint32_t)(S.rw[(size_t)rj * NW + w / 2] >> (32 * (w & 1)));
                 NT a = NT(0), b = NT(0);
                 if ((bits >> lane) & 1u) {
                   a = eri_n[gidx<E4>(o, o, wo, qo, norb)];
@@ -2178,290 +2109,359 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           if (j0 >= n2) break;
           const int j = j0 + lane;
           if (j < n2) {
+            // cells inside J's particles: J -> alpha moves the other two
+            // entries of X to J's two holes outside the batch
             const int r = S.u.l.L12[kChunk - 1 - j];
-            const uint64_t* Jw = rw + (size_t)r * NW;
-            const NT cj = (NT)rc[r];
-            double cjs[kMaxStates];
-            if constexpr (MS) {
-#pragma unroll
-              for (int st = 0; st < kMaxStates; st++) cjs[st] = st < nst ? rc[st * p.rc_stride + r] : 0.0;
-            }
-            const ulonglong2 en = make_ulonglong2(rhm[r], rpt[r]);
-          const uint64_t part = en.y;
+            const uint64_t part = S.rpt[r];
             uint32_t X, T;
             int nx, nt;
-            excitation_sets<NINT, NT>(B, S, part, en.x, &X, &nx, &T, &nt);
-            for_subset_cells<NINT, NT>(B, S, norb, part, [&](int c) {
-              const int cc = c - B.clo;
-              if ((unsigned)cc >= (unsigned)B.nct || ((ban[cc >> 5] >> (cc & 31)) & 1u)) return;
-              int ro, so, x, y;
-              cell_orbitals<NINT, NT>(B, S, c, &ro, &so, &x, &y);
-              const int rcode = B.sa * norb + ro;
-              const int scode = (B.h == 2) ? B.sb * norb + so : -1;
+            excitation_sets<NINT, NT>(B, S, part, S.rhm[r], &X, &nx, &T, &nt);
+            const NT cj = (NT)S.rc[r];
+            uint64_t Jw[NW];
+#pragma unroll
+            for (int w = 0; w < NW; w++) Jw[w] = S.rw[(size_t)r * NW + w];
+#pragma unroll 1
+            for (int k = 0; k < (B.h == 2 ? 6 : 4); k++) {
+              // pairs (0, 1), (0, 2), (1, 2), (0, 3), (1, 3), (2, 3); one-hole batch: single particles
+              const int k1 = B.h == 1 ? k : (k >= 3 ? 3 : k >= 1 ? 2 : 1), k0 = B.h == 1 ? k : (k >= 3 ? k - 3 : k >= 1 ? k - 1 : 0);
+              const int e0 = part_code(part, k0), e1 = part_code(part, k1);
+              if (e0 == kNoPart || e1 == kNoPart) continue;
+              const int sx = e0 >= norb, sy = e1 >= norb;
+              if (B.kind == 2 ? sx == sy : (sx != B.sa || sy != B.sa)) continue;
+              const int vx = S.vidx[sx][e0 - sx * norb], vy = S.vidx[sy][e1 - sy * norb];
+              const int cc = (B.kind == 0 ? vx : B.kind == 1 ? pair_cell(vx, vy) : (sx ? vy * S.nv[1] + vx : vx * S.nv[1] + vy)) - B.clo;
+              if (!live(cc)) continue;
+              int u0 = -1, u1 = -1;
+#pragma unroll
+              for (int i = 0; i < 4; i++) {
+                const int xc = pk(X, i);
+                if (i < nx && xc != e0 && xc != e1) {
+                  if (u0 < 0) u0 = xc;
+                  else u1 = xc;
+                }
+              }
+              const NT v = double_element<NINT, NT, E4>(eri_n, norb, Jw, u0 < u1 ? u0 : u1, u0 < u1 ? u1 : u0, pk(T, 0), pk(T, 1));
               if constexpr (MS) {
-                const double v = (double)element<NINT, NT, E4>(eri_n, h_n, norb, Jw, X, nx, T, nt, rcode, scode);
 #pragma unroll
                 for (int st = 0; st < kMaxStates; st++)
-                  if (st < nst) atomicAdd(&A[st * mc + cc], cjs[st] * v);
+                  if (st < nst) atomicAdd(&A[st * mc + cc], S.rc[st * p.rc_stride + r] * (double)v);
               } else {
                 unsigned long long l;
                 int hh;
-                fix_of(cj * element<NINT, NT, E4>(eri_n, h_n, norb, Jw, X, nx, T, nt, rcode, scode), F, l, hh);
-                fix_atomic_add(Alo, Ahi, cc, l, hh);
+                fix_of(cj * v, F, l, hh);
+                fix_atomic_add(A0, A1, A2, cc, l, hh);
               }
               con++;
-            });
+            }
           }
         }
       }
     }
     __syncthreads();
-  }
 
-  // ---- cells: the perturbers of I in this batch ----
-  if (GRAD) {  // loop 2 is over: the pair tables' storage takes the weights
-    for (int x = tid; x < kMaxOrb; x += kThreads) {
-      S.v.w.rowW2[x] = 0.0;
-      S.v.w.colW2[x] = 0.0;
-    }
-    __syncthreads();
-  }
-  if (p.k > 0) {
-    if (S.tkcnt + B.nct > p.cap) compact_selection<NINT, NT>(p, S, te, ta, tk);
-    if (tid == 0) {
-      const unsigned long long gt = *((volatile unsigned long long*)p.tau_bits);
-      if (gt > S.tau) S.tau = gt;
-    }
-    __syncthreads();
-  }
-  const unsigned long long tau = S.tau;
-  double acc_e = 0.0, acc_s2 = 0.0;
-  unsigned long long acc_na = 0, acc_d0 = 0, acc_d1 = 0, acc_min = ~0ull, acc_tiny = 0;  // acc_min: units of 2^-S
-  double acc_es[kMaxStates], acc_s2s[kMaxStates];  // multi-state form: sums per state
+    // ---- passes over the cells: the terms of the J reaching every cell, a
+    // group of kGroup per pass; in the last pass the cells left are the
+    // perturbers of I in this batch ----
+    const int nt0 = B.h == 2 ? n0 : 0;
+    bool done = false;
+    for (int g0 = 0;; g0 += kGroup) {
+      B = S.bt;
+      const int m = max(0, min(kGroup, nt0 - g0));
+      const bool fin = last_round && (GRAD ? m == 0 : g0 + kGroup >= nt0);
+      if (!fin && m == 0) break;
+      if (g0 > 0 && m > 0) {  // the first group's tables came with the row pass
+        __syncthreads();
+        for (int j = warp; j < m; j += kWarps) build_table(j, S.u.l.L0[g0 + j]);
+        __syncthreads();
+      }
+      if (fin) {
+        if (GRAD) {  // the pair tables' storage takes the weights
+          __syncthreads();
+          for (int x = tid; x < kMaxOrb; x += kThreads) {
+            S.v.w.rowW2[x] = 0.0;
+            S.v.w.colW2[x] = 0.0;
+          }
+          __syncthreads();
+        }
+        if (p.k > 0 && tkcnt + B.nct > p.cap) compact_selection<NINT, NT>(p, S, buf_e(p), buf_a(p), buf_key<NINT>(p));
+      }
+      const unsigned long long tau = S.tau;
+      double acc_e = 0.0, acc_s2 = 0.0;
+      unsigned long long acc_d0 = 0, acc_d1 = 0, acc_min = ~0ull;  // acc_min: units of 2^-S
+      unsigned int acc_na = 0, acc_tiny = 0;
+      double acc_es[kMaxStates], acc_s2s[kMaxStates];  // multi-state form: sums per state
 #pragma unroll
-  for (int st = 0; st < kMaxStates; st++) acc_es[st] = acc_s2s[st] = 0.0;
-  if constexpr (MS) {
-    for (int cc = tid; cc < B.nct; cc += kThreads) {
-      if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
-      int ro, so, x, y;
-      cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
-      double vI = 0.0;  // <I|H|alpha> for the generator's own term
-      if (B.h == 2) {
-        const int a1 = S.iRow[x], b2 = S.iCol[y];
-        if (B.kind == 2) {
-          vI = (double)flip_sign(eri_n[E4 ? S.ibase + (a1 & 0x7fffffff) * norb + (b2 & 0x7fffffff) : tri(a1 & 0x7fffffff, b2 & 0x7fffffff)],
-                                 (a1 ^ b2) < 0);
-        } else {
-          const int a2 = S.iRow[y], b1 = S.iCol[x];
+      for (int st = 0; st < kMaxStates; st++) acc_es[st] = acc_s2s[st] = 0.0;
+      for (int cc = tid; cc < B.nct; cc += kThreads) {
+        if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
+        int ro, so, x, y;
+        cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
+        unsigned long long lo = 0ull;  // exact sum
+        int hi = 0;
+        double accs[kMaxStates];  // multi-state form: one sum per state
+#pragma unroll
+        for (int st = 0; st < kMaxStates; st++) accs[st] = 0.0;
+        if constexpr (!MS) {
+          lo = A0[cc] | ((unsigned long long)A1[cc] << 32);
+          hi = (int)A2[cc];
+        }
+        for (int j = 0; j < m; j++) {
+          const int rt = S.v.g.gRow[j][x], ct = S.v.g.gCol[j][y];
+          if ((rt | ct) & (1 << 30)) continue;
           NT v;
-          if constexpr (E4)
-            v = eri_n[S.ibase + (a1 & 0x7fffffff) * norb + (b2 & 0x7fffffff)] - eri_n[S.ibase + (b2 & 0x7fffffff) * norb + (a1 & 0x7fffffff)];
-          else
-            v = eri_n[tri(a1 & 0x7fffffff, b2 & 0x7fffffff)] - eri_n[tri(a2 & 0x7fffffff, b1 & 0x7fffffff)];
-          const int lo = so < B.qb ? so : B.qb, hi = so < B.qb ? B.qb : so;
-          vI = (double)flip_sign(v, ((a1 ^ b2) < 0 ? 1 : 0) ^ ((ro > lo && ro < hi) ? 1 : 0));
+          bool neg = (rt ^ ct) < 0;
+          if constexpr (E4) {
+            v = eri_n[(rt & 0x3fffffff) + (ct & 0x3fffffff)];
+            if (B.kind == 1) v -= eri_n[S.gB[j] + so * norb + ro];
+          } else {
+            v = eri_n[tri(rt & 0x3fffffff, ct & 0x3fffffff)];
+            if (B.kind == 1) v -= eri_n[tri(S.v.g.gRow[j][y] & 0x3fffffff, S.v.g.gCol[j][x] & 0x3fffffff)];
+          }
+          if (B.kind == 1) {
+            const int x2 = S.gx2[j];
+            neg ^= ro > (so < x2 ? so : x2) && ro < (so < x2 ? x2 : so);
+          }
+          v = flip_sign(v, neg);
+          con++;
+          if constexpr (MS) {
+#pragma unroll
+            for (int st = 0; st < kMaxStates; st++)
+              if (st < nst) accs[st] = fma(ms_gc[j * kMaxStates + st], (double)v, accs[st]);
+          } else {
+            unsigned long long l;
+            int hh;
+            fix_of(S.gcj[j] * v, F, l, hh);
+            fix_add(lo, hi, l, hh);
+          }
         }
-        con++;
-      }
-      long long D0 = S.dx[x];  // E0_0 - H_aa
-      if (B.kind == 2) D0 -= S.u1[y] + p.Ji[ro * norb + so];
-      else if (B.kind == 1) D0 -= S.u0[y] + p.Wi[ro * norb + so];
-      double crit = 0.0, a0 = 0.0;
+        if (!fin) {
+          if constexpr (MS) {
 #pragma unroll
-      for (int st = 0; st < kMaxStates; st++) {
-        if (st >= nst) break;
-        const double a = A[st * mc + cc] + ms_cI[st] * vI;
-        const long long D = D0 + ms_de[st];
-        const double q = div_fix(a, D, E.dscale);
-        const double e = a * q;
-        acc_es[st] += e;
-        acc_s2s[st] += q * q;
-        crit += ms_w[st] * e;  // c_alpha,s A_s / max_I c_Is^2
-        const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
-        acc_min = db < acc_min ? db : acc_min;
-        if (st == 0) a0 = a;
-      }
-      acc_na++;
-      if (abs_bits(a0) < 0x3D06849B86A12B9Bull) acc_tiny++;
-      uint64_t key[NW];
-      const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
-#pragma unroll
-      for (int w = 0; w < NW; w++)
-        key[w] = S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
-      uint64_t hk = 0;
-#pragma unroll
-      for (int w = 0; w < NW; w++) hk = splitmix64(hk ^ key[w]);
-      acc_d0 += hk;
-      acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
-      if (p.k > 0) {
-        const unsigned long long eb = abs_bits(crit);
-        if (eb >= tau) {
-          atomicAdd(&p.sel_hist[sel_bin(eb)], 1u);
-          const int pos = atomicAdd(&S.tkcnt, 1);
-          te[pos] = crit;
-          ta[pos] = a0;
-#pragma unroll
-          for (int w = 0; w < NW; w++) tk[(size_t)pos * NW + w] = key[w];
+            for (int st = 0; st < kMaxStates; st++)
+              if (st < nst) A[st * mc + cc] += accs[st];
+          } else {
+            A0[cc] = (uint32_t)lo;
+            A1[cc] = (uint32_t)(lo >> 32);
+            A2[cc] = (uint32_t)hi;
+          }
+          continue;
         }
-      }
-    }
-    acc_e = acc_es[0];
-    acc_s2 = acc_s2s[0];
-  } else {
-    for (int cc = tid; cc < B.nct; cc += kThreads) {
-      if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
-      int ro, so, x, y;
-      cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
-      double a = fix_to_double(Alo[cc], Ahi[cc], F);
-      if (B.h == 2) {  // the generator's own term c_I <I|H|alpha>
-        NT v;
-        const int a1 = S.iRow[x], b2 = S.iCol[y];
-        if (B.kind == 2) {
-          v = flip_sign(eri_n[E4 ? S.ibase + (a1 & 0x7fffffff) * norb + (b2 & 0x7fffffff) : tri(a1 & 0x7fffffff, b2 & 0x7fffffff)], (a1 ^ b2) < 0);
+        if constexpr (MS) {
+          double vI = 0.0;  // <I|H|alpha> for the generator's own term
+          if (B.h == 2) {
+            const int a1 = S.iRow[x], b2 = S.iCol[y];
+            if (B.kind == 2) {
+              vI = (double)flip_sign(eri_n[E4 ? (a1 & 0x7fffffff) + (b2 & 0x7fffffff) : tri(a1 & 0x7fffffff, b2 & 0x7fffffff)],
+                                     (a1 ^ b2) < 0);
+            } else {
+              const int a2 = S.iRow[y], b1 = S.iCol[x];
+              NT v;
+              if constexpr (E4)
+                v = eri_n[(a1 & 0x7fffffff) + (b2 & 0x7fffffff)] - eri_n[ibase + so * norb + ro];
+              else
+                v = eri_n[tri(a1 & 0x7fffffff, b2 & 0x7fffffff)] - eri_n[tri(a2 & 0x7fffffff, b1 & 0x7fffffff)];
+              const int lo = so < B.qb ? so : B.qb, hi = so < B.qb ? B.qb : so;
+              vI = (double)flip_sign(v, ((a1 ^ b2) < 0 ? 1 : 0) ^ ((ro > lo && ro < hi) ? 1 : 0));
+            }
+            con++;
+          }
+          long long D0 = S.dx[x];  // E0_0 - H_aa
+          if (B.kind == 2) D0 -= S.u1[y] + p.Ji[ro * norb + so];
+          else if (B.kind == 1) D0 -= S.u0[y] + p.Wi[ro * norb + so];
+          double crit = 0.0, a0 = 0.0;
+#pragma unroll
+          for (int st = 0; st < kMaxStates; st++) {
+            if (st >= nst) break;
+            const double a = A[st * mc + cc] + accs[st] + ms_cI[st] * vI;
+            const long long D = D0 + ms_de[st];
+            const double q = div_fix(a, D, E.dscale);
+            const double e = a * q;
+            acc_es[st] += e;
+            acc_s2s[st] += q * q;
+            crit += ms_w[st] * e;  // c_alpha,s A_s / max_I c_Is^2
+            const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
+            acc_min = db < acc_min ? db : acc_min;
+            if (st == 0) a0 = a;
+          }
+          acc_na++;
+          if (abs_bits(a0) < 0x3D06849B86A12B9Bull) acc_tiny++;
+          uint64_t key[NW];
+          const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
+#pragma unroll
+          for (int w = 0; w < NW; w++)
+            key[w] = S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
+          uint64_t hk = 0;
+#pragma unroll
+          for (int w = 0; w < NW; w++) hk = splitmix64(hk ^ key[w]);
+          acc_d0 += hk;
+          acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
+          if (p.k > 0) {
+            const unsigned long long eb = abs_bits(crit);
+            if (eb >= tau) {
+              atomicAdd(&p.sel_hist[sel_bin(eb)], 1u);
+              const int pos = atomicAdd(&S.tkcnt, 1);
+              buf_e(p)[pos] = crit;
+              buf_a(p)[pos] = a0;
+#pragma unroll
+              for (int w = 0; w < NW; w++) buf_key<NINT>(p)[(size_t)pos * NW + w] = key[w];
+            }
+          }
         } else {
-          const int a2 = S.iRow[y], b1 = S.iCol[x];
-          if constexpr (E4)
-            v = eri_n[S.ibase + (a1 & 0x7fffffff) * norb + (b2 & 0x7fffffff)] - eri_n[S.ibase + (b2 & 0x7fffffff) * norb + (a1 & 0x7fffffff)];
-          else
-            v = eri_n[tri(a1 & 0x7fffffff, b2 & 0x7fffffff)] - eri_n[tri(a2 & 0x7fffffff, b1 & 0x7fffffff)];
-          const int lo = so < B.qb ? so : B.qb, hi = so < B.qb ? B.qb : so;
-          v = flip_sign(v, ((a1 ^ b2) < 0 ? 1 : 0) ^ ((ro > lo && ro < hi) ? 1 : 0));
+          double a = fix_to_double(lo, hi, F);
+          if (B.h == 2) {  // the generator's own term c_I <I|H|alpha>
+            NT v;
+            const int a1 = S.iRow[x], b2 = S.iCol[y];
+            if (B.kind == 2) {
+              v = flip_sign(eri_n[E4 ? (a1 & 0x7fffffff) + (b2 & 0x7fffffff) : tri(a1 & 0x7fffffff, b2 & 0x7fffffff)], (a1 ^ b2) < 0);
+            } else {
+              const int a2 = S.iRow[y], b1 = S.iCol[x];
+              if constexpr (E4)
+                v = eri_n[(a1 & 0x7fffffff) + (b2 & 0x7fffffff)] - eri_n[ibase + so * norb + ro];
+              else
+                v = eri_n[tri(a1 & 0x7fffffff, b2 & 0x7fffffff)] - eri_n[tri(a2 & 0x7fffffff, b1 & 0x7fffffff)];
+              const int lo = so < B.qb ? so : B.qb, hi = so < B.qb ? B.qb : so;
+              v = flip_sign(v, ((a1 ^ b2) < 0 ? 1 : 0) ^ ((ro > lo && ro < hi) ? 1 : 0));
+            }
+            a += (double)(S.cI * v);
+            con++;
+          }
+          // D = E0 - H_aa from the per-batch row sums
+          long long D = S.dx[x];
+          if (B.kind == 2) D -= S.u1[y] + p.Ji[ro * norb + so];
+          else if (B.kind == 1) D -= S.u0[y] + p.Wi[ro * norb + so];
+          const double q = div_fix(a, D, E.dscale);
+          acc_e = fma(a, q, acc_e);  // e = A q
+          acc_s2 += q * q;
+          acc_na++;
+          if (GRAD) {
+            // numerator weight 2A/D for loop 3; (A/D)^2 weights the diagonal
+            const unsigned long long wb = (unsigned long long)__double_as_longlong(2.0 * q);
+            A0[cc] = (uint32_t)wb;
+            A1[cc] = (uint32_t)(wb >> 32);
+            const double w2 = q * q;
+            atomicAdd(&S.v.w.rowW2[x], w2);
+            if (B.kind == 2) atomicAdd(&S.v.w.colW2[y], w2);
+            if (B.kind == 1) atomicAdd(&S.v.w.rowW2[y], w2);
+            if (B.h == 2) w_grad(p, ro, B.sa, so, B.sb, w2);
+          }
+          // |a| < 1e-14, compared on the bit pattern (no FP64 compare)
+          if (abs_bits(a) < 0x3D06849B86A12B9Bull) acc_tiny++;
+          const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
+          acc_min = db < acc_min ? db : acc_min;
+          uint64_t key[NW];  // alpha's words; selects keep them in registers
+          const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
+#pragma unroll
+          for (int w = 0; w < NW; w++)
+            key[w] = S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
+          uint64_t hk = 0;
+#pragma unroll
+          for (int w = 0; w < NW; w++) hk = splitmix64(hk ^ key[w]);
+          acc_d0 += hk;
+          acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
+          // e = A q is formed only when it can reach the threshold: with biased
+          // exponents ea, eq of A and q, |A q| < 2^(ea + eq - 2044), so
+          // ea + eq <= et + 1021 (et: the exponent of tau) puts it below tau
+          const int ea = (int)(abs_bits(a) >> 52), eqx = (int)(abs_bits(q) >> 52);
+          if (p.k > 0 && (tau == 0ull || ea + eqx > (int)(tau >> 52) + 1021)) {
+            const double e = a * q;
+            const unsigned long long eb = abs_bits(e);
+            if (eb >= tau) {
+              atomicAdd(&p.sel_hist[sel_bin(eb)], 1u);
+              const int pos = atomicAdd(&S.tkcnt, 1);
+              buf_e(p)[pos] = e;
+              buf_a(p)[pos] = a;
+#pragma unroll
+              for (int w = 0; w < NW; w++) buf_key<NINT>(p)[(size_t)pos * NW + w] = key[w];
+            }
+          }
         }
-        a += (double)(S.cI * v);
-        con++;
       }
-      // D = E0 - H_aa from the per-batch row sums
-      long long D = S.dx[x];
-      if (B.kind == 2) D -= S.u1[y] + p.Ji[ro * norb + so];
-      else if (B.kind == 1) D -= S.u0[y] + p.Wi[ro * norb + so];
-      const double q = div_fix(a, D, E.dscale);
-      acc_e = fma(a, q, acc_e);  // e = A q
-      acc_s2 += q * q;
-      acc_na++;
-      if (GRAD) {
-        // numerator weight 2A/D for loop 3; (A/D)^2 weights the diagonal
-        A[cc] = 2.0 * q;
-        const double w2 = q * q;
-        atomicAdd(&S.v.w.rowW2[x], w2);
-        if (B.kind == 2) atomicAdd(&S.v.w.colW2[y], w2);
-        if (B.kind == 1) atomicAdd(&S.v.w.rowW2[y], w2);
-        if (B.h == 2) w_grad(p, ro, B.sa, so, B.sb, w2);
+      if (!fin) continue;
+      // ---- the item's sums.  The digest, min |D| and the tiny count are the
+      // sweep's: this thread's shares stay in shared memory until the kernel
+      // ends.  e and (A/D)^2 go to the item's own slot (the generator's eps_I and
+      // sum A^2/D^2 are reduced from the slots in item order after the wave, so
+      // they do not depend on which CTA finished first); the last warp to arrive
+      // adds them, thread by thread in a fixed order ----
+      S.td0[tid] += acc_d0;
+      S.td1[tid] ^= acc_d1;
+      if (acc_min < S.tmin[tid]) S.tmin[tid] = acc_min;
+      S.ttiny[tid] += acc_tiny;
+      double* its = p.it_sum + ((size_t)slot * nper + jitem) * p.it_stride;
+      if constexpr (MS) acc_e = acc_es[0], acc_s2 = acc_s2s[0];
+      add_con();
+      const unsigned int wna = __reduce_add_sync(kFull, acc_na);
+      S.u.red_t[0][tid] = acc_e;
+      S.u.red_t[1][tid] = acc_s2;
+      __threadfence_block();
+      __syncwarp();
+      int order = 0;
+      if (lane == 0) {
+        S.red_na[warp] = wna;
+        __threadfence_block();
+        order = atomicAdd(&S.arrive, 1);
       }
-      // |a| < 1e-14, compared on the bit pattern (no FP64 compare)
-      if (abs_bits(a) < 0x3D06849B86A12B9Bull) acc_tiny++;
-      const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
-      acc_min = db < acc_min ? db : acc_min;
-      uint64_t key[NW];  // alpha's words; selects keep them in registers
-      const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
+      order = __shfl_sync(kFull, order, 0);
+      if (order == kWarps - 1) {
+        __threadfence_block();
+        // lanes 0-15 add e, 16-31 (A/D)^2
+        double v = 0.0;
+        const double* src = S.u.red_t[lane >> 4];
+#pragma unroll 4
+        for (int i = lane & 15; i < kThreads; i += 16) v += src[i];
 #pragma unroll
-      for (int w = 0; w < NW; w++)
-        key[w] = S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
-      uint64_t hk = 0;
-#pragma unroll
-      for (int w = 0; w < NW; w++) hk = splitmix64(hk ^ key[w]);
-      acc_d0 += hk;
-      acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
-      // e = A q is formed only when it can reach the threshold: with biased
-      // exponents ea, eq of A and q, |A q| < 2^(ea + eq - 2044), so
-      // ea + eq <= et + 1021 (et: the exponent of tau) puts it below tau
-      const int ea = (int)(abs_bits(a) >> 52), eqx = (int)(abs_bits(q) >> 52);
-      if (p.k > 0 && (tau == 0ull || ea + eqx > (int)(tau >> 52) + 1021)) {
-        const double e = a * q;
-        const unsigned long long eb = abs_bits(e);
-        if (eb >= tau) {
-          atomicAdd(&p.sel_hist[sel_bin(eb)], 1u);
-          const int pos = atomicAdd(&S.tkcnt, 1);
-          te[pos] = e;
-          ta[pos] = a;
-#pragma unroll
-          for (int w = 0; w < NW; w++) tk[(size_t)pos * NW + w] = key[w];
+        for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+        const double vs = __shfl_sync(kFull, v, 16);
+        unsigned long long tn = lane < kWarps ? S.red_na[lane] : 0ull, tc = lane < kWarps ? S.red_con[lane] : 0ull;
+        tn = warp_sum_u(tn);
+        tc = warp_sum_u(tc);
+        if (lane == 0) {
+          its[0] = v;
+          its[1] = vs;
+          S.sw2 = vs;
+          S.arrive = 0;
+          if (tn) {
+            atomicAdd(&p.na[M->g], tn);
+            atomicAdd(&p.ncon[M->g], tc);
+          }
         }
       }
+      if constexpr (MS) {  // the other states' eps and s2, one at a time
+#pragma unroll
+        for (int st = 1; st < kMaxStates; st++) {
+          if (st >= nst) break;
+          __syncthreads();
+          S.u.red_t[0][tid] = acc_es[st];
+          S.u.red_t[1][tid] = acc_s2s[st];
+          __syncthreads();
+          if (warp == 0) {
+            double ue = 0.0, us = 0.0;
+            for (int i = lane; i < kThreads; i += 32) {
+              ue += S.u.red_t[0][i];
+              us += S.u.red_t[1][i];
+            }
+            ue = warp_sum(ue);
+            us = warp_sum(us);
+            if (lane == 0) {
+              its[2 * st] = ue;
+              its[2 * st + 1] = us;
+            }
+          }
+        }
+      }
+      done = true;
+      break;
     }
-  }
-  // ---- per-item reduction into the generator's totals ----
-  {
-    // FP64 sums through shared memory and one warp: a shuffle tree in every
-    // warp would spend five FP64 adds per lane per quantity
-    S.u.red_t[0][tid] = acc_e;
-    S.u.red_t[1][tid] = acc_s2;
-    const unsigned long long na = warp_sum_u(acc_na), nc = warp_sum_u(con), d0 = warp_sum_u(acc_d0);
-    const unsigned long long d1 = warp_xor_u(acc_d1), mn = warp_min_u(acc_min), tiny = warp_sum_u(acc_tiny);
-    if (lane == 0) {
-      S.red_u[warp][0] = na;
-      S.red_u[warp][1] = nc;
-      S.red_u[warp][2] = d0;
-      S.red_u[warp][3] = d1;
-      S.red_u[warp][4] = mn;
-      S.red_u[warp][5] = tiny;
-    }
+    if (done) break;
+    add_con();
     __syncthreads();
-    double se = 0.0, ss = 0.0;
-    if (warp == 0) {
-      for (int i = lane; i < kThreads; i += 32) {
-        se += S.u.red_t[0][i];
-        ss += S.u.red_t[1][i];
-      }
-      se = warp_sum(se);
-      ss = warp_sum(ss);
-    }
-    if (tid == 0) {
-      const double te_ = se, ts = ss;
-      unsigned long long tn = 0, tc = 0, x0 = 0, x1 = 0, m = ~0ull, tt = 0;
-      for (int w = 0; w < kWarps; w++) {
-        tn += S.red_u[w][0];
-        tc += S.red_u[w][1];
-        x0 += S.red_u[w][2];
-        x1 ^= S.red_u[w][3];
-        m = S.red_u[w][4] < m ? S.red_u[w][4] : m;
-        tt += S.red_u[w][5];
-      }
-      S.sw2 = ts;
-      // the item's FP64 sums go to its own slot; the generator's eps_I
-      // and sum A^2/D^2 are reduced from the slots in item order after the
-      // wave (reduce_items_kernel), so they do not depend on which CTA
-      // finished first
-      double* its = p.it_sum + ((size_t)slot * nper + j) * p.it_stride;
-      its[0] = te_;
-      its[1] = ts;
-      if (tn) {
-        atomicAdd(&p.na[g], tn);
-        atomicAdd(&p.ncon[g], tc);
-        atomicAdd(&p.digest[0], x0);
-        atomicXor(&p.digest[1], x1);
-        atomicMin(p.min_den_bits, (unsigned long long)__double_as_longlong(den_double(m, E.dscale)));
-        if (tt) atomicAdd(p.n_tiny, tt);
-      }
-    }
-    if constexpr (MS) {  // the other states' eps and s2, one at a time
-#pragma unroll
-      for (int st = 1; st < kMaxStates; st++) {
-        if (st >= nst) break;
-        __syncthreads();
-        S.u.red_t[0][tid] = acc_es[st];
-        S.u.red_t[1][tid] = acc_s2s[st];
-        __syncthreads();
-        if (warp == 0) {
-          double ue = 0.0, us = 0.0;
-          for (int i = lane; i < kThreads; i += 32) {
-            ue += S.u.red_t[0][i];
-            us += S.u.red_t[1][i];
-          }
-          ue = warp_sum(ue);
-          us = warp_sum(us);
-          if (lane == 0) {
-            double* its = p.it_sum + ((size_t)slot * nper + j) * p.it_stride;
-            its[2 * st] = ue;
-            its[2 * st + 1] = us;
-          }
-        }
-      }
-    }
+    if (tid == 0) S.n0 = S.n1 = S.n2 = S.cnext = 0;
+    __syncthreads();
   }
   if (GRAD) {
     __syncthreads();
     // ---- loop 3: c_J (2A/D) d<J|H|alpha> over the same (J, cell) pairs ----
-    for (int c0 = 0; c0 < total; c0 += kChunk) {
+    for (int c0 = 0; c0 < S.seg_s[3]; c0 += kChunk) {
       if (tid == 0) {
         S.n0 = 0;
         S.n1 = 0;
@@ -2469,17 +2469,17 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         S.cnext = 0;
       }
       __syncthreads();
-      const int c1 = min(c0 + kChunk, total);
+      const int c1 = min(c0 + kChunk, S.seg_s[3]);
       for (int i = c0 + tid; i < c1; i += kThreads) {
         const int o = entry(i);
-        const ulonglong2 en = ehp[o];
+        const ulonglong2 en = S.ehp[o];
         const uint64_t hmr = en.x, part = en.y;
         if (part & kBeforeBit) continue;
         if (dup(i, hmr)) continue;
         const int t = __popcll(hmr & ~B.hm);
         if (t > 2) continue;
         const bool all = (B.h == 1) ? (t <= 1) : (t == 0);
-        const int rec = (int)(erec[o] & 0x7FFFFFFFu);
+        const int rec = (int)(S.erec[o] & 0x7FFFFFFFu);
         if (all) S.u.l.L0[atomicAdd(&S.n0, 1)] = rec;
         else if (t == 1) {
           if (row_live<NINT, NT>(B, S, norb, part)) S.u.l.L12[atomicAdd(&S.n1, 1)] = rec;
@@ -2489,17 +2489,17 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       __syncthreads();
       for (int j = 0; j < S.n0; j++) {
         const int r = S.u.l.L0[j];
-        const uint64_t* Jw = rw + (size_t)r * NW;
-        const double cj = rc[r];
+        const uint64_t* Jw = S.rw + (size_t)r * NW;
+        const double cj = S.rc[r];
         uint32_t X, T;
         int nx, nt;
-        const ulonglong2 en = make_ulonglong2(rhm[r], rpt[r]);
+        const ulonglong2 en = make_ulonglong2(S.rhm[r], S.rpt[r]);
         excitation_sets<NINT, NT>(B, S, en.y, en.x, &X, &nx, &T, &nt);
         for (int cc = tid; cc < B.nct; cc += kThreads) {
           if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
           int ro, so, x, y;
           cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
-          element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, B.sa * norb + ro, (B.h == 2) ? B.sb * norb + so : -1, cj * A[cc]);
+          element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, B.sa * norb + ro, (B.h == 2) ? B.sb * norb + so : -1, cj * a2d(cc));
         }
       }
       {  // row-reaching J (a warp each), then subset-reaching J (32 per draw), drawn dynamically
@@ -2511,9 +2511,9 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           if (jd < n1) {
             const int j = jd;
             const int r = S.u.l.L12[j];
-            const uint64_t* Jw = rw + (size_t)r * NW;
-            const double cj = rc[r];
-            const ulonglong2 en = make_ulonglong2(rhm[r], rpt[r]);
+            const uint64_t* Jw = S.rw + (size_t)r * NW;
+            const double cj = S.rc[r];
+            const ulonglong2 en = make_ulonglong2(S.rhm[r], S.rpt[r]);
           const uint64_t part = en.y;
             uint32_t X, T;
             int nx, nt;
@@ -2521,7 +2521,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             for_row_cells<NINT, NT>(B, S, norb, part, lane, [&](int c, int pc, int zc) {
               const int cc = c - B.clo;
               if ((unsigned)cc >= (unsigned)B.nct || ((ban[cc >> 5] >> (cc & 31)) & 1u)) return;
-              element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, pc, zc, cj * A[cc]);
+              element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, pc, zc, cj * a2d(cc));
             });
           } else {
             const int j0 = (jd - n1) * 32;
@@ -2529,9 +2529,9 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             const int j = j0 + lane;
             if (j < n2) {
               const int r = S.u.l.L12[kChunk - 1 - j];
-              const uint64_t* Jw = rw + (size_t)r * NW;
-              const double cj = rc[r];
-              const ulonglong2 en = make_ulonglong2(rhm[r], rpt[r]);
+              const uint64_t* Jw = S.rw + (size_t)r * NW;
+              const double cj = S.rc[r];
+              const ulonglong2 en = make_ulonglong2(S.rhm[r], S.rpt[r]);
           const uint64_t part = en.y;
               uint32_t X, T;
               int nx, nt;
@@ -2542,7 +2542,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
                 int ro, so, x, y;
                 cell_orbitals<NINT, NT>(B, S, c, &ro, &so, &x, &y);
                 element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, B.sa * norb + ro, (B.h == 2) ? B.sb * norb + so : -1,
-                                   cj * A[cc]);
+                                   cj * a2d(cc));
               });
             }
           }
@@ -2553,6 +2553,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     // ---- diagonal: H_aa = H_II - F(a) [- F(b) + W(a,b)] + F(r) [+ F(s)]
     //      - W(r,a) [- W(r,b) - W(s,a) - W(s,b) + W(r,s)]; the W(r,s) terms
     //      were scattered per cell, the rest goes by row sums ----
+    const int g = M->g;
     double* wF = p.g_wF + (size_t)g * 2 * norb;
     const int s1 = B.sa, s2 = (B.h == 2) ? B.sb : B.sa;
     for (int x = tid; x < S.nv[s1]; x += kThreads) {
@@ -2584,6 +2585,75 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   }
 }
 
+// This CTA's digest, min |D| and tiny counts into the sweep's totals.
+template <int NINT, typename NT>
+__device__ __forceinline__ void flush_totals(const SweepParams& p, BatchShared<NINT, NT>& S, int dscale) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const unsigned long long d0 = warp_sum_u(S.td0[tid]), d1 = warp_xor_u(S.td1[tid]), mn = warp_min_u(S.tmin[tid]);
+  const unsigned int tiny = __reduce_add_sync(kFull, S.ttiny[tid]);
+  if (lane == 0 && mn != ~0ull) {
+    atomicAdd(&p.digest[0], d0);
+    atomicXor(&p.digest[1], d1);
+    atomicMin(p.min_den_bits, (unsigned long long)__double_as_longlong(den_double(mn, dscale)));
+    if (tiny) atomicAdd(p.n_tiny, (unsigned long long)tiny);
+  }
+}
+
+// The shared state of a CTA for the sweep of p.
+template <int NINT, typename NT>
+__device__ __forceinline__ void begin_sweep(const SweepParams& p, BatchShared<NINT, NT>& S) {
+  const int tid = threadIdx.x;
+  S.td0[tid] = S.td1[tid] = 0ull;
+  S.tmin[tid] = ~0ull;
+  S.ttiny[tid] = 0u;
+  if (tid == 0) {
+    S.tkcnt = p.tk_cnt[blockIdx.x];
+    S.tau = p.tk_tau[blockIdx.x];
+    S.arrive = 0;
+    S.nv[0] = p.norb - p.nalpha;
+    S.nv[1] = p.norb - p.nbeta;
+    S.inv_nv1 = S.nv[1] > 0 ? 1.0f / (float)S.nv[1] : 0.0f;
+  }
+}
+
+// Thread 0's draws from the queue of live items (prep_slot's list): an item
+// is published one item ahead, its list entry loaded two ahead and its queue
+// position drawn three ahead, so that no latency of the queue is waited for.
+struct Drawer {
+  int pos, nxt;  // the position drawn last; the next item to publish (-1: none)
+  // take(n): the first of n queue positions
+  template <typename BS, typename Fn>
+  __device__ __forceinline__ void draw(BS& S, int chunk, Fn&& take) {
+    if (S.inext >= S.iend) {
+      const int b0 = take(chunk);
+      S.inext = b0;
+      S.iend = b0 + chunk;
+    }
+    pos = S.inext++;
+  }
+  template <typename BS>
+  __device__ __forceinline__ int entry(const BS& S, const SweepParams& p) const {
+    return (unsigned)pos < (unsigned)S.nlive ? (int)p.live[pos] : -1;
+  }
+  // The first item of the sweep of p.
+  template <typename BS, typename Fn>
+  __device__ __forceinline__ void begin(BS& S, const SweepParams& p, int chunk, Fn&& take) {
+    S.nlive = *p.live_cnt;
+    S.inext = S.iend = 0;
+    draw(S, chunk, take);
+    S.item[0] = entry(S, p);
+    draw(S, chunk, take);
+    nxt = entry(S, p);
+    draw(S, chunk, take);
+  }
+  template <typename BS, typename Fn>
+  __device__ __forceinline__ void advance(BS& S, const SweepParams& p, int par, int chunk, Fn&& take) {
+    S.item[par ^ 1] = nxt;
+    nxt = entry(S, p);
+    draw(S, chunk, take);
+  }
+};
+
 // Three CTAs per SM for one word per spin; two words per spin come with
 // larger accumulators (at most two CTAs fit in shared memory), so those
 // kernels take the registers of two CTAs and do not spill.
@@ -2599,46 +2669,41 @@ template <int NINT, typename NT, bool GRAD = false, bool MS = false, bool E4 = t
 __global__ void __launch_bounds__(kThreads, (NINT == 1) ? 3 : 2) batch_kernel(const __grid_constant__ SweepParams p) {
   static_assert(!(MS && GRAD), "the gradient is a one-state form");
   static_assert(!MS || sizeof(NT) == 8, "the multi-state form is FP64");
-  constexpr int NW = 2 * NINT;
   __shared__ BatchShared<NINT, NT> S;
   const int tid = threadIdx.x;
-  const long long nitems = (long long)p.wave_slots * p.nper;
-  double* te = p.tk_e + (size_t)blockIdx.x * (size_t)p.cap;
-  double* ta = p.tk_a + (size_t)blockIdx.x * (size_t)p.cap;
-  uint64_t* tk = p.tk_key + (size_t)blockIdx.x * (size_t)p.cap * NW;
   const ItemEnv E = item_env<MS>(p);
   const NT* eri_n = numer_eri<NT, E4>(p);
   const NT* h_n = numer_h<NT>(p);
 
-  if (tid == 0) {
-    S.tkcnt = p.tk_cnt[blockIdx.x];
-    S.tau = p.tk_tau[blockIdx.x];
-    S.slot = -1;
-    S.inext = S.iend = 0;
-    if (p.timeout_ns) atomicCAS(p.t_start, 0ull, global_ns());
-  }
+  begin_sweep<NINT, NT>(p, S);
   const int F = MS ? 0 : fix_scale(p);  // fixed-point scale of A_alpha (units of 2^-F)
-
-  for (;;) {
-    __syncthreads();
-    if (tid == 0) {  // the next work item: p.chunk of them per draw from the queue
-      if (S.inext >= S.iend) {
-        const long long b0 = atomicAdd(p.queue, p.chunk);
-        S.inext = b0;
-        S.iend = b0 + p.chunk;
-      }
-      S.item = S.inext++;
-      if (p.timeout_ns && global_ns() - *((volatile unsigned long long*)p.t_start) > p.timeout_ns) {
-        atomicOr(p.err, 128);  // watchdog: stop taking work, report the timeout
-        S.item = nitems;
-      }
-    }
-    __syncthreads();
-    const long long item = S.item;
-    if (item >= nitems) break;
-    batch_item<NINT, NT, GRAD, MS, E4>(p, S, item, F, te, ta, tk, E, eri_n, h_n);
+  auto take = [&](int n) { return atomicAdd(p.queue, n); };
+  // watchdog: stop taking work, report the timeout
+  auto expired = [&]() {
+    if (!p.timeout_ns || global_ns() - *((volatile unsigned long long*)p.t_start) <= p.timeout_ns) return false;
+    atomicOr(p.err, 128);
+    return true;
+  };
+  Drawer D;
+  if (tid == 0) {
+    if (p.timeout_ns) atomicCAS(p.t_start, 0ull, global_ns());
+    D.begin(S, p, p.chunk, take);
   }
-  if (p.k > 0 && p.last_wave) compact_selection<NINT, NT>(p, S, te, ta, tk);
+  for (int par = 0;; par ^= 1) {
+    __syncthreads();
+    const int item = S.item[par];
+    if (item < 0) break;
+    if (tid == 0) {
+      if (D.nxt >= 0 && expired()) {
+        S.nlive = 0;
+        D.nxt = -1;
+      }
+      D.advance(S, p, par, p.chunk, take);
+    }
+    batch_item<NINT, NT, GRAD, MS, E4>(p, S, item, F, E, eri_n, h_n);
+  }
+  flush_totals<NINT, NT>(p, S, E.dscale);
+  if (p.k > 0 && p.last_wave) compact_selection<NINT, NT>(p, S, buf_e(p), buf_a(p), buf_key<NINT>(p));
   __syncthreads();
   if (tid == 0) {
     p.tk_cnt[blockIdx.x] = S.tkcnt;
@@ -2658,50 +2723,41 @@ __global__ void __launch_bounds__(kThreads, (NINT == 1) ? 3 : 2) batch_kernel(co
 // wave.
 template <int NINT, typename NT>
 __global__ void __launch_bounds__(kThreads, (NINT == 1) ? 3 : 2) batch_multi_kernel(const __grid_constant__ MultiWaveInline m) {
-  constexpr int NW = 2 * NINT;
   __shared__ BatchShared<NINT, NT> S;
   const int tid = threadIdx.x;
   if (tid == 0 && m.timeout_ns) atomicCAS(m.t_start, 0ull, global_ns());
-  bool stop = false;
   // the pieces one after another, each from its own queue: the piece index
   // is the same in every thread, so its parameters are read like a single
   // sweep's
 #pragma unroll 1
-  for (int pc = 0; pc < m.n && !stop; pc++) {
+  for (int pc = 0; pc < m.n; pc++) {
     const SweepParams& p = m.ps[pc];
-    const long long nitems = m.item_ofs[pc + 1] - m.item_ofs[pc];
     __syncthreads();
-    if (tid == 0) {
-      S.tkcnt = p.tk_cnt[blockIdx.x];
-      S.tau = p.tk_tau[blockIdx.x];
-      S.slot = -1;
-      S.inext = S.iend = 0;
-    }
+    begin_sweep<NINT, NT>(p, S);
     const int F = fix_scale(p);
     const ItemEnv E = item_env<false>(p);
-    double* te = p.tk_e + (size_t)blockIdx.x * (size_t)p.cap;
-    double* ta = p.tk_a + (size_t)blockIdx.x * (size_t)p.cap;
-    uint64_t* tk = p.tk_key + (size_t)blockIdx.x * (size_t)p.cap * NW;
-    for (;;) {
+    auto take = [&](int n) { return (int)atomicAdd(m.queue + pc, (unsigned long long)n); };
+    auto expired = [&]() {
+      if (!m.timeout_ns || global_ns() - *((volatile unsigned long long*)m.t_start) <= m.timeout_ns) return false;
+      atomicOr(m.err, 128);  // watchdog: stop taking work, report the timeout
+      return true;
+    };
+    Drawer D;
+    if (tid == 0) D.begin(S, p, m.chunk, take);
+    for (int par = 0;; par ^= 1) {
       __syncthreads();
+      const int item = S.item[par];
+      if (item < 0) break;
       if (tid == 0) {
-        if (S.inext >= S.iend) {
-          const long long b0 = (long long)atomicAdd(m.queue + pc, (unsigned long long)m.chunk);
-          S.inext = b0;
-          S.iend = b0 + m.chunk;
+        if (D.nxt >= 0 && expired()) {
+          S.nlive = 0;
+          D.nxt = -1;
         }
-        S.item = S.inext++;
-        if (m.timeout_ns && global_ns() - *((volatile unsigned long long*)m.t_start) > m.timeout_ns) {
-          atomicOr(m.err, 128);  // watchdog: stop taking work, report the timeout
-          S.item = -1;
-        }
+        D.advance(S, p, par, m.chunk, take);
       }
-      __syncthreads();
-      const long long item = S.item;
-      if (item < 0) stop = true;
-      if (item < 0 || item >= nitems) break;
-      batch_item<NINT, NT, false, false, true>(p, S, item, F, te, ta, tk, E, numer_eri<NT, true>(p), numer_h<NT>(p));
+      batch_item<NINT, NT, false, false, true>(p, S, item, F, E, numer_eri<NT, true>(p), numer_h<NT>(p));
     }
+    flush_totals<NINT, NT>(p, S, E.dscale);
     __syncthreads();
     if (tid == 0) {
       p.tk_cnt[blockIdx.x] = S.tkcnt;
