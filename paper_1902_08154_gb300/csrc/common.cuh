@@ -107,11 +107,12 @@ __host__ __device__ inline int mask_words(int norb, int na, int nb) {  // even: 
 __host__ __device__ inline int orb_mask_words(int nint, int nel) { return (4 + 3 * nel) * nint; }
 
 // Dynamic shared memory of the one-state batch kernel for mc cells: A_alpha
-// as a 96-bit integer per cell (a 64-bit low word and a 32-bit high word; the
-// exact accumulation in sweep_impl.cuh) and one ban bit per cell.
+// as a 96-bit integer per cell (three 32-bit words; the exact accumulation in
+// sweep_impl.cuh), one ban bit per cell and the list of the cells left (16 bits
+// each).
 __host__ __device__ inline size_t sweep_smem(int mc) {
   const size_t m = (size_t)(mc < 1 ? 1 : mc);
-  return 8 * m + 4 * ((m + 1) & ~(size_t)1) + 4 * ((m + 31) / 32);
+  return 8 * m + 4 * ((m + 1) & ~(size_t)1) + 4 * ((m + 31) / 32) + 2 * m;
 }
 
 struct GenMeta;

@@ -54,7 +54,7 @@ namespace qp {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kChunk = 512;  // bucket entries classified per round
-constexpr int kGroup = 8;     // J reaching every cell, handled together
+constexpr int kGroup = 6;     // J reaching every cell, handled together
 constexpr unsigned kFull = 0xffffffffu;
 // Bit of a bucket entry's particle word that flags a J ranked before I (see
 // part_code below).
@@ -873,11 +873,15 @@ struct BatchShared {
   unsigned char vir[2][kMaxOrb], vidx[2][kMaxOrb];
   int nv[2];  // the sweep's virtual orbitals per spin
   float inv_nv1;
-  // fixed point (den_scale): per-batch row sums for H_aa, E0 - base - u0[x]
-  long long u0[kMaxOrb], u1[kMaxOrb], dx[kMaxOrb];
-  // two-hole batches: <I|H|I - H + R> by pair tables like those of the J
-  // reaching every cell (its particles are the hole pair H itself)
-  int iRow[kMaxOrb], iCol[kMaxOrb];
+  // per virtual orbital of the cells' row and column: d in fixed point
+  // (den_scale), E0 - H_II + ... of the row (E0 - base - u0) and the sum u of
+  // the column for H_aa; the orbital; idx: <I|H|I - H + R> by pair tables like
+  // those of the J reaching every cell (its particles are the hole pair H)
+  struct __align__(16) Side {
+    long long d;
+    int idx, orb;
+  } row[kMaxOrb], col[kMaxOrb];
+  uint64_t hk0[kMaxOrb];  // digest fold of the spin-up words of a row's determinants
   NT cI;
   uint64_t kbase[2 * NINT];  // I with the batch's holes removed
   // rows (and columns) of cells banned as a whole by J ranked before I, bits
@@ -932,9 +936,10 @@ struct BatchShared {
   int arrive;
   unsigned long long red_na[kWarps], red_con[kWarps];
   double sw2;
-  // totals of this thread over the sweep: digest sum and xor, min |D|, |A| < 1e-14
+  // totals over the sweep: digest sum and xor, min |D| (of a thread each), |A| < 1e-14
   unsigned long long td0[kThreads], td1[kThreads], tmin[kThreads];
-  uint32_t ttiny[kThreads];
+  unsigned int tiny;
+  int nlist;  // cells left after the bans
 };
 
 template <int NINT, typename NT>
@@ -1006,17 +1011,22 @@ __device__ __forceinline__ void for_subset_cells(const Batch& B, const BatchShar
   if (B.kind == 0) {
     int np;
     const uint32_t P = particles_of_spin(part, norb, B.sa, &np);
+#pragma unroll 1
     for (int i = 0; i < np; i++) fn(S.vidx[B.sa][pk(P, i)]);
   } else if (B.kind == 1) {
     int np;
     const uint32_t P = particles_of_spin(part, norb, B.sa, &np);
+#pragma unroll 1
     for (int i = 0; i < np; i++)
+#pragma unroll 1
       for (int j = i + 1; j < np; j++) fn(pair_cell(S.vidx[B.sa][pk(P, i)], S.vidx[B.sa][pk(P, j)]));
   } else {
     int na, nb;
     const uint32_t Pa = particles_of_spin(part, norb, 0, &na);
     const uint32_t Pb = particles_of_spin(part, norb, 1, &nb);
+#pragma unroll 1
     for (int i = 0; i < na; i++)
+#pragma unroll 1
       for (int j = 0; j < nb; j++) fn(S.vidx[0][pk(Pa, i)] * S.nv[1] + S.vidx[1][pk(Pb, j)]);
   }
 }
@@ -1454,6 +1464,7 @@ struct ItemEnv {
   double* A;
   uint32_t *A0, *A1, *A2;
   uint32_t* ban;
+  unsigned short* lst;  // one-state form: the cells left, x << 8 | y
   double *ms_gc, *ms_cI, *ms_w;
   long long* ms_de;  // E0_s - E0_0, fixed point
   int mc, nst, norb, nel, nbat, nper;
@@ -1471,6 +1482,7 @@ __device__ __forceinline__ ItemEnv item_env(const SweepParams& p) {
   E.A1 = E.A0 + E.mc;
   E.A2 = E.A1 + E.mc;
   E.ban = MS ? reinterpret_cast<uint32_t*>(E.A + p.nst * E.mc) : E.A2 + ((E.mc + 1) & ~1);
+  E.lst = reinterpret_cast<unsigned short*>(E.ban + (E.mc + 31) / 32);
   E.ms_gc = reinterpret_cast<double*>(E.ban + (((E.mc + 31) / 32 + 1) & ~1));
   E.ms_cI = E.ms_gc + kGroup * kMaxStates;
   E.ms_w = E.ms_cI + kMaxStates;
@@ -1582,6 +1594,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   B.cb = B.h == 2 ? M->occ[B.ib] : -1;
   B.qb = B.h == 2 ? B.cb - B.sb * norb : -1;
   const int ibase = B.h == 2 ? (B.qa * norb + B.qb) * norb * norb : 0;
+#pragma unroll 1
   for (int x = tid; x < 2 * norb; x += kThreads) {  // a thread per orbital and spin
     const int s = x >= norb, q = x - s * norb;
     uint64_t sw[NINT];
@@ -1608,21 +1621,32 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       if (isrow) {  // E0 - base - u0, base = H_II - F(a) [- F(b) + W(a, b)]
         long long base = M->hii - M->F[B.sa][B.qa];
         if (B.h == 2) base += (B.kind == 1 ? p.Wi : p.Ji)[B.qa * norb + B.qb] - M->F[B.sb][B.qb];
-        S.u0[v] = u;
-        S.dx[v] = (E.e0 - base) - u;
-      }
-      if (iscol) S.u1[v] = u;
-      if (B.h == 2) {  // pair tables of J = I: its particles x1, x2 are the holes a, b
-        if (isrow) {
+        int idx = 0;  // pair tables of J = I: its particles x1, x2 are the holes a, b
+        if (B.h == 2) {
           const int par = count_between<NINT>(sw, q < B.qa ? q : B.qa, q < B.qa ? B.qa : q) & 1;
-          S.iRow[v] = (E4 ? ibase + q * norb : tri(B.qa, q)) | (par << 31);
+          idx = (E4 ? ibase + q * norb : tri(B.qa, q)) | (par << 31);
         }
-        if (iscol) {
-          const int lo = q < B.qb ? q : B.qb, hi = q < B.qb ? B.qb : q;
-          int par = count_between<NINT>(sw, lo, hi) & 1;
-          if (B.kind == 1) par ^= (B.qa > lo && B.qa < hi) ? 1 : 0;
-          S.iCol[v] = (E4 ? q : tri(B.qb, q)) | (par << 31);
+        S.row[v].d = (E.e0 - base) - u;
+        S.row[v].idx = idx;
+        S.row[v].orb = q;
+        // spin-up words: of the row's cells (opposite-spin batch), or I's
+        uint64_t hk = 0;
+#pragma unroll
+        for (int w = 0; w < NINT; w++) {
+          uint64_t up = s == 0 ? sw[w] : M->I[w];
+          if (s == 0 && (B.qa >> 6) == w) up &= ~(1ull << (B.qa & 63));
+          if (s == 0 && (q >> 6) == w) up |= 1ull << (q & 63);
+          hk = splitmix64(hk ^ up);
         }
+        S.hk0[v] = hk;
+      }
+      if (iscol) {
+        const int lo = q < B.qb ? q : B.qb, hi = q < B.qb ? B.qb : q;
+        int par = count_between<NINT>(sw, lo, hi) & 1;
+        if (B.kind == 1) par ^= (B.qa > lo && B.qa < hi) ? 1 : 0;
+        S.col[v].d = u;
+        S.col[v].idx = (E4 ? q : tri(B.qb, q)) | (par << 31);
+        S.col[v].orb = q;
       }
     }
   }
@@ -1645,8 +1669,10 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       ms_de[tid] = den_fix(p.st_e0[tid], E.dscale) - E.e0;
     }
     for (int st = 0; st < nst; st++)
+#pragma unroll 1
       for (int c = tid; c < B.nct; c += kThreads) A[st * mc + c] = 0.0;
   } else {
+#pragma unroll 1
     for (int c = tid; c < B.nct; c += kThreads) A0[c] = A1[c] = A2[c] = 0u;
   }
   // bans by J ranked before I: the masks of the slot and the batch's holes
@@ -1660,6 +1686,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     const uint32_t* m2 = gm + mbase + B.ib * md.hs + (B.kind == 2 ? mix : 0);
     const int nw32 = (B.ncell + 31) / 32;
     auto word = [&](int w) { return w < nw32 ? m0[w] | m1[w] | m2[w] : 0u; };
+#pragma unroll 1
     for (int w = tid; w < (B.nct + 31) / 32; w += kThreads) {
       const int at = (B.clo >> 5) + w;
       ban[w] = __funnelshift_r(word(at), (B.clo & 31) ? word(at + 1) : 0u, B.clo & 31);
@@ -1669,6 +1696,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   __syncthreads();
   if (B.h == 1) {
     const uint64_t *b1 = om + (2 + B.sa) * NINT, *h1 = om + (6 + 3 * B.ia) * NINT;
+#pragma unroll 1
     for (int c0 = 0; c0 < B.nct; c0 += kThreads) {
       const int c = c0 + tid, r = c < B.nct ? S.vir[B.sa][c] : 0;
       const unsigned f = __ballot_sync(kFull, c < B.nct && (((b1[r >> 6] | h1[r >> 6]) >> (r & 63)) & 1ull));
@@ -1677,6 +1705,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     __syncthreads();
   }
   if (p.tgt_on) {  // cells outside the target space contribute nothing: ban them
+#pragma unroll 1
     for (int cc = tid; cc < B.nct; cc += kThreads) {
       int ro, so, x, y;
       cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
@@ -1697,6 +1726,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   // ---- loop 1: bans by the entries of the batch's own bucket.  J ranked
   // before I: rows (t = 1) and cells (t = 2); a later J equal to a cell's
   // alpha bans that cell ----
+#pragma unroll 1
   for (int i = tid; i < S.seg_s[0]; i += kThreads) {
     const ulonglong2 en = i < kThreads ? en0 : S.ehp[S.seg_o[0] + i];
     const uint64_t hm = en.x, part = en.y;
@@ -1717,9 +1747,11 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   if (B.h == 2) {  // flagged rows and columns as cell bans: a row per thread, 32 cells at a time
     const int scol = B.kind == 2 ? 1 : B.sa, srow = B.kind == 2 ? 0 : B.sa, nvc = S.nv[scol];
     const int x0 = B.kind == 2 ? B.clo / nvc : 0, x1 = B.kind == 2 ? x0 + B.nct / nvc : nvc;
+#pragma unroll 1
     for (int y = 0; y < nvc; y += 32) {
       const unsigned fw =
           __ballot_sync(kFull, y + lane < nvc && row_banned<NINT, NT>(S, scol, S.vir[scol][(y + lane) & (kMaxOrb - 1)]));
+#pragma unroll 1
       for (int x = x0 + tid; x < x1; x += kThreads) {
         const int len = B.kind == 2 ? nvc : x;  // same spin: the cells (y, x), y < x
         if (y >= len) continue;
@@ -1763,11 +1795,13 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     }
     phase_mask<NINT>(w1, x1, 0, M1);
     phase_mask<NINT>(w2, x2, 0, M2);
+#pragma unroll 1
     for (int v = lane; v < S.nv[sr]; v += 32) {
       const int q = S.vir[sr][v];
       const int ex = q == x1 || (B.kind == 1 && q == x2) ? 1 << 30 : 0;
       S.v.g.gRow[j][v] = (E4 ? gB + q * norb : tri(x1, q)) | ex | ((int)mask_bit<NINT>(M1, q) << 31);
     }
+#pragma unroll 1
     for (int v = lane; v < S.nv[sc]; v += 32) {
       const int q = S.vir[sc][v];
       const int ex = q == x2 || (B.kind == 1 && q == x1) ? 1 << 30 : 0;
@@ -1790,9 +1824,11 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     if (lane == 0) S.red_con[warp] += wcon;
     con = 0;
   };
+#pragma unroll 1
   for (int c0 = 0;; c0 += kChunk) {
     const int total = S.seg_s[3], c1 = min(c0 + kChunk, total);
     const bool last_round = c0 + kChunk >= total;
+#pragma unroll 1
     for (int i = c0 + tid; i < c1; i += kThreads) {
       const int o = entry(i);
       const ulonglong2 en = i < kThreads ? en0 : S.ehp[o];
@@ -1833,7 +1869,10 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       const int nrow = S.n1, n2 = S.n2;
       const int ntab = B.h == 2 ? (n0 < kGroup ? n0 : kGroup) : 0;
       const int nvm = S.nv[0] > S.nv[1] ? S.nv[0] : S.nv[1], nch = (nvm + 31) / 32;
-      const int nall = ntab + n0 * B.h * nch;  // pair tables, then (J, particle slot, 32 cells)
+      // units: the list of the cells left (256 cells each), pair tables, rows of
+      // the J reaching every cell (J, particle slot, 32 cells), row J, the rest
+      const int ncmp = !MS && c0 == 0 ? (B.nct + 255) / 256 : 0;
+      const int nall = ncmp + ntab + n0 * B.h * nch;
       int per = (nrow + kWarps - 1) / kWarps;
       per = per > 8 ? 8 : per;
       const int ndraw = nall + (per ? (nrow + per - 1) / per : 0);
@@ -1856,10 +1895,52 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         int jd = 0;
         if (lane == 0) jd = atomicAdd(&S.cnext, 1);
         jd = __shfl_sync(kFull, jd, 0);
-        if (jd < ntab) {
-          build_table(jd, S.u.l.L0[jd]);
+        if (jd < ncmp) {
+          // cells not banned, in cell order: a byte of the ban bits per lane
+          auto left = [&](int w) {
+            const int n = B.nct - 32 * w;
+            return n <= 0 ? 0u : ~ban[w] & (n >= 32 ? ~0u : (1u << n) - 1u);
+          };
+          const int nw = (B.nct + 31) / 32;
+          unsigned before = 0, all = 0;
+#pragma unroll 1
+          for (int w = lane; w < (jd == 0 ? nw : 8 * jd); w += 32) {
+            const unsigned c = __popc(left(w));
+            all += c;
+            if (w < 8 * jd) before += c;
+          }
+          before = __reduce_add_sync(kFull, before);
+          all = __reduce_add_sync(kFull, all);
+          if (jd == 0 && lane == 0) S.nlist = (int)all;
+          const int hb = 32 * jd + lane;
+          const unsigned bits = (left(hb >> 2) >> (8 * (hb & 3))) & 0xFFu;
+          int at = __popc(bits);
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(kFull, at, o);
+            if (lane >= o) at += t;
+          }
+          at += (int)before - __popc(bits);
+          if (bits) {
+            int ro, so, x, y;
+            cell_orbitals<NINT, NT>(B, S, B.clo + 8 * hb, &ro, &so, &x, &y);
+            const int nv1 = S.nv[1];
+            if (B.kind == 0) y = 0;
+#pragma unroll 1
+            for (int k = 0; k < 8; k++) {
+              if ((bits >> k) & 1u) E.lst[at++] = (unsigned short)(x << 8 | y);
+              if (B.kind == 2) {
+                if (++y == nv1) y = 0, x++;
+              } else if (++x == y && B.kind == 1) {
+                x = 0;
+                y++;
+              }
+            }
+          }
+        } else if (jd < ncmp + ntab) {
+          build_table(jd - ncmp, S.u.l.L0[jd - ncmp]);
         } else if (jd < nall) {
-          const int ju = jd - ntab, j = ju / (B.h * nch), rem = ju - j * (B.h * nch), ip = rem / nch, y = (rem - ip * nch) * 32 + lane;
+          const int ju = jd - ncmp - ntab, j = ju / (B.h * nch), rem = ju - j * (B.h * nch), ip = rem / nch, y = (rem - ip * nch) * 32 + lane;
           const int r = S.u.l.L0[j];
           const uint64_t hm = S.rhm[r], part = S.rpt[r];
           uint32_t X, T;
@@ -1886,10 +1967,11 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           NT v = h_n[uz * norb + z];
           // J's orbitals in ascending order (the FP32 form's sum depends on
           // it), four at a time so that their loads overlap
-#pragma unroll
+#pragma unroll 1
           for (int w = 0; w < NW; w++) {
             uint64_t bits = S.rw[(size_t)r * NW + w];
             const bool sp = w / NINT == sz;
+#pragma unroll 1
             while (bits) {
               int o[4];
               NT a[4], b[4];
@@ -2014,6 +2096,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
               }
             }
           }
+#pragma unroll 1
           for (unsigned m = __ballot_sync(kFull, act); m; m &= m - 1) {
             const int src = __ffs((int)m) - 1;
             const uint32_t iwr = __shfl_sync(kFull, iw, src);
@@ -2029,6 +2112,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             // the integrals at b1 + z and (same spin) b2 + z
             const int b1 = ((uo * norb + uz) * norb + q) * norb, b2 = ((uz * norb + uo) * norb + q) * norb;
             // two rounds of 32 cells at a time, their loads in flight together
+#pragma unroll 1
             for (int y0 = lane; y0 < nz; y0 += 64) {
               int cc[2], zz[2];
               NT v[2], w2[2];
@@ -2063,6 +2147,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
                 }
             }
           }
+#pragma unroll 1
           for (unsigned m = __ballot_sync(kFull, sact); m; m &= m - 1) {
             const int src = __ffs((int)m) - 1;
             const uint32_t sc = __shfl_sync(kFull, scell, src), wq = __shfl_sync(kFull, sw, src);
@@ -2072,6 +2157,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             const int wo = wq & 0xFF, qo = (wq >> 8) & 0xFF, sq = (wq >> 16) & 1;
             NT v = NT(0);
             if constexpr (sizeof(NT) == 8) {  // J's orbitals: I's, with particles in the place of its holes
+#pragma unroll 1
               for (int i = lane; i < nel; i += 32) {
                 int mo = S.occ[i];
                 if ((hmr >> i) & 1ull) mo = part_code(ptr_, __popcll(hmr & ((1ull << i) - 1)));
@@ -2164,6 +2250,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     // perturbers of I in this batch ----
     const int nt0 = B.h == 2 ? n0 : 0;
     bool done = false;
+#pragma unroll 1
     for (int g0 = 0;; g0 += kGroup) {
       B = S.bt;
       const int m = max(0, min(kGroup, nt0 - g0));
@@ -2171,6 +2258,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       if (!fin && m == 0) break;
       if (g0 > 0 && m > 0) {  // the first group's tables came with the row pass
         __syncthreads();
+#pragma unroll 1
         for (int j = warp; j < m; j += kWarps) build_table(j, S.u.l.L0[g0 + j]);
         __syncthreads();
       }
@@ -2188,14 +2276,28 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       const unsigned long long tau = S.tau;
       double acc_e = 0.0, acc_s2 = 0.0;
       unsigned long long acc_d0 = 0, acc_d1 = 0, acc_min = ~0ull;  // acc_min: units of 2^-S
-      unsigned int acc_na = 0, acc_tiny = 0;
+      unsigned int acc_na = 0;  // multi-state form
       double acc_es[kMaxStates], acc_s2s[kMaxStates];  // multi-state form: sums per state
 #pragma unroll
       for (int st = 0; st < kMaxStates; st++) acc_es[st] = acc_s2s[st] = 0.0;
-      for (int cc = tid; cc < B.nct; cc += kThreads) {
-        if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
-        int ro, so, x, y;
-        cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
+      const int nv1 = S.nv[1], nleft = MS ? B.nct : S.nlist;
+#pragma unroll 1
+      for (int i = tid; i < nleft; i += kThreads) {
+        int x, y, cc;
+        if constexpr (MS) {
+          cc = i;
+          if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
+          int ro, so;
+          cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
+          y = y < 0 ? 0 : y;
+        } else {
+          const int xy = E.lst[i];
+          x = xy >> 8;
+          y = xy & 0xFF;
+          cc = (B.kind == 2 ? x * nv1 + y : B.kind == 1 ? y * (y - 1) / 2 + x : x) - B.clo;
+        }
+        const typename BatchShared<NINT, NT>::Side R = S.row[x], C = S.col[y];
+        const int ro = R.orb, so = C.orb;
         unsigned long long lo = 0ull;  // exact sum
         int hi = 0;
         double accs[kMaxStates];  // multi-state form: one sum per state
@@ -2205,6 +2307,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           lo = A0[cc] | ((unsigned long long)A1[cc] << 32);
           hi = (int)A2[cc];
         }
+#pragma unroll 1
         for (int j = 0; j < m; j++) {
           const int rt = S.v.g.gRow[j][x], ct = S.v.g.gCol[j][y];
           if ((rt | ct) & (1 << 30)) continue;
@@ -2249,25 +2352,22 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         if constexpr (MS) {
           double vI = 0.0;  // <I|H|alpha> for the generator's own term
           if (B.h == 2) {
-            const int a1 = S.iRow[x], b2 = S.iCol[y];
-            if (B.kind == 2) {
-              vI = (double)flip_sign(eri_n[E4 ? (a1 & 0x7fffffff) + (b2 & 0x7fffffff) : tri(a1 & 0x7fffffff, b2 & 0x7fffffff)],
-                                     (a1 ^ b2) < 0);
+            NT t;
+            bool neg = (R.idx ^ C.idx) < 0;
+            if constexpr (E4) {
+              t = eri_n[(R.idx & 0x7fffffff) + (C.idx & 0x7fffffff)];
+              if (B.kind == 1) t -= eri_n[ibase + so * norb + ro];
             } else {
-              const int a2 = S.iRow[y], b1 = S.iCol[x];
-              NT v;
-              if constexpr (E4)
-                v = eri_n[(a1 & 0x7fffffff) + (b2 & 0x7fffffff)] - eri_n[ibase + so * norb + ro];
-              else
-                v = eri_n[tri(a1 & 0x7fffffff, b2 & 0x7fffffff)] - eri_n[tri(a2 & 0x7fffffff, b1 & 0x7fffffff)];
-              const int lo = so < B.qb ? so : B.qb, hi = so < B.qb ? B.qb : so;
-              vI = (double)flip_sign(v, ((a1 ^ b2) < 0 ? 1 : 0) ^ ((ro > lo && ro < hi) ? 1 : 0));
+              t = eri_n[tri(R.idx & 0x7fffffff, C.idx & 0x7fffffff)];
+              if (B.kind == 1) t -= eri_n[tri(S.row[y].idx & 0x7fffffff, S.col[x].idx & 0x7fffffff)];
             }
+            if (B.kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
+            t = flip_sign(t, neg);
+            vI = (double)t;
             con++;
           }
-          long long D0 = S.dx[x];  // E0_0 - H_aa
-          if (B.kind == 2) D0 -= S.u1[y] + p.Ji[ro * norb + so];
-          else if (B.kind == 1) D0 -= S.u0[y] + p.Wi[ro * norb + so];
+          long long D0 = R.d;  // E0_0 - H_aa
+          if (B.h == 2) D0 -= C.d + (B.kind == 2 ? p.Ji : p.Wi)[ro * norb + so];
           double crit = 0.0, a0 = 0.0;
 #pragma unroll
           for (int st = 0; st < kMaxStates; st++) {
@@ -2284,7 +2384,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             if (st == 0) a0 = a;
           }
           acc_na++;
-          if (abs_bits(a0) < 0x3D06849B86A12B9Bull) acc_tiny++;
+          if (abs_bits(a0) < 0x3D06849B86A12B9Bull) atomicAdd(&S.tiny, 1u);
           uint64_t key[NW];
           const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
 #pragma unroll
@@ -2308,31 +2408,27 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           }
         } else {
           double a = fix_to_double(lo, hi, F);
-          if (B.h == 2) {  // the generator's own term c_I <I|H|alpha>
-            NT v;
-            const int a1 = S.iRow[x], b2 = S.iCol[y];
-            if (B.kind == 2) {
-              v = flip_sign(eri_n[E4 ? (a1 & 0x7fffffff) + (b2 & 0x7fffffff) : tri(a1 & 0x7fffffff, b2 & 0x7fffffff)], (a1 ^ b2) < 0);
+          // the generator's own term c_I <I|H|alpha>
+          if (B.h == 2) {
+            NT t;
+            bool neg = (R.idx ^ C.idx) < 0;
+            if constexpr (E4) {
+              t = eri_n[(R.idx & 0x7fffffff) + (C.idx & 0x7fffffff)];
+              if (B.kind == 1) t -= eri_n[ibase + so * norb + ro];
             } else {
-              const int a2 = S.iRow[y], b1 = S.iCol[x];
-              if constexpr (E4)
-                v = eri_n[(a1 & 0x7fffffff) + (b2 & 0x7fffffff)] - eri_n[ibase + so * norb + ro];
-              else
-                v = eri_n[tri(a1 & 0x7fffffff, b2 & 0x7fffffff)] - eri_n[tri(a2 & 0x7fffffff, b1 & 0x7fffffff)];
-              const int lo = so < B.qb ? so : B.qb, hi = so < B.qb ? B.qb : so;
-              v = flip_sign(v, ((a1 ^ b2) < 0 ? 1 : 0) ^ ((ro > lo && ro < hi) ? 1 : 0));
+              t = eri_n[tri(R.idx & 0x7fffffff, C.idx & 0x7fffffff)];
+              if (B.kind == 1) t -= eri_n[tri(S.row[y].idx & 0x7fffffff, S.col[x].idx & 0x7fffffff)];
             }
-            a += (double)(S.cI * v);
-            con++;
+            if (B.kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
+            t = flip_sign(t, neg);
+            a += (double)(S.cI * t);
           }
-          // D = E0 - H_aa from the per-batch row sums
-          long long D = S.dx[x];
-          if (B.kind == 2) D -= S.u1[y] + p.Ji[ro * norb + so];
-          else if (B.kind == 1) D -= S.u0[y] + p.Wi[ro * norb + so];
+          // D = E0 - H_aa from the row and column sums
+          long long D = R.d;
+          if (B.h == 2) D -= C.d + (B.kind == 2 ? p.Ji : p.Wi)[ro * norb + so];
           const double q = div_fix(a, D, E.dscale);
           acc_e = fma(a, q, acc_e);  // e = A q
           acc_s2 += q * q;
-          acc_na++;
           if (GRAD) {
             // numerator weight 2A/D for loop 3; (A/D)^2 weights the diagonal
             const unsigned long long wb = (unsigned long long)__double_as_longlong(2.0 * q);
@@ -2345,17 +2441,24 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             if (B.h == 2) w_grad(p, ro, B.sa, so, B.sb, w2);
           }
           // |a| < 1e-14, compared on the bit pattern (no FP64 compare)
-          if (abs_bits(a) < 0x3D06849B86A12B9Bull) acc_tiny++;
+          if (abs_bits(a) < 0x3D06849B86A12B9Bull) atomicAdd(&S.tiny, 1u);
           const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
           acc_min = db < acc_min ? db : acc_min;
-          uint64_t key[NW];  // alpha's words; selects keep them in registers
+          // alpha's word w: the batch's base with the cell's orbitals
           const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
+          auto key = [&](int w) {
+            return S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
+          };
+          // digest: the fold over the spin-up words is the row's where they
+          // depend on the row alone
+          uint64_t hk = S.hk0[x];
+          if (B.kind != 2 && B.sa == 0) {
+            hk = 0;
 #pragma unroll
-          for (int w = 0; w < NW; w++)
-            key[w] = S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
-          uint64_t hk = 0;
+            for (int w = 0; w < NINT; w++) hk = splitmix64(hk ^ key(w));
+          }
 #pragma unroll
-          for (int w = 0; w < NW; w++) hk = splitmix64(hk ^ key[w]);
+          for (int w = NINT; w < NW; w++) hk = splitmix64(hk ^ key(w));
           acc_d0 += hk;
           acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
           // e = A q is formed only when it can reach the threshold: with biased
@@ -2371,7 +2474,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
               buf_e(p)[pos] = e;
               buf_a(p)[pos] = a;
 #pragma unroll
-              for (int w = 0; w < NW; w++) buf_key<NINT>(p)[(size_t)pos * NW + w] = key[w];
+              for (int w = 0; w < NW; w++) buf_key<NINT>(p)[(size_t)pos * NW + w] = key(w);
             }
           }
         }
@@ -2386,11 +2489,10 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       S.td0[tid] += acc_d0;
       S.td1[tid] ^= acc_d1;
       if (acc_min < S.tmin[tid]) S.tmin[tid] = acc_min;
-      S.ttiny[tid] += acc_tiny;
       double* its = p.it_sum + ((size_t)slot * nper + jitem) * p.it_stride;
       if constexpr (MS) acc_e = acc_es[0], acc_s2 = acc_s2s[0];
       add_con();
-      const unsigned int wna = __reduce_add_sync(kFull, acc_na);
+      const unsigned int wna = MS ? __reduce_add_sync(kFull, acc_na) : 0u;
       S.u.red_t[0][tid] = acc_e;
       S.u.red_t[1][tid] = acc_s2;
       __threadfence_block();
@@ -2415,6 +2517,10 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         unsigned long long tn = lane < kWarps ? S.red_na[lane] : 0ull, tc = lane < kWarps ? S.red_con[lane] : 0ull;
         tn = warp_sum_u(tn);
         tc = warp_sum_u(tc);
+        if constexpr (!MS) {  // every cell of the list, each with the generator's own term (two-hole batch)
+          tn = (unsigned long long)S.nlist;
+          if (B.h == 2) tc += tn;
+        }
         if (lane == 0) {
           its[0] = v;
           its[1] = vs;
@@ -2590,13 +2696,12 @@ template <int NINT, typename NT>
 __device__ __forceinline__ void flush_totals(const SweepParams& p, BatchShared<NINT, NT>& S, int dscale) {
   const int tid = threadIdx.x, lane = tid & 31;
   const unsigned long long d0 = warp_sum_u(S.td0[tid]), d1 = warp_xor_u(S.td1[tid]), mn = warp_min_u(S.tmin[tid]);
-  const unsigned int tiny = __reduce_add_sync(kFull, S.ttiny[tid]);
   if (lane == 0 && mn != ~0ull) {
     atomicAdd(&p.digest[0], d0);
     atomicXor(&p.digest[1], d1);
     atomicMin(p.min_den_bits, (unsigned long long)__double_as_longlong(den_double(mn, dscale)));
-    if (tiny) atomicAdd(p.n_tiny, (unsigned long long)tiny);
   }
+  if (tid == 0 && S.tiny) atomicAdd(p.n_tiny, (unsigned long long)S.tiny);
 }
 
 // The shared state of a CTA for the sweep of p.
@@ -2605,8 +2710,8 @@ __device__ __forceinline__ void begin_sweep(const SweepParams& p, BatchShared<NI
   const int tid = threadIdx.x;
   S.td0[tid] = S.td1[tid] = 0ull;
   S.tmin[tid] = ~0ull;
-  S.ttiny[tid] = 0u;
   if (tid == 0) {
+    S.tiny = 0u;
     S.tkcnt = p.tk_cnt[blockIdx.x];
     S.tau = p.tk_tau[blockIdx.x];
     S.arrive = 0;
