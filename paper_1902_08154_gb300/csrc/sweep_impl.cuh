@@ -256,29 +256,22 @@ __device__ __forceinline__ int fix_scale(const SweepParams& p) {
 }
 
 // m * 2^sh as a 96-bit integer (lo, hi), negated when neg; m < 2^53 and
-// m * 2^sh < 2^94; for sh < 0 the bits below 2^0 are rounded (half up).
+// m * 2^sh < 2^94, so sh < 64; for sh < 0 the bits below 2^0 are rounded (half
+// up).
 __device__ __forceinline__ void fix_of_mant(unsigned long long m, int sh, bool neg, unsigned long long& lo,
                                             int& hi) {
   unsigned long long l;
-  unsigned int h;
-  if (sh >= 64) {
-    l = 0ull;
-    h = (unsigned int)(m << (sh - 64));
-  } else if (sh > 0) {
-    l = m << sh;
-    h = (unsigned int)(m >> (64 - sh));
-  } else if (sh == 0) {
-    l = m;
-    h = 0u;
+  unsigned int h = 0u;
+  if (sh <= 0) {
+    const int r = -sh < 63 ? -sh : 63;
+    l = (m + ((1ull << r) >> 1)) >> r;
   } else {
-    const int r = -sh;
-    l = (r < 64) ? (m >> r) + ((m >> (r - 1)) & 1ull) : 0ull;
-    h = 0u;
+    l = m << sh;
+    h = (unsigned int)((m >> 1) >> (63 - sh));
   }
-  if (neg) {
-    l = ~l + 1ull;
-    h = ~h + (l == 0ull ? 1u : 0u);
-  }
+  const unsigned int s = neg ? ~0u : 0u;
+  l = (l ^ (((unsigned long long)s << 32) | s)) + (neg ? 1ull : 0ull);
+  h = (h ^ s) + (neg && l == 0ull ? 1u : 0u);
   lo = l;
   hi = (int)h;
 }
@@ -286,23 +279,16 @@ __device__ __forceinline__ void fix_of_mant(unsigned long long m, int sh, bool n
 __device__ __forceinline__ void fix_of(double x, int F, unsigned long long& lo, int& hi) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7FF);
-  if (e == 0) {  // zero, or below 2^-1022: nothing at 2^-F (F <= 126)
-    lo = 0ull;
-    hi = 0;
-    return;
-  }
-  fix_of_mant((b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull, e - 1075 + F, (b >> 63) != 0ull, lo, hi);
+  // zero, or below 2^-1022: nothing at 2^-F (F <= 126)
+  fix_of_mant(e == 0 ? 0ull : (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull, e - 1075 + F, (b >> 63) != 0ull, lo,
+              hi);
 }
 
 __device__ __forceinline__ void fix_of(float x, int F, unsigned long long& lo, int& hi) {
   const unsigned int b = (unsigned int)__float_as_int(x);
   const int e = (int)((b >> 23) & 0xFF);
-  if (e == 0) {
-    lo = 0ull;
-    hi = 0;
-    return;
-  }
-  fix_of_mant((unsigned long long)((b & 0x7FFFFFu) | 0x800000u), e - 150 + F, (b >> 31) != 0u, lo, hi);
+  fix_of_mant(e == 0 ? 0ull : (unsigned long long)((b & 0x7FFFFFu) | 0x800000u) << 29, e - 179 + F, (b >> 31) != 0u, lo,
+              hi);
 }
 
 __device__ __forceinline__ void fix_add(unsigned long long& lo, int& hi, unsigned long long l2, int h2) {
@@ -960,9 +946,10 @@ __device__ __forceinline__ void cell_orbitals(const Batch& B, const BatchShared<
     *r = S.vir[0][xx];
     *s = S.vir[1][*y];
   } else {
+    // c < 2^13: the square root is exact up to one step
     int yy = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)c)) * 0.5f);
-    while (yy * (yy - 1) / 2 > c) yy--;
-    while ((yy + 1) * yy / 2 <= c) yy++;
+    if (yy * (yy - 1) / 2 > c) yy--;
+    if ((yy + 1) * yy / 2 <= c) yy++;
     *x = c - yy * (yy - 1) / 2;
     *y = yy;
     *r = S.vir[B.sa][*x];
@@ -1464,7 +1451,7 @@ struct ItemEnv {
   double* A;
   uint32_t *A0, *A1, *A2;
   uint32_t* ban;
-  unsigned short* lst;  // one-state form: the cells left, x << 8 | y
+  unsigned short* lst;  // one-state form: the cells left
   double *ms_gc, *ms_cI, *ms_w;
   long long* ms_de;  // E0_s - E0_0, fixed point
   int mc, nst, norb, nel, nbat, nper;
@@ -1848,6 +1835,33 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     __syncthreads();
     const int n0 = S.n0;
     B = S.bt;
+    if (!MS && c0 == 0) {
+      // the list of the cells left, in cell order: every warp scans the ban
+      // words, 32 at a time, and writes the cells of every eighth of them
+      int base = 0;
+#pragma unroll 1
+      for (int w0 = 0; 32 * w0 < B.nct; w0 += 32) {
+        const int n = B.nct - 32 * (w0 + lane);
+        const unsigned left = n <= 0 ? 0u : ~ban[w0 + lane] & (n >= 32 ? ~0u : (1u << n) - 1u);
+        int at = __popc(left);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(kFull, at, o);
+          if (lane >= o) at += t;
+        }
+        const int sum = __shfl_sync(kFull, at, 31);
+        at += base - __popc(left);
+        base += sum;
+#pragma unroll
+        for (int k = 0; k < 32; k += kWarps) {
+          const unsigned bits = __shfl_sync(kFull, left, warp + k);
+          const int b0 = __shfl_sync(kFull, at, warp + k);
+          if ((bits >> lane) & 1u)
+            E.lst[b0 + __popc(bits & ((1u << lane) - 1u))] = (unsigned short)(32 * (w0 + warp + k) + lane);
+        }
+      }
+      if (tid == 0) S.nlist = base;
+    }
     // The rest of the J, drawn by the warps as they free up: the rows of J
     // reaching every cell (a two-hole batch: the cells touching their
     // particles; a one-hole batch: all cells), J reaching rows, and J reaching
@@ -1869,10 +1883,9 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       const int nrow = S.n1, n2 = S.n2;
       const int ntab = B.h == 2 ? (n0 < kGroup ? n0 : kGroup) : 0;
       const int nvm = S.nv[0] > S.nv[1] ? S.nv[0] : S.nv[1], nch = (nvm + 31) / 32;
-      // units: the list of the cells left (256 cells each), pair tables, rows of
-      // the J reaching every cell (J, particle slot, 32 cells), row J, the rest
-      const int ncmp = !MS && c0 == 0 ? (B.nct + 255) / 256 : 0;
-      const int nall = ncmp + ntab + n0 * B.h * nch;
+      // units: pair tables, rows of the J reaching every cell (J, particle slot,
+      // 32 cells), row J, the rest
+      const int nall = ntab + n0 * B.h * nch;
       int per = (nrow + kWarps - 1) / kWarps;
       per = per > 8 ? 8 : per;
       const int ndraw = nall + (per ? (nrow + per - 1) / per : 0);
@@ -1895,52 +1908,10 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         int jd = 0;
         if (lane == 0) jd = atomicAdd(&S.cnext, 1);
         jd = __shfl_sync(kFull, jd, 0);
-        if (jd < ncmp) {
-          // cells not banned, in cell order: a byte of the ban bits per lane
-          auto left = [&](int w) {
-            const int n = B.nct - 32 * w;
-            return n <= 0 ? 0u : ~ban[w] & (n >= 32 ? ~0u : (1u << n) - 1u);
-          };
-          const int nw = (B.nct + 31) / 32;
-          unsigned before = 0, all = 0;
-#pragma unroll 1
-          for (int w = lane; w < (jd == 0 ? nw : 8 * jd); w += 32) {
-            const unsigned c = __popc(left(w));
-            all += c;
-            if (w < 8 * jd) before += c;
-          }
-          before = __reduce_add_sync(kFull, before);
-          all = __reduce_add_sync(kFull, all);
-          if (jd == 0 && lane == 0) S.nlist = (int)all;
-          const int hb = 32 * jd + lane;
-          const unsigned bits = (left(hb >> 2) >> (8 * (hb & 3))) & 0xFFu;
-          int at = __popc(bits);
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, at, o);
-            if (lane >= o) at += t;
-          }
-          at += (int)before - __popc(bits);
-          if (bits) {
-            int ro, so, x, y;
-            cell_orbitals<NINT, NT>(B, S, B.clo + 8 * hb, &ro, &so, &x, &y);
-            const int nv1 = S.nv[1];
-            if (B.kind == 0) y = 0;
-#pragma unroll 1
-            for (int k = 0; k < 8; k++) {
-              if ((bits >> k) & 1u) E.lst[at++] = (unsigned short)(x << 8 | y);
-              if (B.kind == 2) {
-                if (++y == nv1) y = 0, x++;
-              } else if (++x == y && B.kind == 1) {
-                x = 0;
-                y++;
-              }
-            }
-          }
-        } else if (jd < ncmp + ntab) {
-          build_table(jd - ncmp, S.u.l.L0[jd - ncmp]);
+        if (jd < ntab) {
+          build_table(jd, S.u.l.L0[jd]);
         } else if (jd < nall) {
-          const int ju = jd - ncmp - ntab, j = ju / (B.h * nch), rem = ju - j * (B.h * nch), ip = rem / nch, y = (rem - ip * nch) * 32 + lane;
+          const int ju = jd - ntab, j = ju / (B.h * nch), rem = ju - j * (B.h * nch), ip = rem / nch, y = (rem - ip * nch) * 32 + lane;
           const int r = S.u.l.L0[j];
           const uint64_t hm = S.rhm[r], part = S.rpt[r];
           uint32_t X, T;
@@ -2110,41 +2081,40 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             const bool same = (iwr >> 24) & 1u;
             const int nz = S.nv[sz], nv1 = S.nv[1];
             // the integrals at b1 + z and (same spin) b2 + z
-            const int b1 = ((uo * norb + uz) * norb + q) * norb, b2 = ((uz * norb + uo) * norb + q) * norb;
+            const NT* e1 = eri_n + ((uo * norb + uz) * norb + q) * norb;
+            const NT* e2 = eri_n + ((uz * norb + uo) * norb + q) * norb;
+            // cell of z's index y: cb + y cs, or (same spin) a pair
+            const int cs = B.kind == 2 && s ? nv1 : 1;
+            const int cb = (B.kind == 2 ? (s ? x : x * nv1) : 0) - B.clo, xx = x * (x - 1) / 2;
             // two rounds of 32 cells at a time, their loads in flight together
 #pragma unroll 1
             for (int y0 = lane; y0 < nz; y0 += 64) {
-              int cc[2], zz[2];
-              NT v[2], w2[2];
-#pragma unroll
+              int ca = -1, cn = -1;
+              NT va = NT(0), vn = NT(0);
+              auto fetch = [&](int y, int& c, NT& v) {
+                if (y >= nz) return;
+                const int z = S.vir[sz][y];
+                int cc = cb + y * cs;
+                if (B.kind == 1) cc = cb + (y > x ? y * (y - 1) / 2 + x : xx + y);
+                if (mask_bit<NINT>(Er, z) || !live(cc)) return;
+                c = cc;
+                if constexpr (E4) {
+                  v = e1[z];
+                  if (same) v -= e2[z];
+                } else {
+                  v = eri_n[eri_index(uo, q, uz, z)];
+                  if (same) v -= eri_n[eri_index(uz, q, uo, z)];
+                }
+                v = flip_sign(v, mask_bit<NINT>(Mr, z));
+              };
+              fetch(y0, ca, va);
+              fetch(y0 + 32, cn, vn);
+#pragma unroll 1
               for (int i = 0; i < 2; i++) {
-                const int y = y0 + 32 * i;
-                cc[i] = -1;
-                v[i] = w2[i] = NT(0);
-                zz[i] = 0;
-                if (y < nz) {
-                  const int z = S.vir[sz][y];
-                  const int c = (B.kind == 0 ? y : B.kind == 1 ? pair_cell(x, y) : (s ? y * nv1 + x : x * nv1 + y)) - B.clo;
-                  zz[i] = z;
-                  if (!mask_bit<NINT>(Er, z) && live(c)) {
-                    cc[i] = c;
-                    if constexpr (E4) {
-                      v[i] = eri_n[b1 + z];
-                      if (same) w2[i] = eri_n[b2 + z];
-                    } else {
-                      v[i] = eri_n[eri_index(uo, q, uz, z)];
-                      if (same) w2[i] = eri_n[eri_index(uz, q, uo, z)];
-                    }
-                  }
-                }
+                if (ca >= 0) add(ca, va, rj, cjr);
+                ca = cn;
+                va = vn;
               }
-#pragma unroll
-              for (int i = 0; i < 2; i++)
-                if (cc[i] >= 0) {
-                  NT t = v[i];
-                  if (same) t -= w2[i];
-                  add(cc[i], flip_sign(t, mask_bit<NINT>(Mr, zz[i])), rj, cjr);
-                }
             }
           }
 #pragma unroll 1
@@ -2280,22 +2250,17 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       double acc_es[kMaxStates], acc_s2s[kMaxStates];  // multi-state form: sums per state
 #pragma unroll
       for (int st = 0; st < kMaxStates; st++) acc_es[st] = acc_s2s[st] = 0.0;
-      const int nv1 = S.nv[1], nleft = MS ? B.nct : S.nlist;
+      const int nleft = MS ? B.nct : S.nlist;
 #pragma unroll 1
       for (int i = tid; i < nleft; i += kThreads) {
-        int x, y, cc;
+        int cc = i, x, y, ro_, so_;
         if constexpr (MS) {
-          cc = i;
           if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
-          int ro, so;
-          cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
-          y = y < 0 ? 0 : y;
         } else {
-          const int xy = E.lst[i];
-          x = xy >> 8;
-          y = xy & 0xFF;
-          cc = (B.kind == 2 ? x * nv1 + y : B.kind == 1 ? y * (y - 1) / 2 + x : x) - B.clo;
+          cc = E.lst[i];
         }
+        cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro_, &so_, &x, &y);
+        y = y < 0 ? 0 : y;
         const typename BatchShared<NINT, NT>::Side R = S.row[x], C = S.col[y];
         const int ro = R.orb, so = C.orb;
         unsigned long long lo = 0ull;  // exact sum
