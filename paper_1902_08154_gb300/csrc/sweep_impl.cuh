@@ -2263,6 +2263,20 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         y = y < 0 ? 0 : y;
         const typename BatchShared<NINT, NT>::Side R = S.row[x], C = S.col[y];
         const int ro = R.orb, so = C.orb;
+        // the generator's own integrals and the pair's term of D, loaded ahead
+        // of the terms of the J reaching every cell
+        NT own = NT(0), own2 = NT(0);
+        long long dpair = 0;
+        if (fin && B.h == 2) {
+          if constexpr (E4) {
+            own = eri_n[(R.idx & 0x7fffffff) + (C.idx & 0x7fffffff)];
+            if (B.kind == 1) own2 = eri_n[ibase + so * norb + ro];
+          } else {
+            own = eri_n[tri(R.idx & 0x7fffffff, C.idx & 0x7fffffff)];
+            if (B.kind == 1) own2 = eri_n[tri(S.row[y].idx & 0x7fffffff, S.col[x].idx & 0x7fffffff)];
+          }
+          dpair = (B.kind == 2 ? p.Ji : p.Wi)[ro * norb + so];
+        }
         unsigned long long lo = 0ull;  // exact sum
         int hi = 0;
         double accs[kMaxStates];  // multi-state form: one sum per state
@@ -2317,22 +2331,16 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         if constexpr (MS) {
           double vI = 0.0;  // <I|H|alpha> for the generator's own term
           if (B.h == 2) {
-            NT t;
+            NT t = own;
             bool neg = (R.idx ^ C.idx) < 0;
-            if constexpr (E4) {
-              t = eri_n[(R.idx & 0x7fffffff) + (C.idx & 0x7fffffff)];
-              if (B.kind == 1) t -= eri_n[ibase + so * norb + ro];
-            } else {
-              t = eri_n[tri(R.idx & 0x7fffffff, C.idx & 0x7fffffff)];
-              if (B.kind == 1) t -= eri_n[tri(S.row[y].idx & 0x7fffffff, S.col[x].idx & 0x7fffffff)];
-            }
+            if (B.kind == 1) t -= own2;
             if (B.kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
             t = flip_sign(t, neg);
             vI = (double)t;
             con++;
           }
           long long D0 = R.d;  // E0_0 - H_aa
-          if (B.h == 2) D0 -= C.d + (B.kind == 2 ? p.Ji : p.Wi)[ro * norb + so];
+          if (B.h == 2) D0 -= C.d + dpair;
           double crit = 0.0, a0 = 0.0;
 #pragma unroll
           for (int st = 0; st < kMaxStates; st++) {
@@ -2375,22 +2383,16 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           double a = fix_to_double(lo, hi, F);
           // the generator's own term c_I <I|H|alpha>
           if (B.h == 2) {
-            NT t;
+            NT t = own;
             bool neg = (R.idx ^ C.idx) < 0;
-            if constexpr (E4) {
-              t = eri_n[(R.idx & 0x7fffffff) + (C.idx & 0x7fffffff)];
-              if (B.kind == 1) t -= eri_n[ibase + so * norb + ro];
-            } else {
-              t = eri_n[tri(R.idx & 0x7fffffff, C.idx & 0x7fffffff)];
-              if (B.kind == 1) t -= eri_n[tri(S.row[y].idx & 0x7fffffff, S.col[x].idx & 0x7fffffff)];
-            }
+            if (B.kind == 1) t -= own2;
             if (B.kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
             t = flip_sign(t, neg);
             a += (double)(S.cI * t);
           }
           // D = E0 - H_aa from the row and column sums
           long long D = R.d;
-          if (B.h == 2) D -= C.d + (B.kind == 2 ? p.Ji : p.Wi)[ro * norb + so];
+          if (B.h == 2) D -= C.d + dpair;
           const double q = div_fix(a, D, E.dscale);
           acc_e = fma(a, q, acc_e);  // e = A q
           acc_s2 += q * q;
