@@ -56,6 +56,13 @@ cudaError_t launch_prep(int nint, const SweepParams& p, int slots, cudaStream_t 
 cudaError_t launch_batch_packed(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_reduce_items(const SweepParams& p, cudaStream_t st);
 int batch_blocks_per_sm_packed(int nint, size_t smem);
+int64_t count_rank_max();
+int count_select_max();
+cudaError_t launch_count_rank(int nint, int64_t n, int norb, int na, int nb, const uint64_t* dets, const double* coefs,
+                              int32_t* order, int32_t* rank_of, int* err, unsigned long long* cmax,
+                              unsigned long long* min_den, cudaStream_t st);
+cudaError_t launch_count_select(int nint, size_t maxn, const int* ncand, int64_t k, const double* ce, const double* ca,
+                                const uint64_t* ck, uint64_t* sel, double* se, double* sn, cudaStream_t st);
 int report(int code, const char* msg);
 }  // namespace qp
 
@@ -196,7 +203,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   const int64_t cap = k > 0 ? k + max_cells : 1, ngen = ndet;
   const int64_t ent_cap = (int64_t)nd * bucket_entries_per_record(nel);
   const int nper = nbat;
-  size_t maxc = 0, tmp1 = 0, tmp2 = 0;
+  size_t maxc = 0, tmp1 = 0, tmp2 = 0, zeroed = 0;
   int64_t W = 0, nwaves = 0;
   double *d_J = nullptr, *d_K = nullptr, *eps = nullptr, *s2 = nullptr, *tk_e = nullptr;
   double *tk_a = nullptr, *cand_e = nullptr, *cand_a = nullptr, *r_coef = nullptr;
@@ -230,20 +237,22 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     den_tab = cv.take<long long>(2 * (size_t)norb * norb);
     order = cv.take<int32_t>(nd);
     rank_of = cv.take<int32_t>(nd);
-    eps = cv.take<double>(nd);
-    s2 = cv.take<double>(nd);
-    na = cv.take<unsigned long long>(nd);
-    ncon = cv.take<unsigned long long>(nd);
+    // what starts at zero, cleared in one piece
+    zeroed = 32 * nd + 8 * (size_t)grid + 4 * kSelBins + 4 * (size_t)grid;
+    eps = cv.take<double>((zeroed + 7) / 8);
+    s2 = eps + nd;
+    na = reinterpret_cast<unsigned long long*>(s2 + nd);
+    ncon = na + nd;
+    tk_tau = ncon + nd;
+    sel_hist = reinterpret_cast<unsigned int*>(tk_tau + grid);
+    tk_cnt = reinterpret_cast<int*>(sel_hist + kSelBins);
     acc = cv.take<unsigned long long>(9);
     dres = cv.take<DevResult>(1);
     queues = cv.take<int>(2);  // the wave's item counter and live count
     tk_e = cv.take<double>((size_t)cap * grid);
     tk_a = cv.take<double>((size_t)cap * grid);
     tk_key = cv.take<uint64_t>((size_t)cap * grid * nw);
-    tk_cnt = cv.take<int>(grid);
-    tk_tau = cv.take<unsigned long long>(grid);
     d_hmax = cv.take<unsigned long long>(2);
-    sel_hist = cv.take<unsigned int>(kSelBins);
     // the validation's arrays, the waves' and the selection's share the rest,
     // one phase after another on the stream
     Carve c1 = cv, c3 = cv;
@@ -310,13 +319,17 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   absmax_kernel<<<(unsigned)((P + 255) / 256 < 4096 ? (P + 255) / 256 : 4096), 256, 0, st>>>(P, eri, d_hmax + 1);
   jk_kernel<<<(norb * norb + 255) / 256, 256, 0, st>>>(norb, eri, d_J, d_K);
   const int nb = (int)((ndet + 255) / 256);
-  validate_kernel<<<nb, 256, 0, st>>>(ndet, nint, norb, n_alpha, n_beta, dets, coefs, hkey, hidx, rkey, rank_of, d_err,
-                                      acc + 8);
-  NTRY_Q(cudaGetLastError());
-  NTRY_Q(cub::DeviceRadixSort::SortPairs(cub_tmp, tmp1, hkey, hkey2, hidx, hidx2, (int)ndet, 0, 64, st));
-  dup_kernel<<<nb, 256, 0, st>>>(ndet, nint, dets, hkey2, hidx2, d_err);
-  NTRY_Q(cub::DeviceRadixSort::SortPairs(cub_tmp, tmp1, rkey, rkey2, rank_of, order, (int)ndet, 0, 64, st));
-  rank_kernel<<<nb, 256, 0, st>>>(ndet, order, rank_of);
+  if (ndet <= count_rank_max()) {
+    NTRY_Q(launch_count_rank(nint, ndet, norb, n_alpha, n_beta, dets, coefs, order, rank_of, d_err, acc + 8, acc + 2, st));
+  } else {
+    validate_kernel<<<nb, 256, 0, st>>>(ndet, nint, norb, n_alpha, n_beta, dets, coefs, hkey, hidx, rkey, rank_of, d_err,
+                                        acc + 8);
+    NTRY_Q(cudaGetLastError());
+    NTRY_Q(cub::DeviceRadixSort::SortPairs(cub_tmp, tmp1, hkey, hkey2, hidx, hidx2, (int)ndet, 0, 64, st));
+    dup_kernel<<<nb, 256, 0, st>>>(ndet, nint, dets, hkey2, hidx2, d_err);
+    NTRY_Q(cub::DeviceRadixSort::SortPairs(cub_tmp, tmp1, rkey, rkey2, rank_of, order, (int)ndet, 0, 64, st));
+    rank_kernel<<<nb, 256, 0, st>>>(ndet, order, rank_of);
+  }
   int herr = 0;
   NTRY_Q(cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   NTRY_Q(cudaStreamSynchronize(st));
@@ -326,13 +339,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   if (herr & 2) return nfail(QP_EDUP, "duplicate determinant in Psi0");
 
   // ---- the sweep, in waves ----
-  NTRY(cudaMemsetAsync(eps, 0, 8 * nd, st));
-  NTRY(cudaMemsetAsync(s2, 0, 8 * nd, st));
-  NTRY(cudaMemsetAsync(na, 0, 8 * nd, st));
-  NTRY(cudaMemsetAsync(ncon, 0, 8 * nd, st));
-  NTRY(cudaMemsetAsync(tk_cnt, 0, 4 * (size_t)grid, st));
-  NTRY(cudaMemsetAsync(tk_tau, 0, 8 * (size_t)grid, st));
-  NTRY(cudaMemsetAsync(sel_hist, 0, 4 * (size_t)kSelBins, st));
+  NTRY_Q(cudaMemsetAsync(eps, 0, zeroed, st));
   SweepParams p{};
   p.norb = norb;
   p.nalpha = n_alpha;
@@ -414,10 +421,12 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   if (k > 0) {
     gather_kernel<<<grid, 256, 0, st>>>(grid, nint, cap, tk_cnt, tk_e, tk_a, tk_key, p.tau_bits, cand_e, cand_a,
                                         cand_key, d_ncand, (int64_t)maxc, d_err);
+    NTRY_Q(launch_count_select(nint, maxc, d_ncand, k, cand_e, cand_a, cand_key, sel_dets, sel_e, nullptr, st));
     int ncand = 0;
     NTRY_Q(cudaMemcpyAsync(&ncand, d_ncand, sizeof(int), cudaMemcpyDeviceToHost, st));
     NTRY_Q(cudaStreamSynchronize(st));
-    if (ncand > 0) {
+    nsel = ncand < k ? ncand : k;
+    if (ncand > count_select_max()) {
       const int sb = (ncand + 255) / 256;
       iota_kernel<<<sb, 256, 0, st>>>(ncand, perm);
       int32_t *pa = perm, *pb = perm2;
@@ -429,7 +438,6 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
         pa = pb;
         pb = t;
       }
-      nsel = ncand < k ? ncand : k;
       select_out_kernel<<<(int)((nsel + 255) / 256), 256, 0, st>>>((int)nsel, nint, pa, cand_e, cand_a, cand_key,
                                                                  sel_dets, sel_e, nullptr);
       NTRY_Q(cudaGetLastError());

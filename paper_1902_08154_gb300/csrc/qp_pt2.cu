@@ -34,6 +34,13 @@ cudaError_t launch_wave_multi(int nint, int mixed, const MultiWave& m, const Mul
                               int grid, size_t smem, cudaStream_t st);
 cudaError_t launch_compact_multi(int nint, int mixed, const SweepParams* ps, int n, int grid, cudaStream_t st);
 int batch_multi_blocks_per_sm(int nint, int mixed, size_t smem);
+int64_t count_rank_max();
+int count_select_max();
+cudaError_t launch_count_rank(int nint, int64_t n, int norb, int na, int nb, const uint64_t* dets, const double* coefs,
+                              int32_t* order, int32_t* rank_of, int* err, unsigned long long* cmax,
+                              unsigned long long* min_den, cudaStream_t st);
+cudaError_t launch_count_select(int nint, size_t maxn, const int* ncand, int64_t k, const double* ce, const double* ca,
+                                const uint64_t* ck, uint64_t* sel, double* se, double* sn, cudaStream_t st);
 }  // namespace qp
 
 using namespace qp;
@@ -326,7 +333,7 @@ struct qp_pt2_ctx {
   unsigned long long* d_hmax = nullptr;        // bits of max |h|, max |(pq|rs)|
   // workspace
   Buf in_dets, in_coefs, hkey, hkey2, hidx, hidx2, rkey, rkey2, order, rank_of, cub_tmp;
-  Buf eps, s2, na, ncon, acc, res;
+  Buf eps, s2, na, ncon, acc, res, zeroed;
   Buf den_tab, meta, r_words, r_coef, r_hmask, r_part, b_mask, o_mask, b_ofs, e_hp, e_rec, live, queues, it_sum;
   Buf tk_e, tk_a, tk_key, tk_cnt, tk_tau, sel_hist, gen_list, gen_out, st_cmax;
   Buf cand_e, cand_a, cand_key, skey, skey2, perm, perm2, cub_tmp2;
@@ -336,6 +343,7 @@ struct qp_pt2_ctx {
   int64_t launches = 0;
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};  // call start, sweep start, sweep end
   cudaEvent_t ev_end = nullptr;
+  unsigned char* h_pin = nullptr;  // pinned, for the totals read back by every call
   bool timed = false;
 };
 
@@ -379,6 +387,8 @@ static void set_rpt2(qp_pt2_result& r, double e0) {
 
 // accumulator block layout (unsigned long long words)
 enum { kAccDigest0 = 0, kAccDigest1, kAccMinDen, kAccTiny, kAccTau, kAccQueue, kAccErr, kAccNcand, kAccCmax, kAccT0, kAccWords };
+// the accumulators and the states' totals behind them, read back in one copy
+constexpr size_t kAccBytes = 8 * kAccWords + sizeof(DevResult) * kMaxStates;
 
 static bool is_device_ptr(const void* p) {
   if (!p) return false;
@@ -452,6 +462,7 @@ extern "C" int qp_pt2_create(qp_pt2_ctx** out, int norb, int n_alpha, int n_beta
   for (int i = 0; i < 3; i++)
     if (cudaEventCreate(&x->ev[i]) != cudaSuccess) return bail(QP_ECUDA, "cudaEventCreate failed");
   if (cudaEventCreate(&x->ev_end) != cudaSuccess) return bail(QP_ECUDA, "cudaEventCreate failed");
+  if (cudaMallocHost(&x->h_pin, kAccBytes) != cudaSuccess) return bail(QP_ENOMEM, "host allocation failed");
   cudaDeviceGetAttribute(&x->nsm, cudaDevAttrMultiProcessorCount, x->device);
   if (cudaMalloc(&x->d_h, sizeof(double) * norb * norb) != cudaSuccess ||
       cudaMalloc(&x->d_eri, sizeof(double) * P) != cudaSuccess ||
@@ -520,6 +531,7 @@ extern "C" void qp_pt2_destroy(qp_pt2_ctx* x) {
   for (int i = 0; i < 3; i++)
     if (x->ev[i]) cudaEventDestroy(x->ev[i]);
   if (x->ev_end) cudaEventDestroy(x->ev_end);
+  if (x->h_pin) cudaFreeHost(x->h_pin);
   cudaFree(x->d_h);
   cudaFree(x->d_eri);
   cudaFree(x->d_h32);
@@ -530,7 +542,7 @@ extern "C" void qp_pt2_destroy(qp_pt2_ctx* x) {
   cudaFree(x->d_K);
   cudaFree(x->d_hmax);
   Buf* all[] = {&x->in_dets, &x->in_coefs, &x->hkey, &x->hkey2, &x->hidx, &x->hidx2, &x->rkey, &x->rkey2,
-                &x->order, &x->rank_of, &x->cub_tmp, &x->eps, &x->s2, &x->na, &x->ncon, &x->acc,
+                &x->order, &x->rank_of, &x->cub_tmp, &x->eps, &x->s2, &x->na, &x->ncon, &x->acc, &x->zeroed,
                 &x->res, &x->meta, &x->r_words, &x->r_coef, &x->r_hmask, &x->den_tab, &x->r_part, &x->b_mask, &x->o_mask,
                 &x->b_ofs, &x->e_hp, &x->e_rec, &x->it_sum, &x->live, &x->queues, &x->tk_e, &x->tk_a, &x->tk_key, &x->tk_cnt, &x->tk_tau, &x->sel_hist, &x->gen_list, &x->gen_out, &x->cand_e, &x->cand_a, &x->cand_key, &x->skey,
                 &x->skey2, &x->perm, &x->perm2, &x->cub_tmp2, &x->out_sel, &x->out_e, &x->out_num,
@@ -654,6 +666,53 @@ __global__ void gather_gen_kernel(int64_t n, const int32_t* ranks, const double*
   out_ncon[i] = (int64_t)ncon[r];
 }
 
+// Validation of Psi0 and the generator order into x->order and x->rank_of:
+// by counting (order.cu) where that is faster, else by radix sorts.  acc (its
+// error flags, max |c| and min |D| words) is set up here.
+static int enqueue_rank(qp_pt2_ctx* x, int64_t ndet, const uint64_t* d_dets, const double* d_coefs) {
+  cudaStream_t st = x->st;
+  const size_t nd = (size_t)ndet;
+  int rc;
+  if ((rc = x->order.grow(4 * nd)) || (rc = x->rank_of.grow(4 * nd)) || (rc = x->acc.grow(kAccBytes))) return rc;
+  unsigned long long* acc = x->acc.as<unsigned long long>();
+  int* d_err = reinterpret_cast<int*>(acc + kAccErr);
+  CUDA_TRY(cudaMemsetAsync(acc, 0, kAccBytes, st));
+  if (ndet <= count_rank_max()) {
+    CUDA_TRY(launch_count_rank(x->nint, ndet, x->norb, x->nalpha, x->nbeta, d_dets, d_coefs, x->order.as<int32_t>(),
+                               x->rank_of.as<int32_t>(), d_err, acc + kAccCmax, acc + kAccMinDen, st));
+    x->launches++;
+    return QP_OK;
+  }
+  if ((rc = x->hkey.grow(8 * nd)) || (rc = x->hkey2.grow(8 * nd)) || (rc = x->hidx.grow(4 * nd)) ||
+      (rc = x->hidx2.grow(4 * nd)) || (rc = x->rkey.grow(8 * nd)) || (rc = x->rkey2.grow(8 * nd)))
+    return rc;
+  static const unsigned long long inf_bits = 0x7FF0000000000000ull;
+  CUDA_TRY(cudaMemcpyAsync(acc + kAccMinDen, &inf_bits, sizeof(inf_bits), cudaMemcpyHostToDevice, st));
+  const int nb = (int)((ndet + 255) / 256);
+  validate_kernel<<<nb, 256, 0, st>>>(ndet, x->nint, x->norb, x->nalpha, x->nbeta, d_dets, d_coefs,
+                                      x->hkey.as<unsigned long long>(), x->hidx.as<int32_t>(),
+                                      x->rkey.as<unsigned long long>(), x->rank_of.as<int32_t>(), d_err,
+                                      acc + kAccCmax);
+  CUDA_TRY(cudaGetLastError());
+  size_t tmp1 = 0;
+  cub::DeviceRadixSort::SortPairs(nullptr, tmp1, x->hkey.as<unsigned long long>(),
+                                  x->hkey2.as<unsigned long long>(), x->hidx.as<int32_t>(),
+                                  x->hidx2.as<int32_t>(), (int)ndet, 0, 64, st);
+  if ((rc = x->cub_tmp.grow(tmp1))) return rc;
+  CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, tmp1, x->hkey.as<unsigned long long>(),
+                                           x->hkey2.as<unsigned long long>(), x->hidx.as<int32_t>(),
+                                           x->hidx2.as<int32_t>(), (int)ndet, 0, 64, st));
+  dup_kernel<<<nb, 256, 0, st>>>(ndet, x->nint, d_dets, x->hkey2.as<unsigned long long>(), x->hidx2.as<int32_t>(),
+                                 d_err);
+  CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, tmp1, x->rkey.as<unsigned long long>(),
+                                           x->rkey2.as<unsigned long long>(), x->rank_of.as<int32_t>(),
+                                           x->order.as<int32_t>(), (int)ndet, 0, 64, st));
+  rank_kernel<<<nb, 256, 0, st>>>(ndet, x->order.as<int32_t>(), x->rank_of.as<int32_t>());
+  CUDA_TRY(cudaGetLastError());
+  x->launches += 3;
+  return QP_OK;
+}
+
 // The sweep; with gen_ranks (host array of ngen_list distinct ranks) only
 // those generators are swept and their eps, |A_I| and connections are
 // written to gen_eps / gen_na / gen_ncon in list order.  nst > 0 selects
@@ -701,41 +760,10 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   // ---- validation and generator order ----
   const size_t nd = (size_t)ndet;
   NvtxRange nvtx_phase("qp_pt2 validate and rank");
-  if ((rc = x->hkey.grow(8 * nd)) || (rc = x->hkey2.grow(8 * nd)) || (rc = x->hidx.grow(4 * nd)) ||
-      (rc = x->hidx2.grow(4 * nd)) || (rc = x->rkey.grow(8 * nd)) || (rc = x->rkey2.grow(8 * nd)) ||
-      (rc = x->order.grow(4 * nd)) || (rc = x->rank_of.grow(4 * nd)) || (rc = x->acc.grow(8 * kAccWords)))
-    return rc;
+  if ((rc = enqueue_rank(x, ndet, d_dets, d_coefs))) return rc;
   unsigned long long* acc = x->acc.as<unsigned long long>();
-  {
-    unsigned long long init[kAccWords] = {0};
-    init[kAccMinDen] = 0x7FF0000000000000ull;  // +inf
-    CUDA_TRY(cudaMemcpyAsync(acc, init, sizeof(init), cudaMemcpyHostToDevice, st));
-  }
   int* d_err = reinterpret_cast<int*>(acc + kAccErr);
   const int tb = 256;
-  const int nb = (int)((ndet + tb - 1) / tb);
-  validate_kernel<<<nb, tb, 0, st>>>(ndet, nint, x->norb, x->nalpha, x->nbeta, d_dets, d_coefs,
-                                 x->hkey.as<unsigned long long>(), x->hidx.as<int32_t>(),
-                                 x->rkey.as<unsigned long long>(), x->rank_of.as<int32_t>(), d_err,
-                                      acc + kAccCmax);
-  x->launches++;
-  CUDA_TRY(cudaGetLastError());
-  size_t tmp1 = 0;
-  cub::DeviceRadixSort::SortPairs(nullptr, tmp1, x->hkey.as<unsigned long long>(),
-                                  x->hkey2.as<unsigned long long>(), x->hidx.as<int32_t>(),
-                                  x->hidx2.as<int32_t>(), (int)ndet, 0, 64, st);
-  if ((rc = x->cub_tmp.grow(tmp1))) return rc;
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, tmp1, x->hkey.as<unsigned long long>(),
-                                           x->hkey2.as<unsigned long long>(), x->hidx.as<int32_t>(),
-                                           x->hidx2.as<int32_t>(), (int)ndet, 0, 64, st));
-  dup_kernel<<<nb, tb, 0, st>>>(ndet, nint, d_dets, x->hkey2.as<unsigned long long>(), x->hidx2.as<int32_t>(),
-                                d_err);
-  x->launches++;
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, tmp1, x->rkey.as<unsigned long long>(),
-                                           x->rkey2.as<unsigned long long>(), x->rank_of.as<int32_t>(),
-                                           x->order.as<int32_t>(), (int)ndet, 0, 64, st));
-  rank_kernel<<<nb, tb, 0, st>>>(ndet, x->order.as<int32_t>(), x->rank_of.as<int32_t>());
-  x->launches++;
   unsigned long long hcmax[kMaxStates] = {0};
   if (ms) {  // every state's coefficients: finite, and max_I |c_Is|
     if ((rc = x->st_cmax.grow(8 * (size_t)kMaxStates))) return rc;
@@ -746,9 +774,10 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaMemcpyAsync(hcmax, x->st_cmax.p, 8 * (size_t)nst, cudaMemcpyDeviceToHost, st));
   }
-  int herr = 0;
-  CUDA_TRY(cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(x->h_pin, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
+  int herr = 0;
+  memcpy(&herr, x->h_pin, sizeof(int));
   if (herr & kErrOcc) return fail(QP_EINVAL, "a determinant has the wrong occupation or bits beyond norb");
   if (herr & kErrCoef) return fail(QP_EINVAL, "a coefficient is not finite");
   if (herr & kErrDup) return fail(QP_EDUP, "duplicate determinant in Psi0");
@@ -787,29 +816,24 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   if (W > ngen) W = ngen > 0 ? ngen : 1;
   const int64_t nwaves = ngen > 0 ? (ngen + W - 1) / W : 0;
   const size_t ws = (size_t)W;
-  if ((rc = x->eps.grow(8 * nd * nsts)) || (rc = x->s2.grow(8 * nd * nsts)) || (rc = x->na.grow(8 * nd)) ||
-      (rc = x->ncon.grow(8 * nd)) || (rc = x->meta.grow(sizeof(GenMeta) * ws)) ||
+  // what starts at zero, cleared in one piece: per-generator sums and counts,
+  // the CTAs' thresholds and candidate counts, the histogram, the waves'
+  // queue and live counts
+  const size_t z_tau = 8 * nd * (2 * (size_t)nsts + 2), z_hist = z_tau + 8 * (size_t)grid, z_cnt = z_hist + 4 * kSelBins,
+               z_queue = z_cnt + 4 * (size_t)grid, z_end = z_queue + 8 * (size_t)(nwaves + 1);
+  if ((rc = x->zeroed.grow(z_end)) || (rc = x->meta.grow(sizeof(GenMeta) * ws)) ||
       (rc = x->r_words.grow(8 * nd * nw * ws)) || (rc = x->r_coef.grow(8 * nd * ws * nsts)) ||
       (rc = x->r_hmask.grow(8 * nd * ws)) || (rc = x->r_part.grow(8 * nd * ws)) ||
       (rc = x->b_mask.grow(4 * (size_t)mask_words(x->norb, x->nalpha, x->nbeta) * ws)) ||
       (rc = x->o_mask.grow(8 * (size_t)orb_mask_words(nint, x->nel) * ws)) || (rc = x->b_ofs.grow(4 * (size_t)(x->nbat + 2) * ws)) ||
       (rc = x->e_hp.grow(16 * (size_t)ent_cap * ws)) ||
       (rc = x->e_rec.grow(4 * (size_t)ent_cap * ws)) || (rc = x->it_sum.grow(16 * (size_t)nper * nsts * ws)) ||
-      (rc = x->live.grow(4 * (size_t)nper * ws)) || (rc = x->queues.grow(8 * (size_t)(nwaves + 1))) ||
+      (rc = x->live.grow(4 * (size_t)nper * ws)) ||
       (rc = x->tk_e.grow(8 * (size_t)cap * grid)) || (rc = x->tk_a.grow(8 * (size_t)cap * grid)) ||
-      (rc = x->tk_key.grow(8 * (size_t)cap * grid * nw)) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
-      (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
-      (rc = x->res.grow(sizeof(DevResult) * nsts)) ||
-      (rc = x->sel_hist.grow(4 * (size_t)kSelBins)))
+      (rc = x->tk_key.grow(8 * (size_t)cap * grid * nw)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)))
     return rc;
-  CUDA_TRY(cudaMemsetAsync(x->sel_hist.p, 0, 4 * (size_t)kSelBins, st));
-  CUDA_TRY(cudaMemsetAsync(x->eps.p, 0, 8 * nd * nsts, st));
-  CUDA_TRY(cudaMemsetAsync(x->s2.p, 0, 8 * nd * nsts, st));
-  CUDA_TRY(cudaMemsetAsync(x->na.p, 0, 8 * nd, st));
-  CUDA_TRY(cudaMemsetAsync(x->ncon.p, 0, 8 * nd, st));
-  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 8 * (size_t)(nwaves + 1), st));
-  CUDA_TRY(cudaMemsetAsync(x->tk_cnt.p, 0, 4 * (size_t)grid, st));
-  CUDA_TRY(cudaMemsetAsync(x->tk_tau.p, 0, 8 * (size_t)grid, st));
+  unsigned char* zb = x->zeroed.as<unsigned char>();
+  CUDA_TRY(cudaMemsetAsync(zb, 0, z_end, st));
   SweepParams p{};
   p.norb = x->norb;
   p.nalpha = x->nalpha;
@@ -866,10 +890,10 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   p.b_ofs = x->b_ofs.as<int>();
   p.live = x->live.as<uint32_t>();
   p.ent_cap = ent_cap;
-  p.eps = x->eps.as<double>();
-  p.s2 = x->s2.as<double>();
-  p.na = x->na.as<unsigned long long>();
-  p.ncon = x->ncon.as<unsigned long long>();
+  p.eps = reinterpret_cast<double*>(zb);
+  p.s2 = p.eps + nd * nsts;
+  p.na = reinterpret_cast<unsigned long long*>(p.s2 + nd * nsts);
+  p.ncon = p.na + nd;
   p.digest = acc + kAccDigest0;
   p.min_den_bits = acc + kAccMinDen;
   p.n_tiny = acc + kAccTiny;
@@ -878,10 +902,10 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   p.tk_e = x->tk_e.as<double>();
   p.tk_a = x->tk_a.as<double>();
   p.tk_key = x->tk_key.as<uint64_t>();
-  p.tk_cnt = x->tk_cnt.as<int>();
-  p.tk_tau = x->tk_tau.as<unsigned long long>();
+  p.tk_cnt = reinterpret_cast<int*>(zb + z_cnt);
+  p.tk_tau = reinterpret_cast<unsigned long long*>(zb + z_tau);
   p.tau_bits = acc + kAccTau;
-  p.sel_hist = x->sel_hist.as<unsigned int>();
+  p.sel_hist = reinterpret_cast<unsigned int*>(zb + z_hist);
   p.max_cells = x->max_cells;
   p.err = d_err;
   p.it_stride = 2 * nsts;
@@ -896,8 +920,8 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
     p.wave_start = (int)(w * W);
     p.wave_slots = (int)((ngen - w * W) < W ? (ngen - w * W) : W);
     p.last_wave = (w == nwaves - 1);
-    p.queue = x->queues.as<int>() + w;
-    p.live_cnt = x->queues.as<int>() + (nwaves + 1) + w;
+    p.queue = reinterpret_cast<int*>(zb + z_queue) + w;
+    p.live_cnt = p.queue + (nwaves + 1);
     CUDA_TRY(launch_prep(nint, p, p.wave_slots, st));
     if (ms) CUDA_TRY(launch_batch_states(nint, p, grid, smem, st));
     else CUDA_TRY(launch_batch(nint, p, grid, smem, st));
@@ -905,7 +929,7 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
     x->launches += 3;
   }
   CUDA_TRY(cudaEventRecord(x->ev[2], st));
-  DevResult* dres = x->res.as<DevResult>();
+  DevResult* dres = reinterpret_cast<DevResult*>(acc + kAccWords);
   for (int s = 0; s < nsts; s++) {
     finalize_kernel<<<1, 1024, 0, st>>>(ndet, p.eps + (size_t)s * nd, p.s2 + (size_t)s * nd,
                                         reinterpret_cast<const long long*>(p.na),
@@ -914,61 +938,27 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   }
   CUDA_TRY(cudaGetLastError());
 
-  // ---- selection merge ----
+  // ---- selection merge: the candidates gathered and, up to a size, ranked
+  // by counting without waiting for their number ----
   nvtx_phase.next("qp_pt2 selection merge");
-  int64_t nsel = 0;
+  uint64_t* d_sel = nullptr;
+  double *d_se = nullptr, *d_sn = nullptr;
+  bool cb1 = false, cb2 = false, cb3 = false;
   if (k > 0) {
     const size_t maxc = (size_t)grid * (size_t)k;
     if ((rc = x->cand_e.grow(8 * maxc)) || (rc = x->cand_a.grow(8 * maxc)) ||
-        (rc = x->cand_key.grow(8 * maxc * nw)) || (rc = x->skey.grow(8 * maxc)) ||
-        (rc = x->skey2.grow(8 * maxc)) || (rc = x->perm.grow(4 * maxc)) || (rc = x->perm2.grow(4 * maxc)))
+        (rc = x->cand_key.grow(8 * maxc * nw)) ||
+        (rc = out_target(x->out_sel, sel_dets, (size_t)k * nw, &d_sel, &cb1)) ||
+        (rc = out_target(x->out_e, sel_e, (size_t)k, &d_se, &cb2)) ||
+        (rc = out_target(x->out_num, sel_num, (size_t)k, &d_sn, &cb3)))
       return rc;
     int* d_ncand = reinterpret_cast<int*>(acc + kAccNcand);
     gather_kernel<<<grid, 256, 0, st>>>(grid, nint, cap, p.tk_cnt, p.tk_e, p.tk_a, p.tk_key, p.tau_bits,
                                         x->cand_e.as<double>(), x->cand_a.as<double>(),
                                         x->cand_key.as<uint64_t>(), d_ncand, (int64_t)maxc, d_err);
-    x->launches++;
-    int ncand = 0;
-    CUDA_TRY(cudaMemcpyAsync(&ncand, d_ncand, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    if (ncand > 0) {
-      size_t tmp2 = 0;
-      cub::DeviceRadixSort::SortPairs(nullptr, tmp2, x->skey.as<unsigned long long>(),
-                                      x->skey2.as<unsigned long long>(), x->perm.as<int32_t>(),
-                                      x->perm2.as<int32_t>(), ncand, 0, 64, st);
-      if ((rc = x->cub_tmp2.grow(tmp2))) return rc;
-      const int sb = (ncand + 255) / 256;
-      iota_kernel<<<sb, 256, 0, st>>>(ncand, x->perm.as<int32_t>());
-      x->launches++;
-      // least significant first: key words from last to first, then |e|
-      for (int pass = 0; pass <= nw; pass++) {
-        const int word = (pass < nw) ? (nw - 1 - pass) : nw;  // nw means |e|
-        sortkey_kernel<<<sb, 256, 0, st>>>(ncand, nint, word, x->cand_e.as<double>(),
-                                           x->cand_key.as<uint64_t>(), x->perm.as<int32_t>(),
-                                           x->skey.as<unsigned long long>());
-        x->launches++;
-        CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp2.p, tmp2, x->skey.as<unsigned long long>(),
-                                                 x->skey2.as<unsigned long long>(), x->perm.as<int32_t>(),
-                                                 x->perm2.as<int32_t>(), ncand, 0, 64, st));
-        std::swap(x->perm, x->perm2);
-      }
-      nsel = ncand < k ? ncand : k;
-      uint64_t* d_sel;
-      double *d_se, *d_sn;
-      bool cb1, cb2, cb3;
-      if ((rc = out_target(x->out_sel, sel_dets, (size_t)k * nw, &d_sel, &cb1)) ||
-          (rc = out_target(x->out_e, sel_e, (size_t)k, &d_se, &cb2)) ||
-          (rc = out_target(x->out_num, sel_num, (size_t)k, &d_sn, &cb3)))
-        return rc;
-      select_out_kernel<<<(int)((nsel + 255) / 256), 256, 0, st>>>((int)nsel, nint, x->perm.as<int32_t>(),
-                                                                 x->cand_e.as<double>(), x->cand_a.as<double>(),
-                                                                 x->cand_key.as<uint64_t>(), d_sel, d_se, d_sn);
-      x->launches++;
-      CUDA_TRY(cudaGetLastError());
-      if (cb1) CUDA_TRY(cudaMemcpyAsync(sel_dets, d_sel, 8 * nsel * nw, cudaMemcpyDeviceToHost, st));
-      if (cb2) CUDA_TRY(cudaMemcpyAsync(sel_e, d_se, 8 * nsel, cudaMemcpyDeviceToHost, st));
-      if (cb3) CUDA_TRY(cudaMemcpyAsync(sel_num, d_sn, 8 * nsel, cudaMemcpyDeviceToHost, st));
-    }
+    CUDA_TRY(launch_count_select(nint, maxc, d_ncand, k, x->cand_e.as<double>(), x->cand_a.as<double>(),
+                                 x->cand_key.as<uint64_t>(), d_sel, d_se, d_sn, st));
+    x->launches += 2;
   }
 
   // ---- per-generator outputs ----
@@ -994,13 +984,60 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
       return rc;
   }
 
-  DevResult hres[kMaxStates];
-  unsigned long long hacc[kAccWords];
-  CUDA_TRY(cudaMemcpyAsync(hres, dres, sizeof(DevResult) * nsts, cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(hacc, acc, sizeof(hacc), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CUDA_TRY(cudaMemcpyAsync(x->h_pin, acc, kAccBytes, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaEventRecord(x->ev_end, st));
   CUDA_TRY(cudaStreamSynchronize(st));
+  DevResult hres[kMaxStates];
+  unsigned long long hacc[kAccWords];
+  memcpy(hacc, x->h_pin, sizeof(hacc));
+  memcpy(hres, x->h_pin + sizeof(hacc), sizeof(hres));
+  memcpy(&herr, hacc + kAccErr, sizeof(int));
+  int64_t nsel = 0;
+  if (k > 0) {
+    int ncand = 0;
+    memcpy(&ncand, hacc + kAccNcand, sizeof(int));
+    nsel = ncand < k ? ncand : k;
+    if (ncand > count_select_max()) {
+      const size_t n = (size_t)ncand;
+      if ((rc = x->skey.grow(8 * n)) || (rc = x->skey2.grow(8 * n)) || (rc = x->perm.grow(4 * n)) ||
+          (rc = x->perm2.grow(4 * n)))
+        return rc;
+      size_t tmp2 = 0;
+      cub::DeviceRadixSort::SortPairs(nullptr, tmp2, x->skey.as<unsigned long long>(),
+                                      x->skey2.as<unsigned long long>(), x->perm.as<int32_t>(),
+                                      x->perm2.as<int32_t>(), ncand, 0, 64, st);
+      if ((rc = x->cub_tmp2.grow(tmp2))) return rc;
+      const int sb = (ncand + 255) / 256;
+      iota_kernel<<<sb, 256, 0, st>>>(ncand, x->perm.as<int32_t>());
+      x->launches++;
+      // least significant first: key words from last to first, then |e|
+      for (int pass = 0; pass <= nw; pass++) {
+        const int word = (pass < nw) ? (nw - 1 - pass) : nw;  // nw means |e|
+        sortkey_kernel<<<sb, 256, 0, st>>>(ncand, nint, word, x->cand_e.as<double>(),
+                                           x->cand_key.as<uint64_t>(), x->perm.as<int32_t>(),
+                                           x->skey.as<unsigned long long>());
+        x->launches++;
+        CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp2.p, tmp2, x->skey.as<unsigned long long>(),
+                                                 x->skey2.as<unsigned long long>(), x->perm.as<int32_t>(),
+                                                 x->perm2.as<int32_t>(), ncand, 0, 64, st));
+        std::swap(x->perm, x->perm2);
+      }
+      select_out_kernel<<<(int)((nsel + 255) / 256), 256, 0, st>>>((int)nsel, nint, x->perm.as<int32_t>(),
+                                                                 x->cand_e.as<double>(), x->cand_a.as<double>(),
+                                                                 x->cand_key.as<uint64_t>(), d_sel, d_se, d_sn);
+      x->launches++;
+      CUDA_TRY(cudaGetLastError());
+    }
+    if (nsel > 0) {
+      if (cb1) CUDA_TRY(cudaMemcpyAsync(sel_dets, d_sel, 8 * nsel * nw, cudaMemcpyDeviceToHost, st));
+      if (cb2) CUDA_TRY(cudaMemcpyAsync(sel_e, d_se, 8 * nsel, cudaMemcpyDeviceToHost, st));
+      if (cb3) CUDA_TRY(cudaMemcpyAsync(sel_num, d_sn, 8 * nsel, cudaMemcpyDeviceToHost, st));
+    }
+    if (ncand > count_select_max() || cb1 || cb2 || cb3) {
+      CUDA_TRY(cudaEventRecord(x->ev_end, st));
+      CUDA_TRY(cudaStreamSynchronize(st));
+    }
+  }
   x->timed = true;
   if (herr & kErrBucket) return fail(QP_ECUDA, "internal error: bucket capacity exceeded");
   if (herr & kErrRange)
@@ -1142,39 +1179,9 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   if ((rc = stage_in(x, x->in_dets, dets, (size_t)ndet * nw, &d_dets))) return rc;
   if ((rc = stage_in(x, x->in_coefs, coefs, (size_t)ndet, &d_coefs))) return rc;
   const size_t nd = (size_t)ndet;
-  if ((rc = x->hkey.grow(8 * nd)) || (rc = x->hkey2.grow(8 * nd)) || (rc = x->hidx.grow(4 * nd)) ||
-      (rc = x->hidx2.grow(4 * nd)) || (rc = x->rkey.grow(8 * nd)) || (rc = x->rkey2.grow(8 * nd)) ||
-      (rc = x->order.grow(4 * nd)) || (rc = x->rank_of.grow(4 * nd)) || (rc = x->acc.grow(8 * kAccWords)))
-    return rc;
+  if ((rc = enqueue_rank(x, ndet, d_dets, d_coefs))) return rc;
   unsigned long long* acc = x->acc.as<unsigned long long>();
-  {
-    unsigned long long init[kAccWords] = {0};
-    init[kAccMinDen] = 0x7FF0000000000000ull;
-    CUDA_TRY(cudaMemcpyAsync(acc, init, sizeof(init), cudaMemcpyHostToDevice, st));
-  }
   int* d_err = reinterpret_cast<int*>(acc + kAccErr);
-  const int nb = (int)((ndet + 255) / 256);
-  validate_kernel<<<nb, 256, 0, st>>>(ndet, nint, norb, x->nalpha, x->nbeta, d_dets, d_coefs,
-                                      x->hkey.as<unsigned long long>(), x->hidx.as<int32_t>(),
-                                      x->rkey.as<unsigned long long>(), x->rank_of.as<int32_t>(), d_err,
-                                      acc + kAccCmax);
-  x->launches++;
-  CUDA_TRY(cudaGetLastError());
-  size_t tmp1 = 0;
-  cub::DeviceRadixSort::SortPairs(nullptr, tmp1, x->hkey.as<unsigned long long>(),
-                                  x->hkey2.as<unsigned long long>(), x->hidx.as<int32_t>(),
-                                  x->hidx2.as<int32_t>(), (int)ndet, 0, 64, st);
-  if ((rc = x->cub_tmp.grow(tmp1))) return rc;
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, tmp1, x->hkey.as<unsigned long long>(),
-                                           x->hkey2.as<unsigned long long>(), x->hidx.as<int32_t>(),
-                                           x->hidx2.as<int32_t>(), (int)ndet, 0, 64, st));
-  dup_kernel<<<nb, 256, 0, st>>>(ndet, nint, d_dets, x->hkey2.as<unsigned long long>(), x->hidx2.as<int32_t>(), d_err);
-  x->launches++;
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, tmp1, x->rkey.as<unsigned long long>(),
-                                           x->rkey2.as<unsigned long long>(), x->rank_of.as<int32_t>(),
-                                           x->order.as<int32_t>(), (int)ndet, 0, 64, st));
-  rank_kernel<<<nb, 256, 0, st>>>(ndet, x->order.as<int32_t>(), x->rank_of.as<int32_t>());
-  x->launches++;
   int herr = 0;
   CUDA_TRY(cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
   CUDA_TRY(cudaStreamSynchronize(st));
@@ -1466,7 +1473,7 @@ static int plan_instance(BatchInst& b, size_t wave_budget, int64_t W_fixed, bool
                                            (int)b.maxc, 1, (int*)nullptr, (int*)nullptr, 0, 64, x->st);
   if ((rc = x->hkey.grow(8 * nd)) || (rc = x->hkey2.grow(8 * nd)) || (rc = x->hidx.grow(4 * nd)) ||
       (rc = x->hidx2.grow(4 * nd)) || (rc = x->rkey.grow(8 * nd)) || (rc = x->rkey2.grow(8 * nd)) ||
-      (rc = x->order.grow(4 * nd)) || (rc = x->rank_of.grow(4 * nd)) || (rc = x->acc.grow(8 * kAccWords)) ||
+      (rc = x->order.grow(4 * nd)) || (rc = x->rank_of.grow(4 * nd)) || (rc = x->acc.grow(kAccBytes)) ||
       (rc = x->cub_tmp.grow(b.tmp1)) || (rc = x->cub_tmp2.grow(b.tmp2 + 256)) || (rc = x->eps.grow(8 * nd)) ||
       (rc = x->s2.grow(8 * nd)) || (rc = x->na.grow(8 * nd)) || (rc = x->ncon.grow(8 * nd)))
     return rc;
@@ -1584,19 +1591,24 @@ static int enqueue_pre(BatchInst& b, cudaStream_t st) {
   int* d_err = reinterpret_cast<int*>(acc + kAccErr);
   init_acc_kernel<<<1, 32, 0, st>>>(acc);
   CUDA_TRY(cudaMemsetAsync(x->sel_hist.p, 0, 4 * (size_t)kSelBins, st));
-  const int nb = (int)((ndet + 255) / 256);
-  validate_kernel<<<nb, 256, 0, st>>>(ndet, nint, x->norb, x->nalpha, x->nbeta, b.dets, b.coefs,
-                                      x->hkey.as<unsigned long long>(), x->hidx.as<int32_t>(),
-                                      x->rkey.as<unsigned long long>(), x->rank_of.as<int32_t>(), d_err,
-                                      acc + kAccCmax);
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, b.tmp1, x->hkey.as<unsigned long long>(),
-                                           x->hkey2.as<unsigned long long>(), x->hidx.as<int32_t>(),
-                                           x->hidx2.as<int32_t>(), (int)ndet, 0, 64, st));
-  dup_kernel<<<nb, 256, 0, st>>>(ndet, nint, b.dets, x->hkey2.as<unsigned long long>(), x->hidx2.as<int32_t>(), d_err);
-  CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, b.tmp1, x->rkey.as<unsigned long long>(),
-                                           x->rkey2.as<unsigned long long>(), x->rank_of.as<int32_t>(),
-                                           x->order.as<int32_t>(), (int)ndet, 0, 64, st));
-  rank_kernel<<<nb, 256, 0, st>>>(ndet, x->order.as<int32_t>(), x->rank_of.as<int32_t>());
+  if (ndet <= count_rank_max()) {
+    CUDA_TRY(launch_count_rank(nint, ndet, x->norb, x->nalpha, x->nbeta, b.dets, b.coefs, x->order.as<int32_t>(),
+                               x->rank_of.as<int32_t>(), d_err, acc + kAccCmax, acc + kAccMinDen, st));
+  } else {
+    const int nb = (int)((ndet + 255) / 256);
+    validate_kernel<<<nb, 256, 0, st>>>(ndet, nint, x->norb, x->nalpha, x->nbeta, b.dets, b.coefs,
+                                        x->hkey.as<unsigned long long>(), x->hidx.as<int32_t>(),
+                                        x->rkey.as<unsigned long long>(), x->rank_of.as<int32_t>(), d_err,
+                                        acc + kAccCmax);
+    CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, b.tmp1, x->hkey.as<unsigned long long>(),
+                                             x->hkey2.as<unsigned long long>(), x->hidx.as<int32_t>(),
+                                             x->hidx2.as<int32_t>(), (int)ndet, 0, 64, st));
+    dup_kernel<<<nb, 256, 0, st>>>(ndet, nint, b.dets, x->hkey2.as<unsigned long long>(), x->hidx2.as<int32_t>(), d_err);
+    CUDA_TRY(cub::DeviceRadixSort::SortPairs(x->cub_tmp.p, b.tmp1, x->rkey.as<unsigned long long>(),
+                                             x->rkey2.as<unsigned long long>(), x->rank_of.as<int32_t>(),
+                                             x->order.as<int32_t>(), (int)ndet, 0, 64, st));
+    rank_kernel<<<nb, 256, 0, st>>>(ndet, x->order.as<int32_t>(), x->rank_of.as<int32_t>());
+  }
   CUDA_TRY(cudaMemsetAsync(x->eps.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->s2.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->na.p, 0, 8 * nd, st));
