@@ -250,7 +250,9 @@ int qp_pt2_eval_states(qp_pt2_ctx *ctx, int64_t ndet, const uint64_t *dets, int 
  *
  * qp_pt2_sigma: S[k] = H U[k] for nvec vectors (U, S: [nvec][ndet], host or
  * device), H the matrix of Psi0's determinants (Slater-Condon rules,
- * Eqs. Hij).  H is rebuilt on every call (device memory freed on return).
+ * Eqs. Hij).  H is rebuilt on every call; the device memory is the
+ * context's workspace (up to 256 MiB, kept until qp_pt2_destroy) or, beyond
+ * that, freed on return.
  *
  * qp_pt2_davidson: the lowest eigenvalue *e0 and its normalised eigenvector
  * coefs[ndet] (host or device; coefs[0] >= 0), by Davidson's method with the
@@ -260,8 +262,8 @@ int qp_pt2_eval_states(qp_pt2_ctx *ctx, int64_t ndet, const uint64_t *dets, int 
  * Rayleigh quotient of the returned vector.  info (may be NULL) receives the
  * iteration count, the final residual, the number of stored off-diagonal
  * elements and the build and solve times.  Psi0 is validated as for
- * qp_pt2_eval (QP_EINVAL, QP_EDUP).  Allocates device memory for H and the
- * basis (32 vectors). */
+ * qp_pt2_eval (QP_EINVAL, QP_EDUP).  Device memory for H and the
+ * basis (32 vectors) as for qp_pt2_sigma. */
 typedef struct {
   int iterations, converged;
   double residual;

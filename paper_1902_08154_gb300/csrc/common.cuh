@@ -69,8 +69,13 @@ struct CtxView {
   int norb, nalpha, nbeta, nint, nel, device;
   const double *h, *eri, *Jm, *Km;  // device copies, [norb*norb] and packed
   cudaStream_t st;
+  struct ::qp_pt2_ctx* ctx;
 };
-int ctx_view(const struct ::qp_pt2_ctx* x, CtxView* v);
+int ctx_view(struct ::qp_pt2_ctx* x, CtxView* v);
+// The context's workspace for the Hamiltonian and Davidson unit: taken by one
+// call at a time (false: another holds it), given back with the size wanted.
+bool ctx_ws_take(struct ::qp_pt2_ctx* x, void** p, size_t* bytes);
+void ctx_ws_give(struct ::qp_pt2_ctx* x, size_t bytes);
 int report(int code, const char* msg);
 
 // Bucket entries per coarse-filter record with holes Q of I (d = |Q|), at

@@ -6,17 +6,18 @@
 //   * H is built once per call as a CSR matrix of the pairs (I, J) at
 //     excitation degree 1 or 2 (Slater-Condon rules, Eqs. Hij), plus its
 //     diagonal.  Pairs are found through the spin-up and spin-down strings
-//     of the determinants (the paper's DISCIUS-like search, see below), or,
-//     as a cross-check, by a tiled all-pairs test (each CTA keeps a tile of
-//     rows in shared memory and streams every determinant once); they are
-//     written in any order and then sorted by column within each row, so that
-//     the products below add in a fixed order.
-//   * sigma = H u by one warp per row.
+//     of the determinants (the paper's DISCIUS-like search, see below) into
+//     a bit map per row, read off with ascending columns, or, as a
+//     cross-check, by a tiled all-pairs test (each CTA keeps a tile of rows in
+//     shared memory and streams every determinant once) whose pairs are then
+//     sorted by column within each row; the products below add in a fixed order.
+//   * sigma = H u by a warp per row, a block for the longest rows.
 //   * Davidson's method (E. R. Davidson, J. Comput. Phys. 17, 87 (1975)) with
 //     the diagonal preconditioner t = r / (theta - H_II): basis vectors,
 //     their products with H and every dot product stay on the device; only
-//     the small subspace matrix goes to the host, where a cyclic Jacobi
-//     eigensolver (Golub & Van Loan, Sec. 8.5) diagonalises it.
+//     the small subspace matrix goes to the host, where its lowest
+//     eigenpair is found through a tridiagonal matrix (Golub & Van Loan,
+//     Secs. 8.3 and 8.4).
 #include <cuda_runtime.h>
 
 #include <cub/device/device_radix_sort.cuh>
@@ -24,6 +25,7 @@
 #include <cub/device/device_segmented_radix_sort.cuh>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/qp_pt2.h"
@@ -140,7 +142,7 @@ __global__ void diag_kernel(int64_t n, const uint64_t* dets, int norb, const dou
 // otherwise (col, <I|H|J>) pairs go to each row's next free slots.
 template <int NINT, bool COUNT>
 __global__ void pairs_kernel(int64_t n, const uint64_t* dets, int norb, const double* h, const double* eri,
-                             int* rowcnt, const int64_t* rowptr, int* cursor, int* cols, double* vals, int* err) {
+                             int64_t* rowcnt, const int64_t* rowptr, int* cursor, int* cols, double* vals, int* err) {
   constexpr int NW = 2 * NINT;
   __shared__ uint64_t rows[kRows][NW];
   __shared__ int cnt[kRows];
@@ -238,25 +240,27 @@ __global__ void str_index_kernel(int64_t n, int spin, const uint64_t* dets, cons
   }
 }
 
-// Single-excitation neighbours among the distinct strings (count, then fill).
+// Single-excitation neighbours among the distinct strings (count, then fill),
+// a warp per string (a thread per string took 190 us for 3,000 of them).
 template <int NINT, bool COUNT>
 __global__ void str_nb_kernel(int nu, const uint64_t* ukey, int* cnt, const int* nb_ptr, int* nb) {
-  const int u = blockIdx.x * blockDim.x + threadIdx.x;
+  const int u = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (u >= nu) return;
   uint64_t a[NINT];
 #pragma unroll
   for (int w = 0; w < NINT; w++) a[w] = ukey[(size_t)u * NINT + w];
-  int c = 0;
-  for (int v = 0; v < nu; v++) {
+  int c = COUNT ? 0 : nb_ptr[u];
+  for (int v0 = 0; v0 < nu; v0 += 32) {
+    const int v = v0 + lane;
     int d = 0;
+    if (v < nu)
 #pragma unroll
-    for (int w = 0; w < NINT; w++) d += __popcll(a[w] ^ ukey[(size_t)v * NINT + w]);
-    if (d == 2) {
-      if (!COUNT) nb[nb_ptr[u] + c] = v;
-      c++;
-    }
+      for (int w = 0; w < NINT; w++) d += __popcll(a[w] ^ ukey[(size_t)v * NINT + w]);
+    const unsigned hit = __ballot_sync(0xffffffffu, d == 2);
+    if (!COUNT && d == 2) nb[c + __popc(hit & ((1u << lane) - 1u))] = v;
+    c += __popc(hit);
   }
-  if (COUNT) cnt[u] = c;
+  if (COUNT && lane == 0) cnt[u] = c;
 }
 
 template <int NINT>
@@ -267,173 +271,474 @@ __device__ __forceinline__ int spin_degree(const uint64_t* I, const uint64_t* J,
   return d >> 1;
 }
 
-// One warp per row I: COUNT writes the number of connected J, otherwise the
-// (column, <I|H|J>) pairs go to the row's next free slots.
+// One block per row I: the connected J marked in a bit map of the
+// determinants (shared memory; `win` of them at a time), COUNT: their number;
+// otherwise the columns read off the map in ascending order, so that nothing
+// is sorted.  Spin-up neighbour strings with few determinants take a thread
+// each, the others a warp.  (A warp per row that evaluated each element as it
+// found it and drew its slot from a global counter, and a segmented sort of
+// the pairs, took 2.9 ms for 10^4 determinants, 6.2e6 elements; the two passes
+// of this kernel and the values take 0.65.)
+constexpr int kMapThreads = 256;
+constexpr int kMapQueue = 512;
+constexpr int64_t kMapMax = 1 << 20;  // determinants per window: 128 KB of map
+
 template <int NINT, bool COUNT>
-__global__ void str_pairs_kernel(int64_t n, const uint64_t* dets, int norb, const double* h, const double* eri,
-                                 const int* aid, const int* aptr, const int* agrp, const int* anb_ptr,
-                                 const int* anb, const int* bid, const int* bptr, const int* bgrp, int* rowcnt,
-                                 const int64_t* rowptr, int* cursor, int* cols, double* vals, int* err) {
+__global__ void __launch_bounds__(kMapThreads) str_pairs_kernel(
+    int64_t n, int win, const uint64_t* __restrict__ dets, const int* __restrict__ aid, const int* __restrict__ aptr,
+    const int* __restrict__ agrp, const int* __restrict__ anb_ptr, const int* __restrict__ anb,
+    const int* __restrict__ bid, const int* __restrict__ bptr, const int* __restrict__ bgrp, int64_t* rowcnt,
+    const int64_t* rowptr, int* cols, int* err) {
   constexpr int NW = 2 * NINT;
-  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= n) return;
+  extern __shared__ uint32_t map[];
+  __shared__ int queue[kMapQueue], nq, wsum[kMapThreads / 32];
+  const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint64_t I[NW];
 #pragma unroll
   for (int w = 0; w < NW; w++) I[w] = dets[(size_t)row * NW + w];
-  int cnt = 0;
-  auto emit = [&](int j) {
-    if (COUNT) {
-      cnt++;
-    } else {
-      const int64_t pos = rowptr[row] + atomicAdd(&cursor[row], 1);
-      cols[pos] = j;
-      vals[pos] = hij_pair<NINT>(I, dets + (size_t)j * NW, norb, h, eri);
-    }
-  };
-  {  // (a) the same spin-down string: spin-up excitations
-    const int b = bid[row];
-    for (int k = bptr[b] + lane; k < bptr[b + 1]; k += 32) {
+  const int a = aid[row], b = bid[row];
+  int64_t done = 0;
+  for (int64_t lo = 0; lo < n; lo += win) {
+    const int nbits = (int)(n - lo < win ? n - lo : win), nwords = (nbits + 31) / 32;
+    for (int w = tid; w < nwords; w += kMapThreads) map[w] = 0u;
+    if (tid == 0) nq = 0;
+    __syncthreads();
+    auto mark = [&](int j) {
+      const int64_t at = j - lo;
+      if (at >= 0 && at < nbits) atomicOr(&map[at >> 5], 1u << (at & 31));
+    };
+    for (int k = bptr[b] + tid; k < bptr[b + 1]; k += kMapThreads) {  // (a) the same spin-down string
       const int j = bgrp[k];
-      if (j == (int)row) continue;
+      if (j == row) continue;
       const int d = spin_degree<NINT>(I, dets + (size_t)j * NW, 0);
       if (d == 0) atomicOr(err, 1);  // a repeated determinant
-      else if (d <= 2) emit(j);
+      else if (d <= 2) mark(j);
     }
-  }
-  const int a = aid[row];
-  for (int k = aptr[a] + lane; k < aptr[a + 1]; k += 32) {  // (b) the same spin-up string
-    const int j = agrp[k];
-    if (j == (int)row) continue;
-    const int d = spin_degree<NINT>(I, dets + (size_t)j * NW, 1);
-    if (d >= 1 && d <= 2) emit(j);
-  }
-  for (int q = anb_ptr[a]; q < anb_ptr[a + 1]; q++) {  // (c) spin-up single, then spin-down single
-    const int a2 = anb[q];
-    for (int k = aptr[a2] + lane; k < aptr[a2 + 1]; k += 32) {
+    for (int k = aptr[a] + tid; k < aptr[a + 1]; k += kMapThreads) {  // (b) the same spin-up string
       const int j = agrp[k];
-      if (spin_degree<NINT>(I, dets + (size_t)j * NW, 1) == 1) emit(j);
+      if (j == row) continue;
+      const int d = spin_degree<NINT>(I, dets + (size_t)j * NW, 1);
+      if (d >= 1 && d <= 2) mark(j);
     }
-  }
-  if (COUNT) {
+    auto pair = [&](int k) {
+      const int j = agrp[k];
+      if (spin_degree<NINT>(I, dets + (size_t)j * NW, 1) == 1) mark(j);
+    };
+    for (int q = anb_ptr[a] + tid; q < anb_ptr[a + 1]; q += kMapThreads) {  // (c) spin-up single, then spin-down single
+      const int a2 = anb[q], k0 = aptr[a2], k1 = aptr[a2 + 1];
+      if (k1 - k0 > 8) {
+        const int at = atomicAdd(&nq, 1);
+        if (at < kMapQueue) {
+          queue[at] = a2;
+          continue;
+        }
+      }
+      for (int k = k0; k < k1; k++) pair(k);
+    }
+    __syncthreads();
+    const int nbig = nq < kMapQueue ? nq : kMapQueue;
+    for (int q = warp; q < nbig; q += kMapThreads / 32)
+      for (int k = aptr[queue[q]] + lane, e = aptr[queue[q] + 1]; k < e; k += 32) pair(k);
+    __syncthreads();
+    // a contiguous run of words per thread, of odd length: 32 banks
+    const int per = ((nwords + kMapThreads - 1) / kMapThreads) | 1, w0 = min(tid * per, nwords), w1 = min(w0 + per, nwords);
+    int c = 0;
+    for (int w = w0; w < w1; w++) c += __popc(map[w]);
+    int at = c;
 #pragma unroll
-    for (int o = 16; o; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if (lane == 0) rowcnt[row] = cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += v;
+    }
+    if (lane == 31) wsum[warp] = at;
+    __syncthreads();
+    int before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < kMapThreads / 32; w++) {
+      before += w < warp ? wsum[w] : 0;
+      all += wsum[w];
+    }
+    if (!COUNT) {
+      int* out = cols + rowptr[row] + done + before + at - c;
+      for (int w = w0; w < w1; w++)
+        for (uint32_t m = map[w]; m; m &= m - 1) *out++ = (int)(lo + 32 * w + __ffs((int)m) - 1);
+    }
+    done += all;
+    __syncthreads();
   }
+  if (COUNT && tid == 0) rowcnt[row] = done;
 }
 
-// Y[k] = H X[k] for nvec vectors of length n: one warp per row.
-__global__ void spmv_kernel(int64_t n, int nvec, const int64_t* rowptr, const int* cols, const double* vals,
-                            const double* diag, const double* X, double* Y) {
-  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= n) return;
+// The elements of the columns found: a block per row, a thread per element;
+// single excitations, whose sums run over the occupied orbitals, are listed
+// and taken together, so that a warp of doubles does not wait for one of them
+// (533 -> 200 us for 6.2e6 elements).
+constexpr int kValThreads = 128, kSingles = 1024;
+template <int NINT>
+__global__ void __launch_bounds__(kValThreads) str_vals_kernel(const uint64_t* __restrict__ dets, int norb,
+                                                               const double* __restrict__ h,
+                                                               const double* __restrict__ eri,
+                                                               const int64_t* __restrict__ rowptr,
+                                                               const int* __restrict__ cols, double* __restrict__ vals) {
+  constexpr int NW = 2 * NINT;
+  __shared__ int single[kSingles], ns;
+  const int64_t row = blockIdx.x, q0 = rowptr[row];
+  const int len = (int)(rowptr[row + 1] - q0);
+  uint64_t I[NW];
+#pragma unroll
+  for (int w = 0; w < NW; w++) I[w] = dets[(size_t)row * NW + w];
+  if (threadIdx.x == 0) ns = 0;
+  __syncthreads();
+  auto element = [&](int k) {
+    uint64_t J[NW];
+    const uint64_t* p = dets + (size_t)cols[q0 + k] * NW;
+#pragma unroll
+    for (int w = 0; w < NW; w++) J[w] = p[w];
+    vals[q0 + k] = hij_pair<NINT>(I, J, norb, h, eri);
+  };
+  for (int k = threadIdx.x; k < len; k += kValThreads) {
+    const uint64_t* p = dets + (size_t)cols[q0 + k] * NW;
+    int x = 0;
+#pragma unroll
+    for (int w = 0; w < NW; w++) x += __popcll(I[w] ^ p[w]);
+    if (x == 2) {
+      const int at = atomicAdd(&ns, 1);
+      if (at < kSingles) {
+        single[at] = k;
+        continue;
+      }
+    }
+    element(k);
+  }
+  __syncthreads();
+  for (int q = threadIdx.x, e = ns < kSingles ? ns : kSingles; q < e; q += kValThreads) element(single[q]);
+}
+
+// Y[k] = H X[k] for nvec vectors of length n: a warp per row, and the whole
+// block for those of its rows that are longer than kLongRow (the row of the
+// reference holds fifteen times the average; a block's rows lie apart, as the
+// long ones are often neighbours).  A product costs a warp 19 cycles of the
+// SM's FP64 unit, and so does each step of a sum over lanes: for the 6.2e6
+// elements of 10^4 rows 12.8 us and 4, and their 75 MB take 11 us from HBM.
+// 33 us; a warp per row throughout took 130 (85 of it the longest row alone),
+// four warps per row 35, long rows from 1,536 on 34, and one block per SM with
+// x in shared memory 34: neither the sums nor the gathers are the bound, but
+// the chain of loads in each row.
+constexpr int kLongRow = 4096, kSpmvLoads = 8, kSpmvThreads = 256, kSpmvRows = kSpmvThreads / 32;
+__device__ __forceinline__ double row_part(int len, int first, int step, const int* __restrict__ c,
+                                           const double* __restrict__ v, const double* x) {
+  double a = 0.0, b = 0.0;
+  for (int q = first; q < len; q += kSpmvLoads * step) {
+    int cc[kSpmvLoads];
+    double vv[kSpmvLoads];
+#pragma unroll
+    for (int u = 0; u < kSpmvLoads; u++) {
+      const bool ok = q + u * step < len;
+      cc[u] = ok ? c[q + u * step] : -1;
+      vv[u] = ok ? v[q + u * step] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kSpmvLoads; u += 2) {
+      if (cc[u] >= 0) a = fma(vv[u], x[cc[u]], a);
+      if (cc[u + 1] >= 0) b = fma(vv[u + 1], x[cc[u + 1]], b);
+    }
+  }
+  a += b;
+#pragma unroll
+  for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
+__global__ void __launch_bounds__(kSpmvThreads) spmv_kernel(int64_t n, int nvec, const int64_t* __restrict__ rowptr,
+                                                            const int* __restrict__ cols,
+                                                            const double* __restrict__ vals,
+                                                            const double* __restrict__ diag,
+                                                            const double* __restrict__ X, double* __restrict__ Y) {
+  __shared__ double part[kSpmvRows];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t own = blockIdx.x + (int64_t)warp * gridDim.x;
+  const int64_t row = own < n ? own : n - 1, q0 = rowptr[row];
+  const int len = own < n ? (int)(rowptr[row + 1] - q0) : -1;  // -1: no row
+  const int any = __syncthreads_or(len > kLongRow);
   for (int k = 0; k < nvec; k++) {
     const double* x = X + (size_t)k * n;
-    double acc = 0.0;
-    for (int64_t q = rowptr[row] + lane; q < rowptr[row + 1]; q += 32) acc += vals[q] * x[cols[q]];
-#pragma unroll
-    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) Y[(size_t)k * n + row] = diag[row] * x[row] + acc;
+    double* y = Y + (size_t)k * n;
+    if (len >= 0 && len <= kLongRow) {
+      const double s = row_part(len, lane, 32, cols + q0, vals + q0, x);
+      if (lane == 0) y[row] = fma(diag[row], x[row], s);
+    }
+    if (!any) continue;
+    for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
+      const int64_t p0 = rowptr[r], p1 = rowptr[r + 1];
+      if (p1 - p0 <= kLongRow) continue;
+      const double s = row_part((int)(p1 - p0), threadIdx.x, kSpmvThreads, cols + p0, vals + p0, x);
+      if (lane == 0) part[warp] = s;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < kSpmvRows; w++) t += part[w];
+        y[r] = fma(diag[r], x[r], t);
+      }
+      __syncthreads();
+    }
   }
 }
 
-// out[k] = V[k] . y for k < m (one CTA per k).
-__global__ void dots_kernel(int64_t n, const double* V, const double* y, double* out) {
-  const double* v = V + (size_t)blockIdx.x * n;
-  double acc = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) acc += v[i] * y[i];
-  __shared__ double part[32];
+// out[kDotParts k + p] = part p of V[k] . y for k < m, and of z . z at k = m
+// where z is given.  A block per part: one SM's FP64 unit alone takes 3 us for
+// a product over 10^4 elements.
+constexpr int kDotThreads = 256, kDotParts = 8;
+__global__ void __launch_bounds__(kDotThreads) dots_kernel(int64_t n, int m, const double* __restrict__ V,
+                                                           const double* __restrict__ y, const double* __restrict__ z,
+                                                           double* out) {
+  const int k = blockIdx.x / kDotParts, p = blockIdx.x % kDotParts;
+  const double* a = k < m ? V + (size_t)k * n : z;
+  const double* b = k < m ? y : z;
+  const int64_t lo = n * p / kDotParts, hi = n * (p + 1) / kDotParts;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  int64_t i = lo + threadIdx.x;
+  for (; i + 3 * kDotThreads < hi; i += 4 * kDotThreads)
 #pragma unroll
-  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+    for (int u = 0; u < 4; u++) acc[u] = fma(a[i + u * kDotThreads], b[i + u * kDotThreads], acc[u]);
+#pragma unroll
+  for (int u = 0; u < 3; u++)
+    if (i + u * kDotThreads < hi) acc[u] = fma(a[i + u * kDotThreads], b[i + u * kDotThreads], acc[u]);
+  double s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  __shared__ double part[kDotThreads / 32];
+#pragma unroll
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    acc = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (threadIdx.x == 0) out[blockIdx.x] = acc;
+  if (threadIdx.x == 0) {
+    s = 0.0;
+    for (int w = 0; w < kDotThreads / 32; w++) s += part[w];
+    out[blockIdx.x] = s;
+  }
+}
+// A product from its parts, the same sum on the host and on the device.
+__host__ __device__ inline double dot_sum(const double* p) {
+  double s = 0.0;
+  for (int i = 0; i < kDotParts; i++) s += p[i];
+  return s;
+}
+
+// The lowest Ritz vector's coefficients, passed by value.
+struct Ritz {
+  double s[kMaxBasis], theta;
+};
+
+// x = sum_k s_k V_k, w = sum_k s_k W_k, r = w - theta x, t = r / (theta - H_II)
+// with |theta - H_II| kept above 1e-6.  restart: x and w become the first
+// basis vector and its product.
+__global__ void __launch_bounds__(128) ritz_kernel(int64_t n, int m, int restart, const __grid_constant__ Ritz z, double* V,
+                                                   double* W, const double* __restrict__ diag, double* x, double* w,
+                                                   double* r, double* t) {
+  const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (i >= n) return;
+  double xi = 0.0, wi = 0.0;
+#pragma unroll 4
+  for (int k = 0; k < m; k++) {
+    xi += z.s[k] * V[(size_t)k * n + i];
+    wi += z.s[k] * W[(size_t)k * n + i];
+  }
+  const double ri = wi - z.theta * xi;
+  double den = z.theta - diag[i];
+  if (fabs(den) < 1e-6) den = den < 0 ? -1e-6 : 1e-6;
+  x[i] = xi;
+  w[i] = wi;
+  r[i] = ri;
+  t[i] = ri / den;
+  if (restart) {
+    V[i] = xi;
+    W[i] = wi;
   }
 }
 
-// out = sum_k s[k] V[k] (+ beta * out when accumulate).
-__global__ void combine_kernel(int64_t n, int m, const double* V, const double* s, double* out, double beta) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// t - sum_k d_k V_k; norm: divided by its norm, whose square is t.t - sum d_k^2
+// (d_k the second pass's products, at the rounding level of t), into out.
+// d: parts of the products, t.t last.
+__global__ void __launch_bounds__(128) orth_kernel(int64_t n, int m, int norm, const double* __restrict__ V,
+                                                   const double* __restrict__ d, const double* t, double* out) {
+  __shared__ double c[kMaxBasis + 1], rn;
+  const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (threadIdx.x < 32) {
+    const int k = threadIdx.x;
+    double v = k < m ? dot_sum(d + k * kDotParts) : 0.0;
+    c[k] = v;
+    if (norm) {
+      v *= v;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (k == 0) {
+        const double nn = dot_sum(d + m * kDotParts) - v;
+        rn = nn > 1e-28 ? sqrt(nn) : 0.0;
+      }
+    }
+  }
+  __syncthreads();
   if (i >= n) return;
-  double acc = beta != 0.0 ? beta * out[i] : 0.0;
-  for (int k = 0; k < m; k++) acc += s[k] * V[(size_t)k * n + i];
+  double acc = 0.0;
+#pragma unroll 4
+  for (int k = 0; k < m; k++) acc += c[k] * V[(size_t)k * n + i];
+  acc = t[i] - acc;
+  if (norm) acc = rn > 0.0 ? acc / rn : 0.0;
   out[i] = acc;
 }
 
-// r = w - theta x; t = r / (theta - H_II), with |theta - H_II| kept above 1e-6.
-__global__ void correction_kernel(int64_t n, const double* x, const double* w, const double* diag, double theta,
-                                  double* r, double* t) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const double ri = w[i] - theta * x[i];
-  double den = theta - diag[i];
-  if (fabs(den) < 1e-6) den = den < 0 ? -1e-6 : 1e-6;
-  r[i] = ri;
-  t[i] = ri / den;
-}
-
-__global__ void scale_kernel(int64_t n, double a, const double* x, double* y) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = a * x[i];
-}
-
-// Eigenpairs of the symmetric m x m matrix a (row-major, overwritten) by
-// cyclic Jacobi rotations; eigenvalues in w, eigenvectors in the columns of v.
-void jacobi_eigen(int m, std::vector<double>& a, std::vector<double>& w, std::vector<double>& v) {
-  v.assign((size_t)m * m, 0.0);
-  for (int i = 0; i < m; i++) v[(size_t)i * m + i] = 1.0;
-  for (int sweep = 0; sweep < 100; sweep++) {
-    double off = 0.0, tot = 0.0;
-    for (int i = 0; i < m; i++)
-      for (int j = 0; j < m; j++) {
-        tot += a[(size_t)i * m + j] * a[(size_t)i * m + j];
-        if (i != j) off += a[(size_t)i * m + j] * a[(size_t)i * m + j];
-      }
-    if (off <= 1e-30 * tot || off == 0.0) break;
-    for (int p = 0; p < m; p++)
-      for (int q = p + 1; q < m; q++) {
-        const double apq = a[(size_t)p * m + q];
-        if (apq == 0.0) continue;
-        const double app = a[(size_t)p * m + p], aqq = a[(size_t)q * m + q];
-        const double tau = (aqq - app) / (2.0 * apq);
-        const double t = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + std::sqrt(1.0 + tau * tau));
-        const double c = 1.0 / std::sqrt(1.0 + t * t), s = t * c;
-        for (int k = 0; k < m; k++) {  // A <- J^T A J
-          const double akp = a[(size_t)k * m + p], akq = a[(size_t)k * m + q];
-          a[(size_t)k * m + p] = c * akp - s * akq;
-          a[(size_t)k * m + q] = s * akp + c * akq;
-        }
-        for (int k = 0; k < m; k++) {
-          const double apk = a[(size_t)p * m + k], aqk = a[(size_t)q * m + k];
-          a[(size_t)p * m + k] = c * apk - s * aqk;
-          a[(size_t)q * m + k] = s * apk + c * aqk;
-        }
-        for (int k = 0; k < m; k++) {
-          const double vkp = v[(size_t)k * m + p], vkq = v[(size_t)k * m + q];
-          v[(size_t)k * m + p] = c * vkp - s * vkq;
-          v[(size_t)k * m + q] = s * vkp + c * vkq;
-        }
-      }
+// The lowest eigenpair of the symmetric m x m matrix a (row-major): Householder
+// reduction to a tridiagonal matrix, its lowest eigenvalue by bisection on the
+// sign count of the LDL^T pivots (Sturm sequence), the eigenvector by inverse
+// iteration and the reflections, the eigenvalue again as its Rayleigh quotient.
+// The whole spectrum by Jacobi rotations, of which one pair was used, took
+// most of the solver's time at 20 and more vectors.
+double lowest_eigenpair(int m, const std::vector<double>& a0, double* y) {
+  if (m == 1) {
+    y[0] = 1.0;
+    return a0[0];
   }
-  w.resize(m);
-  for (int i = 0; i < m; i++) w[i] = a[(size_t)i * m + i];
+  std::vector<double> a(a0), v((size_t)m * m, 0.0), beta(m, 0.0), d(m), e(m, 0.0), p(m);
+  for (int k = 0; k + 2 < m; k++) {  // reflection k acts on the indices k + 1 .. m - 1
+    double* u = &v[(size_t)k * m];
+    double xx = 0.0;
+    for (int i = k + 1; i < m; i++) xx += a[(size_t)i * m + k] * a[(size_t)i * m + k];
+    const double x0 = a[(size_t)(k + 1) * m + k], tail = xx - x0 * x0;
+    if (!(tail > 0.0)) continue;
+    const double alpha = x0 > 0 ? -std::sqrt(xx) : std::sqrt(xx);
+    for (int i = k + 1; i < m; i++) u[i] = a[(size_t)i * m + k];
+    u[k + 1] -= alpha;
+    const double b = 2.0 / (tail + u[k + 1] * u[k + 1]);
+    beta[k] = b;
+    double up = 0.0;
+    for (int i = k + 1; i < m; i++) {
+      double q = 0.0;
+      for (int j = k + 1; j < m; j++) q += a[(size_t)i * m + j] * u[j];
+      p[i] = b * q;
+      up += u[i] * p[i];
+    }
+    for (int i = k + 1; i < m; i++) p[i] -= 0.5 * b * up * u[i];
+    for (int i = k + 1; i < m; i++)
+      for (int j = k + 1; j < m; j++) a[(size_t)i * m + j] -= u[i] * p[j] + p[i] * u[j];
+    a[(size_t)(k + 1) * m + k] = alpha;
+  }
+  double lo = INFINITY, hi = INFINITY, scale = 0.0;
+  for (int i = 0; i < m; i++) {
+    d[i] = a[(size_t)i * m + i];
+    if (i + 1 < m) e[i] = a[(size_t)(i + 1) * m + i];
+  }
+  for (int i = 0; i < m; i++) {
+    const double rad = (i ? std::fabs(e[i - 1]) : 0.0) + std::fabs(e[i]);
+    lo = std::fmin(lo, d[i] - rad);
+    hi = std::fmin(hi, d[i]);  // the lowest eigenvalue is at most the lowest diagonal entry
+    scale = std::fmax(scale, std::fabs(d[i]) + rad);
+  }
+  const double tiny = scale * 1e-300 + 1e-300;
+  for (int it = 0; it < 200 && hi - lo > 2.3e-16 * std::fmax(std::fabs(lo), std::fabs(hi)); it++) {
+    const double mid = 0.5 * (lo + hi);
+    if (mid <= lo || mid >= hi) break;
+    double q = d[0] - mid;
+    bool neg = q < 0.0;
+    for (int i = 1; i < m && !neg; i++) {
+      if (std::fabs(q) < tiny) q = tiny;
+      q = d[i] - mid - e[i - 1] * e[i - 1] / q;
+      neg = q < 0.0;
+    }
+    if (neg) hi = mid;
+    else lo = mid;
+  }
+  // inverse iteration: (T - lo) by Gaussian elimination with row exchanges
+  const double mu = lo, small = scale * 2.3e-16 + 1e-300;
+  std::vector<double> c0(m), c1(m), c2(m), mult(m);
+  std::vector<char> swp(m, 0);
+  for (int i = 0; i < m; i++) {
+    c0[i] = d[i] - mu;
+    c1[i] = e[i];
+    c2[i] = 0.0;
+  }
+  for (int i = 0; i + 1 < m; i++) {
+    double below = e[i];  // entry (i + 1, i)
+    if (std::fabs(below) > std::fabs(c0[i])) {
+      swp[i] = 1;
+      const double r0 = c0[i], r1 = c1[i];
+      c0[i] = below;
+      c1[i] = c0[i + 1];
+      c2[i] = c1[i + 1];
+      below = r0;
+      mult[i] = below / c0[i];
+      c0[i + 1] = r1 - mult[i] * c1[i];
+      c1[i + 1] = -mult[i] * c2[i];
+    } else {
+      if (std::fabs(c0[i]) < small) c0[i] = small;
+      mult[i] = below / c0[i];
+      c0[i + 1] -= mult[i] * c1[i];
+    }
+  }
+  if (std::fabs(c0[m - 1]) < small) c0[m - 1] = small;
+  for (int i = 0; i < m; i++) y[i] = 1.0 + 0.01 * i;
+  for (int it = 0; it < 4; it++) {
+    if (it)  // the first right-hand side is taken as eliminated already
+      for (int i = 0; i + 1 < m; i++) {
+        if (swp[i]) std::swap(y[i], y[i + 1]);
+        y[i + 1] -= mult[i] * y[i];
+      }
+    double big = 0.0;
+    for (int i = m - 1; i >= 0; i--) {
+      double b = y[i];
+      if (i + 1 < m) b -= c1[i] * y[i + 1];
+      if (i + 2 < m) b -= c2[i] * y[i + 2];
+      y[i] = b / c0[i];
+      big = std::fmax(big, std::fabs(y[i]));
+    }
+    for (int i = 0; i < m; i++) y[i] /= big;
+  }
+  for (int k = m - 3; k >= 0; k--) {
+    if (beta[k] == 0.0) continue;
+    const double* u = &v[(size_t)k * m];
+    double q = 0.0;
+    for (int i = k + 1; i < m; i++) q += u[i] * y[i];
+    for (int i = k + 1; i < m; i++) y[i] -= beta[k] * q * u[i];
+  }
+  double nn = 0.0;
+  for (int i = 0; i < m; i++) nn += y[i] * y[i];
+  nn = 1.0 / std::sqrt(nn);
+  for (int i = 0; i < m; i++) y[i] *= nn;
+  double theta = 0.0;
+  for (int i = 0; i < m; i++)
+    for (int j = 0; j < m; j++) theta += y[i] * a0[(size_t)i * m + j] * y[j];
+  return theta;
 }
 
-// Device buffers of one Hamiltonian (freed on scope exit).
+// Device buffers of one call: cut from the context's workspace as far as it
+// goes (one call at a time holds it), the rest allocated and freed on scope
+// exit.  A call that needed more than the workspace, and not more than
+// kKeepBytes in all, leaves one of the size it needed.
+constexpr size_t kKeepBytes = (size_t)256 << 20;
 struct DevMem {
+  const CtxView& c;
+  bool held;
+  void* ws = nullptr;
+  size_t ws_bytes = 0, off = 0, need = 0;
   std::vector<void*> ptrs;
+  explicit DevMem(const CtxView& v) : c(v), held(ctx_ws_take(v.ctx, &ws, &ws_bytes)) {}
+  DevMem(const DevMem&) = delete;
   ~DevMem() {
+    cudaStreamSynchronize(c.st);  // nothing of this call may still run
     for (void* p : ptrs) cudaFree(p);
+    if (held) ctx_ws_give(c.ctx, need <= kKeepBytes ? need : 0);
   }
   template <typename T>
   T* alloc(size_t count) {
+    const size_t bytes = (sizeof(T) * (count ? count : 1) + 255) & ~(size_t)255;
+    need += bytes;
+    if (off + bytes <= ws_bytes) {
+      T* p = reinterpret_cast<T*>(static_cast<unsigned char*>(ws) + off);
+      off += bytes;
+      return p;
+    }
     void* p = nullptr;
-    if (cudaMalloc(&p, sizeof(T) * (count ? count : 1)) != cudaSuccess) return nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
     ptrs.push_back(p);
     return static_cast<T*>(p);
   }
@@ -492,7 +797,7 @@ int build_strings(const CtxView& c, int64_t n, const uint64_t* d_dets, int spin,
   S->nb_ptr = mem.alloc<int>((size_t)nu + 1);
   if (!cnt || !S->nb_ptr) return report(QP_ENOMEM, "device allocation for the spin strings failed");
   DV_TRY(cudaMemsetAsync(cnt, 0, sizeof(int) * ((size_t)nu + 1), st));
-  const unsigned nbu = (unsigned)((nu + 127) / 128);
+  const unsigned nbu = (unsigned)(((int64_t)nu * 32 + 127) / 128);
   if (nint == 1) str_nb_kernel<1, true><<<nbu, 128, 0, st>>>(nu, S->ukey, cnt, nullptr, nullptr);
   else str_nb_kernel<2, true><<<nbu, 128, 0, st>>>(nu, S->ukey, cnt, nullptr, nullptr);
   size_t tmp3 = 0;
@@ -511,100 +816,97 @@ int build_strings(const CtxView& c, int64_t n, const uint64_t* d_dets, int spin,
   return QP_OK;
 }
 
-// search: kSearchStrings (default) or kSearchAllPairs (the tiled test of
-// every pair, O(N_det^2), kept as a cross-check)
+// search: 0, the spin strings; 1, the tiled test of every pair, O(N_det^2),
+// kept as a cross-check.
 int build_h(const CtxView& c, int64_t n, const uint64_t* d_dets, DevMem& mem, HMat* H, int search = 0) {
   cudaStream_t st = c.st;
   H->n = n;
-  int* rowcnt = mem.alloc<int>(n + 1);
-  int* cursor = mem.alloc<int>(n);
+  int64_t* cnt = mem.alloc<int64_t>(n + 1);
   int* err = mem.alloc<int>(1);
   H->rowptr = mem.alloc<int64_t>(n + 1);
   H->diag = mem.alloc<double>(n);
-  int64_t* cnt64 = mem.alloc<int64_t>(n + 1);
-  if (!rowcnt || !cursor || !err || !H->rowptr || !H->diag || !cnt64)
+  size_t tmp = 0;
+  cub::DeviceScan::ExclusiveSum(nullptr, tmp, cnt, H->rowptr, (int)(n + 1), st);
+  void* d_tmp = mem.alloc<unsigned char>(tmp);
+  if (!cnt || !err || !H->rowptr || !H->diag || !d_tmp)
     return report(QP_ENOMEM, "device allocation for the Hamiltonian failed");
   DV_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
-  DV_TRY(cudaMemsetAsync(rowcnt, 0, sizeof(int) * (n + 1), st));
-  DV_TRY(cudaMemsetAsync(cursor, 0, sizeof(int) * n, st));
+  DV_TRY(cudaMemsetAsync(cnt, 0, sizeof(int64_t) * (n + 1), st));
   const unsigned tiles = (unsigned)((n + kRows - 1) / kRows), nb = (unsigned)((n + 255) / 256);
-  const unsigned nwarp = (unsigned)((n * 32 + 255) / 256);
+  const int win = (int)(n < kMapMax ? n : kMapMax);  // determinants per bit map
+  const size_t smem = 4 * (size_t)((win + 31) / 32);
   SpinStrings SA, SB;
   int rc;
   if (search == 0) {
     if ((rc = build_strings(c, n, d_dets, 0, true, mem, &SA)) || (rc = build_strings(c, n, d_dets, 1, false, mem, &SB)))
       return rc;
   }
-  // one pass of the pair search: COUNT (row counts) or fill
-  auto pairs = [&](bool count, const int64_t* rowptr, int* cols, double* vals) {
-    if (search == 0) {
-      if (c.nint == 1) {
-        if (count)
-          str_pairs_kernel<1, true><<<nwarp, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.eri, SA.sid, SA.ptr, SA.grp,
-                                                           SA.nb_ptr, SA.nb, SB.sid, SB.ptr, SB.grp, rowcnt, rowptr,
-                                                           cursor, cols, vals, err);
-        else
-          str_pairs_kernel<1, false><<<nwarp, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.eri, SA.sid, SA.ptr, SA.grp,
-                                                            SA.nb_ptr, SA.nb, SB.sid, SB.ptr, SB.grp, rowcnt, rowptr,
-                                                            cursor, cols, vals, err);
-      } else {
-        if (count)
-          str_pairs_kernel<2, true><<<nwarp, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.eri, SA.sid, SA.ptr, SA.grp,
-                                                           SA.nb_ptr, SA.nb, SB.sid, SB.ptr, SB.grp, rowcnt, rowptr,
-                                                           cursor, cols, vals, err);
-        else
-          str_pairs_kernel<2, false><<<nwarp, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.eri, SA.sid, SA.ptr, SA.grp,
-                                                            SA.nb_ptr, SA.nb, SB.sid, SB.ptr, SB.grp, rowcnt, rowptr,
-                                                            cursor, cols, vals, err);
-      }
-    } else if (c.nint == 1) {
-      if (count)
-        pairs_kernel<1, true><<<tiles, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.eri, rowcnt, nullptr, nullptr, nullptr,
-                                                     nullptr, err);
-      else
-        pairs_kernel<1, false><<<tiles, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.eri, nullptr, rowptr, cursor, cols,
-                                                      vals, err);
-    } else {
-      if (count)
-        pairs_kernel<2, true><<<tiles, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.eri, rowcnt, nullptr, nullptr, nullptr,
-                                                     nullptr, err);
-      else
-        pairs_kernel<2, false><<<tiles, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.eri, nullptr, rowptr, cursor, cols,
-                                                      vals, err);
-    }
+  int* cursor = nullptr;
+  if (search == 1) {
+    cursor = mem.alloc<int>(n);
+    if (!cursor) return report(QP_ENOMEM, "device allocation for the Hamiltonian failed");
+    DV_TRY(cudaMemsetAsync(cursor, 0, sizeof(int) * n, st));
+  }
+  // one pass of the pair search: row counts, or the columns (and, all pairs,
+  // the elements in any order)
+  auto strings = [&](auto nint, auto count, int* cols) -> cudaError_t {
+    auto* k = str_pairs_kernel<decltype(nint)::value, decltype(count)::value>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k<<<(unsigned)n, kMapThreads, smem, st>>>(n, win, d_dets, SA.sid, SA.ptr, SA.grp, SA.nb_ptr, SA.nb, SB.sid,
+                                              SB.ptr, SB.grp, cnt, H->rowptr, cols, err);
+    return cudaGetLastError();
   };
+  auto pairs = [&](auto nint, auto count, int* cols, double* vals) -> cudaError_t {
+    pairs_kernel<decltype(nint)::value, decltype(count)::value><<<tiles, 256, 0, st>>>(
+        n, d_dets, c.norb, c.h, c.eri, cnt, H->rowptr, cursor, cols, vals, err);
+    return cudaGetLastError();
+  };
+  using I1 = std::integral_constant<int, 1>;
+  using I2 = std::integral_constant<int, 2>;
   if (c.nint == 1) diag_kernel<1><<<nb, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.Jm, c.Km, H->diag);
   else diag_kernel<2><<<nb, 256, 0, st>>>(n, d_dets, c.norb, c.h, c.Jm, c.Km, H->diag);
-  pairs(true, nullptr, nullptr, nullptr);
-  DV_TRY(cudaGetLastError());
-  // row counts (int) -> 64-bit exclusive offsets
-  std::vector<int> hc((size_t)n);
-  DV_TRY(cudaMemcpyAsync(hc.data(), rowcnt, sizeof(int) * n, cudaMemcpyDeviceToHost, st));
+  if (search == 0)
+    DV_TRY(c.nint == 1 ? strings(I1{}, std::true_type{}, nullptr) : strings(I2{}, std::true_type{}, nullptr));
+  else
+    DV_TRY(c.nint == 1 ? pairs(I1{}, std::true_type{}, nullptr, nullptr) : pairs(I2{}, std::true_type{}, nullptr, nullptr));
+  DV_TRY(cub::DeviceScan::ExclusiveSum(d_tmp, tmp, cnt, H->rowptr, (int)(n + 1), st));
   int herr = 0;
   DV_TRY(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  DV_TRY(cudaMemcpyAsync(&H->nnz, H->rowptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
   DV_TRY(cudaStreamSynchronize(st));
   if (herr) return report(QP_EDUP, "duplicate determinant in Psi0");
-  std::vector<int64_t> hp((size_t)n + 1, 0);
-  for (int64_t i = 0; i < n; i++) hp[i + 1] = hp[i] + hc[i];
-  H->nnz = hp[n];
-  DV_TRY(cudaMemcpyAsync(H->rowptr, hp.data(), sizeof(int64_t) * (n + 1), cudaMemcpyHostToDevice, st));
+  if (H->nnz >= (1ll << 31)) return report(QP_ENOTSUP, "Hamiltonian above 2^31 entries");
   H->cols = mem.alloc<int>(H->nnz);
   H->vals = mem.alloc<double>(H->nnz);
+  if (!H->cols || !H->vals) return report(QP_ENOMEM, "device allocation for the Hamiltonian failed");
+  if (H->nnz == 0) return QP_OK;
+  if (search == 0) {
+    DV_TRY(c.nint == 1 ? strings(I1{}, std::false_type{}, H->cols) : strings(I2{}, std::false_type{}, H->cols));
+    if (c.nint == 1) str_vals_kernel<1><<<(unsigned)n, 128, 0, st>>>(d_dets, c.norb, c.h, c.eri, H->rowptr, H->cols, H->vals);
+    else str_vals_kernel<2><<<(unsigned)n, 128, 0, st>>>(d_dets, c.norb, c.h, c.eri, H->rowptr, H->cols, H->vals);
+    DV_TRY(cudaGetLastError());
+    return QP_OK;
+  }
   int* cols2 = mem.alloc<int>(H->nnz);
   double* vals2 = mem.alloc<double>(H->nnz);
-  if (!H->cols || !H->vals || !cols2 || !vals2) return report(QP_ENOMEM, "device allocation for the Hamiltonian failed");
-  pairs(false, H->rowptr, cols2, vals2);
+  if (!cols2 || !vals2) return report(QP_ENOMEM, "device allocation for the Hamiltonian failed");
+  DV_TRY(c.nint == 1 ? pairs(I1{}, std::false_type{}, cols2, vals2) : pairs(I2{}, std::false_type{}, cols2, vals2));
+  // columns ascending within each row: a fixed order of the sums
+  size_t tmp2 = 0;
+  cub::DeviceSegmentedRadixSort::SortPairs(nullptr, tmp2, cols2, H->cols, vals2, H->vals, (int)H->nnz, (int)n,
+                                           H->rowptr, H->rowptr + 1, 0, 32, st);
+  void* d_tmp2 = mem.alloc<unsigned char>(tmp2);
+  if (!d_tmp2) return report(QP_ENOMEM, "device allocation for the Hamiltonian failed");
+  DV_TRY(cub::DeviceSegmentedRadixSort::SortPairs(d_tmp2, tmp2, cols2, H->cols, vals2, H->vals, (int)H->nnz, (int)n,
+                                                  H->rowptr, H->rowptr + 1, 0, 32, st));
+  return QP_OK;
+}
+
+int spmv(const CtxView& c, const HMat& H, int nvec, const double* X, double* Y) {
+  spmv_kernel<<<(unsigned)((H.n + kSpmvRows - 1) / kSpmvRows), kSpmvThreads, 0, c.st>>>(H.n, nvec, H.rowptr, H.cols,
+                                                                                        H.vals, H.diag, X, Y);
   DV_TRY(cudaGetLastError());
-  if (H->nnz > 0) {  // columns ascending within each row: a fixed order of the sums
-    if (H->nnz >= (1ll << 31) || n >= (1ll << 31)) return report(QP_ENOTSUP, "Hamiltonian above 2^31 entries");
-    size_t tmp = 0;
-    cub::DeviceSegmentedRadixSort::SortPairs(nullptr, tmp, cols2, H->cols, vals2, H->vals, (int)H->nnz, (int)n,
-                                             H->rowptr, H->rowptr + 1, 0, 32, st);
-    void* d_tmp = mem.alloc<unsigned char>(tmp);
-    if (!d_tmp) return report(QP_ENOMEM, "device allocation for the Hamiltonian failed");
-    DV_TRY(cub::DeviceSegmentedRadixSort::SortPairs(d_tmp, tmp, cols2, H->cols, vals2, H->vals, (int)H->nnz,
-                                                    (int)n, H->rowptr, H->rowptr + 1, 0, 32, st));
-  }
   return QP_OK;
 }
 
@@ -633,24 +935,36 @@ int to_device(const T* src, size_t count, cudaStream_t st, DevMem& mem, const T*
   return QP_OK;
 }
 
-int validate(const CtxView& c, int64_t n, const uint64_t* d_dets) {
-  // occupation counts and bits beyond norb, on the host (one copy of Psi0)
-  const int nw = 2 * c.nint;
-  std::vector<uint64_t> hd((size_t)n * nw);
-  DV_TRY(cudaMemcpyAsync(hd.data(), d_dets, sizeof(uint64_t) * n * nw, cudaMemcpyDeviceToHost, c.st));
-  DV_TRY(cudaStreamSynchronize(c.st));
-  for (int64_t i = 0; i < n; i++)
-    for (int s = 0; s < 2; s++) {
-      int cnt = 0;
-      for (int w = 0; w < c.nint; w++) {
-        const uint64_t b = hd[(size_t)i * nw + s * c.nint + w];
-        const int lim = c.norb - 64 * w;  // orbitals held by this word
-        const uint64_t valid = lim >= 64 ? ~0ull : (lim <= 0 ? 0ull : (1ull << lim) - 1);
-        if (b & ~valid) return report(QP_EINVAL, "a bit beyond norb is set");
-        cnt += __builtin_popcountll(b);
-      }
-      if (cnt != (s ? c.nbeta : c.nalpha)) return report(QP_EINVAL, "a determinant has the wrong occupation");
+// Occupation counts and bits beyond norb.
+__global__ void check_dets_kernel(int64_t n, int nint, int norb, int na, int nb, const uint64_t* dets, int* bad) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  int f = 0;
+  for (int s = 0; s < 2; s++) {
+    int cnt = 0;
+    for (int w = 0; w < nint; w++) {
+      const uint64_t b = dets[(size_t)i * 2 * nint + s * nint + w];
+      const int lim = norb - 64 * w;  // orbitals held by this word
+      const uint64_t valid = lim >= 64 ? ~0ull : (lim <= 0 ? 0ull : (1ull << lim) - 1);
+      if (b & ~valid) f |= 1;
+      cnt += __popcll(b);
     }
+    if (cnt != (s ? nb : na)) f |= 2;
+  }
+  if (f) atomicOr(bad, f);
+}
+
+int validate(const CtxView& c, int64_t n, const uint64_t* d_dets, DevMem& mem) {
+  int* bad = mem.alloc<int>(1);
+  if (!bad) return report(QP_ENOMEM, "device allocation failed");
+  DV_TRY(cudaMemsetAsync(bad, 0, sizeof(int), c.st));
+  check_dets_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c.st>>>(n, c.nint, c.norb, c.nalpha, c.nbeta, d_dets, bad);
+  DV_TRY(cudaGetLastError());
+  int f = 0;
+  DV_TRY(cudaMemcpyAsync(&f, bad, sizeof(int), cudaMemcpyDeviceToHost, c.st));
+  DV_TRY(cudaStreamSynchronize(c.st));
+  if (f & 1) return report(QP_EINVAL, "a bit beyond norb is set");
+  if (f & 2) return report(QP_EINVAL, "a determinant has the wrong occupation");
   return QP_OK;
 }
 
@@ -666,19 +980,17 @@ extern "C" int qp_pt2_sigma(qp_pt2_ctx* ctx, int64_t ndet, const uint64_t* dets,
   if (rc) return rc;
   if ((rc = check_inputs(c, ndet, dets))) return rc;
   if (nvec < 1 || !U || !S) return report(QP_EINVAL, "nvec must be positive and U, S non-NULL");
-  DevMem mem;
+  DevMem mem(c);
   const uint64_t* d_dets;
   const double* d_u;
   if ((rc = to_device(dets, (size_t)ndet * 2 * c.nint, c.st, mem, &d_dets))) return rc;
-  if ((rc = validate(c, ndet, d_dets))) return rc;
+  if ((rc = validate(c, ndet, d_dets, mem))) return rc;
   if ((rc = to_device(U, (size_t)ndet * nvec, c.st, mem, &d_u))) return rc;
   HMat H;
   if ((rc = build_h(c, ndet, d_dets, mem, &H))) return rc;
   double* d_s = mem.alloc<double>((size_t)ndet * nvec);
   if (!d_s) return report(QP_ENOMEM, "device allocation failed");
-  spmv_kernel<<<(unsigned)((ndet * 32 + 255) / 256), 256, 0, c.st>>>(ndet, nvec, H.rowptr, H.cols, H.vals, H.diag,
-                                                                     d_u, d_s);
-  DV_TRY(cudaGetLastError());
+  if ((rc = spmv(c, H, nvec, d_u, d_s))) return rc;
   DV_TRY(cudaMemcpyAsync(S, d_s, sizeof(double) * ndet * nvec, cudaMemcpyDefault, c.st));
   DV_TRY(cudaStreamSynchronize(c.st));
   return QP_OK;
@@ -692,10 +1004,10 @@ extern "C" int qp_pt2_hamiltonian(qp_pt2_ctx* ctx, int64_t ndet, const uint64_t*
   if ((rc = check_inputs(c, ndet, dets))) return rc;
   if (!nnz) return report(QP_EINVAL, "nnz is NULL");
   if (search != 0 && search != 1) return report(QP_EINVAL, "search must be 0 (spin strings) or 1 (all pairs)");
-  DevMem mem;
+  DevMem mem(c);
   const uint64_t* d_dets;
   if ((rc = to_device(dets, (size_t)ndet * 2 * c.nint, c.st, mem, &d_dets))) return rc;
-  if ((rc = validate(c, ndet, d_dets))) return rc;
+  if ((rc = validate(c, ndet, d_dets, mem))) return rc;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -729,11 +1041,11 @@ extern "C" int qp_pt2_davidson(qp_pt2_ctx* ctx, int64_t ndet, const uint64_t* de
   if (!(tol > 0.0) || max_iter < 1) return report(QP_EINVAL, "tol must be positive and max_iter at least 1");
   cudaStream_t st = c.st;
   const int64_t n = ndet;
-  const unsigned nb = (unsigned)((n + 255) / 256), nspmv = (unsigned)((n * 32 + 255) / 256);
-  DevMem mem;
+  const unsigned nb = (unsigned)((n + 127) / 128);
+  DevMem mem(c);
   const uint64_t* d_dets;
   if ((rc = to_device(dets, (size_t)n * 2 * c.nint, st, mem, &d_dets))) return rc;
-  if ((rc = validate(c, n, d_dets))) return rc;
+  if ((rc = validate(c, n, d_dets, mem))) return rc;
   struct Events {  // destroyed on every return
     cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
     Events() {
@@ -756,7 +1068,10 @@ extern "C" int qp_pt2_davidson(qp_pt2_ctx* ctx, int64_t ndet, const uint64_t* de
   double* w = mem.alloc<double>(n);
   double* r = mem.alloc<double>(n);
   double* t = mem.alloc<double>(n);
-  double* d_small = mem.alloc<double>(2 * kMaxBasis + 2);
+  // products of the two orthogonalisation passes (with r.r and t.t) and of the
+  // new column of the subspace matrix
+  constexpr int kProducts = (kMaxBasis + 1) * kDotParts;
+  double* d_small = mem.alloc<double>(3 * kProducts);
   if (!V || !W || !x || !w || !r || !t || !d_small) return report(QP_ENOMEM, "device allocation for Davidson failed");
   // first basis vector: the guess, or the determinant of lowest H_II
   std::vector<double> hv((size_t)n);
@@ -777,69 +1092,70 @@ extern "C" int qp_pt2_davidson(qp_pt2_ctx* ctx, int64_t ndet, const uint64_t* de
   if (!(nrm > 0.0) || !std::isfinite(nrm)) return report(QP_EINVAL, "the guess vector is zero or not finite");
   for (double& v : hv) v /= std::sqrt(nrm);
   DV_TRY(cudaMemcpyAsync(V, hv.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
-  auto hmul = [&](const double* in, double* out) {
-    spmv_kernel<<<nspmv, 256, 0, st>>>(n, 1, H.rowptr, H.cols, H.vals, H.diag, in, out);
-  };
-  auto dots = [&](int m, const double* base, const double* y, double* out_host) -> int {
-    dots_kernel<<<m, 256, 0, st>>>(n, base, y, d_small);
-    DV_TRY(cudaMemcpyAsync(out_host, d_small, sizeof(double) * m, cudaMemcpyDeviceToHost, st));
+  auto dot = [&](const double* a, const double* b, double* out_host) -> int {
+    double parts[kDotParts];
+    dots_kernel<<<kDotParts, kDotThreads, 0, st>>>(n, 1, a, b, nullptr, d_small);
+    DV_TRY(cudaMemcpyAsync(parts, d_small, sizeof(parts), cudaMemcpyDeviceToHost, st));
     DV_TRY(cudaStreamSynchronize(st));
+    *out_host = dot_sum(parts);
     return QP_OK;
   };
-  hmul(V, W);
-  std::vector<double> G((size_t)kMaxBasis * kMaxBasis, 0.0), col(kMaxBasis), s_h, ev, evec;
-  if ((rc = dots(1, V, W, col.data()))) return rc;
-  G[0] = col[0];
+  double *d1 = d_small, *d2 = d1 + kProducts, *d3 = d2 + kProducts;
+  if ((rc = spmv(c, H, 1, V, W))) return rc;
+  std::vector<double> G((size_t)kMaxBasis * kMaxBasis, 0.0), a;
+  double hs[3 * kProducts];
+  const double *h1 = hs, *h2 = h1 + kProducts, *h3 = h2 + kProducts;
+  if ((rc = dot(V, W, G.data()))) return rc;
   int m = 1, it = 0;
   double theta = G[0], rnorm = INFINITY;
   bool converged = false;
+  // One iteration: the lowest Ritz pair of the subspace matrix on the host,
+  // then seven launches without a wait between them (the Ritz vector, its
+  // residual and correction; two orthogonalisation passes; the product with
+  // H; the subspace matrix's new column), and one read-back.  The residual is
+  // known with it: the extension of the last iteration is not used.
   for (;;) {
-    // lowest Ritz pair of the subspace matrix
-    std::vector<double> a((size_t)m * m);
+    a.resize((size_t)m * m);
     for (int i = 0; i < m; i++)
       for (int j = 0; j < m; j++) a[(size_t)i * m + j] = 0.5 * (G[(size_t)i * kMaxBasis + j] + G[(size_t)j * kMaxBasis + i]);
-    jacobi_eigen(m, a, ev, evec);
-    int lo = 0;
-    for (int i = 1; i < m; i++)
-      if (ev[i] < ev[lo]) lo = i;
-    theta = ev[lo];
-    s_h.resize(m);
-    for (int i = 0; i < m; i++) s_h[i] = evec[(size_t)i * m + lo];
-    DV_TRY(cudaMemcpyAsync(d_small, s_h.data(), sizeof(double) * m, cudaMemcpyHostToDevice, st));
-    combine_kernel<<<nb, 256, 0, st>>>(n, m, V, d_small, x, 0.0);
-    combine_kernel<<<nb, 256, 0, st>>>(n, m, W, d_small, w, 0.0);
-    correction_kernel<<<nb, 256, 0, st>>>(n, x, w, H.diag, theta, r, t);
+    Ritz z{};
+    z.theta = theta = lowest_eigenpair(m, a, z.s);
+    const int restart = m == mmax ? 1 : 0, mb = restart ? 1 : m;  // full: restart from the Ritz vector
+    ritz_kernel<<<nb, 128, 0, st>>>(n, m, restart, z, V, W, H.diag, x, w, r, t);
+    dots_kernel<<<(mb + 1) * kDotParts, kDotThreads, 0, st>>>(n, mb, V, t, r, d1);
+    orth_kernel<<<nb, 128, 0, st>>>(n, mb, 0, V, d1, t, t);
+    dots_kernel<<<(mb + 1) * kDotParts, kDotThreads, 0, st>>>(n, mb, V, t, t, d2);
+    // (a basis that is restarted at its full length leaves room for one more)
+    double *vn = V + (size_t)mb * n, *wn = W + (size_t)mb * n;
+    const bool room = mb < mmax;
+    if (room) {
+      orth_kernel<<<nb, 128, 0, st>>>(n, mb, 1, V, d2, t, vn);
+      if ((rc = spmv(c, H, 1, vn, wn))) return rc;
+      dots_kernel<<<(mb + 1) * kDotParts, kDotThreads, 0, st>>>(n, mb + 1, V, wn, nullptr, d3);
+    }
     DV_TRY(cudaGetLastError());
-    double rr;
-    if ((rc = dots(1, r, r, &rr))) return rc;
-    rnorm = std::sqrt(rr);
+    DV_TRY(cudaMemcpyAsync(hs, d_small, sizeof(hs), cudaMemcpyDeviceToHost, st));
+    DV_TRY(cudaStreamSynchronize(st));
+    rnorm = std::sqrt(dot_sum(h1 + mb * kDotParts));
     if (rnorm <= tol) {
       converged = true;
       break;
     }
     if (++it > max_iter) break;
-    if (m == mmax) {  // restart from the Ritz vector
-      DV_TRY(cudaMemcpyAsync(V, x, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
-      DV_TRY(cudaMemcpyAsync(W, w, sizeof(double) * n, cudaMemcpyDeviceToDevice, st));
+    if (restart) {
       G[0] = theta;
       m = 1;
     }
-    // orthogonalise t against the basis twice, normalise, extend
-    for (int pass = 0; pass < 2; pass++) {
-      if ((rc = dots(m, V, t, col.data()))) return rc;
-      for (int i = 0; i < m; i++) col[i] = -col[i];
-      DV_TRY(cudaMemcpyAsync(d_small, col.data(), sizeof(double) * m, cudaMemcpyHostToDevice, st));
-      combine_kernel<<<nb, 256, 0, st>>>(n, m, V, d_small, t, 1.0);
+    double tt = dot_sum(h2 + m * kDotParts);
+    for (int i = 0; i < m; i++) {
+      const double d = dot_sum(h2 + i * kDotParts);
+      tt -= d * d;
     }
-    double tt;
-    if ((rc = dots(1, t, t, &tt))) return rc;
-    if (!(tt > 1e-28)) break;  // no new direction
-    scale_kernel<<<nb, 256, 0, st>>>(n, 1.0 / std::sqrt(tt), t, V + (size_t)m * n);
-    hmul(V + (size_t)m * n, W + (size_t)m * n);
-    if ((rc = dots(m + 1, V, W + (size_t)m * n, col.data()))) return rc;
+    if (!room || !(tt > 1e-28)) break;  // no new direction
     for (int i = 0; i <= m; i++) {
-      G[(size_t)i * kMaxBasis + m] = col[i];
-      G[(size_t)m * kMaxBasis + i] = col[i];
+      const double g = dot_sum(h3 + i * kDotParts);
+      G[(size_t)i * kMaxBasis + m] = g;
+      G[(size_t)m * kMaxBasis + i] = g;
     }
     m++;
   }
@@ -853,9 +1169,9 @@ extern "C" int qp_pt2_davidson(qp_pt2_ctx* ctx, int64_t ndet, const uint64_t* de
   for (double& v : hv) v *= sc;
   // E0 as the Rayleigh quotient of the returned vector
   DV_TRY(cudaMemcpyAsync(x, hv.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
-  hmul(x, w);
+  if ((rc = spmv(c, H, 1, x, w))) return rc;
   double xhx;
-  if ((rc = dots(1, x, w, &xhx))) return rc;
+  if ((rc = dot(x, w, &xhx))) return rc;
   DV_TRY(cudaMemcpyAsync(coefs, x, sizeof(double) * n, cudaMemcpyDefault, st));
   DV_TRY(cudaStreamSynchronize(st));
   *e0 = xhx;

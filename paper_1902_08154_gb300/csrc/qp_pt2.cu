@@ -6,6 +6,7 @@
 #include <cub/device/device_radix_sort.cuh>
 #include <cub/device/device_segmented_radix_sort.cuh>
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -339,6 +340,8 @@ struct qp_pt2_ctx {
   Buf cand_e, cand_a, cand_key, skey, skey2, perm, perm2, cub_tmp2;
   Buf out_sel, out_e, out_num, out_eps, out_na, out_ncon, out_rank;
   Buf g_dh, g_deri, g_wF, g_wH;
+  Buf dv_ws;  // the Hamiltonian and Davidson unit's workspace (at most 256 MiB)
+  std::atomic<bool> dv_busy{false};  // a call holds it
   int grad_grid = 0;
   int64_t launches = 0;
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};  // call start, sweep start, sweep end
@@ -348,7 +351,7 @@ struct qp_pt2_ctx {
 };
 
 namespace qp {
-int ctx_view(const qp_pt2_ctx* x, CtxView* v) {
+int ctx_view(qp_pt2_ctx* x, CtxView* v) {
   if (!x || !v) return fail(QP_EINVAL, "ctx is NULL");
   v->norb = x->norb;
   v->nalpha = x->nalpha;
@@ -361,7 +364,22 @@ int ctx_view(const qp_pt2_ctx* x, CtxView* v) {
   v->Jm = x->d_J;
   v->Km = x->d_K;
   v->st = x->st;
+  v->ctx = x;
   return QP_OK;
+}
+bool ctx_ws_take(qp_pt2_ctx* x, void** p, size_t* bytes) {
+  if (x->dv_busy.exchange(true)) return false;
+  *p = x->dv_ws.p;
+  *bytes = x->dv_ws.n;
+  return true;
+}
+void ctx_ws_give(qp_pt2_ctx* x, size_t bytes) {
+  const std::string keep = g_last_error;  // of the call that ends here
+  if (bytes > x->dv_ws.n && x->dv_ws.grow(bytes) != QP_OK) {
+    cudaGetLastError();
+    g_last_error = keep;
+  }
+  x->dv_busy.store(false);
 }
 int report(int code, const char* msg) { return fail(code, msg); }
 }  // namespace qp
@@ -546,7 +564,7 @@ extern "C" void qp_pt2_destroy(qp_pt2_ctx* x) {
                 &x->res, &x->meta, &x->r_words, &x->r_coef, &x->r_hmask, &x->den_tab, &x->r_part, &x->b_mask, &x->o_mask,
                 &x->b_ofs, &x->e_hp, &x->e_rec, &x->it_sum, &x->live, &x->queues, &x->tk_e, &x->tk_a, &x->tk_key, &x->tk_cnt, &x->tk_tau, &x->sel_hist, &x->gen_list, &x->gen_out, &x->cand_e, &x->cand_a, &x->cand_key, &x->skey,
                 &x->skey2, &x->perm, &x->perm2, &x->cub_tmp2, &x->out_sel, &x->out_e, &x->out_num,
-                &x->out_eps, &x->out_na, &x->out_ncon, &x->out_rank, &x->g_dh, &x->g_deri, &x->g_wF, &x->g_wH};
+                &x->out_eps, &x->out_na, &x->out_ncon, &x->out_rank, &x->g_dh, &x->g_deri, &x->g_wF, &x->g_wH, &x->dv_ws};
   for (Buf* b : all) b->release();
   delete x;
 }
