@@ -9,6 +9,10 @@ struct qp_pt2_ctx;
 namespace qp {
 
 constexpr int kMaxOrb = 128;
+// bits of a sweep's error word (16 and 32: the no-allocation entry point's
+// symmetry check, the selection's candidate space; 64: coefficients times
+// integrals beyond the exact accumulator's range)
+enum : int { kErrOcc = 1, kErrDup = 2, kErrCoef = 4, kErrBucket = 8, kErrRange = 64, kErrTimeout = 128 };
 constexpr int kMaxElec = 64;   // per determinant (both spins); hole masks are uint64
 constexpr int kMaxBatch = kMaxElec + kMaxElec * (kMaxElec - 1) / 2;
 constexpr int kSelBins = 1024;  // |e| histogram: 128 binary exponents (2^-100 .. 2^27) x 8 sub-bins

@@ -61,12 +61,6 @@ static int fail(int code, const std::string& msg) {
                   std::string(#expr) + ": " + cudaGetErrorString(e_));                     \
   } while (0)
 
-// device error flags
-// (16 and 32: the no-allocation entry point's symmetry check, the selection's
-// candidate space; 64: coefficients times integrals beyond the exact
-// accumulator's range)
-enum : int { kErrOcc = 1, kErrDup = 2, kErrCoef = 4, kErrBucket = 8, kErrRange = 64, kErrTimeout = 128 };
-
 // device memory allowed for the per-generator records and buckets of a wave
 static const size_t kWaveBudget = (size_t)4 << 30;
 

@@ -475,7 +475,10 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   for (int j = tid; j < p.nper * p.it_stride; j += kThreads) p.it_sum[(size_t)slot * p.nper * p.it_stride + j] = 0.0;
   const long long t = (long long)p.wave_start + slot;
   const long long gg = p.gen_list ? (long long)p.gen_list[t] : p.shard_index + t * (long long)p.shard_count;
-  if (gg >= p.ndet) {
+  // determinants of unequal electron counts (a batch's graph runs on after
+  // the check has flagged them): no work, as the particle lists below are
+  // taken to be as long as the hole lists
+  if (gg >= p.ndet || (*p.err & kErrOcc)) {
     if (tid == 0) {
       M->g = -1;
       M->nrec = 0;
