@@ -357,34 +357,55 @@ __device__ __forceinline__ int part_code(uint64_t part, int i) { return (int)((p
 // d = 3: list J with its i-th hole.
 constexpr uint64_t kKeep0 = 1ull << 31, kKeep1 = 1ull << 47, kKeep2 = 1ull << 63;
 
-// Buckets of a record with hole mask hm and particle word pt (see prep_slot);
-// dead: bits of the batches banned as a whole, whose buckets nothing reads.
+// Buckets of a record of degree 3 at most with hole mask hm and particle word
+// pt (see prep_slot); dead: bits of the batches banned as a whole, whose
+// buckets nothing reads.
 template <typename Fn>
 __device__ __forceinline__ void for_buckets(uint64_t hm, uint64_t pt, int nel, int nbat, const uint32_t* dead,
                                             Fn&& fn) {
   const int d = __popcll(hm);
   const bool before = pt & kBeforeBit;
-  int Q[4], n = 0;
+  int Q[3], n = 0;
   uint64_t m = hm;
-  while (m && n < 4) {
+  while (m && n < 3) {
     Q[n++] = __ffsll((long long)m) - 1;
     m &= m - 1;
   }
   if (before && d <= 2) return;  // in the masks as a whole
   if (d == 0 || (d <= 2 && (pt & kKeep0))) fn(nbat);
-  if (!before && d <= 3) {
+  if (!before) {
 #pragma unroll
     for (int i = 0; i < 3; i++)
       if (i < d && (d < 3 || (pt & (kKeep0 << (16 * i))))) fn(Q[i]);
   }
 #pragma unroll
-  for (int i = 0; i < 4; i++)
+  for (int i = 0; i < 3; i++)
 #pragma unroll
-    for (int j = i + 1; j < 4; j++) {
+    for (int j = i + 1; j < 3; j++) {
       if (j >= d) continue;
       const int b = pair_batch(nel, Q[i], Q[j]);
       if (!((dead[b >> 5] >> (b & 31)) & 1u)) fn(b);
     }
+}
+
+// Buckets of a record of degree 4: the six pairs of its holes.
+template <typename Fn>
+__device__ __forceinline__ void for_pairs4(uint64_t hm, int nel, const uint32_t* dead, Fn&& fn) {
+  int Q[4];
+#pragma unroll
+  for (int i = 0; i < 4; i++) {
+    Q[i] = __ffsll((long long)hm) - 1;
+    hm &= hm - 1;
+  }
+#pragma unroll
+  for (int j = 1; j < 4; j++) {
+    const int row = nel + Q[j] * (Q[j] - 1) / 2;
+#pragma unroll
+    for (int i = 0; i < j; i++) {
+      const int b = row + Q[i];
+      if (!((dead[b >> 5] >> (b & 31)) & 1u)) fn(b);
+    }
+  }
 }
 
 struct Batch {
@@ -459,11 +480,12 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   constexpr int NW = 2 * NINT;
   __shared__ int s_cnt[kMaxBatch + 2];
   __shared__ uint32_t s_dead[(kMaxBatch + 31) / 32];
-  __shared__ int s_wsum[kWarps];
   __shared__ uint64_t sI[NW];
   __shared__ int s_occ[kMaxElec];
   __shared__ unsigned char s_vidx[2][kMaxOrb];
   __shared__ double s_F[2 * kMaxOrb];
+  __shared__ int s_nrec[2];    // records of degree 3 at most, of degree 4
+  __shared__ int s_below[NW];  // I's electrons in the words before
   extern __shared__ __align__(16) unsigned char dyn[];
   uint32_t* sm = reinterpret_cast<uint32_t*>(dyn);               // cell masks (MaskDims)
   uint64_t* so = reinterpret_cast<uint64_t*>(sm + p.mask_w);     // orbital masks (orb_mask_words)
@@ -495,7 +517,13 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
         if ((sI[s * NINT + (q >> 6)] >> (q & 63)) & 1ull) s_occ[n++] = s * norb + q;
     M->g = g;
     M->cI = p.coefs[gi];
-    for (int w = 0; w < 4; w++) M->I[w] = w < NW ? sI[w] : 0ull;
+    for (int w = 0, below = 0; w < 4; w++) {
+      M->I[w] = w < NW ? sI[w] : 0ull;
+      if (w >= NW) continue;
+      s_below[w] = below;
+      below += __popcll(sI[w]);
+    }
+    s_nrec[0] = s_nrec[1] = 0;
   }
   __syncthreads();
   if (tid < nel) M->occ[tid] = s_occ[tid];
@@ -528,7 +556,11 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
     M->hii = den_fix(0.5 * e, S);
   }
 
-  // ---- coarse filter: J within degree 4 of I (I itself included) ----
+  // ---- coarse filter: J within degree 4 of I (I itself included): those of
+  // degree 4, most of a large space, from the back of the slot's arrays, the
+  // others from the front, so that the passes below do not run the branches
+  // of one kind with a few lanes of it in every warp (10^4 determinants, 64
+  // orbitals: prep 7.5 -> 5.9 ms, the sweep 81.1 -> 79.5 ms) ----
   const size_t rb = (size_t)slot * (size_t)p.ndet;
   uint64_t* rw = p.r_words + rb * NW;
   double* rc = p.r_coef + rb;
@@ -537,59 +569,76 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   uint64_t Iw[NW];
 #pragma unroll
   for (int w = 0; w < NW; w++) Iw[w] = sI[w];
-  int nrec = 0;
-  for (long long base = 0; base < p.ndet; base += kThreads) {
-    const long long j = base + tid;
-    bool keep = false;
+  const int lane = tid & 31;
+  for (long long base = tid - lane; base < p.ndet; base += kThreads) {
+    const long long j = base + lane;
+    int d = 9;  // degree
     uint64_t Jw[NW];
     if (j < p.ndet) {
-      int d = 0;
+      int x = 0;
 #pragma unroll
       for (int w = 0; w < NW; w++) {
         Jw[w] = p.dets[(size_t)j * NW + w];
-        d += __popcll(Jw[w] ^ Iw[w]);
+        x += __popcll(Jw[w] ^ Iw[w]);
       }
-      keep = d <= 8;
+      d = x >> 1;
     }
-    int total;
-    const int pos = block_scan_flag(keep, s_wsum, &total);
-    if (keep) {
-      const int r = nrec + pos;
+    const unsigned b3 = __ballot_sync(kFull, d <= 3), b4 = __ballot_sync(kFull, d == 4);
+    if (!(b3 | b4)) continue;
+    int at = 0;
+    if (lane < 2) at = atomicAdd(&s_nrec[lane], __popc(lane ? b4 : b3));
+    const int at3 = __shfl_sync(kFull, at, 0), at4 = __shfl_sync(kFull, at, 1);
+    if (d <= 4) {
+      const unsigned before = (1u << lane) - 1u;
+      const size_t r = d == 4 ? (size_t)p.ndet - 1 - (size_t)(at4 + __popc(b4 & before)) : (size_t)(at3 + __popc(b3 & before));
       uint64_t hmask = 0, part = 0x7FFF7FFF7FFF7FFFull;  // four unused fields (kNoPart)
-      int npart = 0;
+      uint64_t miss[NW], extra[NW];
 #pragma unroll
-      for (int s = 0; s < 2; s++) {
-        int below = (s == 0) ? 0 : p.nalpha;
+      for (int w = 0; w < NW; w++) {
+        miss[w] = Iw[w] & ~Jw[w];
+        extra[w] = Jw[w] & ~Iw[w];
+      }
 #pragma unroll
-        for (int w = 0; w < NINT; w++) {
-          const uint64_t iw = Iw[s * NINT + w], jw = Jw[s * NINT + w];
-          uint64_t miss = iw & ~jw;
-          while (miss) {
-            const int b = __ffsll((long long)miss) - 1;
-            miss &= miss - 1;
-            hmask |= 1ull << (below + __popcll(iw & ((1ull << b) - 1)));
+      for (int k = 0; k < 4; k++) {  // the k-th hole and particle, spin up first
+        if (k >= d) break;
+        uint64_t m = miss[NW - 1], iw = Iw[NW - 1], e = extra[NW - 1];
+        int hb = s_below[NW - 1], eb = norb + 64 * (NINT - 1);
+#pragma unroll
+        for (int w = NW - 2; w >= 0; w--) {
+          if (miss[w]) {
+            m = miss[w];
+            iw = Iw[w];
+            hb = s_below[w];
           }
-          uint64_t extra = jw & ~iw;
-          while (extra) {
-            const int b = __ffsll((long long)extra) - 1;
-            extra &= extra - 1;
-            const uint64_t code = (uint64_t)(s * norb + 64 * w + b);
-            if (npart < 4) part = (part & ~(0xFFFFull << (16 * npart))) | (code << (16 * npart));
-            npart++;
+          if (extra[w]) {
+            e = extra[w];
+            eb = (w / NINT) * norb + 64 * (w % NINT);
           }
-          below += __popcll(iw);
+        }
+        const uint64_t low = m & (0ull - m), elow = e & (0ull - e);
+        hmask |= 1ull << (hb + __popcll(iw & (low - 1)));
+        part ^= (uint64_t)(kNoPart ^ (eb + __popcll(elow - 1))) << (16 * k);
+        bool mdone = false, edone = false;
+#pragma unroll
+        for (int w = 0; w < NW; w++) {  // clear the bits taken, in the first words that have any
+          if (!mdone && miss[w]) {
+            miss[w] &= miss[w] - 1;
+            mdone = true;
+          }
+          if (!edone && extra[w]) {
+            extra[w] &= extra[w] - 1;
+            edone = true;
+          }
         }
       }
 #pragma unroll
-      for (int w = 0; w < NW; w++) rw[(size_t)r * NW + w] = Jw[w];
+      for (int w = 0; w < NW; w++) rw[r * NW + w] = Jw[w];
       rc[r] = p.coefs[j];
       for (int st = 1; st < p.nst; st++) rc[st * p.rc_stride + r] = p.coefs[(size_t)st * p.ndet + j];
       rh[r] = hmask;
       rp[r] = part | (p.rank_of[j] < g ? kBeforeBit : 0ull);
     }
-    nrec += total;
   }
-  if (tid == 0) M->nrec = nrec;
 
   // ---- bans by J ranked before I, once per generator.  With Q the holes of
   // J, P its particles and H the holes of a batch, t = |Q - H|:
@@ -628,6 +677,9 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
     s_vidx[s][q] = (unsigned char)(q - below);
   }
   __syncthreads();
+  const int nlow = s_nrec[0], nfour = s_nrec[1];
+  const size_t r4 = (size_t)p.ndet - nfour;  // first record of degree 4
+  if (tid == 0) M->nrec = nlow + nfour;
   // cell of two particles: 0, 1 same spin, 2 opposite; its index in the batch
   auto pair_of = [&](int c0, int c1, int* idx) {
     const int s0 = c0 >= norb, s1 = c1 >= norb;
@@ -654,7 +706,7 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   auto hole_row = [&](int q) { return so + (4 + 3 * q) * NINT; };
   auto hole_one = [&](int q) { return so + (6 + 3 * q) * NINT; };
   auto hole_mask = [&](int q) { return sm + mbase + q * md.hs; };
-  for (int r = tid; r < nrec; r += kThreads) {
+  for (int r = tid; r < nlow; r += kThreads) {
     const uint64_t pt = rp[r], hm = rh[r];
     if (!(pt & kBeforeBit)) continue;
     const int d = __popcll(hm);
@@ -718,7 +770,7 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
 
   // ---- buckets: counting sort of the entries left into the shared list,
   // one list per hole and one bucket per pair of holes ----
-  for (int r = tid; r < nrec; r += kThreads) {
+  for (int r = tid; r < nlow; r += kThreads) {
     const uint64_t hm = rh[r];
     uint64_t pt = rp[r];
     const int d = __popcll(hm);
@@ -762,6 +814,8 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
     }
     for_buckets(hm, pt, nel, nbat, s_dead, [&](int b) { atomicAdd(&s_cnt[b], 1); });
   }
+  for (int r = tid; r < nfour; r += kThreads)
+    for_pairs4(rh[r4 + r], nel, s_dead, [&](int b) { atomicAdd(&s_cnt[b], 1); });
   __syncthreads();
   if (tid < 32) {  // exclusive scan of the counts
     int run = 0;
@@ -793,17 +847,23 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   ulonglong2* e_hp = p.e_hp + (size_t)slot * (size_t)p.ent_cap;
   uint32_t* e_rec = p.e_rec + (size_t)slot * (size_t)p.ent_cap;
   const long long cap = p.ent_cap;
-  for (int r = tid; r < nrec; r += kThreads) {
-    const uint64_t hm = rh[r], pt = rp[r];
-    const uint64_t pe = pt & ~(kKeep0 | kKeep1 | kKeep2);
+  auto put = [&](int b, uint64_t hm, uint64_t pe, uint32_t rec) {
+    const int o = atomicAdd(&s_cnt[b], 1);
+    if (o < cap) {
+      e_hp[o] = make_ulonglong2(hm, pe);
+      e_rec[o] = rec;
+    }
+  };
+  for (int r = tid; r < nlow; r += kThreads) {
+    const uint64_t hm = rh[r], pt = rp[r], pe = pt & ~(kKeep0 | kKeep1 | kKeep2);
     const uint32_t rec = (uint32_t)r | (pt & kBeforeBit ? 1u << 31 : 0u);
-    for_buckets(hm, pt, nel, nbat, s_dead, [&](int b) {
-      const int o = atomicAdd(&s_cnt[b], 1);
-      if (o < cap) {
-        e_hp[o] = make_ulonglong2(hm, pe);
-        e_rec[o] = rec;
-      }
-    });
+    for_buckets(hm, pt, nel, nbat, s_dead, [&](int b) { put(b, hm, pe, rec); });
+  }
+  for (int i = tid; i < nfour; i += kThreads) {
+    const size_t r = r4 + i;
+    const uint64_t hm = rh[r], pt = rp[r];
+    const uint32_t rec = (uint32_t)r | (pt & kBeforeBit ? 1u << 31 : 0u);
+    for_pairs4(hm, nel, s_dead, [&](int b) { put(b, hm, pt, rec); });
   }
 }
 
