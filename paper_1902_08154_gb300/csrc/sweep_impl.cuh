@@ -46,6 +46,7 @@
 #pragma once
 #include <cfloat>
 #include <cstdio>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -978,18 +979,10 @@ struct BatchShared {
   // a group of J reaching every cell, J = K + {x1, x2}: per particle orbital
   // of each slot the offset of its integrals, with the phase parity in bit 31
   // and, for the particles of J, bit 30 (row) or 29 (column), so that a cell's
-  // offset, sign and flags are one sum (the gradient's per-orbital weights use
-  // the same storage in the cells pass and after loop 3)
+  // offset, sign and flags are one sum
   NT gcj[kGroup];
-  int gx2[kGroup], gB[kGroup];
-  union {
-    struct {
-      int gRow[kGroup][kMaxOrb], gCol[kGroup][kMaxOrb];
-    } g;
-    struct {
-      double rowW2[kMaxOrb], colW2[kMaxOrb];  // sums of (A/D)^2 over the cells of each particle orbital
-    } w;
-  } v;
+  int gx1[kGroup], gx2[kGroup], gB[kGroup];
+  int gRow[kGroup][kMaxOrb], gCol[kGroup][kMaxOrb];
   int wsum[kWarps];
   // selection
   int tkcnt;
@@ -1847,6 +1840,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     const int gB = (x1 * norb + x2) * norb * norb;
     if (lane == 0) {
       S.gcj[j] = (NT)S.rc[r];
+      S.gx1[j] = x1;
       S.gx2[j] = x2;
       S.gB[j] = gB;
       if constexpr (MS)
@@ -1865,13 +1859,13 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     for (int v = lane; v < S.nv[sr]; v += 32) {
       const int q = S.vir[sr][v];
       const int ex = q == x1 || (B.kind == 1 && q == x2) ? 1 << 30 : 0;
-      S.v.g.gRow[j][v] = (E4 ? gB + q * norb : tri(x1, q)) | ex | ((int)mask_bit<NINT>(M1, q) << 31);
+      S.gRow[j][v] = (E4 ? gB + q * norb : tri(x1, q)) | ex | ((int)mask_bit<NINT>(M1, q) << 31);
     }
 #pragma unroll 1
     for (int v = lane; v < S.nv[sc]; v += 32) {
       const int q = S.vir[sc][v];
       const int ex = q == x2 || (B.kind == 1 && q == x1) ? 1 << 29 : 0;
-      S.v.g.gCol[j][v] = (E4 ? q : tri(x2, q)) | ex | ((int)mask_bit<NINT>(M2, q) << 31);
+      S.gCol[j][v] = (E4 ? q : tri(x2, q)) | ex | ((int)mask_bit<NINT>(M2, q) << 31);
     }
   };
 
@@ -1890,6 +1884,405 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     if (lane == 0) S.red_con[warp] += wcon;
     con = 0;
   };
+  // The J of a round but for the tables' terms, drawn by the warps as they free
+  // up (G: the gradient's scatter of the same terms): the rows of J
+  // reaching every cell (a two-hole batch: the cells touching their
+  // particles; a one-hole batch: all cells), J reaching rows, and J reaching
+  // a few cells (one lane each, 32 per draw).
+  //
+  // Along a row everything but the cell's orbital z is fixed: the element of
+  // a double substitution is one or two integrals at base + z (consecutive
+  // lanes on consecutive entries) with a sign from a phase mask of J's
+  // string.  A warp draws up to eight row J and sets up their rows side by
+  // side, a lane per (J, particle).  The few cells holding two particles of
+  // such a J (one, in a one-hole batch) are single substitutions of J; their
+  // sum over J's orbitals is spread over the lanes.  A row of a J reaching
+  // every cell holds single substitutions only: a unit of work is 32 of its
+  // cells, each lane summing over J's orbitals, four at a time in flight.
+  // (Each cell through the general element routine, a warp per J, took 8,000
+  // cycles of a warp per J: two masked popcounts per cell, and a lane's chain
+  // of 30 dependent loads wherever a row met a single substitution.)
+  auto row_pass = [&](auto gp) {
+    constexpr bool G = decltype(gp)::value;
+    const int n0 = S.n0, nrow = S.n1, n2 = S.n2;
+    const int ntab = B.h == 2 ? (n0 < kGroup ? n0 : kGroup) : 0;
+    const int nvm = S.nv[0] > S.nv[1] ? S.nv[0] : S.nv[1], nch = (nvm + 31) / 32;
+    // units: pair tables, rows of the J reaching every cell (J, particle slot,
+    // 32 cells), row J, the rest
+    const int nall = ntab + n0 * B.h * nch;
+    int per = (nrow + kWarps - 1) / kWarps;
+    per = per > 8 ? 8 : per;
+    const int ndraw = nall + (per ? (nrow + per - 1) / per : 0);
+    // c_J v into cell cc
+    auto add = [&](int cc, NT v, int rj, NT cjj) {
+      if constexpr (MS) {
+#pragma unroll
+        for (int st = 0; st < kMaxStates; st++)
+          if (st < nst) atomicAdd(&A[st * mc + cc], S.rc[st * p.rc_stride + rj] * (double)v);
+      } else {
+        unsigned long long l;
+        int hh;
+        fix_of(cjj * v, F, l, hh);
+        fix_atomic_add(A0, A1, A2, cc, l, hh);
+      }
+      con++;
+    };
+    auto live = [&](int cc) { return (unsigned)cc < (unsigned)B.nct && !((ban[cc >> 5] >> (cc & 31)) & 1u); };
+    for (;;) {
+      int jd = 0;
+      if (lane == 0) jd = atomicAdd(&S.cnext, 1);
+      jd = __shfl_sync(kFull, jd, 0);
+      if (jd < ntab) {
+        build_table(jd, S.u.l.L0[jd]);
+      } else if (jd < nall) {
+        const int ju = jd - ntab, j = ju / (B.h * nch), rem = ju - j * (B.h * nch), ip = rem / nch, y = (rem - ip * nch) * 32 + lane;
+        const int r = S.u.l.L0[j];
+        const uint64_t hm = S.rhm[r], part = S.rpt[r];
+        uint32_t X, T;
+        int nx, nt;
+        excitation_sets<NINT, NT>(B, S, part, hm, &X, &nx, &T, &nt);
+        // row of particle ip; the hole u of the substitutions u -> z is the
+        // other entry of X (one-hole batch: the only entry)
+        const int code = B.h == 2 ? part_code(part, ip) : -1;
+        if (code == kNoPart) continue;
+        const int s = code >= norb, x = code >= 0 ? S.vidx[s][code - s * norb] : 0;
+        if (B.kind == 1 && s != B.sa) continue;
+        const int sz = B.kind == 2 ? 1 - s : B.sa;
+        if (B.h == 2 && row_banned<NINT, NT>(S, s, code - s * norb)) continue;
+        const int x0 = pk(X, 0), uz = (x0 == code ? pk(X, 1) : x0) - sz * norb;
+        uint64_t wz[NINT], M[NINT];
+#pragma unroll
+        for (int w = 0; w < NINT; w++) wz[w] = S.rw[(size_t)r * NW + sz * NINT + w];
+        phase_mask<NINT>(wz, uz, 0, M);
+        if (y >= S.nv[sz]) continue;
+        const int z = S.vir[sz][y];
+        const int cc = (B.kind == 0 ? y : B.kind == 1 ? pair_cell(x, y) : (s ? y * S.nv[1] + x : x * S.nv[1] + y)) - B.clo;
+        // z a particle of J: that cell is J itself (banned)
+        if (mask_bit<NINT>(wz, z) || (B.kind == 1 && x == y) || !live(cc)) continue;
+        if constexpr (G) {
+          const double ws = flip_sign(S.rc[r] * a2d(cc), mask_bit<NINT>(M, z));
+          atomicAdd(&p.g_dh[uz * norb + z], 0.5 * ws);
+          atomicAdd(&p.g_dh[z * norb + uz], 0.5 * ws);
+#pragma unroll 1
+          for (int w = 0; w < NW; w++) {
+            const bool sp = w / NINT == sz;
+#pragma unroll 1
+            for (uint64_t bits = S.rw[(size_t)r * NW + w]; bits; bits &= bits - 1) {
+              const int o = 64 * (w % NINT) + __ffsll((long long)bits) - 1;
+              atomicAdd(&p.g_deri[eri_index(o, o, uz, z)], ws);
+              if (sp) atomicAdd(&p.g_deri[eri_index(uz, o, o, z)], -ws);
+            }
+          }
+          continue;
+        }
+        NT v = h_n[uz * norb + z];
+        // J's orbitals in ascending order (the FP32 form's sum depends on
+        // it), four at a time so that their loads overlap
+#pragma unroll 1
+        for (int w = 0; w < NW; w++) {
+          uint64_t bits = S.rw[(size_t)r * NW + w];
+          const bool sp = w / NINT == sz;
+#pragma unroll 1
+          while (bits) {
+            int o[4];
+            NT a[4], b[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+              o[i] = bits ? 64 * (w % NINT) + __ffsll((long long)bits) - 1 : -1;
+              bits &= bits - 1;
+              if (o[i] < 0) continue;
+              a[i] = eri_n[gidx<E4>(o[i], o[i], uz, z, norb)];
+              if (sp) b[i] = eri_n[gidx<E4>(uz, o[i], o[i], z, norb)];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+              if (o[i] < 0) continue;
+              v += a[i];
+              if (sp) v -= b[i];
+            }
+          }
+        }
+        add(cc, flip_sign(v, mask_bit<NINT>(M, z)), r, (NT)S.rc[r]);
+      } else if (jd < ndraw) {
+        const int jl = (jd - nall) * per + (lane >> 2), ip = lane & 3;
+        const bool have = (lane >> 2) < per && jl < nrow;
+        int r = 0;
+        NT cj = NT(0);
+        uint64_t part = 0x7FFF7FFF7FFF7FFFull, hm = 0;
+        uint64_t M[NINT];         // phase of the row's substitution by z
+        uint64_t EX[NINT];        // particles of J with the spin of z
+        // orbitals: uz (hole paired with z) | uo (hole paired with q) << 8 |
+        // q << 16 | same spin << 24
+        uint32_t iw = 0;
+        int geo = 0;              // virtual index of the row's particle, its spin << 8
+        bool act = false;
+        // the single substitution of the pair of particles ip: cell and
+        // sign << 31, hole w | q << 8 | spin << 16
+        bool sact = false;
+        uint32_t scell = 0, sw = 0;
+#pragma unroll
+        for (int w = 0; w < NINT; w++) M[w] = EX[w] = 0;
+        if (have) {
+          r = S.u.l.L12[jl];
+          part = S.rpt[r];
+          hm = S.rhm[r];
+          cj = (NT)S.rc[r];
+          uint32_t X, T;
+          int nx, nt;
+          excitation_sets<NINT, NT>(B, S, part, hm, &X, &nx, &T, &nt);
+          const int q = pk(T, 0), sq = q >= norb ? 1 : 0, qo = q - sq * norb;
+          uint64_t Jw[NW];
+#pragma unroll
+          for (int w = 0; w < NW; w++) Jw[w] = S.rw[(size_t)r * NW + w];
+          // the row's particle (a one-hole batch has one row per J and no
+          // fixed particle)
+          const int code = B.h == 2 ? part_code(part, ip) : (ip == 0 ? -1 : kNoPart);
+          if (code != kNoPart) {
+            const int s = code >= norb, x = code >= 0 ? S.vidx[s][code - s * norb] : 0;
+            const int sz = B.kind == 2 ? 1 - s : B.sa;
+            act = B.h == 1 || ((B.kind == 2 || s == B.sa) && !row_banned<NINT, NT>(S, s, code - s * norb));
+            geo = x | (s << 8);
+            int u0 = -1, u1 = -1;  // X without the row's particle
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+              if (i >= nx) break;
+              const int xc = pk(X, i);
+              if (xc != code) {
+                if (u0 < 0) u0 = xc;
+                else u1 = xc;
+              }
+            }
+            const bool same = (u0 >= norb) == (u1 >= norb);
+            const bool second = same || (u1 >= norb) == (sz != 0);
+            const int uz = second ? u1 : u0, uo = second ? u0 : u1;
+            const int so = uo >= norb, zo = uz - sz * norb, oo = uo - so * norb;
+            uint64_t wo[NINT], wz[NINT];
+#pragma unroll
+            for (int w = 0; w < NINT; w++) {
+              wo[w] = so ? Jw[NINT + w] : Jw[w];
+              wz[w] = sz ? Jw[NINT + w] : Jw[w];
+              if (same) {
+                if ((oo >> 6) == w) wz[w] &= ~(1ull << (oo & 63));
+                if ((qo >> 6) == w) wz[w] |= 1ull << (qo & 63);
+              }
+            }
+            const int c = count_between<NINT>(wo, oo < qo ? oo : qo, oo < qo ? qo : oo) & 1;
+            phase_mask<NINT>(wz, zo, c, M);
+            iw = (uint32_t)zo | ((uint32_t)oo << 8) | ((uint32_t)qo << 16) | ((uint32_t)same << 24);
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+              const int pc = part_code(part, i);
+              if (pc == kNoPart || (pc >= norb) != (sz != 0)) continue;
+              const int po = pc - sz * norb;
+#pragma unroll
+              for (int w = 0; w < NINT; w++)
+                if ((po >> 6) == w) EX[w] |= 1ull << (po & 63);
+            }
+          }
+          if (ip < 3) {  // two-hole batch: pairs (0, 1), (0, 2), (1, 2) of J's particles; one-hole: its particles
+            const int c0_ = part_code(part, B.h == 2 && ip == 2 ? 1 : (B.h == 2 ? 0 : ip));
+            const int c1_ = B.h == 2 ? part_code(part, ip == 0 ? 1 : 2) : -1;
+            if (c0_ != kNoPart && c1_ != kNoPart) {
+              const int sx = c0_ >= norb, sy = c1_ >= norb;
+              if (B.kind == 2 ? sx != sy : (sx == B.sa && (c1_ < 0 || sy == B.sa))) {
+                const int vx = S.vidx[sx][c0_ - sx * norb], vy = c1_ < 0 ? 0 : S.vidx[sy][c1_ - sy * norb];
+                const int cc = (B.kind == 0 ? vx : B.kind == 1 ? pair_cell(vx, vy) : (sx ? vy * S.nv[1] + vx : vx * S.nv[1] + vy)) - B.clo;
+                if (live(cc)) {
+                  int w = 0;  // X without the cell's particles: the hole, with q's spin
+#pragma unroll
+                  for (int i = 0; i < 3; i++) {
+                    const int xc = pk(X, i);
+                    if (i < nx && xc != c0_ && xc != c1_) w = xc;
+                  }
+                  const int wo = w - sq * norb;
+                  uint64_t ws[NINT];
+#pragma unroll
+                  for (int i = 0; i < NINT; i++) ws[i] = sq ? Jw[NINT + i] : Jw[i];
+                  const int neg = count_between<NINT>(ws, wo < qo ? wo : qo, wo < qo ? qo : wo) & 1;
+                  sact = true;
+                  scell = (uint32_t)cc | ((uint32_t)neg << 31);
+                  sw = (uint32_t)wo | ((uint32_t)qo << 8) | ((uint32_t)sq << 16);
+                }
+              }
+            }
+          }
+        }
+#pragma unroll 1
+        for (unsigned m = __ballot_sync(kFull, act); m; m &= m - 1) {
+          const int src = __ffs((int)m) - 1;
+          const uint32_t iwr = __shfl_sync(kFull, iw, src);
+          const int gr = __shfl_sync(kFull, geo, src), rj = __shfl_sync(kFull, r, src);
+          const NT cjr = __shfl_sync(kFull, cj, src);
+          uint64_t Mr[NINT], Er[NINT];
+          shfl_words<NINT>(M, src, Mr);
+          shfl_words<NINT>(EX, src, Er);
+          const int x = gr & 0xFF, s = gr >> 8, sz = B.kind == 2 ? 1 - s : B.sa;
+          const int uz = iwr & 0xFF, uo = (iwr >> 8) & 0xFF, q = (iwr >> 16) & 0xFF;
+          const bool same = (iwr >> 24) & 1u;
+          const int nz = S.nv[sz], nv1 = S.nv[1];
+          // the integrals at b1 + z and (same spin) b2 + z
+          const NT* e1 = eri_n + ((uo * norb + uz) * norb + q) * norb;
+          const NT* e2 = eri_n + ((uz * norb + uo) * norb + q) * norb;
+          // cell of z's index y: cb + y cs, or (same spin) a pair
+          const int cs = B.kind == 2 && s ? nv1 : 1;
+          const int cb = (B.kind == 2 ? (s ? x : x * nv1) : 0) - B.clo, xx = x * (x - 1) / 2;
+          if constexpr (G) {
+#pragma unroll 1
+            for (int y = lane; y < nz; y += 32) {
+              const int z = S.vir[sz][y];
+              const int cc = B.kind == 1 ? cb + (y > x ? y * (y - 1) / 2 + x : xx + y) : cb + y * cs;
+              if (mask_bit<NINT>(Er, z) || !live(cc)) continue;
+              const double ws = flip_sign(cjr * a2d(cc), mask_bit<NINT>(Mr, z));
+              atomicAdd(&p.g_deri[eri_index(uo, q, uz, z)], ws);
+              if (same) atomicAdd(&p.g_deri[eri_index(uz, q, uo, z)], -ws);
+            }
+            continue;
+          }
+          // two rounds of 32 cells at a time, their loads in flight together
+#pragma unroll 1
+          for (int y0 = lane; y0 < nz; y0 += 64) {
+            int ca = -1, cn = -1;
+            NT va = NT(0), vn = NT(0);
+            auto fetch = [&](int y, int& c, NT& v) {
+              if (y >= nz) return;
+              const int z = S.vir[sz][y];
+              int cc = cb + y * cs;
+              if (B.kind == 1) cc = cb + (y > x ? y * (y - 1) / 2 + x : xx + y);
+              if (mask_bit<NINT>(Er, z) || !live(cc)) return;
+              c = cc;
+              if constexpr (E4) {
+                v = e1[z];
+                if (same) v -= e2[z];
+              } else {
+                v = eri_n[eri_index(uo, q, uz, z)];
+                if (same) v -= eri_n[eri_index(uz, q, uo, z)];
+              }
+              v = flip_sign(v, mask_bit<NINT>(Mr, z));
+            };
+            fetch(y0, ca, va);
+            fetch(y0 + 32, cn, vn);
+#pragma unroll 1
+            for (int i = 0; i < 2; i++) {
+              if (ca >= 0) add(ca, va, rj, cjr);
+              ca = cn;
+              va = vn;
+            }
+          }
+        }
+#pragma unroll 1
+        for (unsigned m = __ballot_sync(kFull, sact); m; m &= m - 1) {
+          const int src = __ffs((int)m) - 1;
+          const uint32_t sc = __shfl_sync(kFull, scell, src), wq = __shfl_sync(kFull, sw, src);
+          const int rj = __shfl_sync(kFull, r, src);
+          const NT cjr = __shfl_sync(kFull, cj, src);
+          const uint64_t hmr = __shfl_sync(kFull, hm, src), ptr_ = __shfl_sync(kFull, part, src);
+          const int wo = wq & 0xFF, qo = (wq >> 8) & 0xFF, sq = (wq >> 16) & 1;
+          if constexpr (G) {
+            const double ws = flip_sign(cjr * a2d((int)(sc & 0x7fffffffu)), (sc >> 31) != 0u);
+            if (lane < 2) atomicAdd(&p.g_dh[lane ? qo * norb + wo : wo * norb + qo], 0.5 * ws);
+#pragma unroll 1
+            for (int i = lane; i < nel; i += 32) {
+              int mo = S.occ[i];
+              if ((hmr >> i) & 1ull) mo = part_code(ptr_, __popcll(hmr & ((1ull << i) - 1)));
+              const int sm = mo >= norb, o = mo - sm * norb;
+              atomicAdd(&p.g_deri[eri_index(o, o, wo, qo)], ws);
+              if (sm == sq) atomicAdd(&p.g_deri[eri_index(wo, o, o, qo)], -ws);
+            }
+            continue;
+          }
+          NT v = NT(0);
+          if constexpr (sizeof(NT) == 8) {  // J's orbitals: I's, with particles in the place of its holes
+#pragma unroll 1
+            for (int i = lane; i < nel; i += 32) {
+              int mo = S.occ[i];
+              if ((hmr >> i) & 1ull) mo = part_code(ptr_, __popcll(hmr & ((1ull << i) - 1)));
+              const int sm = mo >= norb, o = mo - sm * norb;
+              v += eri_n[gidx<E4>(o, o, wo, qo, norb)];
+              if (sm == sq) v -= eri_n[gidx<E4>(wo, o, o, qo, norb)];
+            }
+            v = warp_sum_nt<NT>(v) + h_n[wo * norb + qo];
+          } else {
+            // FP32: the sum keeps the ascending order of J's orbitals (its
+            // rounding depends on it); the lanes load, one adds
+            v = h_n[wo * norb + qo];
+#pragma unroll
+            for (int w = 0; w < 2 * NW; w++) {
+              const int o = 32 * (w % (2 * NINT)) + lane;
+              const bool sp = w / (2 * NINT) == sq;
+              uint32_t bits = (uint32_t)(S.rw[(size_t)rj * NW + w / 2] >> (32 * (w & 1)));
+              NT a = NT(0), b = NT(0);
+              if ((bits >> lane) & 1u) {
+                a = eri_n[gidx<E4>(o, o, wo, qo, norb)];
+                if (sp) b = eri_n[gidx<E4>(wo, o, o, qo, norb)];
+              }
+              for (; bits; bits &= bits - 1) {
+                const int src2 = __ffs((int)bits) - 1;
+                v += __shfl_sync(kFull, a, src2);
+                const NT bb = __shfl_sync(kFull, b, src2);
+                if (sp) v -= bb;
+              }
+            }
+          }
+          if (lane == 0) add((int)(sc & 0x7fffffffu), flip_sign(v, (sc >> 31) != 0u), rj, cjr);
+        }
+      } else {
+        const int j0 = (jd - ndraw) * 32;
+        if (j0 >= n2) break;
+        const int j = j0 + lane;
+        if (j < n2) {
+          // cells inside J's particles: J -> alpha moves the other two
+          // entries of X to J's two holes outside the batch
+          const int r = S.u.l.L12[kChunk - 1 - j];
+          const uint64_t part = S.rpt[r];
+          uint32_t X, T;
+          int nx, nt;
+          excitation_sets<NINT, NT>(B, S, part, S.rhm[r], &X, &nx, &T, &nt);
+          const NT cj = (NT)S.rc[r];
+          uint64_t Jw[NW];
+#pragma unroll
+          for (int w = 0; w < NW; w++) Jw[w] = S.rw[(size_t)r * NW + w];
+#pragma unroll 1
+          for (int k = 0; k < (B.h == 2 ? 6 : 4); k++) {
+            // pairs (0, 1), (0, 2), (1, 2), (0, 3), (1, 3), (2, 3); one-hole batch: single particles
+            const int k1 = B.h == 1 ? k : (k >= 3 ? 3 : k >= 1 ? 2 : 1), k0 = B.h == 1 ? k : (k >= 3 ? k - 3 : k >= 1 ? k - 1 : 0);
+            const int e0 = part_code(part, k0), e1 = part_code(part, k1);
+            if (e0 == kNoPart || e1 == kNoPart) continue;
+            const int sx = e0 >= norb, sy = e1 >= norb;
+            if (B.kind == 2 ? sx == sy : (sx != B.sa || sy != B.sa)) continue;
+            const int vx = S.vidx[sx][e0 - sx * norb], vy = S.vidx[sy][e1 - sy * norb];
+            const int cc = (B.kind == 0 ? vx : B.kind == 1 ? pair_cell(vx, vy) : (sx ? vy * S.nv[1] + vx : vx * S.nv[1] + vy)) - B.clo;
+            if (!live(cc)) continue;
+            if constexpr (G) {
+              element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, e0, B.h == 2 ? e1 : -1, S.rc[r] * a2d(cc));
+              continue;
+            }
+            int u0 = -1, u1 = -1;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+              const int xc = pk(X, i);
+              if (i < nx && xc != e0 && xc != e1) {
+                if (u0 < 0) u0 = xc;
+                else u1 = xc;
+              }
+            }
+            const NT v = double_element<NINT, NT, E4>(eri_n, norb, Jw, u0 < u1 ? u0 : u1, u0 < u1 ? u1 : u0, pk(T, 0), pk(T, 1));
+            if constexpr (MS) {
+#pragma unroll
+              for (int st = 0; st < kMaxStates; st++)
+                if (st < nst) atomicAdd(&A[st * mc + cc], S.rc[st * p.rc_stride + r] * (double)v);
+            } else {
+              unsigned long long l;
+              int hh;
+              fix_of(cj * v, F, l, hh);
+              fix_atomic_add(A0, A1, A2, cc, l, hh);
+            }
+            con++;
+          }
+        }
+      }
+    }
+  };
+
 #pragma unroll 1
   for (int c0 = 0;; c0 += kChunk) {
     const int total = S.seg_s[3], c1 = min(c0 + kChunk, total);
@@ -1941,357 +2334,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       }
       if (tid == 0) S.nlist = base;
     }
-    // The rest of the J, drawn by the warps as they free up: the rows of J
-    // reaching every cell (a two-hole batch: the cells touching their
-    // particles; a one-hole batch: all cells), J reaching rows, and J reaching
-    // a few cells (one lane each, 32 per draw).
-    //
-    // Along a row everything but the cell's orbital z is fixed: the element of
-    // a double substitution is one or two integrals at base + z (consecutive
-    // lanes on consecutive entries) with a sign from a phase mask of J's
-    // string.  A warp draws up to eight row J and sets up their rows side by
-    // side, a lane per (J, particle).  The few cells holding two particles of
-    // such a J (one, in a one-hole batch) are single substitutions of J; their
-    // sum over J's orbitals is spread over the lanes.  A row of a J reaching
-    // every cell holds single substitutions only: a unit of work is 32 of its
-    // cells, each lane summing over J's orbitals, four at a time in flight.
-    // (Each cell through the general element routine, a warp per J, took 8,000
-    // cycles of a warp per J: two masked popcounts per cell, and a lane's chain
-    // of 30 dependent loads wherever a row met a single substitution.)
-    {
-      const int nrow = S.n1, n2 = S.n2;
-      const int ntab = B.h == 2 ? (n0 < kGroup ? n0 : kGroup) : 0;
-      const int nvm = S.nv[0] > S.nv[1] ? S.nv[0] : S.nv[1], nch = (nvm + 31) / 32;
-      // units: pair tables, rows of the J reaching every cell (J, particle slot,
-      // 32 cells), row J, the rest
-      const int nall = ntab + n0 * B.h * nch;
-      int per = (nrow + kWarps - 1) / kWarps;
-      per = per > 8 ? 8 : per;
-      const int ndraw = nall + (per ? (nrow + per - 1) / per : 0);
-      // c_J v into cell cc
-      auto add = [&](int cc, NT v, int rj, NT cjj) {
-        if constexpr (MS) {
-#pragma unroll
-          for (int st = 0; st < kMaxStates; st++)
-            if (st < nst) atomicAdd(&A[st * mc + cc], S.rc[st * p.rc_stride + rj] * (double)v);
-        } else {
-          unsigned long long l;
-          int hh;
-          fix_of(cjj * v, F, l, hh);
-          fix_atomic_add(A0, A1, A2, cc, l, hh);
-        }
-        con++;
-      };
-      auto live = [&](int cc) { return (unsigned)cc < (unsigned)B.nct && !((ban[cc >> 5] >> (cc & 31)) & 1u); };
-      for (;;) {
-        int jd = 0;
-        if (lane == 0) jd = atomicAdd(&S.cnext, 1);
-        jd = __shfl_sync(kFull, jd, 0);
-        if (jd < ntab) {
-          build_table(jd, S.u.l.L0[jd]);
-        } else if (jd < nall) {
-          const int ju = jd - ntab, j = ju / (B.h * nch), rem = ju - j * (B.h * nch), ip = rem / nch, y = (rem - ip * nch) * 32 + lane;
-          const int r = S.u.l.L0[j];
-          const uint64_t hm = S.rhm[r], part = S.rpt[r];
-          uint32_t X, T;
-          int nx, nt;
-          excitation_sets<NINT, NT>(B, S, part, hm, &X, &nx, &T, &nt);
-          // row of particle ip; the hole u of the substitutions u -> z is the
-          // other entry of X (one-hole batch: the only entry)
-          const int code = B.h == 2 ? part_code(part, ip) : -1;
-          if (code == kNoPart) continue;
-          const int s = code >= norb, x = code >= 0 ? S.vidx[s][code - s * norb] : 0;
-          if (B.kind == 1 && s != B.sa) continue;
-          const int sz = B.kind == 2 ? 1 - s : B.sa;
-          if (B.h == 2 && row_banned<NINT, NT>(S, s, code - s * norb)) continue;
-          const int x0 = pk(X, 0), uz = (x0 == code ? pk(X, 1) : x0) - sz * norb;
-          uint64_t wz[NINT], M[NINT];
-#pragma unroll
-          for (int w = 0; w < NINT; w++) wz[w] = S.rw[(size_t)r * NW + sz * NINT + w];
-          phase_mask<NINT>(wz, uz, 0, M);
-          if (y >= S.nv[sz]) continue;
-          const int z = S.vir[sz][y];
-          const int cc = (B.kind == 0 ? y : B.kind == 1 ? pair_cell(x, y) : (s ? y * S.nv[1] + x : x * S.nv[1] + y)) - B.clo;
-          // z a particle of J: that cell is J itself (banned)
-          if (mask_bit<NINT>(wz, z) || (B.kind == 1 && x == y) || !live(cc)) continue;
-          NT v = h_n[uz * norb + z];
-          // J's orbitals in ascending order (the FP32 form's sum depends on
-          // it), four at a time so that their loads overlap
-#pragma unroll 1
-          for (int w = 0; w < NW; w++) {
-            uint64_t bits = S.rw[(size_t)r * NW + w];
-            const bool sp = w / NINT == sz;
-#pragma unroll 1
-            while (bits) {
-              int o[4];
-              NT a[4], b[4];
-#pragma unroll
-              for (int i = 0; i < 4; i++) {
-                o[i] = bits ? 64 * (w % NINT) + __ffsll((long long)bits) - 1 : -1;
-                bits &= bits - 1;
-                if (o[i] < 0) continue;
-                a[i] = eri_n[gidx<E4>(o[i], o[i], uz, z, norb)];
-                if (sp) b[i] = eri_n[gidx<E4>(uz, o[i], o[i], z, norb)];
-              }
-#pragma unroll
-              for (int i = 0; i < 4; i++) {
-                if (o[i] < 0) continue;
-                v += a[i];
-                if (sp) v -= b[i];
-              }
-            }
-          }
-          add(cc, flip_sign(v, mask_bit<NINT>(M, z)), r, (NT)S.rc[r]);
-        } else if (jd < ndraw) {
-          const int jl = (jd - nall) * per + (lane >> 2), ip = lane & 3;
-          const bool have = (lane >> 2) < per && jl < nrow;
-          int r = 0;
-          NT cj = NT(0);
-          uint64_t part = 0x7FFF7FFF7FFF7FFFull, hm = 0;
-          uint64_t M[NINT];         // phase of the row's substitution by z
-          uint64_t EX[NINT];        // particles of J with the spin of z
-          // orbitals: uz (hole paired with z) | uo (hole paired with q) << 8 |
-          // q << 16 | same spin << 24
-          uint32_t iw = 0;
-          int geo = 0;              // virtual index of the row's particle, its spin << 8
-          bool act = false;
-          // the single substitution of the pair of particles ip: cell and
-          // sign << 31, hole w | q << 8 | spin << 16
-          bool sact = false;
-          uint32_t scell = 0, sw = 0;
-#pragma unroll
-          for (int w = 0; w < NINT; w++) M[w] = EX[w] = 0;
-          if (have) {
-            r = S.u.l.L12[jl];
-            part = S.rpt[r];
-            hm = S.rhm[r];
-            cj = (NT)S.rc[r];
-            uint32_t X, T;
-            int nx, nt;
-            excitation_sets<NINT, NT>(B, S, part, hm, &X, &nx, &T, &nt);
-            const int q = pk(T, 0), sq = q >= norb ? 1 : 0, qo = q - sq * norb;
-            uint64_t Jw[NW];
-#pragma unroll
-            for (int w = 0; w < NW; w++) Jw[w] = S.rw[(size_t)r * NW + w];
-            // the row's particle (a one-hole batch has one row per J and no
-            // fixed particle)
-            const int code = B.h == 2 ? part_code(part, ip) : (ip == 0 ? -1 : kNoPart);
-            if (code != kNoPart) {
-              const int s = code >= norb, x = code >= 0 ? S.vidx[s][code - s * norb] : 0;
-              const int sz = B.kind == 2 ? 1 - s : B.sa;
-              act = B.h == 1 || ((B.kind == 2 || s == B.sa) && !row_banned<NINT, NT>(S, s, code - s * norb));
-              geo = x | (s << 8);
-              int u0 = -1, u1 = -1;  // X without the row's particle
-#pragma unroll
-              for (int i = 0; i < 3; i++) {
-                if (i >= nx) break;
-                const int xc = pk(X, i);
-                if (xc != code) {
-                  if (u0 < 0) u0 = xc;
-                  else u1 = xc;
-                }
-              }
-              const bool same = (u0 >= norb) == (u1 >= norb);
-              const bool second = same || (u1 >= norb) == (sz != 0);
-              const int uz = second ? u1 : u0, uo = second ? u0 : u1;
-              const int so = uo >= norb, zo = uz - sz * norb, oo = uo - so * norb;
-              uint64_t wo[NINT], wz[NINT];
-#pragma unroll
-              for (int w = 0; w < NINT; w++) {
-                wo[w] = so ? Jw[NINT + w] : Jw[w];
-                wz[w] = sz ? Jw[NINT + w] : Jw[w];
-                if (same) {
-                  if ((oo >> 6) == w) wz[w] &= ~(1ull << (oo & 63));
-                  if ((qo >> 6) == w) wz[w] |= 1ull << (qo & 63);
-                }
-              }
-              const int c = count_between<NINT>(wo, oo < qo ? oo : qo, oo < qo ? qo : oo) & 1;
-              phase_mask<NINT>(wz, zo, c, M);
-              iw = (uint32_t)zo | ((uint32_t)oo << 8) | ((uint32_t)qo << 16) | ((uint32_t)same << 24);
-#pragma unroll
-              for (int i = 0; i < 4; i++) {
-                const int pc = part_code(part, i);
-                if (pc == kNoPart || (pc >= norb) != (sz != 0)) continue;
-                const int po = pc - sz * norb;
-#pragma unroll
-                for (int w = 0; w < NINT; w++)
-                  if ((po >> 6) == w) EX[w] |= 1ull << (po & 63);
-              }
-            }
-            if (ip < 3) {  // two-hole batch: pairs (0, 1), (0, 2), (1, 2) of J's particles; one-hole: its particles
-              const int c0_ = part_code(part, B.h == 2 && ip == 2 ? 1 : (B.h == 2 ? 0 : ip));
-              const int c1_ = B.h == 2 ? part_code(part, ip == 0 ? 1 : 2) : -1;
-              if (c0_ != kNoPart && c1_ != kNoPart) {
-                const int sx = c0_ >= norb, sy = c1_ >= norb;
-                if (B.kind == 2 ? sx != sy : (sx == B.sa && (c1_ < 0 || sy == B.sa))) {
-                  const int vx = S.vidx[sx][c0_ - sx * norb], vy = c1_ < 0 ? 0 : S.vidx[sy][c1_ - sy * norb];
-                  const int cc = (B.kind == 0 ? vx : B.kind == 1 ? pair_cell(vx, vy) : (sx ? vy * S.nv[1] + vx : vx * S.nv[1] + vy)) - B.clo;
-                  if (live(cc)) {
-                    int w = 0;  // X without the cell's particles: the hole, with q's spin
-#pragma unroll
-                    for (int i = 0; i < 3; i++) {
-                      const int xc = pk(X, i);
-                      if (i < nx && xc != c0_ && xc != c1_) w = xc;
-                    }
-                    const int wo = w - sq * norb;
-                    uint64_t ws[NINT];
-#pragma unroll
-                    for (int i = 0; i < NINT; i++) ws[i] = sq ? Jw[NINT + i] : Jw[i];
-                    const int neg = count_between<NINT>(ws, wo < qo ? wo : qo, wo < qo ? qo : wo) & 1;
-                    sact = true;
-                    scell = (uint32_t)cc | ((uint32_t)neg << 31);
-                    sw = (uint32_t)wo | ((uint32_t)qo << 8) | ((uint32_t)sq << 16);
-                  }
-                }
-              }
-            }
-          }
-#pragma unroll 1
-          for (unsigned m = __ballot_sync(kFull, act); m; m &= m - 1) {
-            const int src = __ffs((int)m) - 1;
-            const uint32_t iwr = __shfl_sync(kFull, iw, src);
-            const int gr = __shfl_sync(kFull, geo, src), rj = __shfl_sync(kFull, r, src);
-            const NT cjr = __shfl_sync(kFull, cj, src);
-            uint64_t Mr[NINT], Er[NINT];
-            shfl_words<NINT>(M, src, Mr);
-            shfl_words<NINT>(EX, src, Er);
-            const int x = gr & 0xFF, s = gr >> 8, sz = B.kind == 2 ? 1 - s : B.sa;
-            const int uz = iwr & 0xFF, uo = (iwr >> 8) & 0xFF, q = (iwr >> 16) & 0xFF;
-            const bool same = (iwr >> 24) & 1u;
-            const int nz = S.nv[sz], nv1 = S.nv[1];
-            // the integrals at b1 + z and (same spin) b2 + z
-            const NT* e1 = eri_n + ((uo * norb + uz) * norb + q) * norb;
-            const NT* e2 = eri_n + ((uz * norb + uo) * norb + q) * norb;
-            // cell of z's index y: cb + y cs, or (same spin) a pair
-            const int cs = B.kind == 2 && s ? nv1 : 1;
-            const int cb = (B.kind == 2 ? (s ? x : x * nv1) : 0) - B.clo, xx = x * (x - 1) / 2;
-            // two rounds of 32 cells at a time, their loads in flight together
-#pragma unroll 1
-            for (int y0 = lane; y0 < nz; y0 += 64) {
-              int ca = -1, cn = -1;
-              NT va = NT(0), vn = NT(0);
-              auto fetch = [&](int y, int& c, NT& v) {
-                if (y >= nz) return;
-                const int z = S.vir[sz][y];
-                int cc = cb + y * cs;
-                if (B.kind == 1) cc = cb + (y > x ? y * (y - 1) / 2 + x : xx + y);
-                if (mask_bit<NINT>(Er, z) || !live(cc)) return;
-                c = cc;
-                if constexpr (E4) {
-                  v = e1[z];
-                  if (same) v -= e2[z];
-                } else {
-                  v = eri_n[eri_index(uo, q, uz, z)];
-                  if (same) v -= eri_n[eri_index(uz, q, uo, z)];
-                }
-                v = flip_sign(v, mask_bit<NINT>(Mr, z));
-              };
-              fetch(y0, ca, va);
-              fetch(y0 + 32, cn, vn);
-#pragma unroll 1
-              for (int i = 0; i < 2; i++) {
-                if (ca >= 0) add(ca, va, rj, cjr);
-                ca = cn;
-                va = vn;
-              }
-            }
-          }
-#pragma unroll 1
-          for (unsigned m = __ballot_sync(kFull, sact); m; m &= m - 1) {
-            const int src = __ffs((int)m) - 1;
-            const uint32_t sc = __shfl_sync(kFull, scell, src), wq = __shfl_sync(kFull, sw, src);
-            const int rj = __shfl_sync(kFull, r, src);
-            const NT cjr = __shfl_sync(kFull, cj, src);
-            const uint64_t hmr = __shfl_sync(kFull, hm, src), ptr_ = __shfl_sync(kFull, part, src);
-            const int wo = wq & 0xFF, qo = (wq >> 8) & 0xFF, sq = (wq >> 16) & 1;
-            NT v = NT(0);
-            if constexpr (sizeof(NT) == 8) {  // J's orbitals: I's, with particles in the place of its holes
-#pragma unroll 1
-              for (int i = lane; i < nel; i += 32) {
-                int mo = S.occ[i];
-                if ((hmr >> i) & 1ull) mo = part_code(ptr_, __popcll(hmr & ((1ull << i) - 1)));
-                const int sm = mo >= norb, o = mo - sm * norb;
-                v += eri_n[gidx<E4>(o, o, wo, qo, norb)];
-                if (sm == sq) v -= eri_n[gidx<E4>(wo, o, o, qo, norb)];
-              }
-              v = warp_sum_nt<NT>(v) + h_n[wo * norb + qo];
-            } else {
-              // FP32: the sum keeps the ascending order of J's orbitals (its
-              // rounding depends on it); the lanes load, one adds
-              v = h_n[wo * norb + qo];
-#pragma unroll
-              for (int w = 0; w < 2 * NW; w++) {
-                const int o = 32 * (w % (2 * NINT)) + lane;
-                const bool sp = w / (2 * NINT) == sq;
-                uint32_t bits = (uint32_t)(S.rw[(size_t)rj * NW + w / 2] >> (32 * (w & 1)));
-                NT a = NT(0), b = NT(0);
-                if ((bits >> lane) & 1u) {
-                  a = eri_n[gidx<E4>(o, o, wo, qo, norb)];
-                  if (sp) b = eri_n[gidx<E4>(wo, o, o, qo, norb)];
-                }
-                for (; bits; bits &= bits - 1) {
-                  const int src2 = __ffs((int)bits) - 1;
-                  v += __shfl_sync(kFull, a, src2);
-                  const NT bb = __shfl_sync(kFull, b, src2);
-                  if (sp) v -= bb;
-                }
-              }
-            }
-            if (lane == 0) add((int)(sc & 0x7fffffffu), flip_sign(v, (sc >> 31) != 0u), rj, cjr);
-          }
-        } else {
-          const int j0 = (jd - ndraw) * 32;
-          if (j0 >= n2) break;
-          const int j = j0 + lane;
-          if (j < n2) {
-            // cells inside J's particles: J -> alpha moves the other two
-            // entries of X to J's two holes outside the batch
-            const int r = S.u.l.L12[kChunk - 1 - j];
-            const uint64_t part = S.rpt[r];
-            uint32_t X, T;
-            int nx, nt;
-            excitation_sets<NINT, NT>(B, S, part, S.rhm[r], &X, &nx, &T, &nt);
-            const NT cj = (NT)S.rc[r];
-            uint64_t Jw[NW];
-#pragma unroll
-            for (int w = 0; w < NW; w++) Jw[w] = S.rw[(size_t)r * NW + w];
-#pragma unroll 1
-            for (int k = 0; k < (B.h == 2 ? 6 : 4); k++) {
-              // pairs (0, 1), (0, 2), (1, 2), (0, 3), (1, 3), (2, 3); one-hole batch: single particles
-              const int k1 = B.h == 1 ? k : (k >= 3 ? 3 : k >= 1 ? 2 : 1), k0 = B.h == 1 ? k : (k >= 3 ? k - 3 : k >= 1 ? k - 1 : 0);
-              const int e0 = part_code(part, k0), e1 = part_code(part, k1);
-              if (e0 == kNoPart || e1 == kNoPart) continue;
-              const int sx = e0 >= norb, sy = e1 >= norb;
-              if (B.kind == 2 ? sx == sy : (sx != B.sa || sy != B.sa)) continue;
-              const int vx = S.vidx[sx][e0 - sx * norb], vy = S.vidx[sy][e1 - sy * norb];
-              const int cc = (B.kind == 0 ? vx : B.kind == 1 ? pair_cell(vx, vy) : (sx ? vy * S.nv[1] + vx : vx * S.nv[1] + vy)) - B.clo;
-              if (!live(cc)) continue;
-              int u0 = -1, u1 = -1;
-#pragma unroll
-              for (int i = 0; i < 4; i++) {
-                const int xc = pk(X, i);
-                if (i < nx && xc != e0 && xc != e1) {
-                  if (u0 < 0) u0 = xc;
-                  else u1 = xc;
-                }
-              }
-              const NT v = double_element<NINT, NT, E4>(eri_n, norb, Jw, u0 < u1 ? u0 : u1, u0 < u1 ? u1 : u0, pk(T, 0), pk(T, 1));
-              if constexpr (MS) {
-#pragma unroll
-                for (int st = 0; st < kMaxStates; st++)
-                  if (st < nst) atomicAdd(&A[st * mc + cc], S.rc[st * p.rc_stride + r] * (double)v);
-              } else {
-                unsigned long long l;
-                int hh;
-                fix_of(cj * v, F, l, hh);
-                fix_atomic_add(A0, A1, A2, cc, l, hh);
-              }
-              con++;
-            }
-          }
-        }
-      }
-    }
+    row_pass(std::false_type{});
     __syncthreads();
 
     // ---- passes over the cells: the terms of the J reaching every cell, a
@@ -2303,7 +2346,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     for (int g0 = 0;; g0 += kGroup) {
       B = S.bt;
       const int m = max(0, min(kGroup, nt0 - g0));
-      const bool fin = last_round && (GRAD ? m == 0 : g0 + kGroup >= nt0);
+      const bool fin = last_round && g0 + kGroup >= nt0;
       if (!fin && m == 0) break;
       if (g0 > 0 && m > 0) {  // the first group's tables came with the row pass
         __syncthreads();
@@ -2312,14 +2355,6 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         __syncthreads();
       }
       if (fin) {
-        if (GRAD) {  // the pair tables' storage takes the weights
-          __syncthreads();
-          for (int x = tid; x < kMaxOrb; x += kThreads) {
-            S.v.w.rowW2[x] = 0.0;
-            S.v.w.colW2[x] = 0.0;
-          }
-          __syncthreads();
-        }
         if (p.k > 0 && tkcnt + B.nct > p.cap) compact_selection<NINT, NT>(p, S, buf_e(p), buf_a(p), buf_key<NINT>(p));
       }
       const unsigned long long tau = S.tau;
@@ -2367,7 +2402,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
         }
 #pragma unroll 1
         for (int j = 0; j < m; j++) {
-          const int rt = S.v.g.gRow[j][x], ct = S.v.g.gCol[j][y], rc = (int)((unsigned)rt + (unsigned)ct);
+          const int rt = S.gRow[j][x], ct = S.gCol[j][y], rc = (int)((unsigned)rt + (unsigned)ct);
           if ((rt | ct) & (3 << 29)) continue;
           NT v;
           bool neg = rc < 0;
@@ -2376,7 +2411,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             if (B.kind == 1) v -= eri_n[S.gB[j] + so * norb + ro];
           } else {
             v = eri_n[tri(rt & 0x1fffffff, ct & 0x1fffffff)];
-            if (B.kind == 1) v -= eri_n[tri(S.v.g.gRow[j][y] & 0x1fffffff, S.v.g.gCol[j][x] & 0x1fffffff)];
+            if (B.kind == 1) v -= eri_n[tri(S.gRow[j][y] & 0x1fffffff, S.gCol[j][x] & 0x1fffffff)];
           }
           if (B.kind == 1) {
             const int x2 = S.gx2[j];
@@ -2476,15 +2511,20 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           acc_e = fma(a, q, acc_e);  // e = A q
           acc_s2 += q * q;
           if (GRAD) {
-            // numerator weight 2A/D for loop 3; (A/D)^2 weights the diagonal
-            const unsigned long long wb = (unsigned long long)__double_as_longlong(2.0 * q);
+            // numerator weight 2A/D for loop 3, here already for the
+            // generator's own element; (A/D)^2 weights the diagonal
+            const double w1 = 2.0 * q;
+            const unsigned long long wb = (unsigned long long)__double_as_longlong(w1);
             A0[cc] = (uint32_t)wb;
             A1[cc] = (uint32_t)(wb >> 32);
-            const double w2 = q * q;
-            atomicAdd(&S.v.w.rowW2[x], w2);
-            if (B.kind == 2) atomicAdd(&S.v.w.colW2[y], w2);
-            if (B.kind == 1) atomicAdd(&S.v.w.rowW2[y], w2);
-            if (B.h == 2) w_grad(p, ro, B.sa, so, B.sb, w2);
+            if (B.h == 2) {
+              w_grad(p, ro, B.sa, so, B.sb, q * q);
+              bool neg = (R.idx ^ C.idx) < 0;
+              if (B.kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
+              const double ws = flip_sign((double)S.cI * w1, neg);
+              atomicAdd(&p.g_deri[eri_index(B.qa, ro, B.qb, so)], ws);
+              if (B.kind == 1) atomicAdd(&p.g_deri[eri_index(B.qa, so, B.qb, ro)], -ws);
+            }
           }
           // |a| < 1e-14, compared on the bit pattern (no FP64 compare)
           if (abs_bits(a) < 0x3D06849B86A12B9Bull) atomicAdd(&S.tiny, 1u);
@@ -2612,91 +2652,57 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
   }
   if (GRAD) {
     __syncthreads();
-    // ---- loop 3: c_J (2A/D) d<J|H|alpha> over the same (J, cell) pairs ----
+    // ---- loop 3: c_J (2A/D) d<J|H|alpha> over the same (J, cell) pairs, by
+    // the same rows and pair tables ----
     for (int c0 = 0; c0 < S.seg_s[3]; c0 += kChunk) {
-      if (tid == 0) {
-        S.n0 = 0;
-        S.n1 = 0;
-        S.n2 = 0;
-        S.cnext = 0;
-      }
+      if (tid == 0) S.n0 = S.n1 = S.n2 = S.cnext = 0;
       __syncthreads();
       const int c1 = min(c0 + kChunk, S.seg_s[3]);
+#pragma unroll 1
       for (int i = c0 + tid; i < c1; i += kThreads) {
         const int o = entry(i);
         const ulonglong2 en = S.ehp[o];
         const uint64_t hmr = en.x, part = en.y;
-        if (part & kBeforeBit) continue;
-        if (dup(i, hmr)) continue;
+        if ((part & kBeforeBit) || dup(i, hmr)) continue;
+        if (B.h == 2 && hmr == 0ull) continue;  // J = I: in the cells pass
         const int t = __popcll(hmr & ~B.hm);
         if (t > 2) continue;
-        const bool all = (B.h == 1) ? (t <= 1) : (t == 0);
         const int rec = (int)(S.erec[o] & 0x7FFFFFFFu);
-        if (all) S.u.l.L0[atomicAdd(&S.n0, 1)] = rec;
+        if (t == 0) S.u.l.L0[atomicAdd(&S.n0, 1)] = rec;
         else if (t == 1) {
-          if (row_live<NINT, NT>(B, S, norb, part)) S.u.l.L12[atomicAdd(&S.n1, 1)] = rec;
+          if (B.h == 1 || row_live<NINT, NT>(B, S, norb, part)) S.u.l.L12[atomicAdd(&S.n1, 1)] = rec;
         }
         else if (subset_live<NINT, NT>(B, S, norb, part, ban)) S.u.l.L12[kChunk - 1 - atomicAdd(&S.n2, 1)] = rec;
       }
       __syncthreads();
-      for (int j = 0; j < S.n0; j++) {
-        const int r = S.u.l.L0[j];
-        const uint64_t* Jw = S.rw + (size_t)r * NW;
-        const double cj = S.rc[r];
-        uint32_t X, T;
-        int nx, nt;
-        const ulonglong2 en = make_ulonglong2(S.rhm[r], S.rpt[r]);
-        excitation_sets<NINT, NT>(B, S, en.y, en.x, &X, &nx, &T, &nt);
-        for (int cc = tid; cc < B.nct; cc += kThreads) {
-          if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
+      row_pass(std::true_type{});
+      __syncthreads();
+      const int nt0 = B.h == 2 ? S.n0 : 0;
+#pragma unroll 1
+      for (int g0 = 0; g0 < nt0; g0 += kGroup) {
+        const int m = min(kGroup, nt0 - g0);
+        if (g0 > 0) {
+          __syncthreads();
+#pragma unroll 1
+          for (int j = warp; j < m; j += kWarps) build_table(j, S.u.l.L0[g0 + j]);
+          __syncthreads();
+        }
+#pragma unroll 1
+        for (int i = tid; i < S.nlist; i += kThreads) {
+          const int cc = E.lst[i];
           int ro, so, x, y;
           cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro, &so, &x, &y);
-          element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, B.sa * norb + ro, (B.h == 2) ? B.sb * norb + so : -1, cj * a2d(cc));
-        }
-      }
-      {  // row-reaching J (a warp each), then subset-reaching J (32 per draw), drawn dynamically
-        const int n1 = S.n1, n2 = S.n2;
-        for (;;) {
-          int jd = 0;
-          if (lane == 0) jd = atomicAdd(&S.cnext, 1);
-          jd = __shfl_sync(kFull, jd, 0);
-          if (jd < n1) {
-            const int j = jd;
-            const int r = S.u.l.L12[j];
-            const uint64_t* Jw = S.rw + (size_t)r * NW;
-            const double cj = S.rc[r];
-            const ulonglong2 en = make_ulonglong2(S.rhm[r], S.rpt[r]);
-          const uint64_t part = en.y;
-            uint32_t X, T;
-            int nx, nt;
-            excitation_sets<NINT, NT>(B, S, part, en.x, &X, &nx, &T, &nt);
-            for_row_cells<NINT, NT>(B, S, norb, part, lane, [&](int c, int pc, int zc) {
-              const int cc = c - B.clo;
-              if ((unsigned)cc >= (unsigned)B.nct || ((ban[cc >> 5] >> (cc & 31)) & 1u)) return;
-              element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, pc, zc, cj * a2d(cc));
-            });
-          } else {
-            const int j0 = (jd - n1) * 32;
-            if (j0 >= n2) break;
-            const int j = j0 + lane;
-            if (j < n2) {
-              const int r = S.u.l.L12[kChunk - 1 - j];
-              const uint64_t* Jw = S.rw + (size_t)r * NW;
-              const double cj = S.rc[r];
-              const ulonglong2 en = make_ulonglong2(S.rhm[r], S.rpt[r]);
-          const uint64_t part = en.y;
-              uint32_t X, T;
-              int nx, nt;
-              excitation_sets<NINT, NT>(B, S, part, en.x, &X, &nx, &T, &nt);
-              for_subset_cells<NINT, NT>(B, S, norb, part, [&](int c) {
-                const int cc = c - B.clo;
-                if ((unsigned)cc >= (unsigned)B.nct || ((ban[cc >> 5] >> (cc & 31)) & 1u)) return;
-                int ro, so, x, y;
-                cell_orbitals<NINT, NT>(B, S, c, &ro, &so, &x, &y);
-                element_grad<NINT>(p.g_dh, p.g_deri, norb, Jw, X, nx, T, nt, B.sa * norb + ro, (B.h == 2) ? B.sb * norb + so : -1,
-                                   cj * a2d(cc));
-              });
-            }
+          const double w = a2d(cc);
+#pragma unroll 1
+          for (int j = 0; j < m; j++) {
+            const int rt = S.gRow[j][x], ct = S.gCol[j][y];
+            if ((rt | ct) & (3 << 29)) continue;
+            const int x1 = S.gx1[j], x2 = S.gx2[j];
+            bool neg = (rt ^ ct) < 0;
+            if (B.kind == 1) neg ^= ro > (so < x2 ? so : x2) && ro < (so < x2 ? x2 : so);
+            const double ws = flip_sign((double)S.gcj[j] * w, neg);
+            atomicAdd(&p.g_deri[eri_index(x1, ro, x2, so)], ws);
+            if (B.kind == 1) atomicAdd(&p.g_deri[eri_index(x1, so, x2, ro)], -ws);
           }
         }
       }
@@ -2707,24 +2713,34 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     //      were scattered per cell, the rest goes by row sums ----
     const int g = M->g;
     double* wF = p.g_wF + (size_t)g * 2 * norb;
-    const int s1 = B.sa, s2 = (B.h == 2) ? B.sb : B.sa;
-    for (int x = tid; x < S.nv[s1]; x += kThreads) {
-      const double wr = S.v.w.rowW2[x];
-      if (wr == 0.0) continue;
-      const int r = S.vir[s1][x];
-      atomicAdd(&wF[s1 * norb + r], wr);
-      w_grad(p, r, s1, B.qa, B.sa, -wr);
-      if (B.h == 2) w_grad(p, r, s1, B.qb, B.sb, -wr);
-    }
-    if (B.kind == 2)
-      for (int y = tid; y < S.nv[s2]; y += kThreads) {
-        const double wc = S.v.w.colW2[y];
-        if (wc == 0.0) continue;
-        const int sv = S.vir[s2][y];
-        atomicAdd(&wF[s2 * norb + sv], wc);
-        w_grad(p, sv, s2, B.qa, B.sa, -wc);
-        w_grad(p, sv, s2, B.qb, B.sb, -wc);
+    // four lanes per row or column of cells: sums of (A/D)^2 (cells outside the
+    // list are zero).  (Adding each cell's into shared memory was a
+    // compare-and-swap loop of up to 32 lanes on one word.)
+    const int nvc = S.nv[1], nrows = B.kind == 2 ? B.nct / nvc : S.nv[B.sa], x0 = B.kind == 2 ? B.clo / nvc : 0;
+    const int nsum = nrows + (B.kind == 2 ? nvc : 0);
+#pragma unroll 1
+    for (int u0 = 0; u0 < nsum; u0 += kThreads / 4) {
+      const int u = u0 + (tid >> 2), sub = tid & 3;
+      const bool row = u < nrows;
+      double w = 0.0;
+      if (u < nsum) {
+        const int len = B.kind == 0 ? 1 : B.kind == 2 && row ? nvc : nrows;
+#pragma unroll 2
+        for (int v = sub; v < len; v += 4) {
+          if (B.kind == 1 && v == u) continue;
+          const double a = a2d(B.kind == 0 ? u : B.kind == 1 ? pair_cell(u, v) : row ? u * nvc + v : v * nvc + u - nrows);
+          w = fma(a, a, w);
+        }
       }
+      w += __shfl_xor_sync(kFull, w, 1);
+      w += __shfl_xor_sync(kFull, w, 2);
+      w *= 0.25;
+      if (u >= nsum || w == 0.0) continue;
+      const int sr = row ? B.sa : 1, r = S.vir[sr][row ? x0 + u : u - nrows];
+      if (sub == 0) atomicAdd(&wF[sr * norb + r], w);
+      if (sub == 1) w_grad(p, r, sr, B.qa, B.sa, -w);
+      if (sub == 2 && B.h == 2) w_grad(p, r, sr, B.qb, B.sb, -w);
+    }
     if (tid == 0 && S.sw2 != 0.0) {
       const double sw = S.sw2;
       atomicAdd(&p.g_wH[g], sw);
