@@ -398,7 +398,7 @@ int qp_pt2_last_timings(const qp_pt2_ctx *ctx, double *ms);
  * stream capture.  Every call reuses the same array: calls whose GPU work
  * overlaps (other streams, other threads) race and must not be issued.
  * Problems whose integral tables, generator order, per-generator records,
- * selection buffers (one CTA per SM, k + cells entries each) and sort space
+ * selection buffers (at least one CTA per SM, k + cells entries each) and sort space
  * do not fit in the array are refused with QP_EINVAL; as a guide, 64
  * orbitals with 10+10 electrons fit up to roughly 10^3 determinants with
  * k = 10^3. */
