@@ -217,7 +217,7 @@ struct SweepParams {
   // the wave's work items (slot * nper + item), without those of batches
   // banned as a whole, in the order the prep kernel finished the slots
   uint32_t* live;                 // [slots * nper]
-  int* live_cnt;                  // per wave, zero before the prep kernel
+  int* live_cnt;                  // per wave: items listed from the front, from the back; zero before the prep kernel
   int64_t ent_cap;
 
   // exact accumulation of A_alpha: bits of max_I |c_I| (written by the

@@ -249,7 +249,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     tk_cnt = reinterpret_cast<int*>(sel_hist + kSelBins);
     acc = cv.take<unsigned long long>(9);
     dres = cv.take<DevResult>(1);
-    queues = cv.take<int>(2);  // the wave's item counter and live count
+    queues = cv.take<int>(3);  // the wave's item counter and live counts
     tk_e = cv.take<double>((size_t)cap * grid);
     tk_a = cv.take<double>((size_t)cap * grid);
     tk_key = cv.take<uint64_t>((size_t)cap * grid * nw);
@@ -418,7 +418,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     p.last_wave = (w == nwaves - 1);
     p.queue = queues;
     p.live_cnt = queues + 1;
-    NTRY_Q(cudaMemsetAsync(queues, 0, 2 * sizeof(int), st));
+    NTRY_Q(cudaMemsetAsync(queues, 0, 3 * sizeof(int), st));
     NTRY_Q(launch_prep(nint, p, p.wave_slots, st));
     NTRY_Q(launch_batch_packed(nint, p, grid, smem, st));
     NTRY_Q(launch_reduce_items(p, st));

@@ -832,7 +832,7 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   // the CTAs' thresholds and candidate counts, the histogram, the waves'
   // queue and live counts
   const size_t z_tau = 8 * nd * (2 * (size_t)nsts + 2), z_hist = z_tau + 8 * (size_t)grid, z_cnt = z_hist + 4 * kSelBins,
-               z_queue = z_cnt + 4 * (size_t)grid, z_end = z_queue + 8 * (size_t)(nwaves + 1);
+               z_queue = z_cnt + 4 * (size_t)grid, z_end = z_queue + 12 * (size_t)(nwaves + 1);
   if ((rc = x->zeroed.grow(z_end)) || (rc = x->meta.grow(sizeof(GenMeta) * ws)) ||
       (rc = x->r_words.grow(8 * nd * nw * ws)) || (rc = x->r_coef.grow(8 * nd * ws * nsts)) ||
       (rc = x->r_hmask.grow(8 * nd * ws)) || (rc = x->r_part.grow(8 * nd * ws)) ||
@@ -933,7 +933,7 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
     p.wave_slots = (int)((ngen - w * W) < W ? (ngen - w * W) : W);
     p.last_wave = (w == nwaves - 1);
     p.queue = reinterpret_cast<int*>(zb + z_queue) + w;
-    p.live_cnt = p.queue + (nwaves + 1);
+    p.live_cnt = reinterpret_cast<int*>(zb + z_queue) + (nwaves + 1) + 2 * w;
     CUDA_TRY(launch_prep(nint, p, p.wave_slots, st));
     if (ms) CUDA_TRY(launch_batch_states(nint, p, grid, smem, st));
     else CUDA_TRY(launch_batch(nint, p, grid, smem, st));
@@ -1224,7 +1224,7 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
       (rc = x->e_hp.grow(16 * (size_t)ent_cap * wsl)) ||
       (rc = x->e_rec.grow(4 * (size_t)ent_cap * wsl)) || (rc = x->it_sum.grow(16 * (size_t)nper * wsl)) ||
       (rc = x->live.grow(4 * (size_t)nper * wsl)) ||
-      (rc = x->queues.grow(8 * (size_t)(nwaves + 1))) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
+      (rc = x->queues.grow(12 * (size_t)(nwaves + 1))) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
       (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
       (rc = x->res.grow(sizeof(DevResult))) ||
       (rc = x->g_wF.grow(8 * nd * 2 * norb)) || (rc = x->g_wH.grow(8 * nd)))
@@ -1233,7 +1233,7 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   CUDA_TRY(cudaMemsetAsync(x->s2.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->na.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->ncon.p, 0, 8 * nd, st));
-  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 8 * (size_t)(nwaves + 1), st));
+  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 12 * (size_t)(nwaves + 1), st));
   CUDA_TRY(cudaMemsetAsync(x->tk_cnt.p, 0, 4 * (size_t)grid, st));
   CUDA_TRY(cudaMemsetAsync(x->tk_tau.p, 0, 8 * (size_t)grid, st));
   CUDA_TRY(cudaMemsetAsync(x->g_wF.p, 0, 8 * nd * 2 * norb, st));
@@ -1314,7 +1314,7 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
     p.wave_slots = (int)((ngen - w * W) < W ? (ngen - w * W) : W);
     p.last_wave = (w == nwaves - 1);
     p.queue = x->queues.as<int>() + w;
-    p.live_cnt = x->queues.as<int>() + (nwaves + 1) + w;
+    p.live_cnt = x->queues.as<int>() + (nwaves + 1) + 2 * w;
     CUDA_TRY(launch_prep(nint, p, p.wave_slots, st));
     CUDA_TRY(launch_batch_grad(nint, p, grid, x->smem, st));
     CUDA_TRY(launch_reduce_items(p, st));
@@ -1500,7 +1500,7 @@ static int plan_instance(BatchInst& b, size_t wave_budget, int64_t W_fixed, bool
       (rc = x->e_rec.grow(4 * (size_t)b.ent_cap * ws)) ||
       (rc = x->it_sum.grow(16 * (size_t)nper * ws)) || (rc = x->live.grow(4 * (size_t)nper * ws))))
     return rc;
-  if ((rc = x->queues.grow(8 * (size_t)(b.nwaves + 1))) ||
+  if ((rc = x->queues.grow(12 * (size_t)(b.nwaves + 1))) ||
       (rc = x->tk_e.grow(8 * (size_t)b.cap * grid)) || (rc = x->tk_a.grow(8 * (size_t)b.cap * grid)) ||
       (rc = x->tk_key.grow(8 * (size_t)b.cap * grid * nw)) || (rc = x->tk_cnt.grow(4 * (size_t)grid)) ||
       (rc = x->tk_tau.grow(8 * (size_t)grid)) || (rc = x->den_tab.grow(16 * (size_t)x->norb * x->norb)) ||
@@ -1625,7 +1625,7 @@ static int enqueue_pre(BatchInst& b, cudaStream_t st) {
   CUDA_TRY(cudaMemsetAsync(x->s2.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->na.p, 0, 8 * nd, st));
   CUDA_TRY(cudaMemsetAsync(x->ncon.p, 0, 8 * nd, st));
-  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 8 * (size_t)(b.nwaves + 1), st));
+  CUDA_TRY(cudaMemsetAsync(x->queues.p, 0, 12 * (size_t)(b.nwaves + 1), st));
   CUDA_TRY(cudaMemsetAsync(x->tk_cnt.p, 0, 4 * (size_t)b.grid, st));
   CUDA_TRY(cudaMemsetAsync(x->tk_tau.p, 0, 8 * (size_t)b.grid, st));
   return QP_OK;
@@ -1640,7 +1640,7 @@ static int enqueue_waves(BatchInst& b, cudaStream_t st) {
     p.wave_slots = (int)((b.ngen - w * b.W) < b.W ? (b.ngen - w * b.W) : b.W);
     p.last_wave = (w == b.nwaves - 1);
     p.queue = x->queues.as<int>() + w;
-    p.live_cnt = x->queues.as<int>() + (b.nwaves + 1) + w;
+    p.live_cnt = x->queues.as<int>() + (b.nwaves + 1) + 2 * w;
     CUDA_TRY(launch_prep(x->nint, p, p.wave_slots, st));  // it zeroes the wave's per-item sums
     CUDA_TRY(launch_batch(x->nint, p, b.grid, b.smem, st));
     CUDA_TRY(launch_reduce_items(p, st));

@@ -23,25 +23,26 @@
 //      a cell these leave go to one shared list (d <= 2), to a list per hole
 //      (d <= 3) and to a bucket per pair of holes (d >= 2).
 //
-//  batch_kernel (persistent CTAs, one (generator, batch) item at a time,
-//  items of the heaviest generators first)
+//  batch_kernel (persistent CTAs, one (generator, batch) item at a time, in
+//  the order of the prep kernel's list: large waves by kind, see by_kind)
 //    bans:   the masks, then the bucket's J ranked before I; a later J equal
 //            to some alpha bans it;
 //    loop 2: J ranked at or after I add c_J <J|H|alpha> into the shared-memory
 //            accumulator A(R) of the cells they reach that are not banned.
-//            J reaching every cell are spread over the whole CTA, J reaching a
-//            row of cells over a warp, J reaching a few cells over a thread;
+//            A row of cells is a warp's, a lane per cell; J reaching a few
+//            cells are a thread's; J reaching every cell go through pair
+//            tables in the cells pass;
 //    cells:  every cell left is a perturber of I: e = A^2/(E0 - H_aa) with
-//            H_aa from per-batch row sums of the Fock diagonal, added to eps_I
-//            and offered to the CTA's selection buffer.
+//            H_aa from per-batch row and column sums in fixed point, added to
+//            eps_I and offered to the CTA's selection buffer.
 // Matrix elements follow the Slater-Condon rules (Eqs. Hij) with phases from
 // a masked popcount of J's spin string.
 //
 // Numerator precision: the batch kernel is a template on NT, the type of the
 // integrals it gathers and of the products c_J <J|H|alpha>.  NT = double is
 // the plain FP64 sweep; NT = float gathers FP32 integrals and forms FP32
-// products, while each product is still added into the FP64 accumulator
-// A(R) and the denominators, e_alpha and every reduction stay FP64.
+// products, while each product is still added into the exact accumulator
+// A(R) and the denominators, e_alpha and every reduction are those of FP64.
 // sweep.cu instantiates the FP64 kernels, sweep_mixed.cu the mixed ones.
 #pragma once
 #include <cfloat>
@@ -437,6 +438,17 @@ struct Batch {
 };
 
 
+// Work items of a large wave are taken by kind, same-spin and one-hole ones
+// first, so that the code of one kind at a time is in the instruction caches
+// (10^4 determinants, 64 orbitals 78.5 -> 73.9 ms with a cells pass per kind,
+// 79.0 without the order; opposite-spin first 74.4).  Smaller waves are taken
+// as they come: 9,900 items 415 us, by kind 425; 50,400 items of 240
+// generators 10.35 ms, by kind 10.4 to 10.9; 184,000 items 5.28, by kind 5.00.
+constexpr long long kItemsByKind = 65536;
+__device__ __forceinline__ bool by_kind(const SweepParams& p) {
+  return (long long)p.wave_slots * p.nper >= kItemsByKind;
+}
+
 // Batch and tile of work item j of a generator: j < nbat is batch j (the first
 // row tile of a split batch), j >= nbat row tile 1 + (j - nbat) / (n_alpha
 // n_beta) of opposite-spin batch (j - nbat) % (n_alpha n_beta).
@@ -764,22 +776,29 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
     }
   }
   __syncthreads();
-  // the slot's work items, without those of batches banned as a whole
+  // the slot's work items, without those of batches banned as a whole; by
+  // kind: the opposite-spin ones from the back of the list, taken after the
+  // others
+  const bool mixed = !by_kind(p);
   for (int j0 = 0; j0 < p.nper; j0 += kThreads) {
     const int j = j0 + tid;
-    bool live = false;
+    bool live = false, first = false;
     if (j < p.nper) {
       int tile;
       const int b = item_batch(p, j, &tile);
       Batch B;
       batch_geometry(p, b, tile, B);
       live = B.nct > 0 && !((s_dead[b >> 5] >> (b & 31)) & 1u);
+      first = mixed || B.kind != 2;
     }
-    const unsigned lb = __ballot_sync(kFull, live);
+    const unsigned lf = __ballot_sync(kFull, live && first), ll = __ballot_sync(kFull, live && !first);
     int at = 0;
-    if ((tid & 31) == 0 && lb) at = atomicAdd(p.live_cnt, __popc(lb));
-    at = __shfl_sync(kFull, at, 0);
-    if (live) p.live[at + __popc(lb & ((1u << (tid & 31)) - 1))] = (uint32_t)(slot * p.nper + j);
+    if (lane < 2 && (lane ? ll : lf)) at = atomicAdd(p.live_cnt + lane, __popc(lane ? ll : lf));
+    const int af = __shfl_sync(kFull, at, 0), al = __shfl_sync(kFull, at, 1);
+    const unsigned before = (1u << lane) - 1u;
+    if (live)
+      p.live[first ? af + __popc(lf & before) : p.wave_slots * p.nper - 1 - (al + __popc(ll & before))] =
+          (uint32_t)(slot * p.nper + j);
   }
   bool one_alive = false;
   for (int i = 0; i < nel; i++) one_alive |= !((s_dead[i >> 5] >> (i & 31)) & 1u);
@@ -962,7 +981,7 @@ struct BatchShared {
   int seg_o[4], seg_s[4];
   Batch bt;  // the item's batch, read again by each phase
   int item[2];        // this work item and the next (-1: none)
-  int inext, iend, nlive;  // positions left of the last draw; live items of the wave
+  int inext, iend, nlive, nfirst;  // positions left of the last draw; live items of the wave, those listed from the front
   // storage of one phase of a work item at a time: the J lists, the
   // selection histogram, the per-thread sums of the reduction
   union {
@@ -1000,15 +1019,16 @@ struct BatchShared {
   int nlist;  // cells left after the bans
 };
 
-template <int NINT, typename NT>
+template <int NINT, typename NT, int KD = -1>  // KD: the batch's kind where it is known
 __device__ __forceinline__ void cell_orbitals(const Batch& B, const BatchShared<NINT, NT>& S, int c, int* r,
                                               int* s, int* x, int* y) {
-  if (B.kind == 0) {
+  const int kind = KD >= 0 ? KD : B.kind;
+  if (kind == 0) {
     *x = c;
     *y = -1;
     *r = S.vir[B.sa][c];
     *s = -1;
-  } else if (B.kind == 2) {
+  } else if (kind == 2) {
     const int nv1 = S.nv[1];
     int xx = __float2int_rz((float)c * S.inv_nv1);  // c < 2^14: exact up to one step
     if (xx * nv1 > c) xx--;
@@ -2365,206 +2385,218 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
 #pragma unroll
       for (int st = 0; st < kMaxStates; st++) acc_es[st] = acc_s2s[st] = 0.0;
       const int nleft = MS ? B.nct : S.nlist;
+      // a copy per kind: without the tests of it and the values one kind alone
+      // needs, two words per spin 63.0 -> 57.3 ms.  With one word and the kinds
+      // mixed in time three copies are more code in flight than the caches
+      // hold (150 determinants 415 -> 423 us): one copy for all kinds then.
+      auto cells = [&](auto kd) {
+        constexpr int KD = decltype(kd)::value;
+        const int kind = KD >= 0 ? KD : B.kind;
 #pragma unroll 1
-      for (int i = tid; i < nleft; i += kThreads) {
-        int cc = i, x, y, ro_, so_;
-        if constexpr (MS) {
-          if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
-        } else {
-          cc = E.lst[i];
-        }
-        cell_orbitals<NINT, NT>(B, S, B.clo + cc, &ro_, &so_, &x, &y);
-        y = y < 0 ? 0 : y;
-        const typename BatchShared<NINT, NT>::Side R = S.row[x], C = S.col[y];
-        const int ro = R.orb, so = C.orb;
-        // the generator's own integrals and the pair's term of D, loaded ahead
-        // of the terms of the J reaching every cell
-        NT own = NT(0), own2 = NT(0);
-        long long dpair = 0;
-        if (fin && B.h == 2) {
-          if constexpr (E4) {
-            own = eri_n[(R.idx & 0x7fffffff) + (C.idx & 0x7fffffff)];
-            if (B.kind == 1) own2 = eri_n[ibase + so * norb + ro];
+        for (int i = tid; i < nleft; i += kThreads) {
+          int cc = i, x, y, ro_, so_;
+          if constexpr (MS) {
+            if ((ban[cc >> 5] >> (cc & 31)) & 1u) continue;
           } else {
-            own = eri_n[tri(R.idx & 0x7fffffff, C.idx & 0x7fffffff)];
-            if (B.kind == 1) own2 = eri_n[tri(S.row[y].idx & 0x7fffffff, S.col[x].idx & 0x7fffffff)];
+            cc = E.lst[i];
           }
-          dpair = (B.kind == 2 ? p.Ji : p.Wi)[ro * norb + so];
-        }
-        unsigned long long lo = 0ull;  // exact sum
-        int hi = 0;
-        double accs[kMaxStates];  // multi-state form: one sum per state
+          cell_orbitals<NINT, NT, KD>(B, S, B.clo + cc, &ro_, &so_, &x, &y);
+          y = y < 0 ? 0 : y;
+          const typename BatchShared<NINT, NT>::Side R = S.row[x], C = S.col[y];
+          const int ro = R.orb, so = C.orb;
+          // the generator's own integrals and the pair's term of D, loaded ahead
+          // of the terms of the J reaching every cell
+          NT own = NT(0), own2 = NT(0);
+          long long dpair = 0;
+          if (fin && kind > 0) {
+            if constexpr (E4) {
+              own = eri_n[(R.idx & 0x7fffffff) + (C.idx & 0x7fffffff)];
+              if (kind == 1) own2 = eri_n[ibase + so * norb + ro];
+            } else {
+              own = eri_n[tri(R.idx & 0x7fffffff, C.idx & 0x7fffffff)];
+              if (kind == 1) own2 = eri_n[tri(S.row[y].idx & 0x7fffffff, S.col[x].idx & 0x7fffffff)];
+            }
+            dpair = (kind == 2 ? p.Ji : p.Wi)[ro * norb + so];
+          }
+          unsigned long long lo = 0ull;  // exact sum
+          int hi = 0;
+          double accs[kMaxStates];  // multi-state form: one sum per state
 #pragma unroll
-        for (int st = 0; st < kMaxStates; st++) accs[st] = 0.0;
-        if constexpr (!MS) {
-          lo = A0[cc] | ((unsigned long long)A1[cc] << 32);
-          hi = (int)A2[cc];
-        }
+          for (int st = 0; st < kMaxStates; st++) accs[st] = 0.0;
+          if constexpr (!MS) {
+            lo = A0[cc] | ((unsigned long long)A1[cc] << 32);
+            hi = (int)A2[cc];
+          }
 #pragma unroll 1
-        for (int j = 0; j < m; j++) {
-          const int rt = S.gRow[j][x], ct = S.gCol[j][y], rc = (int)((unsigned)rt + (unsigned)ct);
-          if ((rt | ct) & (3 << 29)) continue;
-          NT v;
-          bool neg = rc < 0;
-          if constexpr (E4) {
-            v = eri_n[rc & 0x7fffffff];
-            if (B.kind == 1) v -= eri_n[S.gB[j] + so * norb + ro];
-          } else {
-            v = eri_n[tri(rt & 0x1fffffff, ct & 0x1fffffff)];
-            if (B.kind == 1) v -= eri_n[tri(S.gRow[j][y] & 0x1fffffff, S.gCol[j][x] & 0x1fffffff)];
-          }
-          if (B.kind == 1) {
-            const int x2 = S.gx2[j];
-            neg ^= ro > (so < x2 ? so : x2) && ro < (so < x2 ? x2 : so);
-          }
-          v = flip_sign(v, neg);
-          con++;
-          if constexpr (MS) {
-#pragma unroll
-            for (int st = 0; st < kMaxStates; st++)
-              if (st < nst) accs[st] = fma(ms_gc[j * kMaxStates + st], (double)v, accs[st]);
-          } else {
-            unsigned long long l;
-            int hh;
-            fix_of(S.gcj[j] * v, F, l, hh);
-            fix_add(lo, hi, l, hh);
-          }
-        }
-        if (!fin) {
-          if constexpr (MS) {
-#pragma unroll
-            for (int st = 0; st < kMaxStates; st++)
-              if (st < nst) A[st * mc + cc] += accs[st];
-          } else {
-            A0[cc] = (uint32_t)lo;
-            A1[cc] = (uint32_t)(lo >> 32);
-            A2[cc] = (uint32_t)hi;
-          }
-          continue;
-        }
-        if constexpr (MS) {
-          double vI = 0.0;  // <I|H|alpha> for the generator's own term
-          if (B.h == 2) {
-            NT t = own;
-            bool neg = (R.idx ^ C.idx) < 0;
-            if (B.kind == 1) t -= own2;
-            if (B.kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
-            t = flip_sign(t, neg);
-            vI = (double)t;
+          for (int j = 0; j < m; j++) {
+            const int rt = S.gRow[j][x], ct = S.gCol[j][y], rc = (int)((unsigned)rt + (unsigned)ct);
+            if ((rt | ct) & (3 << 29)) continue;
+            NT v;
+            bool neg = rc < 0;
+            if constexpr (E4) {
+              v = eri_n[rc & 0x7fffffff];
+              if (kind == 1) v -= eri_n[S.gB[j] + so * norb + ro];
+            } else {
+              v = eri_n[tri(rt & 0x1fffffff, ct & 0x1fffffff)];
+              if (kind == 1) v -= eri_n[tri(S.gRow[j][y] & 0x1fffffff, S.gCol[j][x] & 0x1fffffff)];
+            }
+            if (kind == 1) {
+              const int x2 = S.gx2[j];
+              neg ^= ro > (so < x2 ? so : x2) && ro < (so < x2 ? x2 : so);
+            }
+            v = flip_sign(v, neg);
             con++;
-          }
-          long long D0 = R.d;  // E0_0 - H_aa
-          if (B.h == 2) D0 -= C.d + dpair;
-          double crit = 0.0, a0 = 0.0;
+            if constexpr (MS) {
 #pragma unroll
-          for (int st = 0; st < kMaxStates; st++) {
-            if (st >= nst) break;
-            const double a = A[st * mc + cc] + accs[st] + ms_cI[st] * vI;
-            const long long D = D0 + ms_de[st];
+              for (int st = 0; st < kMaxStates; st++)
+                if (st < nst) accs[st] = fma(ms_gc[j * kMaxStates + st], (double)v, accs[st]);
+            } else {
+              unsigned long long l;
+              int hh;
+              fix_of(S.gcj[j] * v, F, l, hh);
+              fix_add(lo, hi, l, hh);
+            }
+          }
+          if (!fin) {
+            if constexpr (MS) {
+#pragma unroll
+              for (int st = 0; st < kMaxStates; st++)
+                if (st < nst) A[st * mc + cc] += accs[st];
+            } else {
+              A0[cc] = (uint32_t)lo;
+              A1[cc] = (uint32_t)(lo >> 32);
+              A2[cc] = (uint32_t)hi;
+            }
+            continue;
+          }
+          if constexpr (MS) {
+            double vI = 0.0;  // <I|H|alpha> for the generator's own term
+            if (kind > 0) {
+              NT t = own;
+              bool neg = (R.idx ^ C.idx) < 0;
+              if (kind == 1) t -= own2;
+              if (kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
+              t = flip_sign(t, neg);
+              vI = (double)t;
+              con++;
+            }
+            long long D0 = R.d;  // E0_0 - H_aa
+            if (kind > 0) D0 -= C.d + dpair;
+            double crit = 0.0, a0 = 0.0;
+#pragma unroll
+            for (int st = 0; st < kMaxStates; st++) {
+              if (st >= nst) break;
+              const double a = A[st * mc + cc] + accs[st] + ms_cI[st] * vI;
+              const long long D = D0 + ms_de[st];
+              const double q = div_fix<MS>(a, D, E.dscale);
+              const double e = a * q;
+              acc_es[st] += e;
+              acc_s2s[st] += q * q;
+              crit += ms_w[st] * e;  // c_alpha,s A_s / max_I c_Is^2
+              const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
+              acc_min = db < acc_min ? db : acc_min;
+              if (st == 0) a0 = a;
+            }
+            acc_na++;
+            if (abs_bits(a0) < 0x3D06849B86A12B9Bull) atomicAdd(&S.tiny, 1u);
+            uint64_t key[NW];
+            const int kwr = B.sa * NINT + (ro >> 6), kws = (kind > 0) ? B.sb * NINT + (so >> 6) : -1;
+#pragma unroll
+            for (int w = 0; w < NW; w++)
+              key[w] = S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
+            uint64_t hk = 0;
+#pragma unroll
+            for (int w = 0; w < NW; w++) hk = splitmix64(hk ^ key[w]);
+            acc_d0 += hk;
+            acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
+            if (p.k > 0) {
+              const unsigned long long eb = abs_bits(crit);
+              if (eb >= tau) {
+                atomicAdd(&p.sel_hist[sel_bin(eb)], 1u);
+                const int pos = atomicAdd(&S.tkcnt, 1);
+                buf_e(p)[pos] = crit;
+                buf_a(p)[pos] = a0;
+#pragma unroll
+                for (int w = 0; w < NW; w++) buf_key<NINT>(p)[(size_t)pos * NW + w] = key[w];
+              }
+            }
+          } else {
+            double a = fix_to_double(lo, hi, F);
+            // the generator's own term c_I <I|H|alpha>
+            if (kind > 0) {
+              NT t = own;
+              bool neg = (R.idx ^ C.idx) < 0;
+              if (kind == 1) t -= own2;
+              if (kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
+              t = flip_sign(t, neg);
+              a += (double)(S.cI * t);
+            }
+            // D = E0 - H_aa from the row and column sums
+            long long D = R.d;
+            if (kind > 0) D -= C.d + dpair;
             const double q = div_fix<MS>(a, D, E.dscale);
-            const double e = a * q;
-            acc_es[st] += e;
-            acc_s2s[st] += q * q;
-            crit += ms_w[st] * e;  // c_alpha,s A_s / max_I c_Is^2
+            acc_e = fma(a, q, acc_e);  // e = A q
+            acc_s2 += q * q;
+            if (GRAD) {
+              // numerator weight 2A/D for loop 3, here already for the
+              // generator's own element; (A/D)^2 weights the diagonal
+              const double w1 = 2.0 * q;
+              const unsigned long long wb = (unsigned long long)__double_as_longlong(w1);
+              A0[cc] = (uint32_t)wb;
+              A1[cc] = (uint32_t)(wb >> 32);
+              if (kind > 0) {
+                w_grad(p, ro, B.sa, so, B.sb, q * q);
+                bool neg = (R.idx ^ C.idx) < 0;
+                if (kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
+                const double ws = flip_sign((double)S.cI * w1, neg);
+                atomicAdd(&p.g_deri[eri_index(B.qa, ro, B.qb, so)], ws);
+                if (kind == 1) atomicAdd(&p.g_deri[eri_index(B.qa, so, B.qb, ro)], -ws);
+              }
+            }
+            // |a| < 1e-14, compared on the bit pattern (no FP64 compare)
+            if (abs_bits(a) < 0x3D06849B86A12B9Bull) atomicAdd(&S.tiny, 1u);
             const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
             acc_min = db < acc_min ? db : acc_min;
-            if (st == 0) a0 = a;
-          }
-          acc_na++;
-          if (abs_bits(a0) < 0x3D06849B86A12B9Bull) atomicAdd(&S.tiny, 1u);
-          uint64_t key[NW];
-          const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
+            // alpha's word w: the batch's base with the cell's orbitals
+            const int kwr = B.sa * NINT + (ro >> 6), kws = (kind > 0) ? B.sb * NINT + (so >> 6) : -1;
+            auto key = [&](int w) {
+              return S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
+            };
+            // digest: the fold over the spin-up words is the row's where they
+            // depend on the row alone
+            uint64_t hk = S.hk0[x];
+            if (kind != 2 && B.sa == 0) {
+              hk = 0;
 #pragma unroll
-          for (int w = 0; w < NW; w++)
-            key[w] = S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
-          uint64_t hk = 0;
-#pragma unroll
-          for (int w = 0; w < NW; w++) hk = splitmix64(hk ^ key[w]);
-          acc_d0 += hk;
-          acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
-          if (p.k > 0) {
-            const unsigned long long eb = abs_bits(crit);
-            if (eb >= tau) {
-              atomicAdd(&p.sel_hist[sel_bin(eb)], 1u);
-              const int pos = atomicAdd(&S.tkcnt, 1);
-              buf_e(p)[pos] = crit;
-              buf_a(p)[pos] = a0;
-#pragma unroll
-              for (int w = 0; w < NW; w++) buf_key<NINT>(p)[(size_t)pos * NW + w] = key[w];
+              for (int w = 0; w < NINT; w++) hk = splitmix64(hk ^ key(w));
             }
-          }
-        } else {
-          double a = fix_to_double(lo, hi, F);
-          // the generator's own term c_I <I|H|alpha>
-          if (B.h == 2) {
-            NT t = own;
-            bool neg = (R.idx ^ C.idx) < 0;
-            if (B.kind == 1) t -= own2;
-            if (B.kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
-            t = flip_sign(t, neg);
-            a += (double)(S.cI * t);
-          }
-          // D = E0 - H_aa from the row and column sums
-          long long D = R.d;
-          if (B.h == 2) D -= C.d + dpair;
-          const double q = div_fix<MS>(a, D, E.dscale);
-          acc_e = fma(a, q, acc_e);  // e = A q
-          acc_s2 += q * q;
-          if (GRAD) {
-            // numerator weight 2A/D for loop 3, here already for the
-            // generator's own element; (A/D)^2 weights the diagonal
-            const double w1 = 2.0 * q;
-            const unsigned long long wb = (unsigned long long)__double_as_longlong(w1);
-            A0[cc] = (uint32_t)wb;
-            A1[cc] = (uint32_t)(wb >> 32);
-            if (B.h == 2) {
-              w_grad(p, ro, B.sa, so, B.sb, q * q);
-              bool neg = (R.idx ^ C.idx) < 0;
-              if (B.kind == 1) neg ^= ro > (so < B.qb ? so : B.qb) && ro < (so < B.qb ? B.qb : so);
-              const double ws = flip_sign((double)S.cI * w1, neg);
-              atomicAdd(&p.g_deri[eri_index(B.qa, ro, B.qb, so)], ws);
-              if (B.kind == 1) atomicAdd(&p.g_deri[eri_index(B.qa, so, B.qb, ro)], -ws);
-            }
-          }
-          // |a| < 1e-14, compared on the bit pattern (no FP64 compare)
-          if (abs_bits(a) < 0x3D06849B86A12B9Bull) atomicAdd(&S.tiny, 1u);
-          const unsigned long long db = D < 0 ? 0ull - (unsigned long long)D : (unsigned long long)D;
-          acc_min = db < acc_min ? db : acc_min;
-          // alpha's word w: the batch's base with the cell's orbitals
-          const int kwr = B.sa * NINT + (ro >> 6), kws = (B.h == 2) ? B.sb * NINT + (so >> 6) : -1;
-          auto key = [&](int w) {
-            return S.kbase[w] | (w == kwr ? 1ull << (ro & 63) : 0ull) | (w == kws ? 1ull << (so & 63) : 0ull);
-          };
-          // digest: the fold over the spin-up words is the row's where they
-          // depend on the row alone
-          uint64_t hk = S.hk0[x];
-          if (B.kind != 2 && B.sa == 0) {
-            hk = 0;
 #pragma unroll
-            for (int w = 0; w < NINT; w++) hk = splitmix64(hk ^ key(w));
-          }
+            for (int w = NINT; w < NW; w++) hk = splitmix64(hk ^ key(w));
+            acc_d0 += hk;
+            acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
+            // e = A q is formed only when it can reach the threshold: with biased
+            // exponents ea, eq of A and q, |A q| < 2^(ea + eq - 2044), so
+            // ea + eq <= et + 1021 (et: the exponent of tau) puts it below tau
+            const int ea = (int)(abs_bits(a) >> 52), eqx = (int)(abs_bits(q) >> 52);
+            if (p.k > 0 && (tau == 0ull || ea + eqx > (int)(tau >> 52) + 1021)) {
+              const double e = a * q;
+              const unsigned long long eb = abs_bits(e);
+              if (eb >= tau) {
+                atomicAdd(&p.sel_hist[sel_bin(eb)], 1u);
+                const int pos = atomicAdd(&S.tkcnt, 1);
+                buf_e(p)[pos] = e;
+                buf_a(p)[pos] = a;
 #pragma unroll
-          for (int w = NINT; w < NW; w++) hk = splitmix64(hk ^ key(w));
-          acc_d0 += hk;
-          acc_d1 ^= splitmix64(hk ^ 0x243F6A8885A308D3ull);
-          // e = A q is formed only when it can reach the threshold: with biased
-          // exponents ea, eq of A and q, |A q| < 2^(ea + eq - 2044), so
-          // ea + eq <= et + 1021 (et: the exponent of tau) puts it below tau
-          const int ea = (int)(abs_bits(a) >> 52), eqx = (int)(abs_bits(q) >> 52);
-          if (p.k > 0 && (tau == 0ull || ea + eqx > (int)(tau >> 52) + 1021)) {
-            const double e = a * q;
-            const unsigned long long eb = abs_bits(e);
-            if (eb >= tau) {
-              atomicAdd(&p.sel_hist[sel_bin(eb)], 1u);
-              const int pos = atomicAdd(&S.tkcnt, 1);
-              buf_e(p)[pos] = e;
-              buf_a(p)[pos] = a;
-#pragma unroll
-              for (int w = 0; w < NW; w++) buf_key<NINT>(p)[(size_t)pos * NW + w] = key(w);
+                for (int w = 0; w < NW; w++) buf_key<NINT>(p)[(size_t)pos * NW + w] = key(w);
+              }
             }
           }
         }
-      }
+      };
+      if (NINT == 1 && !MS && !GRAD && !by_kind(p)) cells(std::integral_constant<int, -1>{});
+      else if (B.kind == 2) cells(std::integral_constant<int, 2>{});
+      else if (B.kind == 1) cells(std::integral_constant<int, 1>{});
+      else cells(std::integral_constant<int, 0>{});
       if (!fin) continue;
       // ---- the item's sums.  The digest, min |D| and the tiny count are the
       // sweep's: this thread's shares stay in shared memory until the kernel
@@ -2800,12 +2832,14 @@ struct Drawer {
   }
   template <typename BS>
   __device__ __forceinline__ int entry(const BS& S, const SweepParams& p) const {
-    return (unsigned)pos < (unsigned)S.nlive ? (int)p.live[pos] : -1;
+    if ((unsigned)pos >= (unsigned)S.nlive) return -1;
+    return (int)p.live[pos < S.nfirst ? pos : p.wave_slots * p.nper - 1 - (pos - S.nfirst)];
   }
   // The first item of the sweep of p.
   template <typename BS, typename Fn>
   __device__ __forceinline__ void begin(BS& S, const SweepParams& p, int chunk, Fn&& take) {
-    S.nlive = *p.live_cnt;
+    S.nfirst = p.live_cnt[0];
+    S.nlive = S.nfirst + p.live_cnt[1];
     S.inext = S.iend = 0;
     draw(S, chunk, take);
     S.item[0] = entry(S, p);
