@@ -45,12 +45,13 @@ L2_FLUSH_BYTES = 256 << 20
 # one FMA of A_alpha += c_J <J|H|alpha>; per perturber the incremental
 # diagonal H_aa (about 20 operations: the Fock-diagonal and two-index terms
 # of the particles and holes), one division and two FMAs (e = A^2/D and the
-# sum of A^2/D^2).  The kernels form H_aa from per-batch row sums in 3 adds
-# and 1/D by a Newton reciprocal; the smallest form the kernels execute,
-# 9 operations per perturber, is reported beside it.
+# sum of A^2/D^2).  The kernels form H_aa, D and A/D in 64-bit integers, so
+# that this count can exceed what the FP64 pipe executes; the FP64 operations
+# they do execute, 4 per perturber (the generator's own product and its
+# addition, e and the sum of A^2/D^2), are reported beside it.
 FP64_OPS_PER_CONNECTION = 1
 FP64_OPS_PER_PERTURBER = 23
-FP64_OPS_PER_PERTURBER_MIN = 9
+FP64_OPS_PER_PERTURBER_MIN = 4
 # Integer work per unit: about 15 XOR/POPC/add operations per connection
 # (excitation degree and phase) per 64-bit word of a spin string, and
 # 2 x 2 x nint XOR+POPC per pair test of the coarse filter (N_det per
@@ -60,7 +61,7 @@ INT_OPS_PER_CONNECTION_PER_WORD = 15
 # waves) over one sweep of the bench workload, from one ncu capture of the
 # current kernels (dram__bytes_read.sum + dram__bytes_write.sum; None when
 # the kernels have changed since the capture).
-TRAFFIC_BYTES_PER_SWEEP = 18.099e9
+TRAFFIC_BYTES_PER_SWEEP = None
 
 
 def load_workload(name=WORKLOAD):
