@@ -61,7 +61,7 @@ INT_OPS_PER_CONNECTION_PER_WORD = 15
 # waves) over one sweep of the bench workload, from one ncu capture of the
 # current kernels (dram__bytes_read.sum + dram__bytes_write.sum; None when
 # the kernels have changed since the capture).
-TRAFFIC_BYTES_PER_SWEEP = None
+TRAFFIC_BYTES_PER_SWEEP = 9.050e9
 
 
 def load_workload(name=WORKLOAD):
