@@ -1,6 +1,7 @@
 // common.cuh -- device helpers and launch parameters of the sm_103a EN-PT2
 // sweep (Quantum Package 2.0, arXiv:1902.08154).  Internal to the library.
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -137,15 +138,29 @@ inline size_t wave_slot_bytes(size_t meta_bytes, int norb, int na, int nb, int n
          4 * (size_t)nper + 16 * (size_t)nper * (size_t)nst;
 }
 
+// The fixed-point unit of a sweep's denominators is 2^-62 of a power of two at
+// most the bound |E0| + n max|h| + n (n - 1) max|(pq|rs)|, n = n_el + 2; a
+// generator has that form where this power is at most kDenRange times the
+// magnitude of its energies (den_form in sweep_impl.cuh).  False: |E0| alone
+// is large enough for that, so that all generators have it.
+constexpr double kDenRange = 128.0;
+inline bool den_maybe_fp64(double hmax, double emax, int nel, double e0_max, double e0_min) {
+  const double n = (double)(nel + 2), bound = e0_max + n * hmax + n * (n - 1.0) * emax;
+  if (!(bound < 0.99e300)) return true;
+  int e;
+  frexp(bound, &e);  // bound < 2^e
+  return !(ldexp(1.0, e - 1 > -838 ? e - 1 : -838) <= kDenRange * e0_min);
+}
+
 // Per-generator data built by the prep kernel and read by the batch kernel.
 struct GenMeta {
   uint64_t I[4];            // generator determinant (2*NINT words used)
   int g;                    // rank of the generator (-1: empty slot)
   int nrec;                 // coarse-filter records
-  long long hii;            // <I|H|I>, fixed point (den_scale in sweep_impl.cuh)
+  long long hii;            // <I|H|I>, fixed point or the bits of FP64 (den_form in sweep_impl.cuh)
   double cI;                // c_I
   int occ[kMaxElec];        // spin-orbital codes s*norb+q of I, ordered
-  long long F[2][kMaxOrb];  // Fock diagonal of I, fixed point
+  long long F[2][kMaxOrb];  // Fock diagonal of I, likewise
 };
 
 struct SweepParams {
@@ -215,7 +230,8 @@ struct SweepParams {
   ulonglong2* e_hp;               // [slots][ent_cap]: hole mask, particles (one 16-byte load)
   uint32_t* e_rec;                // [slots][ent_cap]
   // the wave's work items (slot * nper + item), without those of batches
-  // banned as a whole, in the order the prep kernel finished the slots
+  // banned as a whole, in the order the prep kernel finished the slots (den64:
+  // those of generators with denominators in FP64 from the back)
   uint32_t* live;                 // [slots * nper]
   int* live_cnt;                  // per wave: items listed from the front, from the back; zero before the prep kernel
   int64_t ent_cap;
@@ -254,6 +270,7 @@ struct SweepParams {
   unsigned int* sel_hist;        // [kSelBins] counts of candidates offered to the buffers, by |e| bin
 
   int max_cells;
+  int den64;                     // 1: generators with denominators in FP64 are possible (den_maybe_fp64)
   int* err;                      // device error flags (0 = fine)
 
   // gradient of E_PT2 (Psi0 and E0 fixed); used by the GRAD batch kernel

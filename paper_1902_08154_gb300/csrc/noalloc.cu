@@ -247,13 +247,13 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     tk_tau = ncon + nd;
     sel_hist = reinterpret_cast<unsigned int*>(tk_tau + grid);
     tk_cnt = reinterpret_cast<int*>(sel_hist + kSelBins);
-    acc = cv.take<unsigned long long>(9);
+    acc = cv.take<unsigned long long>(11);
+    d_hmax = acc + 9;
     dres = cv.take<DevResult>(1);
     queues = cv.take<int>(3);  // the wave's item counter and live counts
     tk_e = cv.take<double>((size_t)cap * grid);
     tk_a = cv.take<double>((size_t)cap * grid);
     tk_key = cv.take<uint64_t>((size_t)cap * grid * nw);
-    d_hmax = cv.take<unsigned long long>(2);
     // the validation's arrays, the waves' and the selection's share the rest,
     // one phase after another on the stream
     Carve c1 = cv, c3 = cv;
@@ -318,12 +318,11 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
 
   // ---- clear what must start at zero; integral tables; validation ----
   // accumulator words: 0, 1 digest, 2 min |D|, 3 tiny, 4 threshold, 6 error
-  // flags, 7 candidates, 8 bits of max |c_I|
-  static const unsigned long long init[9] = {0, 0, 0x7FF0000000000000ull, 0, 0, 0, 0, 0, 0};
+  // flags, 7 candidates, 8 bits of max |c_I|, 9, 10 of max |h| and max |(pq|rs)|
+  static const unsigned long long init[11] = {0, 0, 0x7FF0000000000000ull};
   NTRY(cudaMemcpyAsync(acc, init, sizeof(init), cudaMemcpyHostToDevice, st));
   int* d_err = reinterpret_cast<int*>(acc + 6);
   int* d_ncand = reinterpret_cast<int*>(acc + 7);
-  NTRY(cudaMemsetAsync(d_hmax, 0, 2 * sizeof(unsigned long long), st));
   sym_kernel<<<(norb * norb + 255) / 256, 256, 0, st>>>(norb, h, d_err);
   const int64_t npair = (int64_t)norb * (norb + 1) / 2, P = npair * (npair + 1) / 2;
   absmax_kernel<<<(norb * norb + 255) / 256, 256, 0, st>>>((int64_t)norb * norb, h, d_hmax);
@@ -342,8 +341,12 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     rank_kernel<<<nb, 256, 0, st>>>(ndet, order, rank_of);
   }
   int herr = 0;
-  NTRY_Q(cudaMemcpyAsync(&herr, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  unsigned long long hval[5];  // the error flags to max |(pq|rs)|
+  NTRY_Q(cudaMemcpyAsync(hval, acc + 6, sizeof(hval), cudaMemcpyDeviceToHost, st));
   NTRY_Q(cudaStreamSynchronize(st));
+  memcpy(&herr, hval, sizeof(int));
+  double hmax[2];
+  memcpy(hmax, hval + 3, sizeof(hmax));
   if (herr & 16) return nfail(QP_ESYM, "h is not symmetric");
   if (herr & 1) return nfail(QP_EINVAL, "a determinant has the wrong occupation or bits beyond norb");
   if (herr & 4) return nfail(QP_EINVAL, "a coefficient is not finite");
@@ -411,6 +414,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   p.tau_bits = acc + 4;
   p.sel_hist = sel_hist;
   p.max_cells = max_cells;
+  p.den64 = den_maybe_fp64(hmax[0], hmax[1], nel, fabs(e0), fabs(e0));
   p.err = d_err;
   for (int64_t w = 0; w < nwaves; w++) {
     p.wave_start = (int)(w * W);

@@ -326,6 +326,7 @@ struct qp_pt2_ctx {
   double* d_eri4 = nullptr;                      // four-index layout (eri4_index)
   float* d_eri4_32 = nullptr;                    // its FP32 copy, mixed precision only
   unsigned long long* d_hmax = nullptr;        // bits of max |h|, max |(pq|rs)|
+  double hmax[2] = {0.0, 0.0};                 // the same on the host
   // workspace
   Buf in_dets, in_coefs, hkey, hkey2, hidx, hidx2, rkey, rkey2, order, rank_of, cub_tmp;
   Buf eps, s2, na, ncon, acc, res, zeroed;
@@ -506,7 +507,9 @@ extern "C" int qp_pt2_create(qp_pt2_ctx** out, int norb, int n_alpha, int n_beta
       return bail(QP_ENOMEM, "device allocation of the four-index integrals failed");
     eri4_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, x->st>>>(norb, x->d_eri, x->d_eri4, x->d_eri4_32);
   }
-  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(x->st) != cudaSuccess)
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync(x->hmax, x->d_hmax, sizeof(x->hmax), cudaMemcpyDeviceToHost, x->st) != cudaSuccess ||
+      cudaStreamSynchronize(x->st) != cudaSuccess)
     return bail(QP_ECUDA, "integral tables failed");
   if (c.tile < 0) return bail(QP_EINVAL, "tile must be >= 0");
   if (c.work_chunk < 0) return bail(QP_EINVAL, "work_chunk must be >= 0");
@@ -919,12 +922,19 @@ static int eval_core(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, const do
   p.tau_bits = acc + kAccTau;
   p.sel_hist = reinterpret_cast<unsigned int*>(zb + z_hist);
   p.max_cells = x->max_cells;
+  p.den64 = den_maybe_fp64(x->hmax[0], x->hmax[1], x->nel, fabs(e0), fabs(e0));
   p.err = d_err;
   p.it_stride = 2 * nsts;
   if (ms) {
     p.nst = nst;
     p.rc_stride = (int64_t)(nd * ws);
     for (int s = 0; s < nst; s++) p.st_e0[s] = e0s[s];
+    double lo = fabs(e0), hi = lo;
+    for (int s = 1; s < nst; s++) {
+      lo = std::min(lo, fabs(e0s[s]));
+      hi = std::max(hi, fabs(e0s[s]));
+    }
+    p.den64 = den_maybe_fp64(x->hmax[0], x->hmax[1], x->nel, hi, lo);
     p.st_cmax = x->st_cmax.as<unsigned long long>();
   }
   CUDA_TRY(cudaEventRecord(x->ev[1], st));
@@ -1303,6 +1313,7 @@ extern "C" int qp_pt2_grad(qp_pt2_ctx* x, int64_t ndet, const uint64_t* dets, co
   p.tau_bits = acc + kAccTau;
   p.sel_hist = x->sel_hist.as<unsigned int>();
   p.max_cells = x->max_cells;
+  p.den64 = den_maybe_fp64(x->hmax[0], x->hmax[1], x->nel, fabs(e0), fabs(e0));
   p.err = d_err;
   p.g_dh = d_dh;
   p.g_deri = d_deri;
@@ -1589,6 +1600,7 @@ static void make_params(BatchInst& b) {
   p.tau_bits = acc + kAccTau;
   p.sel_hist = x->sel_hist.as<unsigned int>();
   p.max_cells = b.max_cells;
+  p.den64 = den_maybe_fp64(x->hmax[0], x->hmax[1], x->nel, fabs(b.e0), fabs(b.e0));
   p.err = reinterpret_cast<int*>(acc + kAccErr);
   b.p = p;
 }

@@ -107,8 +107,6 @@ int batch_multi_blocks_per_sm(int nint, int mixed, size_t smem) {
 
 template __global__ void prep_kernel<1>(const __grid_constant__ SweepParams);
 template __global__ void prep_kernel<2>(const __grid_constant__ SweepParams);
-template __global__ void batch_kernel<1, double>(const __grid_constant__ SweepParams);
-template __global__ void batch_kernel<2, double>(const __grid_constant__ SweepParams);
 template __global__ void grad_gen_kernel<1>(const __grid_constant__ SweepParams);
 template __global__ void grad_gen_kernel<2>(const __grid_constant__ SweepParams);
 
@@ -140,14 +138,7 @@ cudaError_t launch_prep(int nint, const SweepParams& p, int slots, cudaStream_t 
 
 cudaError_t launch_batch(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
   if (p.mixed) return launch_batch_mixed(nint, p, grid, smem, st);
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_kernel<1, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    batch_kernel<1, double><<<grid, kThreads, smem, st>>>(p);
-  } else {
-    cudaFuncSetAttribute(batch_kernel<2, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    batch_kernel<2, double><<<grid, kThreads, smem, st>>>(p);
-  }
-  return cudaGetLastError();
+  return batch_launch<double>(nint, p, grid, smem, st);
 }
 
 int batch_blocks_per_sm(int nint, int mixed, size_t smem) {

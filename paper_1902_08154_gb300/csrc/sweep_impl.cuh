@@ -134,21 +134,31 @@ __device__ __forceinline__ const float* numer_h<float>(const SweepParams& p) { r
 // (a 64-bit integer add 1, a high 64-bit product 5.5), so the two FP64
 // additions of D and the five operations of its reciprocal were most of the
 // cells pass.  S is the same for a whole sweep:
-// |D| <= |E0| + n_el max|h| + n_el (n_el - 1) max|(pq|rs)| < 2^(62 - S), and
-// sums of table entries on the way may wrap.  The units are finer than the
-// rounding of the same sums in FP64 (2^-51 Eh against 2^-45 on 64 orbitals).
+// |D| <= |E0| + n_el max|h| + n_el (n_el - 1) max|(pq|rs)| < 2^(63 - S), and
+// sums of table entries on the way may wrap.
+// That bound is over all orbitals, whichever a perturber has: one large entry
+// of h or of the integrals (a level-shifted orbital, a tight virtual one) makes
+// the unit coarse for every D, while FP64 sums lose digits only where they
+// contain it.  So a generator has this form only where the unit is at most
+// 2^-55 of the sums that make up its H_II (or of E0 where that is larger),
+// whose rounding each of its FP64 denominators carries; otherwise its energies
+// and denominators stay in FP64 (den_form) and its items go to the FP64 form
+// of the batch kernel.  2^62 units against those sums: 2^2.4 to 2^4.7 on the
+// workloads of 14 to 64 orbitals and 3 to 26 electrons, up to 2^7.2 with 64
+// electrons; with one h_pp of 10^4 2^12, where D is up to 18 times further off
+// than in FP64, with one of 10^6 2^19 and 8,000 times.
 // Two states at once, 2,000 determinants, 64 orbitals: 43 to 33.8 ms (two
 // quotients per cell); one state, 10^4 determinants 113.3 to 111.8 ms; 10^3
 // determinants, 128 orbitals 87.1 to 84.1 ms.
 // ---------------------------------------------------------------------------
-constexpr int kBadScale = 1 << 20;  // integrals not finite: every quotient is NaN
+constexpr int kDenFp64 = 1 << 20;  // in the place of S: energies as the bits of FP64 numbers
 __device__ __forceinline__ int den_scale(const SweepParams& p) {
   const double hmx = __longlong_as_double((long long)p.hmax_bits[0]);
   const double emx = __longlong_as_double((long long)p.hmax_bits[1]);
   double e0 = fabs(p.e0);
   for (int s = 0; s < p.nst; s++) e0 = fmax(e0, fabs(p.st_e0[s]));
   const double n = (double)(p.nel + 2), bound = e0 + n * hmx + n * (n - 1.0) * emx;
-  if (!(bound < 1e300)) return kBadScale;
+  if (!(bound < 1e300)) return kDenFp64;  // or not finite
   const int e = (int)((((unsigned long long)__double_as_longlong(bound)) >> 52) & 0x7FF) - 1023;
   return 62 - e < 900 ? 62 - e : 900;
 }
@@ -156,18 +166,22 @@ __device__ __forceinline__ int den_scale(const SweepParams& p) {
 __device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 // x in units of 2^-S.
 __device__ __forceinline__ long long den_fix(double x, int S) {
-  return S == kBadScale ? 0ll : __double2ll_rn(x * pow2(S));
+  return S == kDenFp64 ? 0ll : __double2ll_rn(x * pow2(S));
 }
-__device__ __forceinline__ double den_double(unsigned long long um, int S) {
-  return S == kBadScale ? __longlong_as_double(0x7FF8000000000000ll) : (double)um * pow2(-S);
+__device__ __forceinline__ double den_double(unsigned long long um, int S) { return (double)um * pow2(-S); }
+// The form of a generator's denominators: S, or kDenFp64 where that unit is
+// too coarse.  sum: of |h_ii| and |F(i)| over its orbitals, twice what H_II's
+// partial sums reach.
+__device__ __forceinline__ int den_form(const SweepParams& p, int S, double sum) {
+  if (S == kDenFp64) return S;
+  double e0 = fabs(p.nst > 0 ? p.st_e0[0] : p.e0);
+  for (int s = 1; s < p.nst; s++) e0 = fmin(e0, fabs(p.st_e0[s]));
+  return pow2(62 - S) <= kDenRange * fmax(e0, 0.5 * sum) ? S : kDenFp64;
 }
 
 // a / (d 2^-S) for a quotient outside the normal range, a zero denominator
 // or operands that are not finite.
-static __device__ __noinline__ double div_slow(double a, long long d, int S) {
-  if (S == kBadScale) return __longlong_as_double(0x7FF8000000000000ll);
-  return a / ((double)d * pow2(-S));
-}
+static __device__ __noinline__ double div_slow(double a, long long d, int S) { return a / ((double)d * pow2(-S)); }
 
 // a / (d 2^-S): the reciprocal of the normalised 64-bit magnitude m of d from
 // the FP32 approximation of its top 24 bits (relative error e below 2^-21) by
@@ -204,7 +218,7 @@ __device__ __forceinline__ double div_core(double a, long long d, int S, bool* b
   return __longlong_as_double((long long)(v | ((ab ^ (unsigned long long)d) & 0x8000000000000000ull)));
 }
 __device__ __forceinline__ double div_rest(double a, long long d, int S) {
-  if (((__double_as_longlong(a) >> 52) & 0x7FF) == 0 && d != 0 && S != kBadScale) return 0.0;
+  if (((__double_as_longlong(a) >> 52) & 0x7FF) == 0 && d != 0) return 0.0;
   return div_slow(a, d, S);
 }
 template <bool SMALL>
@@ -444,9 +458,10 @@ struct Batch {
 // 79.0 without the order; opposite-spin first 74.4).  Smaller waves are taken
 // as they come: 9,900 items 415 us, by kind 425; 50,400 items of 240
 // generators 10.35 ms, by kind 10.4 to 10.9; 184,000 items 5.28, by kind 5.00.
+// (Not where the back of the list is the FP64 form's, den64.)
 constexpr long long kItemsByKind = 65536;
 __device__ __forceinline__ bool by_kind(const SweepParams& p) {
-  return (long long)p.wave_slots * p.nper >= kItemsByKind;
+  return !p.den64 && (long long)p.wave_slots * p.nper >= kItemsByKind;
 }
 
 // Batch and tile of work item j of a generator: j < nbat is batch j (the first
@@ -513,6 +528,8 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   __shared__ unsigned char s_vidx[2][kMaxOrb];
   __shared__ double s_F[2 * kMaxOrb];
   __shared__ int s_nrec[2];    // records of degree 3 at most, of degree 4
+  __shared__ int s_form;       // den_form of I, and H_II (with den64)
+  __shared__ double s_hii;
   __shared__ int s_below[NW];  // I's electrons in the words before
   extern __shared__ __align__(16) unsigned char dyn[];
   uint32_t* sm = reinterpret_cast<uint32_t*>(dyn);               // cell masks (MaskDims)
@@ -582,6 +599,15 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
       e += p.h[q * norb + q] + s_F[c];
     }
     M->hii = den_fix(0.5 * e, S);
+    if (p.den64) s_hii = 0.5 * e;
+  } else if (p.den64 && tid >> 5 == 1) {
+    double sum = 0.0;
+    for (int i = tid & 31; i < nel; i += 32) {
+      const int c = s_occ[i], q = c >= norb ? c - norb : c;
+      sum += fabs(p.h[q * norb + q]) + fabs(s_F[c]);
+    }
+    sum = warp_sum(sum);
+    if (tid == 32) s_form = den_form(p, S, sum);
   }
 
   // ---- coarse filter: J within degree 4 of I (I itself included): those of
@@ -705,6 +731,11 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
     s_vidx[s][q] = (unsigned char)(q - below);
   }
   __syncthreads();
+  const bool den64 = p.den64 && s_form == kDenFp64;
+  if (den64) {
+    for (int x = tid; x < 2 * norb; x += kThreads) M->F[x >= norb][x >= norb ? x - norb : x] = __double_as_longlong(s_F[x]);
+    if (tid == 0) M->hii = __double_as_longlong(s_hii);
+  }
   const int nlow = s_nrec[0], nfour = s_nrec[1];
   const size_t r4 = (size_t)p.ndet - nfour;  // first record of degree 4
   if (tid == 0) M->nrec = nlow + nfour;
@@ -778,7 +809,7 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
   __syncthreads();
   // the slot's work items, without those of batches banned as a whole; by
   // kind: the opposite-spin ones from the back of the list, taken after the
-  // others
+  // others (den64: those of FP64 generators from the back)
   const bool mixed = !by_kind(p);
   for (int j0 = 0; j0 < p.nper; j0 += kThreads) {
     const int j = j0 + tid;
@@ -789,7 +820,7 @@ __device__ __forceinline__ void prep_slot(const SweepParams& p, const int slot) 
       Batch B;
       batch_geometry(p, b, tile, B);
       live = B.nct > 0 && !((s_dead[b >> 5] >> (b & 31)) & 1u);
-      first = mixed || B.kind != 2;
+      first = mixed ? !den64 : B.kind != 2;
     }
     const unsigned lf = __ballot_sync(kFull, live && first), ll = __ballot_sync(kFull, live && !first);
     int at = 0;
@@ -1047,6 +1078,46 @@ __device__ __forceinline__ void cell_orbitals(const Batch& B, const BatchShared<
     *r = S.vir[B.sa][*x];
     *s = S.vir[B.sa][yy];
   }
+}
+
+// The FP64 form of the denominators (kDenFp64): the rows' and columns' terms,
+// u = F - W(q, a) [- W(q, b)] of a column, (E0 - base) - u of a row, base = H_II -
+// F(a) [- F(b) + W(a, b)]; all threads, with S.vir set.
+template <int NINT, typename NT>
+__device__ __forceinline__ void den64_sides(const SweepParams& p, BatchShared<NINT, NT>& S, const Batch& B,
+                                            const GenMeta* M, double e0) {
+  const int norb = p.norb;
+  auto F = [&](int s, int q) { return __longlong_as_double(M->F[s][q]); };
+  auto W = [&](int x, int sx, int y, int sy) {
+    const double j = p.Jm[x * norb + y];
+    return sx == sy ? j - p.Km[x * norb + y] : j;
+  };
+  double base = __longlong_as_double(M->hii) - F(B.sa, B.qa);
+  if (B.h == 2) base = base - F(B.sb, B.qb) + W(B.qa, B.sa, B.qb, B.sb);
+  for (int c = 0; c < B.h; c++) {
+    const int s = c ? B.sb : B.sa;
+    for (int v = threadIdx.x; v < S.nv[s]; v += kThreads) {
+      const int q = S.vir[s][v];
+      double u = F(s, q) - W(q, s, B.qa, B.sa);
+      if (B.h == 2) u -= W(q, s, B.qb, B.sb);
+      if (c) S.col[v].d = __double_as_longlong(u);
+      else S.row[v].d = __double_as_longlong((e0 - base) - u);
+    }
+  }
+}
+// a / D, D = (row - column - pair) + de of a cell with the orbitals of r and c
+// (kind 0: row + de); *D becomes the bits of |D|.
+template <typename Side>
+__device__ __forceinline__ double den64_quot(const SweepParams& p, double a, const Side& r, const Side& c, int kind,
+                                             double de, long long* D) {
+  double d = __longlong_as_double(r.d);
+  if (kind > 0) {
+    const int at = r.orb * p.norb + c.orb;
+    d -= __longlong_as_double(c.d) + (kind == 1 ? p.Jm[at] - p.Km[at] : p.Jm[at]);
+  }
+  d += de;
+  *D = __double_as_longlong(fabs(d));
+  return a / d;
 }
 
 // Bans cell c (an index over the whole batch) when it lies in this item's tile.
@@ -1598,7 +1669,7 @@ __device__ __forceinline__ uint64_t* buf_key(const SweepParams& p) {
   return p.tk_key + (size_t)blockIdx.x * (size_t)p.cap * (2 * NINT);
 }
 
-template <int NINT, typename NT, bool GRAD, bool MS, bool E4>
+template <int NINT, typename NT, bool GRAD, bool MS, bool E4, bool FP>
 __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NINT, NT>& S, const long long item,
                                            const int F, const ItemEnv& E,
                                            const NT* eri_n, const NT* h_n) {
@@ -1773,6 +1844,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
     if (tid < NW) S.rowban[tid] = om[tid] | om[(4 + 3 * B.ia) * NINT + tid] | om[(4 + 3 * B.ib) * NINT + tid];
   }
   __syncthreads();
+  if constexpr (FP) den64_sides<NINT, NT>(p, S, B, M, MS ? p.st_e0[0] : p.e0);
   if (B.h == 1) {
     const uint64_t *b1 = om + (2 + B.sa) * NINT, *h1 = om + (6 + 3 * B.ia) * NINT;
 #pragma unroll 1
@@ -2379,7 +2451,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
       }
       const unsigned long long tau = S.tau;
       double acc_e = 0.0, acc_s2 = 0.0;
-      unsigned long long acc_d0 = 0, acc_d1 = 0, acc_min = ~0ull;  // acc_min: units of 2^-S
+      unsigned long long acc_d0 = 0, acc_d1 = 0, acc_min = ~0ull;  // acc_min: units of 2^-S (FP: bits of |D|)
       unsigned int acc_na = 0;  // multi-state form
       double acc_es[kMaxStates], acc_s2s[kMaxStates];  // multi-state form: sums per state
 #pragma unroll
@@ -2487,8 +2559,8 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             for (int st = 0; st < kMaxStates; st++) {
               if (st >= nst) break;
               const double a = A[st * mc + cc] + accs[st] + ms_cI[st] * vI;
-              const long long D = D0 + ms_de[st];
-              const double q = div_fix<MS>(a, D, E.dscale);
+              long long D = D0 + ms_de[st];
+              const double q = FP ? den64_quot(p, a, R, C, kind, p.st_e0[st] - p.st_e0[0], &D) : div_fix<MS>(a, D, E.dscale);
               const double e = a * q;
               acc_es[st] += e;
               acc_s2s[st] += q * q;
@@ -2534,7 +2606,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
             // D = E0 - H_aa from the row and column sums
             long long D = R.d;
             if (kind > 0) D -= C.d + dpair;
-            const double q = div_fix<MS>(a, D, E.dscale);
+            const double q = FP ? den64_quot(p, a, R, C, kind, 0.0, &D) : div_fix<MS>(a, D, E.dscale);
             acc_e = fma(a, q, acc_e);  // e = A q
             acc_s2 += q * q;
             if (GRAD) {
@@ -2593,7 +2665,7 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
           }
         }
       };
-      if (NINT == 1 && !MS && !GRAD && !by_kind(p)) cells(std::integral_constant<int, -1>{});
+      if (FP || (NINT == 1 && !MS && !GRAD && !by_kind(p))) cells(std::integral_constant<int, -1>{});
       else if (B.kind == 2) cells(std::integral_constant<int, 2>{});
       else if (B.kind == 1) cells(std::integral_constant<int, 1>{});
       else cells(std::integral_constant<int, 0>{});
@@ -2786,14 +2858,14 @@ __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NIN
 }
 
 // This CTA's digest, min |D| and tiny counts into the sweep's totals.
-template <int NINT, typename NT>
+template <int NINT, typename NT, bool FP>
 __device__ __forceinline__ void flush_totals(const SweepParams& p, BatchShared<NINT, NT>& S, int dscale) {
   const int tid = threadIdx.x, lane = tid & 31;
   const unsigned long long d0 = warp_sum_u(S.td0[tid]), d1 = warp_xor_u(S.td1[tid]), mn = warp_min_u(S.tmin[tid]);
   if (lane == 0 && mn != ~0ull) {
     atomicAdd(&p.digest[0], d0);
     atomicXor(&p.digest[1], d1);
-    atomicMin(p.min_den_bits, (unsigned long long)__double_as_longlong(den_double(mn, dscale)));
+    atomicMin(p.min_den_bits, FP ? mn : (unsigned long long)__double_as_longlong(den_double(mn, dscale)));
   }
   if (tid == 0 && S.tiny) atomicAdd(p.n_tiny, (unsigned long long)S.tiny);
 }
@@ -2835,11 +2907,12 @@ struct Drawer {
     if ((unsigned)pos >= (unsigned)S.nlive) return -1;
     return (int)p.live[pos < S.nfirst ? pos : p.wave_slots * p.nper - 1 - (pos - S.nfirst)];
   }
-  // The first item of the sweep of p.
-  template <typename BS, typename Fn>
+  // The first item of the sweep of p.  FP: of the items listed for the FP64
+  // form (den64), else of the others.
+  template <bool FP, typename BS, typename Fn>
   __device__ __forceinline__ void begin(BS& S, const SweepParams& p, int chunk, Fn&& take) {
-    S.nfirst = p.live_cnt[0];
-    S.nlive = S.nfirst + p.live_cnt[1];
+    S.nfirst = FP ? 0 : p.live_cnt[0];
+    S.nlive = S.nfirst + (FP == (p.den64 != 0) ? p.live_cnt[1] : 0);
     S.inext = S.iend = 0;
     draw(S, chunk, take);
     S.item[0] = entry(S, p);
@@ -2860,6 +2933,10 @@ struct Drawer {
 // kernels take the registers of two CTAs and do not spill; so does the
 // gradient's, whose row pass is there twice (17.8 -> 17.5 ms).
 //
+// FP = true: the items of the generators whose denominators are in FP64
+// (den_form), which another launch runs after the others' items; as a branch of
+// one kernel that form took 2% of every sweep's time.
+//
 // MS = true: the multi-state form (several states at once, FP64 only).
 // Each state s has its own accumulator A_s (dynamic shared memory, one
 // stride of max_cells each); a (J, cell) element is formed once and added
@@ -2867,7 +2944,7 @@ struct Drawer {
 // for every state, sums each into its own eps and s2, and offers the
 // determinant to the selection with the criterion sum_s w_s e_s,
 // w_s = 1/max_I c_Is^2 (Sec. "Selected CI", the criterion of Angeli et al.).
-template <int NINT, typename NT, bool GRAD = false, bool MS = false, bool E4 = true>
+template <int NINT, typename NT, bool GRAD = false, bool MS = false, bool E4 = true, bool FP = false>
 __global__ void __launch_bounds__(kThreads, (NINT == 1 && !GRAD) ? 3 : 2) batch_kernel(const __grid_constant__ SweepParams p) {
   static_assert(!(MS && GRAD), "the gradient is a one-state form");
   static_assert(!MS || sizeof(NT) == 8, "the multi-state form is FP64");
@@ -2889,7 +2966,7 @@ __global__ void __launch_bounds__(kThreads, (NINT == 1 && !GRAD) ? 3 : 2) batch_
   Drawer D;
   if (tid == 0) {
     if (p.timeout_ns) atomicCAS(p.t_start, 0ull, global_ns());
-    D.begin(S, p, p.chunk, take);
+    D.begin<FP>(S, p, p.chunk, take);
   }
   for (int par = 0;; par ^= 1) {
     __syncthreads();
@@ -2902,9 +2979,9 @@ __global__ void __launch_bounds__(kThreads, (NINT == 1 && !GRAD) ? 3 : 2) batch_
       }
       D.advance(S, p, par, p.chunk, take);
     }
-    batch_item<NINT, NT, GRAD, MS, E4>(p, S, item, F, E, eri_n, h_n);
+    batch_item<NINT, NT, GRAD, MS, E4, FP>(p, S, item, F, E, eri_n, h_n);
   }
-  flush_totals<NINT, NT>(p, S, E.dscale);
+  flush_totals<NINT, NT, FP>(p, S, E.dscale);
   if (p.k > 0 && p.last_wave) compact_selection<NINT, NT>(p, S, buf_e(p), buf_a(p), buf_key<NINT>(p));
   __syncthreads();
   if (tid == 0) {
@@ -2923,7 +3000,7 @@ __global__ void __launch_bounds__(kThreads, (NINT == 1 && !GRAD) ? 3 : 2) batch_
 // Every instance has its own candidate buffers for each CTA of the launch;
 // they are compacted to k entries by compact_multi_kernel after the last
 // wave.
-template <int NINT, typename NT>
+template <int NINT, typename NT, bool FP = false>
 __global__ void __launch_bounds__(kThreads, (NINT == 1) ? 3 : 2) batch_multi_kernel(const __grid_constant__ MultiWaveInline m) {
   __shared__ BatchShared<NINT, NT> S;
   const int tid = threadIdx.x;
@@ -2945,7 +3022,7 @@ __global__ void __launch_bounds__(kThreads, (NINT == 1) ? 3 : 2) batch_multi_ker
       return true;
     };
     Drawer D;
-    if (tid == 0) D.begin(S, p, m.chunk, take);
+    if (tid == 0) D.begin<FP>(S, p, m.chunk, take);
     for (int par = 0;; par ^= 1) {
       __syncthreads();
       const int item = S.item[par];
@@ -2957,9 +3034,9 @@ __global__ void __launch_bounds__(kThreads, (NINT == 1) ? 3 : 2) batch_multi_ker
         }
         D.advance(S, p, par, m.chunk, take);
       }
-      batch_item<NINT, NT, false, false, true>(p, S, item, F, E, numer_eri<NT, true>(p), numer_h<NT>(p));
+      batch_item<NINT, NT, false, false, true, FP>(p, S, item, F, E, numer_eri<NT, true>(p), numer_h<NT>(p));
     }
-    flush_totals<NINT, NT>(p, S, E.dscale);
+    flush_totals<NINT, NT, FP>(p, S, E.dscale);
     __syncthreads();
     if (tid == 0) {
       p.tk_cnt[blockIdx.x] = S.tkcnt;
@@ -2990,21 +3067,52 @@ __global__ void __launch_bounds__(kThreads) compact_multi_kernel(const SweepPara
   }
 }
 
+// The batch launches of one wave: with den64 the FP64 form's items after the
+// others, from the queue again.
+template <int NINT, typename NT, bool GRAD, bool MS, bool E4>
+static cudaError_t batch_launch_nint(const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
+  auto go = [&](auto* k) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k<<<grid, kThreads, smem, st>>>(p);
+  };
+  go(batch_kernel<NINT, NT, GRAD, MS, E4, false>);
+  if (p.den64) {
+    const cudaError_t e = cudaMemsetAsync(p.queue, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    go(batch_kernel<NINT, NT, GRAD, MS, E4, true>);
+  }
+  return cudaGetLastError();
+}
+template <typename NT, bool GRAD = false, bool MS = false, bool E4 = true>
+static cudaError_t batch_launch(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
+  return nint == 1 ? batch_launch_nint<1, NT, GRAD, MS, E4>(p, grid, smem, st)
+                   : batch_launch_nint<2, NT, GRAD, MS, E4>(p, grid, smem, st);
+}
+
 // Launch helpers of the multi-instance batch kernels, instantiated for FP64
 // in sweep.cu and for the mixed form in sweep_mixed.cu (the prep kernel is
 // launched from sweep.cu only).
+template <int NINT, typename NT>
+static cudaError_t multi_launch_nint(const MultiWaveInline& m, int grid, size_t smem, cudaStream_t st) {
+  auto go = [&](auto* k) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k<<<grid, kThreads, smem, st>>>(m);
+  };
+  go(batch_multi_kernel<NINT, NT, false>);
+  bool den64 = false;
+  for (int i = 0; i < m.n; i++) den64 |= m.ps[i].den64 != 0;
+  if (den64) {
+    const cudaError_t e = cudaMemsetAsync(m.queue, 0, sizeof(unsigned long long) * m.n, st);
+    if (e != cudaSuccess) return e;
+    go(batch_multi_kernel<NINT, NT, true>);
+  }
+  return cudaGetLastError();
+}
 template <typename NT>
 static cudaError_t multi_wave_launch(int nint, const MultiWaveInline& m, int total_slots, int grid, size_t smem,
                                      cudaStream_t st) {
   if (total_slots <= 0) return cudaSuccess;
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_multi_kernel<1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    batch_multi_kernel<1, NT><<<grid, kThreads, smem, st>>>(m);
-  } else {
-    cudaFuncSetAttribute(batch_multi_kernel<2, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    batch_multi_kernel<2, NT><<<grid, kThreads, smem, st>>>(m);
-  }
-  return cudaGetLastError();
+  return nint == 1 ? multi_launch_nint<1, NT>(m, grid, smem, st) : multi_launch_nint<2, NT>(m, grid, smem, st);
 }
 
 template <typename NT>

@@ -4,18 +4,8 @@
 
 namespace qp {
 
-template __global__ void batch_kernel<1, float>(const __grid_constant__ SweepParams);
-template __global__ void batch_kernel<2, float>(const __grid_constant__ SweepParams);
-
 cudaError_t launch_batch_mixed(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_kernel<1, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    batch_kernel<1, float><<<grid, kThreads, smem, st>>>(p);
-  } else {
-    cudaFuncSetAttribute(batch_kernel<2, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    batch_kernel<2, float><<<grid, kThreads, smem, st>>>(p);
-  }
-  return cudaGetLastError();
+  return batch_launch<float>(nint, p, grid, smem, st);
 }
 
 cudaError_t launch_wave_multi_mixed(int nint, const MultiWaveInline& m, int total_slots, int grid, size_t smem,

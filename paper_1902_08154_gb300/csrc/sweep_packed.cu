@@ -6,20 +6,8 @@
 
 namespace qp {
 
-template __global__ void batch_kernel<1, double, false, false, false>(const __grid_constant__ SweepParams);
-template __global__ void batch_kernel<2, double, false, false, false>(const __grid_constant__ SweepParams);
-
 cudaError_t launch_batch_packed(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_kernel<1, double, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    batch_kernel<1, double, false, false, false><<<grid, kThreads, smem, st>>>(p);
-  } else {
-    cudaFuncSetAttribute(batch_kernel<2, double, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    batch_kernel<2, double, false, false, false><<<grid, kThreads, smem, st>>>(p);
-  }
-  return cudaGetLastError();
+  return batch_launch<double, false, false, false>(nint, p, grid, smem, st);
 }
 
 int batch_blocks_per_sm_packed(int nint, size_t smem) {

@@ -5,9 +5,6 @@
 
 namespace qp {
 
-template __global__ void batch_kernel<1, double, false, true>(const __grid_constant__ SweepParams);
-template __global__ void batch_kernel<2, double, false, true>(const __grid_constant__ SweepParams);
-
 // Dynamic shared memory of the multi-state form: nst accumulators of
 // max_cells doubles, the ban bitmap (rounded to 8 bytes), the group's
 // per-state coefficients, c_I per state, the weights and
@@ -40,16 +37,7 @@ int batch_blocks_per_sm_states(int nint, size_t smem) {
 }
 
 cudaError_t launch_batch_states(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_kernel<1, double, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    batch_kernel<1, double, false, true><<<grid, kThreads, smem, st>>>(p);
-  } else {
-    cudaFuncSetAttribute(batch_kernel<2, double, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    batch_kernel<2, double, false, true><<<grid, kThreads, smem, st>>>(p);
-  }
-  return cudaGetLastError();
+  return batch_launch<double, false, true>(nint, p, grid, smem, st);
 }
 
 }  // namespace qp
