@@ -117,7 +117,8 @@ typedef struct {
     int tile;           /* tiles of rows each opposite-spin two-hole batch is split
                            into (its accumulator shrinks by that factor, so more
                            CTAs share an SM); 0 = chosen by the library (2 when
-                           the whole accumulator fits only once per SM, else 1) */
+                           the whole accumulator fits only once per SM, else 1);
+                           1 is taken as 2 where one does not fit on an SM */
     double timeout_s;   /* device watchdog: 0 = none; otherwise CTAs stop taking
                            work items once timeout_s seconds of device time have
                            passed since the call's sweep started, and the call

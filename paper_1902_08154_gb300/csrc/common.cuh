@@ -116,6 +116,16 @@ __host__ __device__ inline int mask_words(int norb, int na, int nb) {  // even: 
 // [2][nint] and one-hole cells [nint].
 __host__ __device__ inline int orb_mask_words(int nint, int nel) { return (4 + 3 * nel) * nint; }
 
+// Cells of the largest work item when the opposite-spin batches are split
+// into t tiles of rows.
+inline int cells_for_tile(int norb, int n_alpha, int n_beta, int t) {
+  const int va = norb - n_alpha, vb = norb - n_beta;
+  int m = (n_alpha > 0 && n_beta > 0) ? ((va + t - 1) / t) * vb : 0;
+  const int others[4] = {va, vb, va * (va - 1) / 2, vb * (vb - 1) / 2};
+  for (int o : others) m = o > m ? o : m;
+  return m < 1 ? 1 : m;
+}
+
 // Dynamic shared memory of the one-state batch kernel for mc cells: A_alpha
 // as a 96-bit integer per cell (three 32-bit words; the exact accumulation in
 // sweep_impl.cuh), one ban bit per cell and the list of the cells left (16 bits

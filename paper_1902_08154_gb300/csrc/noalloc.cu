@@ -120,18 +120,6 @@ bool on_device(const void* p, int dev) {
   return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
-int cells_max(int norb, int na, int nb) {
-  const int va = norb - na, vb = norb - nb;
-  int m = va > vb ? va : vb;
-  int t = va * (va - 1) / 2;
-  m = t > m ? t : m;
-  t = vb * (vb - 1) / 2;
-  m = t > m ? t : m;
-  t = va * vb;
-  m = t > m ? t : m;
-  return m < 1 ? 1 : m;
-}
-
 }  // namespace
 
 // The fixed device array all calls share (see the file header).
@@ -194,16 +182,25 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   // ---- sizes and layout ----
   const int nint = (norb - 1) / 64 + 1, nw = 2 * nint, nel = n_alpha + n_beta;
   const int nbat = nel + nel * (nel - 1) / 2;
-  const int max_cells = cells_max(norb, n_alpha, n_beta);
-  const size_t smem = sweep_smem(max_cells);
-  const int bps = batch_blocks_per_sm_packed(nint, smem);
+  // the opposite-spin batches in two tiles of rows where their accumulator
+  // does not fit on an SM (above 14,830 cells: 125 orbitals and more with a few
+  // electrons)
+  int ntile = 1, max_cells = cells_for_tile(norb, n_alpha, n_beta, 1);
+  size_t smem = sweep_smem(max_cells);
+  int bps = batch_blocks_per_sm_packed(nint, smem);
+  if (bps < 1 && n_alpha > 0 && n_beta > 0) {
+    ntile = 2;
+    max_cells = cells_for_tile(norb, n_alpha, n_beta, 2);
+    smem = sweep_smem(max_cells);
+    bps = batch_blocks_per_sm_packed(nint, smem);
+  }
   if (bps < 1) return nfail(QP_ENOTSUP, "batch accumulator exceeds shared memory");
   int nsm = 0;
   NTRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const size_t nd = (size_t)ndet;
   const int64_t cap = k > 0 ? k + max_cells : 1, ngen = ndet;
   const int64_t ent_cap = (int64_t)nd * bucket_entries_per_record(nel);
-  const int nper = nbat;
+  const int nper = nbat + (ntile - 1) * n_alpha * n_beta;
   size_t maxc = 0, tmp1 = 0, tmp2 = 0, zeroed = 0;
   int64_t W = 0, nwaves = 0;
   double *d_J = nullptr, *d_K = nullptr, *eps = nullptr, *s2 = nullptr, *tk_e = nullptr;
@@ -360,7 +357,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   p.nbeta = n_beta;
   p.nel = nel;
   p.nbat = nbat;
-  p.ntile = 1;
+  p.ntile = ntile;
   p.chunk = 1;
   p.timeout_ns = 0ull;
   p.t_start = nullptr;

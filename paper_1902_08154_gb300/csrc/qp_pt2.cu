@@ -413,16 +413,6 @@ static bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Cells of the largest work item when the opposite-spin batches are split
-// into t tiles of rows.
-static int cells_for_tile(int norb, int n_alpha, int n_beta, int t) {
-  const int va = norb - n_alpha, vb = norb - n_beta;
-  int m = (n_alpha > 0 && n_beta > 0) ? ((va + t - 1) / t) * vb : 0;
-  const int others[4] = {va, vb, va * (va - 1) / 2, vb * (vb - 1) / 2};
-  for (int o : others) m = o > m ? o : m;
-  return m < 1 ? 1 : m;
-}
-
 extern "C" int qp_pt2_create(qp_pt2_ctx** out, int norb, int n_alpha, int n_beta, const double* h,
                              const double* eri, const qp_pt2_config* cfg) {
   if (!out) return fail(QP_EINVAL, "out is NULL");
@@ -525,9 +515,11 @@ extern "C" int qp_pt2_create(qp_pt2_ctx** out, int norb, int n_alpha, int n_beta
   x->max_cells = cells_tiled(x->ntile);
   x->smem = sweep_smem(x->max_cells);
   int bps = batch_blocks_per_sm(x->nint, c.precision == QP_MIXED, x->smem);
-  if (c.tile == 0 && x->nint == 2 && bps < 2 && n_alpha > 0 && n_beta > 0 && cells_tiled(2) < x->max_cells) {
+  if (((c.tile == 0 && x->nint == 2 && bps < 2) || (x->ntile == 1 && bps < 1)) && n_alpha > 0 && n_beta > 0 &&
+      cells_tiled(2) < x->max_cells) {
     // the opposite-spin accumulator fits only once per SM: split those
-    // batches in two tiles of rows, so that two CTAs share the SM
+    // batches in two tiles of rows, so that two CTAs share the SM (or, with
+    // tile = 1, not at all: above 14,830 cells)
     x->ntile = 2;
     x->max_cells = cells_tiled(2);
     x->smem = sweep_smem(x->max_cells);
@@ -1952,6 +1944,12 @@ extern "C" int qp_pt2_batch_create_ex(qp_pt2_batch** out, int n, qp_pt2_ctx* con
       b.ntile = (x->nalpha > 0 && x->nbeta > 0) ? std::min(o.tile, std::max(va, 1)) : 1;
       b.max_cells = cells_for_tile(x->norb, x->nalpha, x->nbeta, b.ntile);
       b.smem = sweep_smem(b.max_cells);
+      if (b.ntile == 1 && x->nalpha > 0 && x->nbeta > 0 &&
+          batch_blocks_per_sm(x->nint, x->cfg.precision == QP_MIXED, b.smem) < 1) {  // as qp_pt2_create does
+        b.ntile = 2;
+        b.max_cells = cells_for_tile(x->norb, x->nalpha, x->nbeta, 2);
+        b.smem = sweep_smem(b.max_cells);
+      }
     }
     b.nper = x->nbat + (b.ntile - 1) * x->nalpha * x->nbeta;
     b.ngen = b.ndet;
