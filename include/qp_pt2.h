@@ -392,7 +392,8 @@ int qp_pt2_last_timings(const qp_pt2_ctx *ctx, double *ms);
  * and the call returns once it has finished.  Results equal those of
  * qp_pt2_eval for the same inputs (same rules, same tolerances).
  *
- * Scratch: one 64 MiB device array inside the library (static storage),
+ * Scratch: one 64 MiB device array inside the library (static storage; 256 KB
+ * of tables beside it),
  * which every GPU that loads the library holds until the process exits.  The
  * first call on a device looks up that array's device address
  * (cudaGetSymbolAddress) and caches it; make that first call before any

@@ -75,6 +75,7 @@ constexpr int kMaxDevices = 64;
 
 std::mutex g_mu;
 unsigned char* g_base[kMaxDevices] = {nullptr};
+long long* g_den[kMaxDevices] = {nullptr};
 
 // Failures are reported through the library's error channel, so that
 // qp_pt2_last_error() names them.
@@ -124,6 +125,9 @@ bool on_device(const void* p, int dev) {
 
 // The fixed device array all calls share (see the file header).
 static __device__ __align__(256) unsigned char qp_noalloc_scratch[kScratchBytes];
+// The denominators' fixed-point tables beside it: in the scratch array they
+// would take the room of 1,200 determinants of three electrons in 128 orbitals.
+static __device__ __align__(256) long long qp_noalloc_den[2 * kMaxOrb * kMaxOrb];
 
 #define NTRY(expr)                                                                     \
   do {                                                                                 \
@@ -167,16 +171,20 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   // ---- the static array of this device ----
   if (dev < 0 || dev >= kMaxDevices) return nfail(QP_ENOTSUP, "device index too large");
   unsigned char* base;
+  long long* den_tab;
   {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!g_base[dev]) {
-      void* ptr = nullptr;
-      const cudaError_t e = cudaGetSymbolAddress(&ptr, qp_noalloc_scratch);
-      if (e != cudaSuccess || !ptr)
+      void *ptr = nullptr, *den = nullptr;
+      cudaError_t e = cudaGetSymbolAddress(&den, qp_noalloc_den);
+      if (e == cudaSuccess) e = cudaGetSymbolAddress(&ptr, qp_noalloc_scratch);
+      if (e != cudaSuccess || !ptr || !den)
         return nfail(QP_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
+      g_den[dev] = static_cast<long long*>(den);
       g_base[dev] = static_cast<unsigned char*>(ptr);
     }
     base = g_base[dev];
+    den_tab = g_den[dev];
   }
 
   // ---- sizes and layout ----
@@ -211,7 +219,6 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   unsigned long long *skey2 = nullptr;
   int32_t *hidx = nullptr, *hidx2 = nullptr, *order = nullptr, *rank_of = nullptr, *perm = nullptr, *perm2 = nullptr;
   unsigned char *cub_tmp = nullptr, *cub_tmp2 = nullptr;
-  long long *den_tab = nullptr;
   DevResult *dres = nullptr;
   int *queues = nullptr, *tk_cnt = nullptr, *b_ofs = nullptr;
   uint64_t *tk_key = nullptr, *cand_key = nullptr, *r_words = nullptr, *r_hmask = nullptr;
@@ -232,7 +239,6 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     Carve cv{base};
     d_J = cv.take<double>((size_t)norb * norb);
     d_K = cv.take<double>((size_t)norb * norb);
-    den_tab = cv.take<long long>(2 * (size_t)norb * norb);
     order = cv.take<int32_t>(nd);
     rank_of = cv.take<int32_t>(nd);
     // what starts at zero, cleared in one piece
@@ -271,9 +277,9 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
     cub_tmp2 = c3.take<unsigned char>(tmp2);
     if (!cv.ok || !c1.ok || !c3.ok) return 1;
     const size_t per_slot = wave_slot_bytes(sizeof(GenMeta), norb, n_alpha, n_beta, nbat, nd, 1, nper);
-    // each of the 13 per-slot arrays carved below may start with up to 255
-    // bytes of alignment padding: keep 13 x 256 bytes aside for them
-    const size_t left = kScratchBytes > cv.off + 13 * 256 ? kScratchBytes - cv.off - 13 * 256 : 0;
+    // each of the 12 per-slot arrays carved below may start with up to 255
+    // bytes of alignment padding: keep 12 x 256 bytes aside for them
+    const size_t left = kScratchBytes > cv.off + 12 * 256 ? kScratchBytes - cv.off - 12 * 256 : 0;
     W = (int64_t)(left / per_slot);
     if (W < 1) return 2;
     if (W > ngen) W = ngen;
@@ -296,7 +302,7 @@ extern "C" int qp_pt2_eval_noalloc(int norb, int n_alpha, int n_beta, const doub
   };
   // one CTA per SM keeps the selection buffers small; a few CTAs less where a
   // generator slot would not fit otherwise (with k > 0 the buffer of one or
-  // two CTAs is larger than the ban masks and denominator tables); as many per
+  // two CTAs is larger than the ban masks); as many per
   // SM as fit there where their buffers leave room for as many slots per wave
   // (32 orbitals, 300 determinants, k = 300: 1,210 us with one, 711 with three)
   int grid = nsm, lay = layout(grid);
