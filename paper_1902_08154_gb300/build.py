@@ -17,7 +17,7 @@ SO = os.path.join(OUT, "libqp_pt2.so")
 PEAKS_SO = os.path.join(OUT, "libqp_peaks.so")
 UNITS = ["qp_pt2.cu", "sweep.cu", "sweep_mixed.cu", "sweep_grad.cu", "sweep_states.cu", "sweep_packed.cu",
          "noalloc.cu", "davidson.cu", "order.cu"]
-HEADERS = ["common.cuh", "sweep_impl.cuh"]
+HEADERS = ["common.cuh", "sweep_impl.cuh", "lowest_eigenpair.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
