@@ -2920,6 +2920,12 @@ struct Drawer {
     nxt = entry(S, p);
     draw(S, chunk, take);
   }
+  // No further item is published (the watchdog).
+  template <typename BS>
+  __device__ __forceinline__ void stop(BS& S) {
+    S.nlive = 0;
+    nxt = -1;
+  }
   template <typename BS, typename Fn>
   __device__ __forceinline__ void advance(BS& S, const SweepParams& p, int par, int chunk, Fn&& take) {
     S.item[par ^ 1] = nxt;
@@ -2967,16 +2973,17 @@ __global__ void __launch_bounds__(kThreads, (NINT == 1 && !GRAD) ? 3 : 2) batch_
   if (tid == 0) {
     if (p.timeout_ns) atomicCAS(p.t_start, 0ull, global_ns());
     D.begin<FP>(S, p, p.chunk, take);
+    if (S.item[0] >= 0 && expired()) {
+      S.item[0] = -1;
+      D.stop(S);
+    }
   }
   for (int par = 0;; par ^= 1) {
     __syncthreads();
     const int item = S.item[par];
     if (item < 0) break;
     if (tid == 0) {
-      if (D.nxt >= 0 && expired()) {
-        S.nlive = 0;
-        D.nxt = -1;
-      }
+      if (D.nxt >= 0 && expired()) D.stop(S);
       D.advance(S, p, par, p.chunk, take);
     }
     batch_item<NINT, NT, GRAD, MS, E4, FP>(p, S, item, F, E, eri_n, h_n);
@@ -3022,16 +3029,19 @@ __global__ void __launch_bounds__(kThreads, (NINT == 1) ? 3 : 2) batch_multi_ker
       return true;
     };
     Drawer D;
-    if (tid == 0) D.begin<FP>(S, p, m.chunk, take);
+    if (tid == 0) {
+      D.begin<FP>(S, p, m.chunk, take);
+      if (S.item[0] >= 0 && expired()) {
+        S.item[0] = -1;
+        D.stop(S);
+      }
+    }
     for (int par = 0;; par ^= 1) {
       __syncthreads();
       const int item = S.item[par];
       if (item < 0) break;
       if (tid == 0) {
-        if (D.nxt >= 0 && expired()) {
-          S.nlive = 0;
-          D.nxt = -1;
-        }
+        if (D.nxt >= 0 && expired()) D.stop(S);
         D.advance(S, p, par, m.chunk, take);
       }
       batch_item<NINT, NT, false, false, true, FP>(p, S, item, F, E, numer_eri<NT, true>(p), numer_h<NT>(p));
