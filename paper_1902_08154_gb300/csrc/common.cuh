@@ -1,6 +1,7 @@
 // common.cuh -- device helpers and launch parameters of the sm_103a EN-PT2
 // sweep (Quantum Package 2.0, arXiv:1902.08154).  Internal to the library.
 #pragma once
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -133,6 +134,35 @@ inline int cells_for_tile(int norb, int n_alpha, int n_beta, int t) {
 __host__ __device__ inline size_t sweep_smem(int mc) {
   const size_t m = (size_t)(mc < 1 ? 1 : mc);
   return 8 * m + 4 * ((m + 1) & ~(size_t)1) + 4 * ((m + 31) / 32) + 2 * m;
+}
+
+// Lets kernel K have all the dynamic shared memory that its static part leaves
+// of a block's.  The limit belongs to the process: a size per launch would let
+// one thread's smaller launch lower it between another's call and launch.
+template <auto* K>
+inline cudaError_t allow_smem() {
+  static std::atomic<int> room{0};
+  if (!room) {
+    int dev = 0, all = 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&all, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, K);
+    if (e != cudaSuccess) return e;
+    room = all - (int)a.sharedSizeBytes;
+  }
+  return cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
+}
+// CTAs of kernel K per SM, 0 when one does not fit.
+template <auto* K>
+inline int blocks_per_sm(int threads, size_t smem) {
+  int n = 0;
+  if (allow_smem<K>() != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, K, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
 }
 
 struct GenMeta;

@@ -729,8 +729,8 @@ int build_h(const CtxView& c, int64_t n, const uint64_t* d_dets, DevMem& mem, HM
   // one pass of the pair search: row counts, or the columns (and, all pairs,
   // the elements in any order)
   auto strings = [&](auto nint, auto count, int* cols) -> cudaError_t {
-    auto* k = str_pairs_kernel<decltype(nint)::value, decltype(count)::value>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr auto* k = str_pairs_kernel<decltype(nint)::value, decltype(count)::value>;
+    const cudaError_t e = allow_smem<k>();
     if (e != cudaSuccess) return e;
     k<<<(unsigned)n, kMapThreads, smem, st>>>(n, win, d_dets, SA.sid, SA.ptr, SA.grp, SA.nb_ptr, SA.nb, SB.sid,
                                               SB.ptr, SB.grp, cnt, H->rowptr, cols, err);

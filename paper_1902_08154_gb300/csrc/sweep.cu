@@ -84,13 +84,9 @@ cudaError_t launch_wave_multi(int nint, int mixed, const MultiWave& m, const Mul
     const size_t b = 4 * (size_t)mi.ps[i].mask_w + 8 * (size_t)mi.ps[i].orb_w;
     ps = b > ps ? b : ps;
   }
-  if (nint == 1) {
-    cudaFuncSetAttribute(prep_multi_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps);
-    prep_multi_kernel<1><<<total_slots, kThreads, ps, st>>>(m);
-  } else {
-    cudaFuncSetAttribute(prep_multi_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps);
-    prep_multi_kernel<2><<<total_slots, kThreads, ps, st>>>(m);
-  }
+  const cudaError_t e = nint == 1 ? launch_smem<prep_multi_kernel<1>>(m, total_slots, ps, st)
+                                  : launch_smem<prep_multi_kernel<2>>(m, total_slots, ps, st);
+  if (e != cudaSuccess) return e;
   if (mixed) return launch_wave_multi_mixed(nint, mi, total_slots, grid, smem, st);
   return multi_wave_launch<double>(nint, mi, total_slots, grid, smem, st);
 }
@@ -126,14 +122,7 @@ static size_t prep_smem(const SweepParams& p) { return 4 * (size_t)p.mask_w + 8 
 
 cudaError_t launch_prep(int nint, const SweepParams& p, int slots, cudaStream_t st) {
   const size_t smem = prep_smem(p);
-  if (nint == 1) {
-    cudaFuncSetAttribute(prep_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    prep_kernel<1><<<slots, kThreads, smem, st>>>(p);
-  } else {
-    cudaFuncSetAttribute(prep_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    prep_kernel<2><<<slots, kThreads, smem, st>>>(p);
-  }
-  return cudaGetLastError();
+  return nint == 1 ? launch_smem<prep_kernel<1>>(p, slots, smem, st) : launch_smem<prep_kernel<2>>(p, slots, smem, st);
 }
 
 cudaError_t launch_batch(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
@@ -143,15 +132,7 @@ cudaError_t launch_batch(int nint, const SweepParams& p, int grid, size_t smem, 
 
 int batch_blocks_per_sm(int nint, int mixed, size_t smem) {
   if (mixed) return batch_blocks_per_sm_mixed(nint, smem);
-  int n = 0;
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_kernel<1, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<1, double>, kThreads, smem);
-  } else {
-    cudaFuncSetAttribute(batch_kernel<2, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<2, double>, kThreads, smem);
-  }
-  return n;
+  return nint == 1 ? blocks_per_sm<batch_kernel<1, double>>(kThreads, smem) : blocks_per_sm<batch_kernel<2, double>>(kThreads, smem);
 }
 
 int sweep_threads() { return kThreads; }

@@ -3079,19 +3079,19 @@ __global__ void __launch_bounds__(kThreads) compact_multi_kernel(const SweepPara
 
 // The batch launches of one wave: with den64 the FP64 form's items after the
 // others, from the queue again.
+template <auto* K, typename P>
+static cudaError_t launch_smem(const P& p, int grid, size_t smem, cudaStream_t st) {
+  const cudaError_t e = allow_smem<K>();
+  if (e != cudaSuccess) return e;
+  K<<<grid, kThreads, smem, st>>>(p);
+  return cudaGetLastError();
+}
 template <int NINT, typename NT, bool GRAD, bool MS, bool E4>
 static cudaError_t batch_launch_nint(const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
-  auto go = [&](auto* k) {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<grid, kThreads, smem, st>>>(p);
-  };
-  go(batch_kernel<NINT, NT, GRAD, MS, E4, false>);
-  if (p.den64) {
-    const cudaError_t e = cudaMemsetAsync(p.queue, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    go(batch_kernel<NINT, NT, GRAD, MS, E4, true>);
-  }
-  return cudaGetLastError();
+  cudaError_t e = launch_smem<batch_kernel<NINT, NT, GRAD, MS, E4, false>>(p, grid, smem, st);
+  if (e != cudaSuccess || !p.den64) return e;
+  if ((e = cudaMemsetAsync(p.queue, 0, sizeof(int), st)) != cudaSuccess) return e;
+  return launch_smem<batch_kernel<NINT, NT, GRAD, MS, E4, true>>(p, grid, smem, st);
 }
 template <typename NT, bool GRAD = false, bool MS = false, bool E4 = true>
 static cudaError_t batch_launch(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
@@ -3104,19 +3104,12 @@ static cudaError_t batch_launch(int nint, const SweepParams& p, int grid, size_t
 // launched from sweep.cu only).
 template <int NINT, typename NT>
 static cudaError_t multi_launch_nint(const MultiWaveInline& m, int grid, size_t smem, cudaStream_t st) {
-  auto go = [&](auto* k) {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k<<<grid, kThreads, smem, st>>>(m);
-  };
-  go(batch_multi_kernel<NINT, NT, false>);
+  cudaError_t e = launch_smem<batch_multi_kernel<NINT, NT, false>>(m, grid, smem, st);
   bool den64 = false;
   for (int i = 0; i < m.n; i++) den64 |= m.ps[i].den64 != 0;
-  if (den64) {
-    const cudaError_t e = cudaMemsetAsync(m.queue, 0, sizeof(unsigned long long) * m.n, st);
-    if (e != cudaSuccess) return e;
-    go(batch_multi_kernel<NINT, NT, true>);
-  }
-  return cudaGetLastError();
+  if (e != cudaSuccess || !den64) return e;
+  if ((e = cudaMemsetAsync(m.queue, 0, sizeof(unsigned long long) * m.n, st)) != cudaSuccess) return e;
+  return launch_smem<batch_multi_kernel<NINT, NT, true>>(m, grid, smem, st);
 }
 template <typename NT>
 static cudaError_t multi_wave_launch(int nint, const MultiWaveInline& m, int total_slots, int grid, size_t smem,
@@ -3135,15 +3128,8 @@ static cudaError_t multi_compact_launch(int nint, const SweepParams* ps, int n, 
 
 template <typename NT>
 static int multi_blocks_per_sm(int nint, size_t smem) {
-  int n = 0;
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_multi_kernel<1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_multi_kernel<1, NT>, kThreads, smem);
-  } else {
-    cudaFuncSetAttribute(batch_multi_kernel<2, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_multi_kernel<2, NT>, kThreads, smem);
-  }
-  return n;
+  return nint == 1 ? blocks_per_sm<batch_multi_kernel<1, NT>>(kThreads, smem)
+                   : blocks_per_sm<batch_multi_kernel<2, NT>>(kThreads, smem);
 }
 
 // Per generator: wH * dH_II + sum_{s,x} wF[s][x] * dF^I_s(x), with

@@ -20,15 +20,7 @@ cudaError_t launch_compact_multi_mixed(int nint, const SweepParams* ps, int n, i
 int batch_multi_blocks_per_sm_mixed(int nint, size_t smem) { return multi_blocks_per_sm<float>(nint, smem); }
 
 int batch_blocks_per_sm_mixed(int nint, size_t smem) {
-  int n = 0;
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_kernel<1, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<1, float>, kThreads, smem);
-  } else {
-    cudaFuncSetAttribute(batch_kernel<2, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<2, float>, kThreads, smem);
-  }
-  return n;
+  return nint == 1 ? blocks_per_sm<batch_kernel<1, float>>(kThreads, smem) : blocks_per_sm<batch_kernel<2, float>>(kThreads, smem);
 }
 
 }  // namespace qp

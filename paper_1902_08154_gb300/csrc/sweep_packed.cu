@@ -11,17 +11,8 @@ cudaError_t launch_batch_packed(int nint, const SweepParams& p, int grid, size_t
 }
 
 int batch_blocks_per_sm_packed(int nint, size_t smem) {
-  int n = 0;
-  if (nint == 1) {
-    cudaFuncSetAttribute(batch_kernel<1, double, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<1, double, false, false, false>, kThreads, smem);
-  } else {
-    cudaFuncSetAttribute(batch_kernel<2, double, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<2, double, false, false, false>, kThreads, smem);
-  }
-  return n;
+  return nint == 1 ? blocks_per_sm<batch_kernel<1, double, false, false, false>>(kThreads, smem)
+                   : blocks_per_sm<batch_kernel<2, double, false, false, false>>(kThreads, smem);
 }
 
 }  // namespace qp

@@ -16,24 +16,8 @@ size_t states_smem(int max_cells, int nst) {
 }
 
 int batch_blocks_per_sm_states(int nint, size_t smem) {
-  int n = 0;
-  cudaError_t e;
-  if (nint == 1) {
-    e = cudaFuncSetAttribute(batch_kernel<1, double, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<1, double, false, true>, kThreads, smem);
-  } else {
-    e = cudaFuncSetAttribute(batch_kernel<2, double, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<2, double, false, true>, kThreads, smem);
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return n;
+  return nint == 1 ? blocks_per_sm<batch_kernel<1, double, false, true>>(kThreads, smem)
+                   : blocks_per_sm<batch_kernel<2, double, false, true>>(kThreads, smem);
 }
 
 cudaError_t launch_batch_states(int nint, const SweepParams& p, int grid, size_t smem, cudaStream_t st) {
