@@ -272,16 +272,21 @@ __device__ __forceinline__ int spin_degree(const uint64_t* I, const uint64_t* J,
   return d >> 1;
 }
 
-// One block per row I: the connected J marked in a bit map of the
-// determinants (shared memory; `win` of them at a time), COUNT: their number;
-// otherwise the columns read off the map in ascending order, so that nothing
-// is sorted.  Spin-up neighbour strings with few determinants take a thread
+// One block per row I.  COUNT: the number of connected J; otherwise they are
+// marked in a bit map of the determinants (shared memory; `win` of them at a
+// time) and the columns read off it in ascending order, so that nothing is
+// sorted.  A row with so few that the map's words would cost more than
+// comparing them with each other is ranked by counting instead (10^6
+// determinants without connections to speak of: 138 ms with the map for every
+// row and in both passes, 22.9 for a warp per row and the sort, 12.7 so).
+// Spin-up neighbour strings with few determinants take a thread
 // each, the others a warp.  (A warp per row that evaluated each element as it
 // found it and drew its slot from a global counter, and a segmented sort of
 // the pairs, took 2.9 ms for 10^4 determinants, 6.2e6 elements; the two passes
 // of this kernel and the values take 0.65.)
 constexpr int kMapThreads = 256;
 constexpr int kMapQueue = 512;
+constexpr int kFew = 512;  // columns ranked by counting at most
 constexpr int64_t kMapMax = 1 << 20;  // determinants per window: 128 KB of map
 
 template <int NINT, bool COUNT>
@@ -292,19 +297,33 @@ __global__ void __launch_bounds__(kMapThreads) str_pairs_kernel(
     const int64_t* rowptr, int* cols, int* err) {
   constexpr int NW = 2 * NINT;
   extern __shared__ uint32_t map[];
-  __shared__ int queue[kMapQueue], nq, wsum[kMapThreads / 32];
+  __shared__ int queue[kMapQueue], nq, wsum[kMapThreads / 32], hit[COUNT ? 1 : kFew], nhit;
   const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint64_t I[NW];
 #pragma unroll
   for (int w = 0; w < NW; w++) I[w] = dets[(size_t)row * NW + w];
   const int a = aid[row], b = bid[row];
+  const int64_t q0 = COUNT ? 0 : rowptr[row], len = COUNT ? 0 : rowptr[row + 1] - q0;
+  if (!COUNT && len == 0) return;
+  // comparisons against three passes over the map's words
+  const bool few = !COUNT && len <= kFew && len * ((len + kMapThreads - 1) / kMapThreads * kMapThreads) <= 3 * (n / 32);
+  int found = 0;  // COUNT: by this thread
   int64_t done = 0;
-  for (int64_t lo = 0; lo < n; lo += win) {
-    const int nbits = (int)(n - lo < win ? n - lo : win), nwords = (nbits + 31) / 32;
+  for (int64_t lo = 0; lo < n; lo += COUNT || few ? n : win) {
+    const int nbits = (int)(n - lo < win ? n - lo : win), nwords = COUNT || few ? 0 : (nbits + 31) / 32;
     for (int w = tid; w < nwords; w += kMapThreads) map[w] = 0u;
-    if (tid == 0) nq = 0;
+    if (tid == 0) nq = nhit = 0;
     __syncthreads();
     auto mark = [&](int j) {
+      if (COUNT) {
+        found++;
+        return;
+      }
+      if (few) {
+        const int at = atomicAdd(&nhit, 1);
+        if (at < kFew) hit[COUNT ? 0 : at] = j;
+        return;
+      }
       const int64_t at = j - lo;
       if (at >= 0 && at < nbits) atomicOr(&map[at >> 5], 1u << (at & 31));
     };
@@ -341,6 +360,17 @@ __global__ void __launch_bounds__(kMapThreads) str_pairs_kernel(
     for (int q = warp; q < nbig; q += kMapThreads / 32)
       for (int k = aptr[queue[q]] + lane, e = aptr[queue[q] + 1]; k < e; k += 32) pair(k);
     __syncthreads();
+    if (few) {
+      for (int i = tid; i < (int)len; i += kMapThreads) {
+        const int j = hit[COUNT ? 0 : i];
+        int before = 0;
+#pragma unroll 4
+        for (int k = 0; k < (int)len; k++) before += hit[COUNT ? 0 : k] < j;
+        cols[q0 + before] = j;
+      }
+      return;
+    }
+    if (COUNT) break;
     // a contiguous run of words per thread, of odd length: 32 banks
     const int per = ((nwords + kMapThreads - 1) / kMapThreads) | 1, w0 = min(tid * per, nwords), w1 = min(w0 + per, nwords);
     int c = 0;
@@ -359,15 +389,22 @@ __global__ void __launch_bounds__(kMapThreads) str_pairs_kernel(
       before += w < warp ? wsum[w] : 0;
       all += wsum[w];
     }
-    if (!COUNT) {
-      int* out = cols + rowptr[row] + done + before + at - c;
-      for (int w = w0; w < w1; w++)
-        for (uint32_t m = map[w]; m; m &= m - 1) *out++ = (int)(lo + 32 * w + __ffs((int)m) - 1);
-    }
+    int* out = cols + q0 + done + before + at - c;
+    for (int w = w0; w < w1; w++)
+      for (uint32_t m = map[w]; m; m &= m - 1) *out++ = (int)(lo + 32 * w + __ffs((int)m) - 1);
     done += all;
     __syncthreads();
   }
-  if (COUNT && tid == 0) rowcnt[row] = done;
+  if (COUNT) {
+    found = __reduce_add_sync(0xffffffffu, found);
+    if (lane == 0) wsum[warp] = found;
+    __syncthreads();
+    if (tid == 0) {
+      int64_t all = 0;
+      for (int w = 0; w < kMapThreads / 32; w++) all += wsum[w];
+      rowcnt[row] = all;
+    }
+  }
 }
 
 // The elements of the columns found: a block per row, a thread per element;
@@ -729,10 +766,11 @@ int build_h(const CtxView& c, int64_t n, const uint64_t* d_dets, DevMem& mem, HM
   // one pass of the pair search: row counts, or the columns (and, all pairs,
   // the elements in any order)
   auto strings = [&](auto nint, auto count, int* cols) -> cudaError_t {
-    constexpr auto* k = str_pairs_kernel<decltype(nint)::value, decltype(count)::value>;
+    constexpr bool kCount = decltype(count)::value;
+    constexpr auto* k = str_pairs_kernel<decltype(nint)::value, kCount>;
     const cudaError_t e = allow_smem<k>();
     if (e != cudaSuccess) return e;
-    k<<<(unsigned)n, kMapThreads, smem, st>>>(n, win, d_dets, SA.sid, SA.ptr, SA.grp, SA.nb_ptr, SA.nb, SB.sid,
+    k<<<(unsigned)n, kMapThreads, kCount ? 0 : smem, st>>>(n, win, d_dets, SA.sid, SA.ptr, SA.grp, SA.nb_ptr, SA.nb, SB.sid,
                                               SB.ptr, SB.grp, cnt, H->rowptr, cols, err);
     return cudaGetLastError();
   };
