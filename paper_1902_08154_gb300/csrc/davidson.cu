@@ -283,7 +283,7 @@ __device__ __forceinline__ int spin_degree(const uint64_t* I, const uint64_t* J,
 // each, the others a warp.  (A warp per row that evaluated each element as it
 // found it and drew its slot from a global counter, and a segmented sort of
 // the pairs, took 2.9 ms for 10^4 determinants, 6.2e6 elements; the two passes
-// of this kernel and the values take 0.65.)
+// of this kernel and the values take 0.58.)
 constexpr int kMapThreads = 256;
 constexpr int kMapQueue = 512;
 constexpr int kFew = 512;  // columns ranked by counting at most

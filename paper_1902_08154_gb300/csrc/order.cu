@@ -3,16 +3,22 @@
 // n^2 comparisons in one launch beat the radix sorts of 64-bit keys (8 passes
 // each, two for the generators, one per key word and |e| for the selection)
 // up to some 10^4 elements: 50 determinants and 100 candidates take 5 + 4 us
-// instead of five single-tile sorts of 14.5 us and their 7 helper kernels;
-// 10^4 determinants 40 us instead of two sorts of about 45 us.
+// instead of five single-tile sorts of 14.5 us and their 7 helper kernels.
 #include <cuda_runtime.h>
 
 #include "common.cuh"
 
 namespace qp {
 
-// Above these sizes the radix sorts are faster (measured on both sides).
+// A call that sweeps one generator, counting against sorting: 4,096
+// determinants 183 against 340 us, 10^4 386 against 439 (count_rank_kernel 168
+// of it), 12,288 443 against 458, 16,384 606 against 485; two words per spin
+// 12,288 531 against 549, 16,384 677 against 559.
 constexpr int64_t kCountRankMax = 12288;
+// A sweep of 60 determinants, 40 orbitals: 1,000 candidates 486 against 598 us,
+// 4,000 601 against 949, 8,000 803 against 1,080 (two words 1,024 against
+// 1,510).  Counting was still ahead with 20,000 (1,747 against 1,830), where
+// its n^2 is near the sorts' cost; the line keeps a margin.
 constexpr int kCountSelectMax = 8192;
 
 int64_t count_rank_max() { return kCountRankMax; }

@@ -33,8 +33,9 @@
 //            cells are a thread's; J reaching every cell go through pair
 //            tables in the cells pass;
 //    cells:  every cell left is a perturber of I: e = A^2/(E0 - H_aa) with
-//            H_aa from per-batch row and column sums in fixed point, added to
-//            eps_I and offered to the CTA's selection buffer.
+//            H_aa from per-batch row and column sums in fixed point (FP64 where
+//            its unit is too coarse), added to eps_I and offered to the CTA's
+//            selection buffer.
 // Matrix elements follow the Slater-Condon rules (Eqs. Hij) with phases from
 // a masked popcount of J's spin string.
 //
@@ -42,7 +43,8 @@
 // integrals it gathers and of the products c_J <J|H|alpha>.  NT = double is
 // the plain FP64 sweep; NT = float gathers FP32 integrals and forms FP32
 // products, while each product is still added into the exact accumulator
-// A(R) and the denominators, e_alpha and every reduction are those of FP64.
+// A(R), and the denominators, e_alpha and every reduction are those of the
+// FP64 sweep.
 // sweep.cu instantiates the FP64 kernels, sweep_mixed.cu the mixed ones.
 #pragma once
 #include <cfloat>
@@ -149,7 +151,9 @@ __device__ __forceinline__ const float* numer_h<float>(const SweepParams& p) { r
 // than in FP64, with one of 10^6 2^19 and 8,000 times.
 // Two states at once, 2,000 determinants, 64 orbitals: 43 to 33.8 ms (two
 // quotients per cell); one state, 10^4 determinants 113.3 to 111.8 ms; 10^3
-// determinants, 128 orbitals 87.1 to 84.1 ms.
+// determinants, 128 orbitals 87.1 to 84.1 ms.  The FP64 form of the present
+// kernels (all generators of 10^4 determinants, 64 orbitals, one h_pp of 10^6):
+// 95.0 ms against 73.4, two states 44.1 against 23.6.
 // ---------------------------------------------------------------------------
 constexpr int kDenFp64 = 1 << 20;  // in the place of S: energies as the bits of FP64 numbers
 __device__ __forceinline__ int den_scale(const SweepParams& p) {
@@ -455,9 +459,13 @@ struct Batch {
 // Work items of a large wave are taken by kind, same-spin and one-hole ones
 // first, so that the code of one kind at a time is in the instruction caches
 // (10^4 determinants, 64 orbitals 78.5 -> 73.9 ms with a cells pass per kind,
-// 79.0 without the order; opposite-spin first 74.4).  Smaller waves are taken
-// as they come: 9,900 items 415 us, by kind 425; 50,400 items of 240
-// generators 10.35 ms, by kind 10.4 to 10.9; 184,000 items 5.28, by kind 5.00.
+// 79.0 without the order; opposite-spin first 74.4).  By kind against as they
+// come: 67,200 items 2.88 against 3.05 ms, 84,000 items of 400 generators of a
+// space of 10^4 12.2 against 12.9, 184,000 4.90 against 5.27.  Below the line
+// it depends on the items: 50,400 2.23 against 2.35 ms (64 orbitals) and 22,950
+// 0.83 against 0.87, but 25,200 items of 120 heavy generators 9.1 against 8.1
+// and 9,900 425 against 415 us; so the line lies above all sizes at which the
+// order was seen to lose.  The last wave of a large sweep may fall below it.
 // (Not where the back of the list is the FP64 form's, den64.)
 constexpr long long kItemsByKind = 65536;
 __device__ __forceinline__ bool by_kind(const SweepParams& p) {
@@ -1227,50 +1235,6 @@ __device__ __forceinline__ bool row_live(const Batch& B, const BatchShared<NINT,
   return live;
 }
 
-// Cells touching the particles of J (two-hole batch, t = 1): visited by the
-// 32 lanes of a warp, each cell once.  Rows and columns banned as a whole are
-// skipped (a cell they share with another row is banned too).  fn(c, pc, zc)
-// gets the cell index, the spin-orbital code of the particle of J whose row
-// it is and the code of the cell's other orbital.
-template <int NINT, typename NT, typename Fn>
-__device__ __forceinline__ void for_row_cells(const Batch& B, const BatchShared<NINT, NT>& S, int norb,
-                                              uint64_t part, int lane, Fn&& fn) {
-  if (B.kind == 1) {
-    int np;
-    const uint32_t P = particles_of_spin(part, norb, B.sa, &np);
-    const int nv = S.nv[B.sa];
-    for (int i = 0; i < np; i++) {
-      const int x = S.vidx[B.sa][pk(P, i)];
-      if (row_banned<NINT, NT>(S, B.sa, pk(P, i))) continue;
-      for (int y = lane; y < nv; y += 32) {
-        if (y == x) continue;
-        bool dup = false;  // pair {P[j], P[i]}, j < i, was visited from P[j]
-        for (int j = 0; j < i; j++) dup |= (S.vidx[B.sa][pk(P, j)] == y);
-        if (!dup) fn(pair_cell(x, y), B.sa * norb + pk(P, i), B.sa * norb + S.vir[B.sa][y]);
-      }
-    }
-  } else {  // kind 2
-    int na, nb;
-    const uint32_t Pa = particles_of_spin(part, norb, 0, &na);
-    const uint32_t Pb = particles_of_spin(part, norb, 1, &nb);
-    const int nv0 = S.nv[0], nv1 = S.nv[1];
-    for (int i = 0; i < na; i++) {
-      const int x = S.vidx[0][pk(Pa, i)];
-      if (row_banned<NINT, NT>(S, 0, pk(Pa, i))) continue;
-      for (int y = lane; y < nv1; y += 32) fn(x * nv1 + y, pk(Pa, i), norb + S.vir[1][y]);
-    }
-    for (int j = 0; j < nb; j++) {
-      const int y = S.vidx[1][pk(Pb, j)];
-      if (row_banned<NINT, NT>(S, 1, pk(Pb, j))) continue;
-      for (int x = lane; x < nv0; x += 32) {
-        bool dup = false;  // rows of Pa were visited above
-        for (int i = 0; i < na; i++) dup |= (S.vidx[0][pk(Pa, i)] == x);
-        if (!dup) fn(x * nv1 + y, norb + pk(Pb, j), S.vir[0][x]);
-      }
-    }
-  }
-}
-
 // X = (particles of J) + (holes of H that J keeps); T = holes of J not in H.
 // Both sets are spin-orbital codes, packed (see pk).
 template <int NINT, typename NT>
@@ -1372,8 +1336,8 @@ __device__ __forceinline__ NT warp_sum_nt(NT v) {
 }
 
 // Gradient of one matrix element: adds w * d<J|H|alpha>/d(theta) into dh
-// (symmetric halves) and the packed integrals, with the same case analysis
-// as element().
+// (symmetric halves) and the packed integrals, by the cases of the
+// excitation degree.
 template <int NINT>
 __device__ __noinline__ void element_grad(double* g_dh, double* g_deri, int norb, const uint64_t* Jw, uint32_t X,
                                           int nx, uint32_t T, int nt, int r, int s, double w) {
@@ -1647,20 +1611,6 @@ __device__ __forceinline__ ItemEnv item_env(const SweepParams& p) {
   return E;
 }
 
-// One work item of the sweep of p (a generator slot's hole-set batch, or a
-// row tile of one): bans, the accumulation of A_alpha, the cells pass and the
-// item's sums.  Used by the kernel of one sweep and by the kernel whose queue
-// spans the waves of several instances.
-//
-// What bounds an item is latency, not a pipe (issue slots half used, FP64
-// 23%): 256 threads share about 2,000 cells, and every phase that few of them
-// work in, every dependent global load and every barrier shows.  So the
-// set-up reads the generator straight from global memory in two dependent
-// steps, the first round of bucket entries is in registers before the bans
-// are, tables of the J reaching every cell are units of the row pass, their
-// terms are formed in the cells pass, and the item's sums are finished by the
-// last warp to arrive while the others begin the next item: five barriers
-// where there were fifteen.
 // This CTA's candidate buffers of the selection.
 __device__ __forceinline__ double* buf_e(const SweepParams& p) { return p.tk_e + (size_t)blockIdx.x * (size_t)p.cap; }
 __device__ __forceinline__ double* buf_a(const SweepParams& p) { return p.tk_a + (size_t)blockIdx.x * (size_t)p.cap; }
@@ -1669,6 +1619,21 @@ __device__ __forceinline__ uint64_t* buf_key(const SweepParams& p) {
   return p.tk_key + (size_t)blockIdx.x * (size_t)p.cap * (2 * NINT);
 }
 
+// One work item of the sweep of p (a generator slot's hole-set batch, or a
+// row tile of one): bans, the accumulation of A_alpha, the cells pass and the
+// item's sums.  Used by the kernel of one sweep and by the kernel whose queue
+// spans the waves of several instances.  FP: its generator's denominators are
+// in FP64.
+//
+// What bounds an item is latency, not a pipe (issue slots half used, FP64
+// 26%): 256 threads share about 2,000 cells, and every phase that few of them
+// work in, every dependent global load and every barrier shows.  So the
+// set-up reads the generator straight from global memory in two dependent
+// steps, the first round of bucket entries is in registers before the bans
+// are, tables of the J reaching every cell are units of the row pass, their
+// terms are formed in the cells pass, and the item's sums are finished by the
+// last warp to arrive while the others wait at the next item's first barrier:
+// five barriers where there were fifteen.
 template <int NINT, typename NT, bool GRAD, bool MS, bool E4, bool FP>
 __device__ __forceinline__ void batch_item(const SweepParams& p, BatchShared<NINT, NT>& S, const long long item,
                                            const int F, const ItemEnv& E,

@@ -1,5 +1,6 @@
 // sweep_mixed.cu -- the mixed-precision batch kernels (FP32 integral gathers and
-// products, FP64 accumulation, denominators and reductions); see sweep_impl.cuh.
+// products; exact accumulation, denominators and reductions as in the FP64
+// sweep); see sweep_impl.cuh.
 #include "sweep_impl.cuh"
 
 namespace qp {
