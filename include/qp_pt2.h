@@ -69,6 +69,15 @@
  * rank order: the same inputs give the same bits on every run, every grid
  * size and every work-queue order.
  *
+ * Denominators: D = E0 - H_aa is formed in 64-bit integers of one unit per call
+ * (2^-62 of a power of two at most |E0| + n max|h| + n (n - 1) max|(pq|rs)|,
+ * n = n_el + 2) and A/D by integer arithmetic, correctly rounded to within a
+ * hundredth of an ulp.  Generators whose energies that unit is too coarse for
+ * (above 2^-55 of |E0| and of the sums that make up H_II; integrals of very
+ * wide range, as a level-shifted orbital gives) have D and A/D in FP64 instead,
+ * so that no D is further off than its plain FP64 sum.  Integrals that are not
+ * finite give FP64's results too.
+ *
  * Errors: every entry point returns QP_OK (0) or a negative code; no call
  * aborts, traps or throws.  qp_pt2_strerror() names a code;
  * qp_pt2_last_error() gives the message of the last failing call of this
@@ -94,12 +103,13 @@ extern "C" {
 #define QP_ENOTSUP (-8)    /* configuration not supported by the library */
 #define QP_ENOTCONV (-9)  /* Davidson stopped above its residual tolerance */
 
-#define QP_FP64 0          /* every step in FP64 */
+#define QP_FP64 0          /* numerators in FP64, summed exactly; denominators in
+                              64-bit fixed point or FP64 (below); reductions in FP64 */
 #define QP_MIXED 1         /* numerator <J|H|alpha> gathers and products c_J<J|H|alpha> in
                               FP32 (FP32 copies of h and eri); the products are summed
                               exactly into A_alpha (as in QP_FP64, below) and A_alpha is
                               rounded once to FP64; denominators E0 - H_aa, e_alpha and
-                              every reduction in FP64.  Error bound per result: about
+                              every reduction as in QP_FP64.  Error bound per result: about
                               2^-24 * sum_alpha 2|A_alpha| sum_J |c_J H_Jalpha| / |D_alpha|. */
 
 typedef struct qp_pt2_ctx qp_pt2_ctx; /* opaque, library-owned */
